@@ -150,7 +150,8 @@ def _pack(w, arch, F):
     return blob
 
 
-def _models(case, gen):
+def _weights(case, gen):
+    """Weight tensors of target and draft (None: the draft is the target's first layers)."""
     F = FAMILIES[case["family"]]
     ta, da = tsfm.tsfm_arch(*F["target"]), tsfm.tsfm_arch(*F["draft"])
     tracking = case["op"] == "spec" and F["dtype"] == "bf16"
@@ -161,7 +162,7 @@ def _models(case, gen):
         damp = lambda l: POINT_CORRECTION if F["P_in"] else CORRECTION  # noqa: E731
     t = _model(ta, F, gen, damp)
     if F["mode"] == "layer_skip":
-        return ta, da, _pack(t, ta, F), None
+        return t, None
     if F["mode"] == "perturbed":
         d = {k: v if v.dim() == 1 else v + PERTURBATION * v.std() * torch.randn(v.shape, device="cuda", generator=gen)
              for k, v in t.items()}
@@ -170,7 +171,14 @@ def _models(case, gen):
         if tracking:
             for w in (t, d):
                 _persistence(w[-1, "W_emb"], w[-1, "W_head"], F["P"], gen)
-    return ta, da, _pack(t, ta, F), _pack(d, da, F)
+    return t, d
+
+
+def _models(case, gen):
+    F = FAMILIES[case["family"]]
+    ta, da = tsfm.tsfm_arch(*F["target"]), tsfm.tsfm_arch(*F["draft"])
+    t, d = _weights(case, gen)
+    return ta, da, _pack(t, ta, F), None if d is None else _pack(d, da, F)
 
 
 def _series(B, n, gen):
@@ -238,6 +246,74 @@ def run(st):
         f = tsfm.tsfm_spec_forecast_host if c["host"] else tsfm.tsfm_spec_forecast
         f(st.handle, st.x, c["B"], n, c["H"], c["K"], st.F["tau"], st.seed, st.out, stats)
     return st.out
+
+
+# ------------------------------------------------------------------------------------------ the same in 64 bits
+def _rotate(t, cos, sin):
+    a, b = t.chunk(2, -1)
+    return torch.cat([a * cos - b * sin, b * cos + a * sin], -1)
+
+
+def _norm(x, g):
+    return g * x * torch.rsqrt((x * x).mean(-1, keepdim=True) + 1e-6)
+
+
+class _Plain:
+    """Pre-norm decoder with rotary positions and a key/value cache, plain torch in 64 bits."""
+
+    def __init__(self, w, arch, B, cap):
+        self.w, (self.L, d, self.heads, _) = w, arch
+        self.dh, self.pos = d // self.heads, 0
+        angle = torch.arange(cap, device="cuda", dtype=torch.float64)[:, None] * 1e4 ** (
+            -2.0 * torch.arange(self.dh // 2, device="cuda", dtype=torch.float64) / self.dh)
+        self.cos, self.sin = angle.cos(), angle.sin()
+        self.kv = torch.empty(self.L, 2, B, self.heads, cap, self.dh, device="cuda", dtype=torch.float64)
+
+    def __call__(self, z):
+        """z [B, n, values per token] behind what was given before -> next-patch means [B, n, P]."""
+        w, (B, n, _), p = self.w, z.shape, self.pos
+        split = lambda t: t.view(B, n, self.heads, self.dh).transpose(1, 2)  # noqa: E731
+        cos, sin = self.cos[p:p + n], self.sin[p:p + n]
+        mask = torch.ones(n, p + n, device="cuda", dtype=torch.bool).tril(p)
+        x = z @ w[-1, "W_emb"].T
+        for l in range(self.L):
+            a = _norm(x, w[l, "g1"])
+            K, V = self.kv[l, 0, :, :, :p + n], self.kv[l, 1, :, :, :p + n]
+            K[:, :, p:] = _rotate(split(a @ w[l, "Wk"].T), cos, sin)
+            V[:, :, p:] = split(a @ w[l, "Wv"].T)
+            s = _rotate(split(a @ w[l, "Wq"].T), cos, sin) @ K.transpose(2, 3) / math.sqrt(self.dh)
+            s = s.masked_fill(~mask, -math.inf).softmax(-1)
+            x = x + (s @ V).transpose(1, 2).reshape(B, n, -1) @ w[l, "Wo"].T
+            h = torch.nn.functional.gelu(_norm(x, w[l, "g2"]) @ w[l, "W1"].T)
+            x = x + h @ w[l, "W2"].T
+        self.pos = p + n
+        return _norm(x, w[-1, "g_f"]) @ w[-1, "W_head"].T
+
+
+@torch.no_grad()
+def exact(case, seed):
+    """Scoring and plain forecasts.  A speculative forecast has none: a decision that falls within rounding of its
+    threshold has two valid outcomes."""
+    if case["op"] == "spec":
+        return None
+    F = FAMILIES[case["family"]]
+    gen = torch.Generator(device="cuda").manual_seed(seed)
+    w, _ = _weights(case, gen)
+    w = {k: (v.to(torch.bfloat16) if F["dtype"] == "bf16" and v.dim() == 2 else v).double() for k, v in w.items()}
+    B, P = case["B"], F["P"]
+    P_in = F["P_in"] or P
+    s = _series(B, case["ctx"] * P, gen).double()
+    T = -(-case["H"] // P)
+    model = _Plain(w, F["target"], B, (case["ctx"] + T) * P // P_in)
+    if case["op"] == "forward":
+        return model(s.view(B, -1, P_in))
+    mean, sd = s.mean(1, keepdim=True), (s.var(1, keepdim=True, unbiased=False) + 1e-5).sqrt()
+    z, patches = (s - mean) / sd, []
+    for _ in range(T):
+        z = model(z.view(B, -1, P_in))[:, -1]
+        patches.append(z)
+    out = (torch.cat(patches, 1) * sd + mean)[:, :case["H"]].contiguous()
+    return out.cpu().numpy() if case["host"] else out
 
 
 # ------------------------------------------------------------------------------------------ what a pass needs at least

@@ -23,6 +23,7 @@
 #include "gemm_tc.cuh"
 #include "gemm_sk.cuh"
 #include "gemm_ws.cuh"
+#include "gemm_f32.cuh"
 
 using namespace tsfm;
 
@@ -370,6 +371,8 @@ void prefer_max_smem_all() {
   prefer_max_smem(gemm_sk_kernel<2, false>);
   prefer_max_smem(gemm_ws_kernel<false>);
   prefer_max_smem(gemm_ws_kernel<true>);
+  prefer_max_smem(gemm_f32_kernel<16, 16>);
+  prefer_max_smem(gemm_f32_kernel<32, 32>);
   prefer_max_smem(attn_flash_kernel<32, 3>);
   prefer_max_smem(attn_flash_kernel<32, kFlashStShort>);
   prefer_max_smem(attn_flash_kernel<64, 3>);
@@ -437,10 +440,12 @@ void launch_gemm_simt(cudaStream_t s, bool pdl, const T *A, const T *W, void *C,
   }
 }
 
-// C (op)= A . W^T through the tensor-core kernel when a plan exists, else the FMA kernel.
+// C (op)= A . W^T through the tensor-core kernel when a plan exists, else an FMA kernel.  row_gain (fp32
+// models whose rows gemm_f32_kernel takes): A is the residual stream, normalised by the contraction itself.
 template <typename T>
 void gemm(tsfm_spec *h, GemmSkPlan *plan, const void *A, const void *W, void *C, int M, int N,
-          int K, int epi, const SkNorm *norm = nullptr, LiveRows lr = LiveRows{nullptr, 0}) {
+          int K, int epi, const SkNorm *norm = nullptr, LiveRows lr = LiveRows{nullptr, 0},
+          const float *row_gain = nullptr, float eps = 0.f) {
   const double e = sizeof(T);
   const double out_b = (epi == EPI_F32 || epi == EPI_ATOMIC) ? 4.0 : epi == EPI_RESID ? 8.0 : e;
   const double bytes = ((double)N * K + (double)M * K) * e + (double)M * N * out_b;
@@ -469,6 +474,17 @@ void gemm(tsfm_spec *h, GemmSkPlan *plan, const void *A, const void *W, void *C,
     return;
   }
   KTimer kt(h, KC_GEMM_SIMT, bytes, flops);
+  if constexpr (sizeof(T) == 4) {
+    if (gemm_f32_eligible(W, K)) {
+      if (gemm_f32_launch(h->ls, h->pdl, (const float *)A, (const float *)W, (float *)C, M, N, K, epi, row_gain, eps, lr)) {
+        LAUNCHED();
+      } else if (h->enqueue_err == TSFM_OK) {
+        h->enqueue_err = TSFM_ERR_CUDA;
+        g_cuda_err = std::string("fp32 contraction could not be launched: ") + cudaGetErrorString(cudaGetLastError());
+      }
+      return;
+    }
+  }
   launch_gemm_simt<T>(h->ls, h->pdl, (const T *)A, (const T *)W, C, M, N, K, epi);
 }
 
@@ -553,6 +569,8 @@ void run_pass(tsfm_spec *h, ModelDev &m, int B, const PassGeom &g, int head_mode
   // epilogue work.  With the large tiles' TMA epilogues a producer would have to load its block of x
   // back after the reduction: measured on C2-C4, that costs what the RMSNorm kernel costs.)
   const bool fold = sizeof(T) == 2 && h->use_tc && m.layers[0].tc_qkv.valid && M <= 512;
+  // fp32 models with rows short enough normalise them inside the contraction that reads them.
+  const bool fold32 = sizeof(T) == 4 && gemm_f32_eligible(m.layers[0].Wqkv, d);
   const int L = m.arch.n_layers;
   const LiveRows lr{g.n_live, g.q_len};
   // the RMSNorm of passes of a few thousand rows is a link in a chain: constants before the wait
@@ -575,11 +593,12 @@ void run_pass(tsfm_spec *h, ModelDev &m, int B, const PassGeom &g, int head_mode
   consume.eps = eps;
   for (int l = 0; l < L; ++l) {
     LayerDev &ly = m.layers[l];
-    if (!fold) {
+    if (!fold && !fold32) {
       KTimer kt(h, KC_RMSNORM, norm_bytes, 3.0 * M * d);
       launch_ex(s, h->pdl, norm_kernel, dim3((M + 7) / 8), dim3(256), 0, h->x, ly.g1, M, d, eps, (T *)h->a, lr);
     }
-    gemm<T>(h, &ly.tc_qkv, h->a, ly.Wqkv, h->qkv, M, 3 * d, d, EPI_F32, fold ? &consume : nullptr, lr);
+    gemm<T>(h, &ly.tc_qkv, fold32 ? (const void *)h->x : h->a, ly.Wqkv, h->qkv, M, 3 * d, d, EPI_F32,
+            fold ? &consume : nullptr, lr, fold32 ? ly.g1 : nullptr, eps);
     if (m.dh == 32) launch_attn<T, 32>(h, m, l, B, g);
     else if (m.dh == 64) launch_attn<T, 64>(h, m, l, B, g);
     else launch_attn<T, 128>(h, m, l, B, g);
@@ -589,11 +608,12 @@ void run_pass(tsfm_spec *h, ModelDev &m, int B, const PassGeom &g, int head_mode
     produce.a_out = (bf16 *)h->a;
     produce.gain = ly.g2;
     gemm<T>(h, &ly.tc_o, h->ao, ly.Wo, h->x, M, d, d, EPI_RESID, fold ? &produce : nullptr, lr);
-    if (!fold) {
+    if (!fold && !fold32) {
       KTimer kt(h, KC_RMSNORM, norm_bytes, 3.0 * M * d);
       launch_ex(s, h->pdl, norm_kernel, dim3((M + 7) / 8), dim3(256), 0, h->x, ly.g2, M, d, eps, (T *)h->a, lr);
     }
-    gemm<T>(h, &ly.tc_1, h->a, ly.W1, h->hbuf, M, f, d, EPI_GELU_T, fold ? &consume : nullptr, lr);
+    gemm<T>(h, &ly.tc_1, fold32 ? (const void *)h->x : h->a, ly.W1, h->hbuf, M, f, d, EPI_GELU_T,
+            fold ? &consume : nullptr, lr, fold32 ? ly.g2 : nullptr, eps);
     produce.gain = l + 1 < L ? m.layers[l + 1].g1 : nullptr;
     if (l + 1 == L) produce.a_out = nullptr, produce.ssq_out = nullptr;   // the head kernel norms the final rows itself
     gemm<T>(h, &ly.tc_2, h->hbuf, ly.W2, h->x, M, d, f, EPI_RESID, fold && l + 1 < L ? &produce : nullptr, lr);
@@ -1091,6 +1111,7 @@ int tsfm_spec_create(const tsfm_weights *target_w, const tsfm_weights *draft_w, 
       return fail(TSFM_ERR_CUDA);
   }
   prefer_max_smem_all();
+  if (cfg->dtype == TSFM_F32 && (rc = gemm_f32_init())) return fail(rc);
   if (h->use_tc) {
     if ((rc = gemm_sk_init())) return fail(rc);
     if ((rc = gemm_ws_init())) return fail(rc);

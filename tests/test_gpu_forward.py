@@ -47,6 +47,19 @@ def test_fp32_forward_matches_oracle(target, draft, P, n):
     assert np.abs(gd - wd).max() < 1e-4
 
 
+@pytest.mark.parametrize("target,n", [
+    (Arch(1, 64, 1, 64), 1),          # K = 64: two vectors per warp; five rows of a 16-row tile
+    (Arch(1, 64, 2, 128), 150),       # 750 rows: ragged last 16-row tile
+    (Arch(1, 320, 5, 768), 60),       # 300 rows x 960 features: 32 x 32 tiles, ragged rows; K = 768 is the longest row
+    (Arch(1, 832, 13, 832), 3),       # rows beyond it: the 64 x 64 tile and a separate norm
+])
+def test_fp32_contraction_tiles(target, n):
+    wl = small_workload("f32", target, Arch(1, 64, 2, 128), 32)
+    gt, wt, gd, wd = run_forward_case(wl, 0, n)
+    assert np.abs(gt - wt).max() < 1e-4        # as above: rounding of fp32 sums
+    assert np.abs(gd - wd).max() < 1e-4
+
+
 @pytest.mark.parametrize("backend", [1, 0], ids=["simt", "tcgen05"])
 @pytest.mark.parametrize("target,draft,P,n,mode", [
     (Arch(3, 256, 4, 1024), Arch(2, 128, 4, 256), 96, 9, "separate"),      # few tokens: folded norms, K split

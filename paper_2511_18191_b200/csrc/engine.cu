@@ -344,8 +344,8 @@ template <typename T> void prefer_max_smem_typed() {
   prefer_max_smem(rmsnorm_kernel<T, true>);
   prefer_max_smem(head_kernel<T>);
   prefer_max_smem(embed_rows_kernel<T>);
-  prefer_max_smem(head_rows_kernel<T>);
-  cudaFuncSetAttribute(head_rows_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+  prefer_max_smem(gemm_f32_kernel<T, 16, 16>);
+  prefer_max_smem(gemm_f32_kernel<T, 32, 32>);
   prefer_max_smem(gemm_simt_kernel<T, EPI_F32>);
   prefer_max_smem(gemm_simt_kernel<T, EPI_T>);
   prefer_max_smem(gemm_simt_kernel<T, EPI_GELU_T>);
@@ -371,8 +371,6 @@ void prefer_max_smem_all() {
   prefer_max_smem(gemm_sk_kernel<2, false>);
   prefer_max_smem(gemm_ws_kernel<false>);
   prefer_max_smem(gemm_ws_kernel<true>);
-  prefer_max_smem(gemm_f32_kernel<16, 16>);
-  prefer_max_smem(gemm_f32_kernel<32, 32>);
   prefer_max_smem(attn_flash_kernel<32, 3>);
   prefer_max_smem(attn_flash_kernel<32, kFlashStShort>);
   prefer_max_smem(attn_flash_kernel<64, 3>);
@@ -476,7 +474,13 @@ void gemm(tsfm_spec *h, GemmSkPlan *plan, const void *A, const void *W, void *C,
   KTimer kt(h, KC_GEMM_SIMT, bytes, flops);
   if constexpr (sizeof(T) == 4) {
     if (gemm_f32_eligible(W, K)) {
-      if (gemm_f32_launch(h->ls, h->pdl, (const float *)A, (const float *)W, (float *)C, M, N, K, epi, row_gain, eps, lr)) {
+      RowsArgs ra{};
+      ra.mode = ROWS_PLAIN;
+      ra.epi = epi;
+      ra.gain = row_gain;
+      ra.eps = eps;
+      ra.lr = lr;
+      if (gemm_f32_launch(h->ls, h->pdl, (const float *)A, (const float *)W, (float *)C, M, N, K, ra)) {
         LAUNCHED();
       } else if (h->enqueue_err == TSFM_OK) {
         h->enqueue_err = TSFM_ERR_CUDA;
@@ -540,9 +544,12 @@ void launch_attn(tsfm_spec *h, ModelDev &m, int l, int B, const PassGeom &g) {
 }
 
 enum { HEAD_NONE = 0, HEAD_LAST_TO_HIST = 1, HEAD_ALL_TO_VOUT = 2 };
-// Passes of at least this many rows take the embedding and head kernels that share each weight
-// load between 8 rows; below it there are too few rows to fill the SMs that way.
+// Passes of at least this many rows take the embedding kernel that shares each weight load between 8
+// rows where a token is too short for the tiled contraction (point tokens).
 constexpr int kManyRows = 1024;
+// From this many rows on the head is a tiled contraction (gemm_f32_kernel) on the bf16 path too; below
+// it one CTA per row and eight outputs, with constants fetched before the dependency wait, is shorter.
+constexpr int kHeadTileRows = 192;
 // Up to this many rows the separate RMSNorm kernel fetches its constants before the dependency wait.
 constexpr int kNormEarlyMaxRows = 2048;
 
@@ -573,11 +580,27 @@ void run_pass(tsfm_spec *h, ModelDev &m, int B, const PassGeom &g, int head_mode
   const bool fold32 = sizeof(T) == 4 && gemm_f32_eligible(m.layers[0].Wqkv, d);
   const int L = m.arch.n_layers;
   const LiveRows lr{g.n_live, g.q_len};
+  auto launched = [&](bool ok, const char *what) {
+    if (ok) {
+      LAUNCHED();
+    } else if (h->enqueue_err == TSFM_OK) {
+      h->enqueue_err = TSFM_ERR_CUDA;
+      g_cuda_err = std::string(what) + " could not be launched: " + cudaGetErrorString(cudaGetLastError());
+    }
+  };
   // the RMSNorm of passes of a few thousand rows is a link in a chain: constants before the wait
   auto *norm_kernel = M <= kNormEarlyMaxRows && d <= 1280 ? rmsnorm_kernel<T, true> : rmsnorm_kernel<T, false>;
   {
     KTimer kt(h, KC_EMBED, (double)M * Pi * 4 + (double)d * Pi * sizeof(T) + (double)M * d * 4, 2.0 * M * Pi * d);
-    if (!fold && M >= kManyRows)
+    if (!fold && gemm_f32_eligible(m.W_emb, Pi)) {
+      RowsArgs ra{};
+      ra.mode = ROWS_EMBED;
+      ra.epi = EPI_F32;
+      ra.g = g;
+      ra.opens_round = opens_round ? 1 : 0;
+      ra.stamp = stamp;
+      launched(gemm_f32_launch(s, h->pdl, (const float *)h->hist, (const T *)m.W_emb, h->x, M, d, Pi, ra), "embedding");
+    } else if (!fold && M >= kManyRows)
       launch_ex(s, h->pdl, embed_rows_kernel<T>, dim3((M + 7) / 8, (d + 127) / 128), dim3(128), 8 * Pi * sizeof(float),
                 h->hist, g, M, Pi, d, (const T *)m.W_emb, h->x, stamp);
     else
@@ -622,17 +645,24 @@ void run_pass(tsfm_spec *h, ModelDev &m, int B, const PassGeom &g, int head_mode
   const double rows = head_mode == HEAD_LAST_TO_HIST ? B : Mb;
   KTimer kt(h, head_mode == HEAD_NONE ? -1 : KC_HEAD, rows * d * 4 + (double)P * d * sizeof(T) + rows * P * 4,
             2.0 * rows * P * d);
-  const bool rows_fit = (size_t)8 * d * sizeof(float) <= 200 * 1024;
-  // (The last-token head keeps one CTA per series and eight outputs also with a thousand series:
-  // sharing each weight load between 8 series, as the verification head does, measured slower --
-  // C3 target-only decode 15.98 vs 15.13 ms.)
-  if (head_mode == HEAD_LAST_TO_HIST) {
+  if (head_mode != HEAD_NONE && (fold32 || rows >= kHeadTileRows) && gemm_f32_eligible(m.W_head, d)) {
+    RowsArgs ra{};
+    ra.mode = head_mode == HEAD_LAST_TO_HIST ? ROWS_HEAD_LAST : ROWS_HEAD_ALL;
+    ra.epi = EPI_F32;
+    ra.gain = m.g_f;
+    ra.eps = eps;
+    ra.g = g;
+    ra.tok_len = Pi;
+    ra.st = ds.k_pos >= 0 ? h->st : nullptr;
+    ra.muq = h->muq;
+    ra.k_pos = ds.k_pos;
+    ra.Kblk = ds.K;
+    launched(gemm_f32_launch(s, h->pdl, (const float *)h->x, (const T *)m.W_head, head_mode == HEAD_LAST_TO_HIST ? h->hist : vout,
+                             (int)rows, P, d, ra), "head");
+  } else if (head_mode == HEAD_LAST_TO_HIST) {
     launch_ex(s, h->pdl, head_kernel<T>, dim3(B, (P + 7) / 8), dim3(256), d * sizeof(float), h->x, m.g_f,
               (const T *)m.W_head, d, P, eps, g, 1, h->hist, (float *)nullptr,
               ds.k_pos >= 0 ? (const DevState *)h->st : (const DevState *)nullptr, h->muq, ds.k_pos, ds.K, Pi);
-  } else if (head_mode == HEAD_ALL_TO_VOUT && Mb >= kManyRows && rows_fit) {
-    launch_ex(s, h->pdl, head_rows_kernel<T>, dim3((Mb + 7) / 8, (P + 31) / 32), dim3(256), (size_t)8 * d * sizeof(float),
-              h->x, m.g_f, (const T *)m.W_head, Mb, d, P, eps, vout, g);
   } else if (head_mode == HEAD_ALL_TO_VOUT) {
     launch_ex(s, h->pdl, head_kernel<T>, dim3(Mb, (P + 7) / 8), dim3(256), d * sizeof(float), h->x, m.g_f,
               (const T *)m.W_head, d, P, eps, g, 0, (float *)nullptr, vout, (const DevState *)nullptr, (float *)nullptr, 0, 0,
@@ -1111,7 +1141,7 @@ int tsfm_spec_create(const tsfm_weights *target_w, const tsfm_weights *draft_w, 
       return fail(TSFM_ERR_CUDA);
   }
   prefer_max_smem_all();
-  if (cfg->dtype == TSFM_F32 && (rc = gemm_f32_init())) return fail(rc);
+  if ((rc = cfg->dtype == TSFM_F32 ? gemm_f32_init<float>() : gemm_f32_init<bf16>())) return fail(rc);
   if (h->use_tc) {
     if ((rc = gemm_sk_init())) return fail(rc);
     if ((rc = gemm_ws_init())) return fail(rc);

@@ -1,21 +1,23 @@
-// fp32 contraction with whole rows in shared memory, the RMSNorm of its input folded in.
+// Contractions of fp32 activations in fp32 FMAs: every contraction of the fp32 models, and the patch
+// embedding and the mean head of both kinds of model (weights fp32 or bf16).
 //
 //   C[t, f] (op)= sum_k A'[t, k] * W[f, k]       A' = A, or gain * A / sqrt(mean(A^2) + eps)
 //
-// The fp32 models are small (rows of 64 ... 512 features), so a contraction is a link of a chain of
-// dependent launches and costs what its memory round trips cost.  The 64 x 64 tile of
-// gemm_simt_kernel makes one such round trip per 16 features of K; here a CTA requests its weight
-// rows before the dependency wait and its whole activation rows in one go behind it, and since it
-// holds the rows it also normalises them: the RMSNorm launch in front of the contraction goes away.
-//   * tile MT tokens x FN features over the whole K; the eight warps take the 4-feature vectors of K
-//     in turn (vector w, w + 8, ...), each lane accumulating (MT / 4) x (FN / 8) outputs in fp32 FMAs;
-//     the partial tiles are summed through shared memory in warp order, so every epilogue sees
-//     complete sums and the order of the additions is fixed;
+// For the small fp32 models a contraction is a link of a chain of dependent launches and costs what its
+// memory round trips cost; a CTA therefore requests its weight rows before the dependency wait and its
+// activation rows in one go behind it, and since it holds the rows it also normalises them (no RMSNorm
+// launch in front).  For the embedding and the head of passes of many rows it is a matter of reading
+// every weight once per tile of rows instead of once per row or eight rows.
+//   * tile MT tokens x FN features, K in chunks of KC (all of it in one chunk where that fits); the eight
+//     warps take the 4-feature vectors of a chunk in turn (vector w, w + 8, ...), each lane accumulating
+//     (MT / 4) x (FN / 8) outputs in registers; the partial tiles are summed through shared memory in warp
+//     order, so every epilogue sees complete sums and the order of the additions is fixed;
+//   * the norm's factor 1 / sqrt(...) is common to a row: the sums run over gain * A and are scaled at the end;
 //   * rows are padded by 16 bytes: the four token rows and eight feature rows that a warp reads at a
 //     time fall into different banks.
-// Bound: latency (launch, one L2 round trip, the 8-way sum); 3.5 us a link inside a captured forecast where
-// the 64 x 64 tile took 8 to 31 us (M = 37 ... 185, K = 128, 512).  Forecast of one series with the 2-layer
-// d = 128 model: 636 -> 260 us; of 37 series 2.55 -> 0.90 ms.
+// Bound: latency for small shapes (launch, one L2 round trip, the 8-way sum; 3.5 us a link inside a captured
+// forecast where the 64 x 64 tile took 8 to 31 us at M = 37 ... 185, K = 128, 512: forecast of one series
+// with the 2-layer d = 128 model 636 -> 260 us, of 37 series 2.55 -> 0.90 ms), FMA rate for many rows.
 // grid = (ceil(N / FN), ceil(M / MT)), block = 256.  K a multiple of 16.
 #pragma once
 #include "common.cuh"
@@ -23,63 +25,118 @@
 
 namespace tsfm {
 
-template <int MT, int FN> constexpr int f32_smem_bytes(int K) {
-  const int rows = (MT + FN) * (K + 4) * 4, red = 8 * MT * FN * 4;      // the partial sums reuse the rows
+// Where the rows of A come from and where results go.
+enum : int {
+  ROWS_PLAIN = 0,        // A[t, :], C[t, :] with an epilogue EPI_F32 / EPI_GELU_T / EPI_RESID
+  ROWS_EMBED = 1,        // A = token t of the pass in the series' history, C[t, :]
+  ROWS_HEAD_LAST = 2,    // A = the last token of slot t, C = the series' history behind the pass (see head_kernel)
+  ROWS_HEAD_ALL = 3,     // A = boundary token t of the pass, C = vout[series, boundary, :]
+};
+struct RowsArgs {
+  int mode, epi;
+  const float *gain;               // [K] or NULL: no norm
+  float eps;
+  LiveRows lr;                     // ROWS_PLAIN
+  PassGeom g;                      // the other modes
+  int opens_round;                 // ROWS_EMBED: the slots are looked up after the wait
+  unsigned long long *stamp;       // ROWS_EMBED
+  int tok_len;                     // ROWS_HEAD_LAST: values per token; sampled proposals:
+  const DevState *st;
+  float *muq;
+  int k_pos, Kblk;
+};
+
+template <typename T, int MT, int FN> constexpr int f32_smem_bytes(int KC) {
+  const int rows = MT * (KC + 4) * 4 + FN * (KC * (int)sizeof(T) + 16), red = 8 * MT * FN * 4;   // the partial sums reuse the rows
   return rows > red ? rows : red;
 }
 
-template <int MT, int FN>
+__device__ __forceinline__ float4 f32_vec4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
+__device__ __forceinline__ float4 f32_vec4(const bf16 *p) {
+  const uint2 u = *reinterpret_cast<const uint2 *>(p);
+  return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xffff0000u), __uint_as_float(u.y << 16),
+                     __uint_as_float(u.y & 0xffff0000u));
+}
+
+template <typename T, int MT, int FN>
 __global__ void __launch_bounds__(256)
-gemm_f32_kernel(const float *A, const float *__restrict__ W, float *C, int M, int N, int K, int epi,
-                const float *__restrict__ gain, float eps, const LiveRows lr) {
-  constexpr int RM = MT / 4, RF = FN / 8;
+gemm_f32_kernel(const float *A, const T *__restrict__ W, float *C, int M, int N, int K, int KC, const RowsArgs ra) {
+  constexpr int RM = MT / 4, RF = FN / 8, VW = 16 / sizeof(T);
   extern __shared__ __align__(16) float f32_smem[];
+  __shared__ long long src_off[MT], dst_off[MT];               // row offsets in A and C; src -1: no such row
+  __shared__ int row_series[MT];
+  __shared__ float row_ss[MT];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const int f0 = blockIdx.x * FN, t0 = blockIdx.y * MT;
+  const PassGeom &g = ra.g;
+  const int nb = ra.mode == ROWS_HEAD_LAST ? 1 : ra.mode == ROWS_HEAD_ALL ? g.q_len / g.head_step : g.q_len;   // rows per slot
   // rows in use (active-series compaction): read before the dependency wait, see gemm_sk_kernel
-  if (lr.n_live) {
-    M = min(M, *reinterpret_cast<const volatile int *>(lr.n_live) * lr.q_len);
+  if (ra.mode == ROWS_PLAIN) {
+    if (ra.lr.n_live) M = min(M, *reinterpret_cast<const volatile int *>(ra.lr.n_live) * ra.lr.q_len);
     if (t0 >= M) return;
   }
-  const int ld = K + 4, vpr = K >> 2;
-  float *Ws = f32_smem, *As = f32_smem + FN * ld;
-  for (int i = tid; i < FN * vpr; i += 256) {
-    const int r = i / vpr, c = (i % vpr) * 4;
-    if (f0 + r < N) cp_async16(Ws + r * ld + c, W + (size_t)(f0 + r) * K + c);
-    else *reinterpret_cast<float4 *>(Ws + r * ld + c) = make_float4(0.f, 0.f, 0.f, 0.f);
+  auto lookup = [&]() {                                        // slots of the other modes: see slot_lookup
+    if (tid < MT) {
+      const int t = t0 + tid;
+      long long so = -1, dof = 0;
+      if (t < M) {
+        const int slot = t / nb, i = t % nb;
+        const SlotPos sp = slot_lookup(g, slot);
+        if (!sp.dead) {
+          row_series[tid] = sp.b;
+          if (ra.mode == ROWS_EMBED) {
+            so = ((long long)sp.b * g.cap + sp.p0 + i) * K;
+            dof = (long long)t * N;
+          } else {
+            const int j = ra.mode == ROWS_HEAD_LAST ? g.q_len - 1 : (i + 1) * g.head_step - 1;
+            so = ((long long)slot * g.q_len + j) * K;
+            dof = ra.mode == ROWS_HEAD_LAST ? ((long long)sp.b * g.cap + sp.p0 + g.q_len) * ra.tok_len
+                                            : ((long long)sp.b * nb + i) * N;
+          }
+        }
+      }
+      src_off[tid] = so;
+      dst_off[tid] = dof;
+    }
+  };
+  const int lda = KC + 4, ldw = KC + VW;
+  float *As = f32_smem;
+  T *Ws = reinterpret_cast<T *>(f32_smem + MT * lda);
+  auto load_w = [&](int k0, int kc) {
+    const int cpr = kc / VW;
+    for (int i = tid; i < FN * cpr; i += 256) {
+      const int r = i / cpr, c = (i % cpr) * VW;
+      if (f0 + r < N) cp_async16(Ws + r * ldw + c, W + (size_t)(f0 + r) * K + k0 + c);
+      else *reinterpret_cast<uint4 *>(Ws + r * ldw + c) = make_uint4(0u, 0u, 0u, 0u);
+    }
+  };
+  load_w(0, min(KC, K));
+  const bool early = ra.mode != ROWS_PLAIN && !ra.opens_round;
+  if (ra.mode == ROWS_PLAIN) {
+    if (tid < MT) {
+      src_off[tid] = t0 + tid < M ? (long long)(t0 + tid) * K : -1;
+      dst_off[tid] = (long long)(t0 + tid) * N;
+    }
+  } else if (early) {
+    lookup();
   }
+  if (tid < MT) row_ss[tid] = 0.f;
   pdl_sync();
-  for (int i = tid; i < MT * vpr; i += 256) {
-    const int r = i / vpr, c = (i % vpr) * 4;
-    if (t0 + r < M) cp_async16(As + r * ld + c, A + (size_t)(t0 + r) * K + c);
-    else *reinterpret_cast<float4 *>(As + r * ld + c) = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (ra.stamp && blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) *ra.stamp = globaltimer_ns();
+  if (ra.mode != ROWS_PLAIN && !early) lookup();
+  if (!__syncthreads_or(tid < MT && src_off[tid] >= 0)) {      // a tile of dead slots
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    return;
   }
-  // the old values of this thread's outputs (residual epilogue), while the copies fly
-  constexpr int OUT = MT * FN / 256;                           // outputs per thread, consecutive features
-  const int orow = tid * OUT / FN, ocol = tid * OUT % FN;
-  const int t = t0 + orow, f = f0 + ocol;
+
+  // this thread's outputs: consecutive features of one row; their old values (residual epilogue) fly with the copies
+  constexpr int OUT = MT * FN / 256;
+  const int orow = tid * OUT / FN, f = f0 + tid * OUT % FN;
+  const bool live = src_off[orow] >= 0;
+  float *dst = C + dst_off[orow];
   float old[OUT];
 #pragma unroll
-  for (int i = 0; i < OUT; ++i) old[i] = (epi == EPI_RESID && t < M && f + i < N) ? C[(size_t)t * N + f + i] : 0.f;
-  asm volatile("cp.async.wait_all;" ::: "memory");
-  __syncthreads();
-  if (gain) {
-    for (int r = w; r < MT; r += 8) {                          // one warp per row
-      float ss = 0.f;
-      for (int v = lane; v < vpr; v += 32) {
-        const float4 a = *reinterpret_cast<const float4 *>(As + r * ld + v * 4);
-        ss = fmaf(a.x, a.x, fmaf(a.y, a.y, fmaf(a.z, a.z, fmaf(a.w, a.w, ss))));
-      }
-      const float rstd = rsqrtf(warp_sum(ss) / K + eps);
-      for (int v = lane; v < vpr; v += 32) {
-        float4 a = *reinterpret_cast<const float4 *>(As + r * ld + v * 4);
-        const float4 g = *reinterpret_cast<const float4 *>(gain + v * 4);
-        a.x = g.x * a.x * rstd; a.y = g.y * a.y * rstd; a.z = g.z * a.z * rstd; a.w = g.w * a.w * rstd;
-        *reinterpret_cast<float4 *>(As + r * ld + v * 4) = a;
-      }
-    }
-    __syncthreads();
-  }
+  for (int i = 0; i < OUT; ++i) old[i] = (ra.epi == EPI_RESID && live && f + i < N) ? dst[f + i] : 0.f;
 
   // lane (tr, tf): token rows tr, tr + 4, ..., feature rows tf, tf + 8, ...
   const int tr = lane >> 3, tf = lane & 7;
@@ -88,17 +145,46 @@ gemm_f32_kernel(const float *A, const float *__restrict__ W, float *C, int M, in
   for (int i = 0; i < RM; ++i)
 #pragma unroll
     for (int j = 0; j < RF; ++j) acc[i][j] = 0.f;
-  for (int v = w; v < vpr; v += 8) {
-    float4 a[RM], b[RF];
+  for (int k0 = 0; k0 < K; k0 += KC) {
+    const int kc = min(KC, K - k0), vpr = kc >> 2;
+    if (k0) {
+      __syncthreads();                                         // the previous chunk is done with
+      load_w(k0, kc);
+    }
+    for (int i = tid; i < MT * vpr; i += 256) {
+      const int r = i / vpr, c = (i % vpr) * 4;
+      if (src_off[r] >= 0) cp_async16(As + r * lda + c, A + src_off[r] + k0 + c);
+      else *reinterpret_cast<float4 *>(As + r * lda + c) = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    if (ra.gain) {
+      for (int r = w; r < MT; r += 8) {                        // one warp per row
+        float ss = 0.f;
+        for (int v = lane; v < vpr; v += 32) {
+          float4 a = *reinterpret_cast<const float4 *>(As + r * lda + v * 4);
+          const float4 gg = *reinterpret_cast<const float4 *>(ra.gain + k0 + v * 4);
+          ss = fmaf(a.x, a.x, fmaf(a.y, a.y, fmaf(a.z, a.z, fmaf(a.w, a.w, ss))));
+          a.x *= gg.x; a.y *= gg.y; a.z *= gg.z; a.w *= gg.w;
+          *reinterpret_cast<float4 *>(As + r * lda + v * 4) = a;
+        }
+        ss = warp_sum(ss);
+        if (lane == 0) row_ss[r] += ss;
+      }
+      __syncthreads();
+    }
+    for (int v = w; v < vpr; v += 8) {
+      float4 a[RM], b[RF];
 #pragma unroll
-    for (int i = 0; i < RM; ++i) a[i] = *reinterpret_cast<const float4 *>(As + (tr + 4 * i) * ld + v * 4);
+      for (int i = 0; i < RM; ++i) a[i] = *reinterpret_cast<const float4 *>(As + (tr + 4 * i) * lda + v * 4);
 #pragma unroll
-    for (int j = 0; j < RF; ++j) b[j] = *reinterpret_cast<const float4 *>(Ws + (tf + 8 * j) * ld + v * 4);
+      for (int j = 0; j < RF; ++j) b[j] = f32_vec4(Ws + (tf + 8 * j) * ldw + v * 4);
 #pragma unroll
-    for (int i = 0; i < RM; ++i)
+      for (int i = 0; i < RM; ++i)
 #pragma unroll
-      for (int j = 0; j < RF; ++j)
-        acc[i][j] = fmaf(a[i].x, b[j].x, fmaf(a[i].y, b[j].y, fmaf(a[i].z, b[j].z, fmaf(a[i].w, b[j].w, acc[i][j]))));
+        for (int j = 0; j < RF; ++j)
+          acc[i][j] = fmaf(a[i].x, b[j].x, fmaf(a[i].y, b[j].y, fmaf(a[i].z, b[j].z, fmaf(a[i].w, b[j].w, acc[i][j]))));
+    }
   }
   __syncthreads();                                             // the rows are done with: their space takes the partial tiles
   float *red = f32_smem + w * (MT * FN);
@@ -107,46 +193,56 @@ gemm_f32_kernel(const float *A, const float *__restrict__ W, float *C, int M, in
 #pragma unroll
     for (int j = 0; j < RF; ++j) red[(tr + 4 * i) * FN + tf + 8 * j] = acc[i][j];
   __syncthreads();
-  if (t >= M) return;
+  if (!live) return;
+  const float rstd = ra.gain ? rsqrtf(row_ss[orow] / K + ra.eps) : 1.f;
+  const bool sampled = ra.mode == ROWS_HEAD_LAST && ra.st && (ra.st->flags & VAR_SAMPLE_PROPOSALS);
 #pragma unroll
   for (int i = 0; i < OUT; ++i) {
+    if (f + i >= N) break;
     float v = 0.f;
 #pragma unroll
     for (int k = 0; k < 8; ++k) v += f32_smem[k * (MT * FN) + tid * OUT + i];
-    if (f + i < N) C[(size_t)t * N + f + i] = epi == EPI_RESID ? old[i] + v : epi == EPI_GELU_T ? gelu_erf(v) : v;
+    v *= rstd;
+    if (ra.epi == EPI_RESID) v += old[i];
+    else if (ra.epi == EPI_GELU_T) v = gelu_erf(v);
+    if (sampled) {     // proposal x = mu_q + sigma_q eps (Sec. 3.3); the mean is kept for the statistic
+      ra.muq[((size_t)row_series[orow] * ra.Kblk + ra.k_pos) * N + f + i] = v;
+      v += ra.st->sigma_q * head_normal(ra.st, row_series[orow], ra.k_pos, f + i);
+    }
+    dst[f + i] = v;
   }
 }
 
 // ------------------------------------------------------------------ host side
-// The shapes it takes: rows of which a 32 x 32 tile fits in shared memory (K <= 768: 198 KB), operands
-// 16-byte aligned; longer rows keep gemm_simt_kernel.  32 x 32 tiles (twice the flops per shared-memory
-// read) where the 16 x 16 ones would be more than one wave at four CTAs per SM.
-constexpr int F32_MAX_K = 768;
-
-static int gemm_f32_init() {
-  if (cudaFuncSetAttribute(gemm_f32_kernel<16, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess ||
-      cudaFuncSetAttribute(gemm_f32_kernel<32, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess)
+template <typename T> static int gemm_f32_init() {
+  if (cudaFuncSetAttribute(gemm_f32_kernel<T, 16, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024) != cudaSuccess ||
+      cudaFuncSetAttribute(gemm_f32_kernel<T, 32, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024) != cudaSuccess)
     return -4;
   return 0;
 }
-static bool gemm_f32_eligible(const void *W, int K) { return K % 16 == 0 && K >= 16 && K <= F32_MAX_K && !((uintptr_t)W & 15); }
+// Rows that 16-byte copies can fetch.
+static bool gemm_f32_eligible(const void *W, int K) { return K % 16 == 0 && K >= 16 && !((uintptr_t)W & 15); }
 
-static bool gemm_f32_launch(cudaStream_t st, bool pdl, const float *A, const float *W, float *C, int M, int N, int K, int epi,
-                            const float *gain, float eps, LiveRows lr) {
+// 32 x 32 tiles (twice the flops per shared-memory read) where the 16 x 16 ones would be more than one
+// wave at four CTAs per SM.  Rows of up to 768 values stay whole (one memory round trip; the longest
+// take one CTA per SM); longer ones go through in chunks of 256, four CTAs per SM.
+template <typename T>
+static bool gemm_f32_launch(cudaStream_t st, bool pdl, const float *A, const T *W, float *C, int M, int N, int K, const RowsArgs &ra) {
   const bool small = (long)((N + 15) / 16) * ((M + 15) / 16) <= 4 * 148;
-  const int T = small ? 16 : 32;
+  const int tile = small ? 16 : 32;
+  const int KC = K <= (small ? 768 : 512) ? K : 256;
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((N + T - 1) / T, (M + T - 1) / T);
+  cfg.gridDim = dim3((N + tile - 1) / tile, (M + tile - 1) / tile);
   cfg.blockDim = dim3(256);
-  cfg.dynamicSmemBytes = small ? f32_smem_bytes<16, 16>(K) : f32_smem_bytes<32, 32>(K);
+  cfg.dynamicSmemBytes = small ? f32_smem_bytes<T, 16, 16>(KC) : f32_smem_bytes<T, 32, 32>(KC);
   cfg.stream = st;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = pdl ? 1 : 0;
-  return (small ? cudaLaunchKernelEx(&cfg, gemm_f32_kernel<16, 16>, A, W, C, M, N, K, epi, gain, eps, lr)
-                : cudaLaunchKernelEx(&cfg, gemm_f32_kernel<32, 32>, A, W, C, M, N, K, epi, gain, eps, lr)) == cudaSuccess;
+  return (small ? cudaLaunchKernelEx(&cfg, gemm_f32_kernel<T, 16, 16>, A, W, C, M, N, K, KC, ra)
+                : cudaLaunchKernelEx(&cfg, gemm_f32_kernel<T, 32, 32>, A, W, C, M, N, K, KC, ra)) == cudaSuccess;
 }
 
 }  // namespace tsfm

@@ -877,68 +877,4 @@ head_kernel(const float *x, const float *__restrict__ gain, const T *__restrict_
   }
 }
 
-// The head for the boundary tokens of a pass of many rows (verification: vout[b, i, :]): 8 rows
-// per CTA (one warp normalises one row into shared memory), then each warp produces 4 of the CTA's
-// 32 outputs for all 8 rows, so that a weight vector is loaded once per 8 rows.  M counts boundary
-// rows (series x boundaries per series).
-// grid = (ceil(M / 8), ceil(P / 32)), block = 256, dynamic shared memory 8 * d floats.
-template <typename T>
-__global__ void __launch_bounds__(256)
-head_rows_kernel(const float *x, const float *__restrict__ gain, const T *__restrict__ Wh, int M,
-                 int d, int P, float eps, float *__restrict__ vout, PassGeom g) {
-  constexpr int R = 8;
-  extern __shared__ __align__(16) float xs[];                  // [R][d] normalised rows
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int row0 = blockIdx.x * R;
-  const int nb = g.q_len / g.head_step;                        // boundaries per series
-  // live rows: read before the dependency wait (written when the previous round closed, a whole
-  // pass of kernels back)
-  if (g.n_live) M = min(M, *reinterpret_cast<const volatile int *>(g.n_live) * nb);
-  if (row0 >= M) return;
-  pdl_sync();
-  {
-    const int row = row0 + w;
-    float *xw = xs + (size_t)w * d;
-    float ss = 0.f;
-    if (row < M) {
-      const float *xr = x + ((size_t)(row / nb) * g.q_len + (row % nb + 1) * g.head_step - 1) * d;
-      for (int i = lane; i < d; i += 32) {
-        const float v = xr[i];
-        xw[i] = v;
-        ss = fmaf(v, v, ss);
-      }
-    } else {
-      for (int i = lane; i < d; i += 32) xw[i] = 0.f;
-    }
-    const float rstd = rsqrtf(warp_sum(ss) / d + eps);
-    for (int i = lane; i < d; i += 32) xw[i] = gain[i] * xw[i] * rstd;   // each lane rewrites what it wrote
-  }
-  __syncthreads();
-  constexpr int V = Vec16<T>::N;
-  for (int q = 0; q < 4; ++q) {
-    const int p = blockIdx.y * 32 + q * 8 + w;
-    if (p >= P) break;
-    const T *wr = Wh + (size_t)p * d;
-    float acc[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) acc[r] = 0.f;
-    for (int i = lane * V; i < d; i += 32 * V) {
-      float wv[V];
-      Vec16<T>::load(wr + i, wv);
-#pragma unroll
-      for (int r = 0; r < R; ++r)
-#pragma unroll
-        for (int c = 0; c < V; ++c) acc[r] = fmaf(wv[c], xs[(size_t)r * d + i + c], acc[r]);
-    }
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const float o = warp_sum(acc[r]);
-      if (lane == 0 && row0 + r < M) {                         // vout is indexed by series, rows by slot
-        const int row = row0 + r, b = series_of(g, row / nb);
-        vout[((size_t)b * nb + row % nb) * P + p] = o;
-      }
-    }
-  }
-}
-
 }  // namespace tsfm

@@ -48,10 +48,10 @@ def test_fp32_forward_matches_oracle(target, draft, P, n):
 
 
 @pytest.mark.parametrize("target,n", [
-    (Arch(1, 64, 1, 64), 1),          # K = 64: two vectors per warp; five rows of a 16-row tile
+    (Arch(1, 64, 1, 64), 2),          # K = 64: two vectors per warp; ten rows of a 16-row tile
     (Arch(1, 64, 2, 128), 150),       # 750 rows: ragged last 16-row tile
-    (Arch(1, 320, 5, 768), 60),       # 300 rows x 960 features: 32 x 32 tiles, ragged rows; K = 768 is the longest row
-    (Arch(1, 832, 13, 832), 3),       # rows beyond it: the 64 x 64 tile and a separate norm
+    (Arch(1, 320, 5, 768), 60),       # 300 rows x 960 features: 32 x 32 tiles, ragged rows; K = 768 whole and in chunks
+    (Arch(1, 832, 13, 832), 3),       # longer rows: chunks of 256 with a short last one
 ])
 def test_fp32_contraction_tiles(target, n):
     wl = small_workload("f32", target, Arch(1, 64, 2, 128), 32)

@@ -23,6 +23,7 @@
 #include "gemm_tc.cuh"
 #include "gemm_sk.cuh"
 #include "gemm_ws.cuh"
+#include "gemm_pair.cuh"
 #include "gemm_f32.cuh"
 
 using namespace tsfm;
@@ -369,6 +370,7 @@ void prefer_max_smem_all() {
   prefer_max_smem(gemm_sk_kernel<1, false>);
   prefer_max_smem(gemm_sk_kernel<1, true>);
   prefer_max_smem(gemm_sk_kernel<2, false>);
+  prefer_max_smem(gemm_pair_kernel);
   prefer_max_smem(gemm_ws_kernel<false>);
   prefer_max_smem(gemm_ws_kernel<true>);
   prefer_max_smem(attn_flash_kernel<32, 3>);
@@ -438,6 +440,12 @@ void launch_gemm_simt(cudaStream_t s, bool pdl, const T *A, const T *W, void *C,
   }
 }
 
+// From this many tokens on a contraction runs on pairs of SMs (gemm_pair_kernel against gemm_sk_kernel, graph
+// replay of dependent launches, us: M = 576: 9.5 / 9.7, 6.5 / 8.7, 12.6 / 14.8, 14.7 / 14.6 for the four
+// contractions of a d = 1280 layer; M = 1024, d = 768: 7.7 / 7.5, 5.5 / 6.5, 10.8 / 11.9, 10.3 / 11.6;
+// M = 6000, d = 1024: 32 / 47, 16 / 21, 47 / 74, 43 / 61).
+constexpr int kPairMinRows = 513;
+
 // C (op)= A . W^T through the tensor-core kernel when a plan exists, else an FMA kernel.  row_gain (fp32
 // models whose rows gemm_f32_kernel takes): A is the residual stream, normalised by the contraction itself.
 template <typename T>
@@ -461,7 +469,9 @@ void gemm(tsfm_spec *h, GemmSkPlan *plan, const void *A, const void *W, void *C,
   }
   if (sizeof(T) == 2 && h->use_tc && plan && plan->valid) {
     KTimer kt(h, M <= 512 ? KC_GEMM_TC_SMALL : M < 4096 ? KC_GEMM_TC_MID : KC_GEMM_TC_LARGE, bytes, flops);
-    if (gemm_sk_launch(h->ls, h->pdl, *plan, C, M, epi, h->dev_status, norm, lr)) {
+    const bool pair = !norm && M >= kPairMinRows && gemm_pair_eligible(*plan, C);
+    if (pair ? gemm_pair_launch(h->ls, h->pdl, *plan, C, M, epi, h->dev_status, lr)
+             : gemm_sk_launch(h->ls, h->pdl, *plan, C, M, epi, h->dev_status, norm, lr)) {
       LAUNCHED();
     } else if (h->enqueue_err == TSFM_OK) {
       // No silent fallback: the FMA kernel knows nothing of a folded norm, and a pass that mixes
@@ -1145,6 +1155,7 @@ int tsfm_spec_create(const tsfm_weights *target_w, const tsfm_weights *draft_w, 
   if (h->use_tc) {
     if ((rc = gemm_sk_init())) return fail(rc);
     if ((rc = gemm_ws_init())) return fail(rc);
+    if ((rc = gemm_pair_init())) return fail(rc);
     for (ModelDev *m : {&h->tgt, &h->drf}) {
       const int d = m->arch.d_model, f = m->arch.d_ff;
       for (LayerDev &ly : m->layers) {
@@ -1383,7 +1394,13 @@ int tsfm_gemm_bf16(void *stream, const void *A, const void *W, float *C, int32_t
     cudaFree(status);
     CU_TRY(e0);
   }
-  const bool ok = gemm_sk_launch(s, false, plan, C, M, EPI_F32, status);
+  const bool pair = M >= kPairMinRows && gemm_pair_eligible(plan, C);
+  if (pair && gemm_pair_init()) {
+    cudaFree(status);
+    return TSFM_ERR_CUDA;
+  }
+  const bool ok = pair ? gemm_pair_launch(s, false, plan, C, M, EPI_F32, status, LiveRows{nullptr, 0})
+                       : gemm_sk_launch(s, false, plan, C, M, EPI_F32, status);
   if (ok) LAUNCHED();
   int hs = 0;
   cudaError_t e1 = cudaMemcpyAsync(&hs, status, sizeof(int), cudaMemcpyDeviceToHost, s);

@@ -187,15 +187,18 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant__
     pdl_sync();
     for (int kb = 0; kb < pre; ++kb)
       tma_load_2d(tiles + kb * stage_bytes + w_bytes, &mapA, (kb_lo + kb) * TC_BK, t0, full0 + 8 * kb);
+    // (stage and phase are counted, not divided out of kb: two divisions by a run-time value cost more
+    // than the rest of a block step's issue)
+    int s = 0;
+    uint32_t ph = 0;
     for (int kb = pre; kb < KB; ++kb) {
-      const int s = kb % stages;
-      const uint32_t ph = (uint32_t)(kb / stages) & 1u;
-      if (!mbar_wait(empty0 + 8 * s, ph ^ 1u)) { atomicExch(status, DEV_TIMEOUT_TMA); break; }
+      if (!mbar_wait(empty0 + 8 * s, ph)) { atomicExch(status, DEV_TIMEOUT_TMA); break; }
       const uint32_t dst = tiles + s * stage_bytes;
       mbar_expect_tx(full0 + 8 * s, (uint32_t)stage_bytes);
       for (int q = 0; q < wt; ++q)
         tma_load_2d(dst + q * TC_W_BYTES, &mapW, (kb_lo + kb) * TC_BK, f0 + q * TC_BM, full0 + 8 * s);
       tma_load_2d(dst + w_bytes, &mapA, (kb_lo + kb) * TC_BK, t0, full0 + 8 * s);
+      if (++s == stages) { s = 0; ph ^= 1u; }
     }
   } else {
     if (NORM && nm.a_out && warp < 4) {
@@ -222,9 +225,9 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant__
     // ---------------- MMA issuer
     const uint32_t idesc = umma_idesc_rt(BN);
     bool ok = true;
+    int s = 0;
+    uint32_t ph = 0;
     for (int kb = 0; kb < KB && ok; ++kb) {
-      const int s = kb % stages;
-      const uint32_t ph = (uint32_t)(kb / stages) & 1u;
       if (!mbar_wait(full0 + 8 * s, ph)) { atomicExch(status, DEV_TIMEOUT_MMA); ok = false; break; }
       tc_fence_after();
       const uint32_t sw = tiles + s * stage_bytes;
@@ -235,6 +238,7 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant__
         if (wt == 2) umma_bf16(tmem + BN, dw2 + 2 * k, da + 2 * k, idesc, (kb | k) ? 1u : 0u);
       }
       umma_commit(empty0 + 8 * s);
+      if (++s == stages) { s = 0; ph ^= 1u; }
     }
     if (ok) umma_commit(accum);
   }
@@ -428,6 +432,8 @@ struct GemmSkPlan {
   CUtensorMap mapW;
   CUtensorMap mapA[16];            // box (BN = 16 * (i + 1)) x 64, encoded on first use
   bool haveA[16] = {false};
+  CUtensorMap mapA2[8];            // box 16 * (i + 1) x 64: one rank's half of a pair's token tile
+  bool haveA2[8] = {false};
   // outputs written by the TMA unit (fp32 residual stream, bf16 activations): one map per
   // (buffer, M, rows per box, element type)
   struct CMap { const void *C; int M, rows; bool is_bf16; CUtensorMap map; };
@@ -466,6 +472,7 @@ static int gemm_sk_plan(GemmSkPlan *plan, const void *W, int N, int K, const voi
   plan->valid = false;
   plan->N = N; plan->K = K; plan->M_max = M_max; plan->A = A;
   for (bool &b : plan->haveA) b = false;
+  for (bool &b : plan->haveA2) b = false;
   plan->mapC.clear();
   if (K % 8 || K < 16 || N < 1 || M_max < 1) return 0;
   if (((uintptr_t)W & 15) || ((uintptr_t)A & 15)) return 0;
@@ -564,6 +571,17 @@ static void gemm_sk_geometry(int N, int K, int M, int epi, int *BN, int *S, int 
   *S = s;
 }
 
+// The map of an output written by the TMA unit (box of `rows` tokens x 128 features), encoded on first use;
+// valid until the next call.
+static const CUtensorMap *sk_map_c(GemmSkPlan &p, void *C, int M, int rows, bool is_bf16) {
+  for (const auto &c : p.mapC)
+    if (c.C == C && c.M == M && c.rows == rows && c.is_bf16 == is_bf16) return &c.map;
+  GemmSkPlan::CMap c{C, M, rows, is_bf16, {}};
+  if (sk_encode_c(&c.map, C, M, p.N, rows, is_bf16)) return nullptr;
+  p.mapC.push_back(c);
+  return &p.mapC.back().map;
+}
+
 static bool gemm_sk_launch(cudaStream_t st, bool pdl, GemmSkPlan &p, void *C, int M, int epi, int *status,
                            const SkNorm *norm = nullptr, LiveRows lr = LiveRows{nullptr, 0}) {
   if (!p.valid || M < 1 || M > p.M_max) return false;
@@ -585,18 +603,8 @@ static bool gemm_sk_launch(cudaStream_t st, bool pdl, GemmSkPlan &p, void *C, in
   }
   const CUtensorMap *mapC = &p.mapW;                         // placeholder when unused
   if (tma_c) {
-    const int rows = BN / S;
-    const bool hb = tma_c == SK_TMA_BF16;
-    const GemmSkPlan::CMap *hit = nullptr;
-    for (const auto &c : p.mapC)
-      if (c.C == C && c.M == M && c.rows == rows && c.is_bf16 == hb) { hit = &c; break; }
-    if (!hit) {
-      GemmSkPlan::CMap c{C, M, rows, hb, {}};
-      if (sk_encode_c(&c.map, C, M, p.N, rows, hb)) return false;
-      p.mapC.push_back(c);
-      hit = &p.mapC.back();
-    }
-    mapC = &hit->map;
+    mapC = sk_map_c(p, C, M, BN / S, tma_c == SK_TMA_BF16);
+    if (!mapC) return false;
   }
   const SkShape sh = sk_shape(BN, (KB + S - 1) / S, S > 1 || tma_c, wt, stg);
   if (sh.smem_bytes > 227 * 1024) return false;

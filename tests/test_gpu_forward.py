@@ -109,6 +109,24 @@ def test_tensor_core_gemm_matches_fp64_product_and_fma_kernel(M, N, K):
     assert np.abs(outs["tc"] - outs["simt"]).max() < 2e-5 * K ** 0.5 + 1e-5
 
 
+@pytest.mark.parametrize("M,N,K", [(512, 256, 128), (513, 128, 64), (600, 256, 80), (777, 640, 128), (1500, 384, 1088), (6000, 1024, 256),
+                                   (9001, 2304, 64)])
+def test_many_token_gemm_matches_fp64_product(M, N, K):
+    """The kernel on pairs of SMs (from 513 tokens): half a feature tile over, K that is no whole block or no whole
+    ring, ragged token tiles, several tiles per pair."""
+    import paper_2511_18191_b200 as tsfm
+    g = torch.Generator(device="cpu").manual_seed(M * 13 + N)
+    A = torch.randn((M, K), generator=g).to(torch.bfloat16)
+    W = (torch.randn((N, K), generator=g) / K ** 0.5).to(torch.bfloat16)
+    Cd = torch.full((M, N), float("nan"), device="cuda")
+    tsfm.tsfm_gemm_bf16(torch.cuda.current_stream().cuda_stream, A.cuda(), W.cuda(), Cd, M, N, K, tsfm.TSFM_GEMM_AUTO)
+    torch.cuda.synchronize()
+    got = Cd.cpu().double()
+    want = A.double() @ W.double().T
+    assert torch.isfinite(got).all()
+    assert (got - want).abs().max() < 2e-5 * K ** 0.5 + 1e-5
+
+
 @pytest.mark.parametrize("M,N,K", [(1, 128, 64), (16, 130, 64), (32, 1536, 512), (33, 96, 128), (40, 512, 192), (64, 384, 1536),
                                    (128, 1152, 384), (31, 512, 2048), (256, 66, 448), (160, 1536, 512)])
 def test_small_batch_gemm_matches_fp64_product(M, N, K):

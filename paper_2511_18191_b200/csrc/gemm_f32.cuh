@@ -10,8 +10,10 @@
 // every weight once per tile of rows instead of once per row or eight rows.
 //   * tile MT tokens x FN features, K in chunks of KC (all of it in one chunk where that fits); the eight
 //     warps take the 4-feature vectors of a chunk in turn (vector w, w + 8, ...), each lane accumulating
-//     (MT / 4) x (FN / 8) outputs in registers; the partial tiles are summed through shared memory in warp
-//     order, so every epilogue sees complete sums and the order of the additions is fixed;
+//     (MT / 4) x (FN / 8) outputs in registers; the partial tiles are summed through shared memory, so
+//     every epilogue sees complete sums.  Vectors of four products are summed before they are added, the eight
+//     partial sums as a tree: short chains of additions keep the rounding error of a sum at that of a
+//     warp-wide tree;
 //   * the norm's factor 1 / sqrt(...) is common to a row: the sums run over gain * A and are scaled at the end;
 //   * rows are padded by 16 bytes: the four token rows and eight feature rows that a warp reads at a
 //     time fall into different banks.
@@ -183,7 +185,7 @@ gemm_f32_kernel(const float *A, const T *__restrict__ W, float *C, int M, int N,
       for (int i = 0; i < RM; ++i)
 #pragma unroll
         for (int j = 0; j < RF; ++j)
-          acc[i][j] = fmaf(a[i].x, b[j].x, fmaf(a[i].y, b[j].y, fmaf(a[i].z, b[j].z, fmaf(a[i].w, b[j].w, acc[i][j]))));
+          acc[i][j] += fmaf(a[i].x, b[j].x, fmaf(a[i].y, b[j].y, fmaf(a[i].z, b[j].z, a[i].w * b[j].w)));
     }
   }
   __syncthreads();                                             // the rows are done with: their space takes the partial tiles
@@ -199,10 +201,10 @@ gemm_f32_kernel(const float *A, const T *__restrict__ W, float *C, int M, int N,
 #pragma unroll
   for (int i = 0; i < OUT; ++i) {
     if (f + i >= N) break;
-    float v = 0.f;
+    float p[8];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) v += f32_smem[k * (MT * FN) + tid * OUT + i];
-    v *= rstd;
+    for (int k = 0; k < 8; ++k) p[k] = f32_smem[k * (MT * FN) + tid * OUT + i];
+    float v = (((p[0] + p[1]) + (p[2] + p[3])) + ((p[4] + p[5]) + (p[6] + p[7]))) * rstd;
     if (ra.epi == EPI_RESID) v += old[i];
     else if (ra.epi == EPI_GELU_T) v = gelu_erf(v);
     if (sampled) {     // proposal x = mu_q + sigma_q eps (Sec. 3.3); the mean is kept for the statistic

@@ -172,8 +172,9 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant__
   tc_fence_after();
   const uint32_t tmem = *slot_ptr;
 
-  float g_direct = 0.f;
   float4 g_vec = make_float4(0.f, 0.f, 0.f, 0.f);
+  constexpr int SK_OLD = 8;                             // rows per thread whose old values are fetched early
+  float4 x_old[NORM ? SK_OLD : 1];
   if (warp == 4 && lane == 0) {
     // ---------------- TMA producer.  The weights do not depend on the preceding kernel: the
     // first ring-full of weight tiles is requested before waiting for it, the activation tiles
@@ -202,19 +203,39 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant__
     }
   } else {
     if (NORM && nm.a_out && warp < 4) {
-      // gains of the features this thread finishes in either epilogue: constants, fetched before the wait
-      const int fd = f0 + threadIdx.x, fv = f0 + (threadIdx.x & 31) * 4;
-      if (fd < N) g_direct = nm.gain[fd];
+      // gains of the features this thread finishes: constants, fetched before the wait
+      const int fv = f0 + (threadIdx.x & 31) * 4;
       if (N % 4 == 0 && fv + 3 < N) g_vec = *reinterpret_cast<const float4 *>(nm.gain + fv);
     }
     pdl_sync();
     if (warp < 4) {
-      if (NORM && nm.ssq_in) {                                // overlaps the main loop
-        for (int i = threadIdx.x; i < BN; i += 128) {
+      if (NORM && nm.ssq_in) {
+        // Four threads per row, 16-byte loads all in flight (d % 64 == 0: whole quads): overlaps the main
+        // loop.  (One thread per row, four bytes at a time, took longer than the loop: K = 1280, 80 slices,
+        // 20 round trips.)
+        const int n4 = nm.n_part >> 2, part = threadIdx.x & 3;
+        for (int i = threadIdx.x >> 2; i < BN; i += 32) {
           float acc = 0.f;
-          if (t0 + i < M)
-            for (int j = 0; j < nm.n_part; ++j) acc += nm.ssq_in[(size_t)(t0 + i) * nm.n_part + j];
-          rs[i] = rsqrtf(acc * nm.inv_d + nm.eps);
+          if (t0 + i < M) {
+            const float4 *src = reinterpret_cast<const float4 *>(nm.ssq_in + (size_t)(t0 + i) * nm.n_part);
+#pragma unroll 8
+            for (int j = part; j < n4; j += 4) {
+              const float4 q = src[j];
+              acc += (q.x + q.y) + (q.z + q.w);
+            }
+          }
+          acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+          acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+          if (part == 0) rs[i] = rsqrtf(acc * nm.inv_d + nm.eps);
+        }
+      }
+      if (NORM && epi == EPI_RESID && N % 4 == 0) {
+        // old values of the rows this thread finishes (part 2 of the epilogue), while the main loop runs
+        const int f = f0 + (threadIdx.x & 31) * 4;
+#pragma unroll
+        for (int i = 0; i < SK_OLD; ++i) {
+          const int tl = rank + S * ((threadIdx.x >> 5) + 4 * i);
+          if (tl < BN && t0 + tl < M && f + 3 < N) x_old[i] = __ldcg(reinterpret_cast<const float4 *>((const float *)C + (size_t)(t0 + tl) * N + f));
         }
       }
       if (NORM) asm volatile("bar.sync 1, 128;" ::: "memory");
@@ -243,7 +264,7 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant__
     if (ok) umma_commit(accum);
   }
   // ---------------- epilogue, part 1: drain the accumulator(s), one weight tile at a time
-  const bool staged = S > 1 || tma_c;                  // through shared memory ([token][128 features] fp32)
+  const bool staged = NORM || S > 1 || tma_c;          // through shared memory ([token][128 features] fp32)
   bool acc_ok = false;
   if (warp < 4) {
     acc_ok = KB > 0 && mbar_wait(accum, 0);
@@ -276,28 +297,8 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant__
 #pragma unroll
           for (int j = 0; j < 16; ++j)
             if (t0 + cc + j < M) {
-              const size_t o = (size_t)(t0 + cc + j) * N + f;
-              if (NORM && nm.ssq_in) v[j] *= rs[cc + j];
-              if (NORM && epi == EPI_RESID && nm.a_out) {
-                const float xn = ((float *)C)[o] + v[j];
-                ((float *)C)[o] = xn;
-                nm.a_out[o] = __float2bfloat16_rn(g_direct * xn);
-                v[j] = xn * xn;
-              } else {
-                sk_store_rt(C, o, v[j], epi);
-              }
+              sk_store_rt(C, (size_t)(t0 + cc + j) * N + f, v[j], epi);
             }
-        }
-        if (NORM && epi == EPI_RESID && nm.a_out) {          // sums of squares over slices of 16 features (N % 32 == 0)
-#pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            float sq = v[j];
-            sq += __shfl_xor_sync(0xffffffffu, sq, 1);
-            sq += __shfl_xor_sync(0xffffffffu, sq, 2);
-            sq += __shfl_xor_sync(0xffffffffu, sq, 4);
-            sq += __shfl_xor_sync(0xffffffffu, sq, 8);
-            if ((lane & 15) == 0 && f < N && t0 + cc + j < M) nm.ssq_out[(size_t)(t0 + cc + j) * (N >> 4) + (f >> 4)] = sq;
-          }
         }
       }
     }
@@ -313,10 +314,12 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant__
     }
   }
   __syncwarp();
-  if (S > 1) {
+  if (S > 1 || NORM) {
     // ---------------- epilogue, part 2: reduce the S partial tiles through distributed shared memory
+    // (folded norms take this form also where K is not split)
     tc_fence_before();
-    cluster_sync_all();
+    if (S > 1) cluster_sync_all();
+    else if (warp < 4) asm volatile("bar.sync 2, 128;" ::: "memory");
     if (warp < 4 && (tma_c == SK_TMA_ADD || tma_c == SK_TMA_F32)) {
       // CTA r sums its block of BN / S rows over the S partial tiles, in place in its own tile,
       // and hands the block to the TMA unit
@@ -359,7 +362,9 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant__
         asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote[r]) : "r"(a), "r"((uint32_t)(r < S ? r : 0)));
       }
       const bool vec = (N % 4 == 0) && (f + 3 < N);
-      for (int tl = rank + S * rg; tl < BN; tl += 4 * S) {
+      int it = 0;
+#pragma unroll 1
+      for (int tl = rank + S * rg; tl < BN; tl += 4 * S, ++it) {
         const int t = t0 + tl;
         if (t >= M) break;
         float4 v[SK_MAX_SPLIT];
@@ -379,7 +384,14 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant__
           if (epi == EPI_F32) {
             *reinterpret_cast<float4 *>((float *)C + o) = sum;
           } else if (epi == EPI_RESID) {
-            float4 old = *reinterpret_cast<float4 *>((float *)C + o);
+            float4 old;
+            if (NORM && it < SK_OLD) {
+#pragma unroll
+              for (int i = 0; i < SK_OLD; ++i)
+                if (i == it) old = x_old[NORM ? i : 0];        // (registers: selected, not indexed)
+            } else {
+              old = *reinterpret_cast<float4 *>((float *)C + o);
+            }
             old.x += sum.x; old.y += sum.y; old.z += sum.z; old.w += sum.w;
             *reinterpret_cast<float4 *>((float *)C + o) = old;
             if (NORM && nm.a_out) {
@@ -414,7 +426,7 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant__
         }
       }
     }
-    cluster_sync_all();          // no CTA leaves while a peer may still read its tile
+    if (S > 1) cluster_sync_all();          // no CTA leaves while a peer may still read its tile
   }
   tc_fence_before();
   __syncthreads();
@@ -606,7 +618,7 @@ static bool gemm_sk_launch(cudaStream_t st, bool pdl, GemmSkPlan &p, void *C, in
     mapC = sk_map_c(p, C, M, BN / S, tma_c == SK_TMA_BF16);
     if (!mapC) return false;
   }
-  const SkShape sh = sk_shape(BN, (KB + S - 1) / S, S > 1 || tma_c, wt, stg);
+  const SkShape sh = sk_shape(BN, (KB + S - 1) / S, S > 1 || tma_c || norm, wt, stg);
   if (sh.smem_bytes > 227 * 1024) return false;
   const int ring_bytes = sh.smem_bytes - 1024 - 256 - 1024;
   const SkNorm nm = norm ? *norm : SkNorm{};

@@ -84,8 +84,14 @@ gemm_ws_kernel(const bf16 *A, const bf16 *__restrict__ W, void *C, int M, int N,
   if (epi == EPI_RESID && live) old = *reinterpret_cast<const float2 *>((const float *)C + (size_t)t * N + f);
   if (NORM && nm.ssq_in) {
     float acc = 0.f;
-    if (t < M)
-      for (int j = tid & 7; j < nm.n_part; j += 8) acc += nm.ssq_in[(size_t)t * nm.n_part + j];
+    if (t < M) {
+      const float4 *src = reinterpret_cast<const float4 *>(nm.ssq_in + (size_t)t * nm.n_part);   // (d % 64 == 0: whole quads)
+#pragma unroll 4
+      for (int j = tid & 7; j < (nm.n_part >> 2); j += 8) {
+        const float4 q = src[j];
+        acc += (q.x + q.y) + (q.z + q.w);
+      }
+    }
     acc += __shfl_xor_sync(0xffffffffu, acc, 1);
     acc += __shfl_xor_sync(0xffffffffu, acc, 2);
     acc += __shfl_xor_sync(0xffffffffu, acc, 4);

@@ -1,4 +1,5 @@
-// Causal attention over a bf16 KV cache with a running softmax (one pass over the keys).
+// Causal attention of passes of at most 16 tokens (one query tile) over a bf16 KV cache with a running softmax
+// (one pass over the keys); longer passes: attn_tiles.cuh.
 //
 // Work unit = one warp: 16 queries (the M side of mma.sync m16n8k16) against a range of keys of
 // one (series, head).  The warp streams its keys in chunks of 32 through a private ring of
@@ -6,19 +7,15 @@
 // running maximum m, the running sum l of exp(s - m) and the unnormalised output o in registers:
 //     m' = max(m, max_t s_t),  l' = l e^(m - m') + sum_t e^(s_t - m'),  o' = o e^(m - m') + sum_t e^(s_t - m') v_t.
 // No block-wide barrier is needed while the keys stream.
-//   mode FLASH_TILES: passes of more than 16 tokens.  kv_append_kernel has put the keys and values
-//              of the pass into the cache; the four warps of a CTA take four consecutive query
-//              tiles (64 queries), each over all keys its queries may see.
-//              grid = (heads, B, ceil(q_len / 64)).
-//   mode FLASH_SPLIT: passes of at most 16 tokens (one query tile), long rows.  The cached keys
+//   mode FLASH_SPLIT: long rows.  The cached keys
 //              [0, pos0) are dealt out over the four warps; the last warp also takes the keys of
 //              the pass itself, which it rotates, rounds, puts into a stage of its ring and
 //              appends to the cache; the four (m, l, o) are merged through shared memory.
 //              grid = (heads, B, 1).
-//   mode FLASH_WARP: the same passes on short rows with many (series, head) pairs: each warp
+//   mode FLASH_WARP: short rows, or many (series, head) pairs: each warp
 //              takes one pair on its own (cached keys, then the keys of the pass).
 //              grid = (ceil(B * heads / 4), 1, 1).
-//   NB = 1, 2 (the last two modes, caches of at most 32 NB rows): a warp's cached keys and the
+//   NB = 1, 2 (caches of at most 32 NB rows): a warp's cached keys and the
 //              keys of the pass share one stage of 32 NB rows and are processed as NB chunks; the
 //              CTA then asks for 8 NB KB per warp (head size 64) instead of a ring of 24 KB, so
 //              that more of these latency-bound warps fit on an SM.  NB = 0: the ring.
@@ -31,11 +28,11 @@
 
 namespace tsfm {
 
-enum { FLASH_WARP = 0, FLASH_TILES = 1, FLASH_SPLIT = 4 };
+enum { FLASH_WARP = 0, FLASH_SPLIT = 4 };
 
 template <int DH, int ST = 3> struct FlashGeom {
   static constexpr int CHUNK = 32;                              // keys per stage
-  static constexpr int STAGES = ST;                             // ring depth (3: prefill tiles; 2: one-tile passes)
+  static constexpr int STAGES = ST;                             // ring depth
   static constexpr int ROW_BYTES = DH * 2;
   static constexpr int TILE_BYTES = CHUNK * ROW_BYTES;          // keys (or values) of one stage
   static constexpr int STAGE_BYTES = 2 * TILE_BYTES;
@@ -65,6 +62,97 @@ __device__ __forceinline__ void flash_cp16(uint32_t dst, const void *src) {
 __device__ __forceinline__ void flash_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N> __device__ __forceinline__ void flash_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
+// 2^x in one instruction (scores are in base-2 units; exp2f adds a range correction for results below 2^-126,
+// which a probability that is rounded to bf16 and summed beside the row's maximum of 1 does not need).
+__device__ __forceinline__ float flash_ex2(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+// One step of the running softmax: 32 keys whose keys sit at shared-memory rows kst.. and values at vst.., for the
+// warp's 16 queries.  mask(s) sets the scores of invisible keys to -inf.  Row addresses for ldmatrix are formed
+// once: 16-byte chunk c of a row sits at chunk c ^ f(row), and f depends on the lane alone, so that every
+// address is one XOR away (key rows: ka, value rows: va, relative to the stage).
+template <int DH> struct FlashLane {
+  uint32_t ka, va;
+  __device__ __forceinline__ FlashLane(int lane) {
+    const int krow = (lane & 7) + ((lane >> 4) & 1) * 8, vrow = (lane & 7) + ((lane >> 3) & 1) * 8;
+    ka = (uint32_t)(krow * DH * 2 + flash_swz<DH>(krow, (lane >> 3) & 1) * 16);
+    va = (uint32_t)(vrow * DH * 2 + flash_swz<DH>(vrow, lane >> 4) * 16);
+  }
+};
+template <int DH, typename Mask>
+__device__ __forceinline__ void flash_step(uint32_t kst, uint32_t vst, const FlashLane<DH> &fl, const uint32_t (&qhi)[DH / 16][4],
+                                           const uint32_t (&qlo)[DH / 16][4], float (&o)[DH / 8][4], float (&m_run)[2],
+                                           float (&l_run)[2], Mask mask) {
+  constexpr int KS = DH / 16, RB = DH * 2;
+  // ---- scores of 16 queries x 32 keys
+  float s[4][4];
+#pragma unroll
+  for (int n = 0; n < 4; ++n) s[n][0] = s[n][1] = s[n][2] = s[n][3] = 0.f;
+  const uint32_t ka = kst + fl.ka;
+#pragma unroll
+  for (int ks = 0; ks < KS; ++ks) {
+    const uint32_t a = ka ^ (uint32_t)(ks * 32);
+    uint32_t b0[4], b1[4];
+    flash_ldsm4(a, b0);
+    flash_ldsm4(a + 16 * RB, b1);
+    mma_bf16_16816(s[0], qhi[ks], b0[0], b0[1]);
+    mma_bf16_16816(s[1], qhi[ks], b0[2], b0[3]);
+    mma_bf16_16816(s[2], qhi[ks], b1[0], b1[1]);
+    mma_bf16_16816(s[3], qhi[ks], b1[2], b1[3]);
+    mma_bf16_16816(s[0], qlo[ks], b0[0], b0[1]);
+    mma_bf16_16816(s[1], qlo[ks], b0[2], b0[3]);
+    mma_bf16_16816(s[2], qlo[ks], b1[0], b1[1]);
+    mma_bf16_16816(s[3], qlo[ks], b1[2], b1[3]);
+  }
+  mask(s);
+  // ---- running softmax
+  uint32_t pa[2][4];
+  float alpha[2];
+#pragma unroll
+  for (int rr = 0; rr < 2; ++rr) {
+    float mx = fmaxf(fmaxf(fmaxf(s[0][rr * 2], s[0][rr * 2 + 1]), fmaxf(s[1][rr * 2], s[1][rr * 2 + 1])),
+                     fmaxf(fmaxf(s[2][rr * 2], s[2][rr * 2 + 1]), fmaxf(s[3][rr * 2], s[3][rr * 2 + 1])));
+    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+    const float m_new = fmaxf(m_run[rr], mx);
+    const float m_use = m_new == -INFINITY ? 0.f : m_new;      // nothing visible yet: every p below is 0
+    alpha[rr] = flash_ex2(m_run[rr] - m_use);
+    m_run[rr] = m_new;
+    float sum = 0.f;
+#pragma unroll
+    for (int n = 0; n < 4; ++n) {
+      const float p0v = flash_ex2(s[n][rr * 2] - m_use), p1v = flash_ex2(s[n][rr * 2 + 1] - m_use);
+      sum += p0v + p1v;
+      pa[n >> 1][(n & 1) * 2 + rr] = pack_bf16x2(p0v, p1v);
+    }
+    l_run[rr] = fmaf(l_run[rr], alpha[rr], sum);
+  }
+  // (a maximum that stays leaves the outputs as they are: factor 1)
+  if (__any_sync(0xffffffffu, !(alpha[0] == 1.f && alpha[1] == 1.f))) {
+#pragma unroll
+    for (int n = 0; n < DH / 8; ++n) {
+      o[n][0] *= alpha[0]; o[n][1] *= alpha[0];
+      o[n][2] *= alpha[1]; o[n][3] *= alpha[1];
+    }
+  }
+  // ---- o += P V
+  const uint32_t va = vst + fl.va;
+#pragma unroll
+  for (int n0 = 0; n0 < DH / 8; n0 += 2) {
+    const uint32_t a = va ^ (uint32_t)(n0 * 16);
+    uint32_t b0[4], b1[4];
+    flash_ldsm4_trans(a, b0);
+    flash_ldsm4_trans(a + 16 * RB, b1);
+    mma_bf16_16816(o[n0], pa[0], b0[0], b0[1]);
+    mma_bf16_16816(o[n0 + 1], pa[0], b0[2], b0[3]);
+    mma_bf16_16816(o[n0], pa[1], b1[0], b1[1]);
+    mma_bf16_16816(o[n0 + 1], pa[1], b1[2], b1[3]);
+  }
+}
+
 template <int DH, int NB, int ST>
 __device__ __forceinline__ void
 attn_flash_body(const float *qkv, bf16 *__restrict__ Kc, bf16 *__restrict__ Vc,
@@ -74,7 +162,7 @@ attn_flash_body(const float *qkv, bf16 *__restrict__ Kc, bf16 *__restrict__ Vc,
   using G = FlashGeom<DH, ST>;
   constexpr int S_TILE = (NB > 0 ? NB : 1) * G::TILE_BYTES;     // key (or value) rows of the single stage
   constexpr int HALF = DH / 2, KS = DH / 16, CPR = DH / 8;     // k-steps of Q K^T, 16-byte chunks per row
-  extern __shared__ __align__(128) unsigned char flash_smem[];
+  extern __shared__ __align__(256) unsigned char flash_smem[];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int gr = lane >> 2, q4 = lane & 3;                     // fragment row group, column pair
   const int d = n_heads * DH;
@@ -89,34 +177,26 @@ attn_flash_body(const float *qkv, bf16 *__restrict__ Kc, bf16 *__restrict__ Vc,
   unsigned char *ring = flash_smem + (size_t)w * warp_bytes;
   const uint32_t ring32 = (uint32_t)__cvta_generic_to_shared(ring);
   const SlotPos sp = slot_lookup(g, slot);                     // before the dependency wait: see SlotPos
-  // Passes of one query tile also start streaming their cached keys before the dependency wait: rows
-  // below pos0 of this layer's cache were written by this layer's attention in an earlier pass, a
-  // whole layer of kernels ago at least.  Passes of several tiles read the rows that the directly
-  // preceding kernel (kv_append_kernel) has just appended: they wait first.
-  if (mode == FLASH_TILES) pdl_sync();
+  // The cached keys start streaming before the dependency wait too: rows below pos0 of this layer's cache were
+  // written by this layer's attention in an earlier pass, a whole layer of kernels ago at least.
   if (sp.dead) return;                                         // per warp (FLASH_WARP) or per CTA: no barrier is pending
   const int b = sp.b, p0 = sp.p0;
   const size_t row0 = (size_t)slot * g.q_len;
   bf16 *Kb = Kc + ((size_t)b * n_heads + h) * g.cap * DH;
   bf16 *Vb = Vc + ((size_t)b * n_heads + h) * g.cap * DH;
 
-  // this warp's queries [jq, jq + 16), cached keys [t_beg, t_end), and whether it takes the
+  // this warp's cached keys [t_beg, t_end), and whether it takes the
   // keys of the pass itself as one more chunk
-  int jq = 0, t_beg = 0, t_end = p0;
+  int t_beg = 0, t_end = p0;
   bool own_pass_keys = true;
-  if (mode == FLASH_TILES) {
-    jq = (blockIdx.z * 4 + w) * 16;
-    if (jq >= g.q_len) return;                                 // no block-wide barrier in this mode
-    t_end = p0 + min(jq + 16, g.q_len);
-    own_pass_keys = false;
-  } else if (mode == FLASH_SPLIT) {
+  if (mode == FLASH_SPLIT) {
     // whole chunks, the keys of the pass counted as one more chunk at the end
     const int R = (((p0 + G::CHUNK - 1) / G::CHUNK + 1 + 3) / 4) * G::CHUNK;
     t_beg = min(w * R, p0);
     t_end = min(t_beg + R, p0);
     own_pass_keys = w == 3;
   }
-  const int nq = min(16, g.q_len - jq);
+  const int nq = g.q_len;
   const int n_c = t_end - t_beg;                               // cached keys of this warp
   const int nch = single ? 0 : (n_c + G::CHUNK - 1) / G::CHUNK;   // chunks that go through the ring
 
@@ -150,7 +230,7 @@ attn_flash_body(const float *qkv, bf16 *__restrict__ Kc, bf16 *__restrict__ Vc,
   // q, k, v of the pass come from the preceding kernel.  They are read with ld.global.cg: their
   // addresses are known before the wait, and a load on the read-only path (what a plain load through
   // a const __restrict__ pointer compiles to) may be scheduled ahead of it.
-  if (mode != FLASH_TILES) pdl_sync();
+  pdl_sync();
 
   // rotated, scaled queries as A fragments (rows gr and gr + 8), high and low bf16 parts
   uint32_t qhi[KS][4], qlo[KS][4];
@@ -158,10 +238,10 @@ attn_flash_body(const float *qkv, bf16 *__restrict__ Kc, bf16 *__restrict__ Vc,
     const float sc = rsqrtf((float)DH) * 1.4426950408889634f;
 #pragma unroll
     for (int rr = 0; rr < 2; ++rr) {
-      const int i = gr + rr * 8, j = jq + i;
+      const int i = gr + rr * 8;
       const bool live = i < nq;
-      const float *src = qkv + (row0 + (live ? j : jq)) * 3 * d + h * DH;
-      const float2 *rp = rope + (size_t)(p0 + (live ? j : jq)) * HALF;
+      const float *src = qkv + (row0 + (live ? i : 0)) * 3 * d + h * DH;
+      const float2 *rp = rope + (size_t)(p0 + (live ? i : 0)) * HALF;
 #pragma unroll
       for (int ks = 0; ks < KS / 2; ++ks)
 #pragma unroll
@@ -183,74 +263,23 @@ attn_flash_body(const float *qkv, bf16 *__restrict__ Kc, bf16 *__restrict__ Vc,
 #pragma unroll
   for (int n = 0; n < DH / 8; ++n) o[n][0] = o[n][1] = o[n][2] = o[n][3] = 0.f;
   float m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};
-  const int qpos0 = p0 + jq + gr;                              // position of row gr; row gr + 8 is 8 further
+  const int qpos0 = p0 + gr;                              // position of row gr; row gr + 8 is 8 further
 
   // one chunk: 32 keys at positions t0.. from the stage at kst (values at vst); keys at or past
   // t_lim, and keys after a query's own position, are masked
+  const FlashLane<DH> fl(lane);
   auto chunk = [&](uint32_t kst, uint32_t vst, int t0, int t_lim) {
-    // ---- scores of 16 queries x 32 keys
-    float s[4][4];
+    flash_step<DH>(kst, vst, fl, qhi, qlo, o, m_run, l_run, [&](float (&s)[4][4]) {
+      if (t0 + G::CHUNK > t_lim || t0 + G::CHUNK - 1 > p0) {   // (only chunks that reach either)
 #pragma unroll
-    for (int n = 0; n < 4; ++n) s[n][0] = s[n][1] = s[n][2] = s[n][3] = 0.f;
+        for (int n = 0; n < 4; ++n)
 #pragma unroll
-    for (int n2 = 0; n2 < 2; ++n2) {
-      const int r = n2 * 16 + (lane & 7) + ((lane >> 4) & 1) * 8;        // key row this lane addresses
-#pragma unroll
-      for (int ks = 0; ks < KS; ++ks) {
-        uint32_t bk[4];
-        flash_ldsm4(kst + (uint32_t)(r * G::ROW_BYTES + flash_swz<DH>(r, ks * 2 + ((lane >> 3) & 1)) * 16), bk);
-        mma_bf16_16816(s[n2 * 2], qhi[ks], bk[0], bk[1]);
-        mma_bf16_16816(s[n2 * 2], qlo[ks], bk[0], bk[1]);
-        mma_bf16_16816(s[n2 * 2 + 1], qhi[ks], bk[2], bk[3]);
-        mma_bf16_16816(s[n2 * 2 + 1], qlo[ks], bk[2], bk[3]);
+          for (int e = 0; e < 4; ++e) {
+            const int t = t0 + n * 8 + q4 * 2 + (e & 1);
+            if (t >= t_lim || t > qpos0 + (e >> 1) * 8) s[n][e] = -INFINITY;
+          }
       }
-    }
-    // ---- causal mask and range end (only chunks that reach either)
-    if (t0 + G::CHUNK > t_lim || t0 + G::CHUNK - 1 > p0 + jq) {
-#pragma unroll
-      for (int n = 0; n < 4; ++n)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const int t = t0 + n * 8 + q4 * 2 + (e & 1);
-          if (t >= t_lim || t > qpos0 + (e >> 1) * 8) s[n][e] = -INFINITY;
-        }
-    }
-    // ---- running softmax
-    uint32_t pa[2][4];
-#pragma unroll
-    for (int rr = 0; rr < 2; ++rr) {
-      float mx = -INFINITY;
-#pragma unroll
-      for (int n = 0; n < 4; ++n) mx = fmaxf(mx, fmaxf(s[n][rr * 2], s[n][rr * 2 + 1]));
-      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-      const float m_new = fmaxf(m_run[rr], mx);
-      const float m_use = m_new == -INFINITY ? 0.f : m_new;    // nothing visible yet: every p below is 0
-      const float alpha = exp2f(m_run[rr] - m_use);
-      m_run[rr] = m_new;
-      float sum = 0.f;
-#pragma unroll
-      for (int n = 0; n < 4; ++n) {
-        const float p0v = exp2f(s[n][rr * 2] - m_use), p1v = exp2f(s[n][rr * 2 + 1] - m_use);
-        sum += p0v + p1v;
-        pa[n >> 1][(n & 1) * 2 + rr] = pack_bf16x2(p0v, p1v);
-      }
-      l_run[rr] = fmaf(l_run[rr], alpha, sum);
-#pragma unroll
-      for (int n = 0; n < DH / 8; ++n) { o[n][rr * 2] *= alpha; o[n][rr * 2 + 1] *= alpha; }
-    }
-    // ---- o += P V
-#pragma unroll
-    for (int kk = 0; kk < 2; ++kk) {
-      const int r = kk * 16 + (lane & 7) + ((lane >> 3) & 1) * 8;
-#pragma unroll
-      for (int n0 = 0; n0 < DH / 8; n0 += 2) {
-        uint32_t bv[4];
-        flash_ldsm4_trans(vst + (uint32_t)(r * G::ROW_BYTES + flash_swz<DH>(r, n0 + (lane >> 4)) * 16), bv);
-        mma_bf16_16816(o[n0], pa[kk], bv[0], bv[1]);
-        mma_bf16_16816(o[n0 + 1], pa[kk], bv[2], bv[3]);
-      }
-    }
+    });
   };
 
   // Keys and values of this pass (at most 16 tokens) first, while the copies of the first cached
@@ -330,7 +359,7 @@ attn_flash_body(const float *qkv, bf16 *__restrict__ Kc, bf16 *__restrict__ Vc,
       const int i = gr + rr * 8;
       if (i >= nq) continue;
       const float inv = 1.f / l_run[rr];
-      uint32_t *dst = reinterpret_cast<uint32_t *>(out + (row0 + jq + i) * d + h * DH);
+      uint32_t *dst = reinterpret_cast<uint32_t *>(out + (row0 + i) * d + h * DH);
 #pragma unroll
       for (int n = 0; n < DH / 8; ++n) dst[n * 4 + q4] = pack_bf16x2(o[n][rr * 2] * inv, o[n][rr * 2 + 1] * inv);
     }
@@ -367,7 +396,7 @@ attn_flash_body(const float *qkv, bf16 *__restrict__ Kc, bf16 *__restrict__ Vc,
       oy = fmaf(ov.y, sc, oy);
     }
     const float inv = 1.f / l;
-    *reinterpret_cast<uint32_t *>(out + (row0 + jq + i) * d + h * DH + c) = pack_bf16x2(ox * inv, oy * inv);
+    *reinterpret_cast<uint32_t *>(out + (row0 + i) * d + h * DH + c) = pack_bf16x2(ox * inv, oy * inv);
   }
 }
 

@@ -1,0 +1,134 @@
+// Causal attention of passes of more than 16 tokens (prefill, scoring, verification of point tokens) over a
+// bf16 KV cache.  kv_append_kernel has put the keys and values of the pass into the cache.
+//
+// A CTA takes up to 64 consecutive queries of one (series, head), 16 per warp (the M side of mma.sync
+// m16n8k16), and streams the keys they may see in tiles of 64 through two shared-memory stages that all its
+// warps read.  (Every warp streaming its own keys, as attn_flash_kernel does for single query tiles, brings
+// each key in four times and leaves room for eight warps on an SM: 166 us for 64 series x 20 heads x 255
+// tokens, 65 us for 16 x 8 x 256 tokens behind 768 to 1000 keys, 44 us for 200 x 16 x 30 tokens; now 122, 52
+// and 27 us.)
+//   * running softmax per query row in registers, 32 keys at a time, as in attn_flash_body: queries split
+//     into bf16 high and low parts, scores in base-2 units, probabilities rounded to bf16 for P V;
+//   * warps skip the half tiles behind their last query; only the rows of a half tile that holds a visible
+//     key are fetched;
+//   * the query blocks with the most keys start first.
+// Bound: latency of a block's first loads and of the mma.sync chains with 16 warps per SM (tensor pipe 40 %
+// busy on the long case).
+// grid = (heads, B, ceil(q_len / (16 warps))), block = 32 x warps, warps = 2 where q_len <= 32, else 4.
+#pragma once
+#include "attn_flash.cuh"
+
+namespace tsfm {
+
+template <int DH> struct TilesGeom {
+  static constexpr int KEYS = 64, HALF_KEYS = 32, ROW_BYTES = DH * 2;
+  static constexpr int TILE_BYTES = KEYS * ROW_BYTES, STAGE_BYTES = 2 * TILE_BYTES, SMEM_BYTES = 2 * STAGE_BYTES;
+};
+
+template <int DH>
+__global__ void __launch_bounds__(128, DH <= 64 ? 4 : 2)
+attn_tiles_kernel(const float *qkv, const bf16 *Kc, const bf16 *Vc, const float2 *__restrict__ rope, PassGeom g, int n_heads,
+                  bf16 *__restrict__ out) {
+  using G = TilesGeom<DH>;
+  constexpr int HALF = DH / 2, KS = DH / 16, CPR = DH / 8;
+  extern __shared__ __align__(256) unsigned char tiles_smem[];
+  const uint32_t ring = (uint32_t)__cvta_generic_to_shared(tiles_smem);
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
+  const int gr = lane >> 2, q4 = lane & 3, d = n_heads * DH;
+  const int h = blockIdx.x, slot = blockIdx.y, qb = (gridDim.z - 1 - blockIdx.z) * n_warps * 16;
+  const SlotPos sp = slot_lookup(g, slot);                     // before the dependency wait: see SlotPos
+  pdl_sync();                                                  // (the rows of the pass come from the preceding kernel)
+  if (sp.dead) return;
+  const int p0 = sp.p0;
+  const size_t row0 = (size_t)slot * g.q_len;
+  const bf16 *Kb = Kc + ((size_t)sp.b * n_heads + h) * g.cap * DH, *Vb = Vc + ((size_t)sp.b * n_heads + h) * g.cap * DH;
+  const int jq = qb + w * 16, nq = min(16, g.q_len - jq);      // this warp's queries (nq <= 0: none)
+  const int n_keys = p0 + min(qb + n_warps * 16, g.q_len);     // keys the block's last query sees
+  const int n_tiles = (n_keys + G::KEYS - 1) / G::KEYS;
+
+  auto issue = [&](int tile) {
+    if (tile < n_tiles) {
+      const int t0 = tile * G::KEYS, rows = min(G::KEYS, (n_keys - t0 + G::HALF_KEYS - 1) & ~(G::HALF_KEYS - 1));
+      const uint32_t kst = ring + (uint32_t)((tile & 1) * G::STAGE_BYTES), vst = kst + G::TILE_BYTES;
+      for (int idx = threadIdx.x; idx < rows * CPR; idx += blockDim.x) {
+        const int r = idx / CPR, ch = idx % CPR;
+        const size_t src = (size_t)min(t0 + r, n_keys - 1) * DH + ch * 8;   // rows past the range repeat its last key (masked below)
+        const uint32_t off = (uint32_t)(r * G::ROW_BYTES + flash_swz<DH>(r, ch) * 16);
+        flash_cp16(kst + off, Kb + src);
+        flash_cp16(vst + off, Vb + src);
+      }
+    }
+    flash_commit();
+  };
+  issue(0);
+
+  // rotated, scaled queries as A fragments (rows gr and gr + 8), high and low bf16 parts
+  uint32_t qhi[KS][4], qlo[KS][4];
+  {
+    const float sc = rsqrtf((float)DH) * 1.4426950408889634f;
+#pragma unroll
+    for (int rr = 0; rr < 2; ++rr) {
+      const int i = gr + rr * 8;
+      const bool live = i < nq;
+      const int j = live ? jq + i : 0;
+      const float *src = qkv + (row0 + j) * 3 * d + h * DH;
+      const float2 *rp = rope + (size_t)(p0 + j) * HALF;
+#pragma unroll
+      for (int ks = 0; ks < KS / 2; ++ks)
+#pragma unroll
+        for (int hh = 0; hh < 2; ++hh) {
+          const int c = ks * 16 + hh * 8 + q4 * 2;             // first-half dims c, c + 1; partners c + HALF
+          const float2 q1 = __ldcg(reinterpret_cast<const float2 *>(src + c));
+          const float2 q2 = __ldcg(reinterpret_cast<const float2 *>(src + c + HALF));
+          const float4 cs = *reinterpret_cast<const float4 *>(rp + c);      // cos0 sin0 cos1 sin1
+          float a0 = (q1.x * cs.x - q2.x * cs.y) * sc, a1 = (q1.y * cs.z - q2.y * cs.w) * sc;
+          float b0 = (q2.x * cs.x + q1.x * cs.y) * sc, b1 = (q2.y * cs.z + q1.y * cs.w) * sc;
+          if (!live) a0 = a1 = b0 = b1 = 0.f;
+          split_bf16x2(a0, a1, qhi[ks][hh * 2 + rr], qlo[ks][hh * 2 + rr]);
+          split_bf16x2(b0, b1, qhi[ks + KS / 2][hh * 2 + rr], qlo[ks + KS / 2][hh * 2 + rr]);
+        }
+    }
+  }
+  float o[DH / 8][4];
+#pragma unroll
+  for (int n = 0; n < DH / 8; ++n) o[n][0] = o[n][1] = o[n][2] = o[n][3] = 0.f;
+  float m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};
+  const int qpos0 = p0 + jq + gr;                              // position of row gr; row gr + 8 is 8 further
+  const FlashLane<DH> fl(lane);
+
+  for (int tile = 0; tile < n_tiles; ++tile) {
+    issue(tile + 1);
+    flash_wait<1>();
+    __syncthreads();
+    const uint32_t stage = ring + (uint32_t)((tile & 1) * G::STAGE_BYTES);
+#pragma unroll 1
+    for (int half = 0; half < 2; ++half) {
+      const int t0 = tile * G::KEYS + half * G::HALF_KEYS;
+      if (nq <= 0 || t0 > p0 + jq + nq - 1) break;             // no key of this half is visible to this warp
+      const uint32_t kst = stage + (uint32_t)(half * G::HALF_KEYS * G::ROW_BYTES), vst = kst + G::TILE_BYTES;
+      flash_step<DH>(kst, vst, fl, qhi, qlo, o, m_run, l_run, [&](float (&s)[4][4]) {
+        if (t0 + G::HALF_KEYS - 1 > p0 + jq) {                 // (only halves that reach past the first query)
+#pragma unroll
+          for (int n = 0; n < 4; ++n)
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+              if (t0 + n * 8 + q4 * 2 + (e & 1) > qpos0 + (e >> 1) * 8) s[n][e] = -INFINITY;
+        }
+      });
+    }
+    __syncthreads();                                           // the stage is free for the tile after next
+  }
+#pragma unroll
+  for (int rr = 0; rr < 2; ++rr) {
+    l_run[rr] += __shfl_xor_sync(0xffffffffu, l_run[rr], 1);
+    l_run[rr] += __shfl_xor_sync(0xffffffffu, l_run[rr], 2);
+    const int i = gr + rr * 8;
+    if (i >= nq) continue;
+    const float inv = 1.f / l_run[rr];
+    uint32_t *dst = reinterpret_cast<uint32_t *>(out + (row0 + jq + i) * d + h * DH);
+#pragma unroll
+    for (int n = 0; n < DH / 8; ++n) dst[n * 4 + q4] = pack_bf16x2(o[n][rr * 2] * inv, o[n][rr * 2 + 1] * inv);
+  }
+}
+
+}  // namespace tsfm

@@ -19,6 +19,7 @@
 #include "common.cuh"
 #include "kernels_simt.cuh"
 #include "attn_flash.cuh"
+#include "attn_tiles.cuh"
 #include "accept.cuh"
 #include "gemm_tc.cuh"
 #include "gemm_sk.cuh"
@@ -313,7 +314,7 @@ constexpr int kFlashWarpLongMinPairs = 1024;
 // one-tile passes: a two-stage ring (each warp has a few chunks only, and a third CTA fits on the SM)
 constexpr int kFlashStShort = 2;
 template <int DH> int flash_set_attr() {
-  CU_TRY(cudaFuncSetAttribute(attn_flash_kernel<DH, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, FlashGeom<DH, 3>::SMEM_BYTES));
+  CU_TRY(cudaFuncSetAttribute(attn_tiles_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, TilesGeom<DH>::SMEM_BYTES));
   CU_TRY(cudaFuncSetAttribute(attn_flash_kernel<DH, kFlashStShort>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               FlashGeom<DH, kFlashStShort>::SMEM_BYTES));
   CU_TRY(cudaFuncSetAttribute(attn_flash_single_kernel<DH, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, FlashGeom<DH>::single_bytes(1)));
@@ -373,11 +374,11 @@ void prefer_max_smem_all() {
   prefer_max_smem(gemm_pair_kernel);
   prefer_max_smem(gemm_ws_kernel<false>);
   prefer_max_smem(gemm_ws_kernel<true>);
-  prefer_max_smem(attn_flash_kernel<32, 3>);
+  prefer_max_smem(attn_tiles_kernel<32>);
   prefer_max_smem(attn_flash_kernel<32, kFlashStShort>);
-  prefer_max_smem(attn_flash_kernel<64, 3>);
+  prefer_max_smem(attn_tiles_kernel<64>);
   prefer_max_smem(attn_flash_kernel<64, kFlashStShort>);
-  prefer_max_smem(attn_flash_kernel<128, 3>);
+  prefer_max_smem(attn_tiles_kernel<128>);
   prefer_max_smem(attn_flash_kernel<128, kFlashStShort>);
   prefer_max_smem(attn_flash_single_kernel<32, 1>);
   prefer_max_smem(attn_flash_single_kernel<32, 2>);
@@ -518,22 +519,24 @@ void launch_attn(tsfm_spec *h, ModelDev &m, int l, int B, const PassGeom &g) {
               h->qkv, Kc, Vc, m.rope, g, m.arch.n_heads);
   if constexpr (sizeof(T) == 2) {
     const int pairs = B * m.arch.n_heads;
-    const int mode = pre ? FLASH_TILES
-                         : ((h->cap <= kFlashWarpMaxCap && pairs >= kFlashWarpMinPairs) || pairs >= kFlashWarpLongMinPairs)
-                               ? FLASH_WARP : FLASH_SPLIT;
-    const dim3 grid = mode == FLASH_WARP ? dim3((pairs + 3) / 4)
-                                         : dim3(m.arch.n_heads, B, pre ? (g.q_len + 4 * ATTN_QT - 1) / (4 * ATTN_QT) : 1);
+    if (pre) {
+      const int warps = g.q_len <= 32 ? 2 : 4;
+      launch_ex(h->ls, h->pdl, attn_tiles_kernel<DH>, dim3(m.arch.n_heads, B, (g.q_len + 16 * warps - 1) / (16 * warps)),
+                dim3(32 * warps), (size_t)TilesGeom<DH>::SMEM_BYTES, h->qkv, (const bf16 *)Kc, (const bf16 *)Vc, m.rope, g,
+                m.arch.n_heads, (bf16 *)h->ao);
+      return;
+    }
+    const int mode = ((h->cap <= kFlashWarpMaxCap && pairs >= kFlashWarpMinPairs) || pairs >= kFlashWarpLongMinPairs)
+                         ? FLASH_WARP : FLASH_SPLIT;
+    const dim3 grid = mode == FLASH_WARP ? dim3((pairs + 3) / 4) : dim3(m.arch.n_heads, B);
     // short caches: one stage of 32 or 64 rows per warp instead of the ring, more warps per SM
-    const int nb = pre ? 0 : h->cap <= FlashGeom<DH>::CHUNK ? 1 : h->cap <= 2 * FlashGeom<DH>::CHUNK ? 2 : 0;
+    const int nb = h->cap <= FlashGeom<DH>::CHUNK ? 1 : h->cap <= 2 * FlashGeom<DH>::CHUNK ? 2 : 0;
     if (nb == 1)
       launch_ex(h->ls, h->pdl, attn_flash_single_kernel<DH, 1>, grid, dim3(128), (size_t)FlashGeom<DH>::single_bytes(1),
                 h->qkv, (bf16 *)Kc, (bf16 *)Vc, m.rope, g, m.arch.n_heads, pairs, mode, (bf16 *)h->ao);
     else if (nb == 2)
       launch_ex(h->ls, h->pdl, attn_flash_single_kernel<DH, 2>, grid, dim3(128), (size_t)FlashGeom<DH>::single_bytes(2),
                 h->qkv, (bf16 *)Kc, (bf16 *)Vc, m.rope, g, m.arch.n_heads, pairs, mode, (bf16 *)h->ao);
-    else if (pre)
-      launch_ex(h->ls, h->pdl, attn_flash_kernel<DH, 3>, grid, dim3(128), (size_t)FlashGeom<DH, 3>::SMEM_BYTES, h->qkv,
-                (bf16 *)Kc, (bf16 *)Vc, m.rope, g, m.arch.n_heads, pairs, mode, (bf16 *)h->ao);
     else      // one query tile: each warp has a few chunks only, a two-stage ring lets a third CTA onto the SM
       launch_ex(h->ls, h->pdl, attn_flash_kernel<DH, kFlashStShort>, grid, dim3(128),
                 (size_t)FlashGeom<DH, kFlashStShort>::SMEM_BYTES, h->qkv, (bf16 *)Kc, (bf16 *)Vc, m.rope, g,

@@ -77,6 +77,18 @@ def test_bf16_forward_matches_oracle(backend, target, draft, P, n, mode):
     assert parity.value_error("rel_rms", gd, wd) < 2e-2
 
 
+@pytest.mark.parametrize("n", [17, 32, 33, 64, 65, 129])
+def test_bf16_attention_tiles_of_queries_and_keys(n):
+    """Passes of more than 16 tokens: edges of the 16-query warps, of the two- and four-warp blocks, of the 32-key
+    halves and 64-key tiles; head sizes 64 (target) and 32 (draft)."""
+    wl = small_workload("bf16", Arch(1, 128, 2, 128), Arch(1, 128, 4, 128), 32)
+    gt, wt, gd, wd = run_forward_case(wl, 0, n)
+    for got, want in ((gt, wt), (gd, wd)):
+        assert np.isfinite(got).all()
+        for b in range(got.shape[0]):          # as below: bf16 operands, relative rms 3e-2
+            assert np.sqrt(np.mean((got[b] - want[b]) ** 2)) <= 3e-2 * np.sqrt(np.mean(want[b] ** 2))
+
+
 @pytest.mark.parametrize("dtype,P,P_in,n", [("f32", 16, 1, 70), ("f32", 32, 8, 19), ("bf16", 64, 1, 300), ("bf16", 32, 16, 40)])
 def test_forward_with_input_tokens_shorter_than_the_patch(dtype, P, P_in, n):
     """Embedding of P_in-step tokens ([d, P_in] weights; 16-byte loads or element by element) under a

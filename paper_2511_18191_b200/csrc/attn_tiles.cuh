@@ -1,5 +1,7 @@
 // Causal attention of passes of more than 16 tokens (prefill, scoring, verification of point tokens) over a
-// bf16 KV cache.  kv_append_kernel has put the keys and values of the pass into the cache.
+// bf16 KV cache.  The keys and values of the pass are in the cache: the QKV contraction put them there and
+// rotated and scaled the queries (rotated = 1, see PairRope), or kv_append_kernel did (rotated = 0: the queries
+// are rotated here).
 //
 // A CTA takes up to 64 consecutive queries of one (series, head), 16 per warp (the M side of mma.sync
 // m16n8k16), and streams the keys they may see in tiles of 64 through two shared-memory stages that all its
@@ -28,7 +30,7 @@ template <int DH> struct TilesGeom {
 template <int DH>
 __global__ void __launch_bounds__(128, DH <= 64 ? 4 : 2)
 attn_tiles_kernel(const float *qkv, const bf16 *Kc, const bf16 *Vc, const float2 *__restrict__ rope, PassGeom g, int n_heads,
-                  bf16 *__restrict__ out) {
+                  int rotated, bf16 *__restrict__ out) {
   using G = TilesGeom<DH>;
   constexpr int HALF = DH / 2, KS = DH / 16, CPR = DH / 8;
   extern __shared__ __align__(256) unsigned char tiles_smem[];
@@ -80,9 +82,11 @@ attn_tiles_kernel(const float *qkv, const bf16 *Kc, const bf16 *Vc, const float2
           const int c = ks * 16 + hh * 8 + q4 * 2;             // first-half dims c, c + 1; partners c + HALF
           const float2 q1 = __ldcg(reinterpret_cast<const float2 *>(src + c));
           const float2 q2 = __ldcg(reinterpret_cast<const float2 *>(src + c + HALF));
-          const float4 cs = *reinterpret_cast<const float4 *>(rp + c);      // cos0 sin0 cos1 sin1
+          float4 cs = make_float4(0.f, 0.f, 0.f, 0.f);                     // cos0 sin0 cos1 sin1
+          if (!rotated) cs = *reinterpret_cast<const float4 *>(rp + c);
           float a0 = (q1.x * cs.x - q2.x * cs.y) * sc, a1 = (q1.y * cs.z - q2.y * cs.w) * sc;
           float b0 = (q2.x * cs.x + q1.x * cs.y) * sc, b1 = (q2.y * cs.z + q1.y * cs.w) * sc;
+          if (rotated) { a0 = q1.x; a1 = q1.y; b0 = q2.x; b1 = q2.y; }
           if (!live) a0 = a1 = b0 = b1 = 0.f;
           split_bf16x2(a0, a1, qhi[ks][hh * 2 + rr], qlo[ks][hh * 2 + rr]);
           split_bf16x2(b0, b1, qhi[ks + KS / 2][hh * 2 + rr], qlo[ks + KS / 2][hh * 2 + rr]);

@@ -127,4 +127,48 @@ __device__ __forceinline__ float gelu_erf_fast(float v) {
   return v * (v >= 0.f ? 1.0f - half_erfc : half_erfc);
 }
 
+// Two of them at once, rounded to bf16 (low half: a), for the epilogues of many tokens, whose pace is set by the
+// instructions of this function: packed fp32 arithmetic (two values per instruction), and
+// v Phi(v) = max(v, 0) - |v| erfc(|v| / sqrt(2)) / 2 on both sides, so that nothing is selected.
+__device__ __forceinline__ uint64_t f32x2(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ uint32_t gelu_erf_fast2(float a, float b) {
+  const uint64_t v = f32x2(fabsf(a), fabsf(b));
+  const uint64_t w = fma2(v, f32x2(0.3275911f * 0.70710678118654752440f, 0.3275911f * 0.70710678118654752440f), f32x2(1.f, 1.f));
+  float w0, w1, t0, t1, e0, e1;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(w0), "=f"(w1) : "l"(w));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t0) : "f"(w0));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t1) : "f"(w1));
+  const uint64_t t = f32x2(t0, t1);
+  // the coefficients of A&S 7.1.26, halved
+  uint64_t p = fma2(t, f32x2(0.5f * 1.061405429f, 0.5f * 1.061405429f), f32x2(0.5f * -1.453152027f, 0.5f * -1.453152027f));
+  p = fma2(t, p, f32x2(0.5f * 1.421413741f, 0.5f * 1.421413741f));
+  p = fma2(t, p, f32x2(0.5f * -0.284496736f, 0.5f * -0.284496736f));
+  p = fma2(t, p, f32x2(0.5f * 0.254829592f, 0.5f * 0.254829592f));
+  // exp(-v^2 / 2) = 2^(-(log2(e) / 2) v^2)
+  const uint64_t x = mul2(mul2(v, f32x2(-0.72134752044448170368f, -0.72134752044448170368f)), v);
+  float x0, x1;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(x0), "=f"(x1) : "l"(x));
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e0) : "f"(x0));
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e1) : "f"(x1));
+  const uint64_t he = mul2(mul2(t, p), f32x2(e0, e1));         // erfc / 2
+  float h0, h1;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(h0), "=f"(h1) : "l"(he));
+  const __nv_bfloat162 r = __floats2bfloat162_rn(fmaf(-fabsf(a), h0, fmaxf(a, 0.f)), fmaf(-fabsf(b), h1, fmaxf(b, 0.f)));
+  return *reinterpret_cast<const uint32_t *>(&r);
+}
+
 }  // namespace tsfm

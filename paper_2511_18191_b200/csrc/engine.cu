@@ -447,12 +447,17 @@ void launch_gemm_simt(cudaStream_t s, bool pdl, const T *A, const T *W, void *C,
 // M = 6000, d = 1024: 32 / 47, 16 / 21, 47 / 74, 43 / 61).
 constexpr int kPairMinRows = 513;
 
+// Up to this many tokens their norms are folded in as well: the epilogues that do it cost 1 us per contraction at
+// 576 to 2048 tokens, where an RMSNorm launch is a link of 4 us, and 3 to 6 us at 6000 (scoring, d = 1024: 153 us a
+// layer folded, 136 + 2 x 8 with the kernel).
+constexpr int kPairFoldMaxRows = 3072;
+
 // C (op)= A . W^T through the tensor-core kernel when a plan exists, else an FMA kernel.  row_gain (fp32
 // models whose rows gemm_f32_kernel takes): A is the residual stream, normalised by the contraction itself.
 template <typename T>
 void gemm(tsfm_spec *h, GemmSkPlan *plan, const void *A, const void *W, void *C, int M, int N,
           int K, int epi, const SkNorm *norm = nullptr, LiveRows lr = LiveRows{nullptr, 0},
-          const float *row_gain = nullptr, float eps = 0.f) {
+          const float *row_gain = nullptr, float eps = 0.f, const PairRope *rope = nullptr) {
   const double e = sizeof(T);
   const double out_b = (epi == EPI_F32 || epi == EPI_ATOMIC) ? 4.0 : epi == EPI_RESID ? 8.0 : e;
   const double bytes = ((double)N * K + (double)M * K) * e + (double)M * N * out_b;
@@ -470,8 +475,8 @@ void gemm(tsfm_spec *h, GemmSkPlan *plan, const void *A, const void *W, void *C,
   }
   if (sizeof(T) == 2 && h->use_tc && plan && plan->valid) {
     KTimer kt(h, M <= 512 ? KC_GEMM_TC_SMALL : M < 4096 ? KC_GEMM_TC_MID : KC_GEMM_TC_LARGE, bytes, flops);
-    const bool pair = !norm && M >= kPairMinRows && gemm_pair_eligible(*plan, C);
-    if (pair ? gemm_pair_launch(h->ls, h->pdl, *plan, C, M, epi, h->dev_status, lr)
+    const bool pair = M >= kPairMinRows && gemm_pair_eligible(*plan, C);
+    if (pair ? gemm_pair_launch(h->ls, h->pdl, *plan, C, M, epi, h->dev_status, lr, norm, rope)
              : gemm_sk_launch(h->ls, h->pdl, *plan, C, M, epi, h->dev_status, norm, lr)) {
       LAUNCHED();
     } else if (h->enqueue_err == TSFM_OK) {
@@ -503,8 +508,10 @@ void gemm(tsfm_spec *h, GemmSkPlan *plan, const void *A, const void *W, void *C,
   launch_gemm_simt<T>(h->ls, h->pdl, (const T *)A, (const T *)W, C, M, N, K, epi);
 }
 
+// appended: the QKV contraction has rotated the queries and put the pass's keys and values into the cache;
+// cache_only: nothing reads the attention's output (last layer of a prefill).
 template <typename T, int DH>
-void launch_attn(tsfm_spec *h, ModelDev &m, int l, int B, const PassGeom &g) {
+void launch_attn(tsfm_spec *h, ModelDev &m, int l, int B, const PassGeom &g, bool appended, bool cache_only) {
   T *Kc = (T *)m.Kc + (size_t)l * m.kv_layer_elems;
   T *Vc = (T *)m.Vc + (size_t)l * m.kv_layer_elems;
   // algorithmic bytes: q/k/v of the pass + the cached keys and values (lower bound: done = 0)
@@ -514,16 +521,17 @@ void launch_attn(tsfm_spec *h, ModelDev &m, int l, int B, const PassGeom &g) {
             4.0 * Mr * (std::max(g.base, 0) + 0.5 * g.q_len) * m.arch.d_model);
   // several query tiles: the pass's keys and values go to the cache first, once
   const int pre = g.q_len > ATTN_QT ? 1 : 0;
-  if (pre)
+  if (pre && !appended)
     launch_ex(h->ls, h->pdl, kv_append_kernel<T, DH>, dim3(m.arch.n_heads, B, (g.q_len + 15) / 16), dim3(128), 0,
               h->qkv, Kc, Vc, m.rope, g, m.arch.n_heads);
+  if (pre && cache_only) return;
   if constexpr (sizeof(T) == 2) {
     const int pairs = B * m.arch.n_heads;
     if (pre) {
       const int warps = g.q_len <= 32 ? 2 : 4;
       launch_ex(h->ls, h->pdl, attn_tiles_kernel<DH>, dim3(m.arch.n_heads, B, (g.q_len + 16 * warps - 1) / (16 * warps)),
                 dim3(32 * warps), (size_t)TilesGeom<DH>::SMEM_BYTES, h->qkv, (const bf16 *)Kc, (const bf16 *)Vc, m.rope, g,
-                m.arch.n_heads, (bf16 *)h->ao);
+                m.arch.n_heads, appended ? 1 : 0, (bf16 *)h->ao);
       return;
     }
     const int mode = ((h->cap <= kFlashWarpMaxCap && pairs >= kFlashWarpMinPairs) || pairs >= kFlashWarpLongMinPairs)
@@ -577,18 +585,17 @@ void run_pass(tsfm_spec *h, ModelDev &m, int B, const PassGeom &g, int head_mode
   const int M = B * g.q_len, d = m.arch.d_model, f = m.arch.d_ff, P = h->cfg.patch_len, Pi = h->P_in;
   cudaStream_t s = h->ls;
   const float eps = h->cfg.rms_eps;
-  // On the tensor-core path the RMSNorms are folded into the contractions around them (SkNorm):
-  // whoever produces the residual stream also writes the next operand a' = bf16(gain * x) and the
-  // rows' slice sums of squares; whoever consumes a' scales its result rows by rstd.
-  // (Only for passes of few tokens, where a launch costs more than the extra epilogue work: with
-  // large tiles the epilogue is the bottleneck and the separate RMSNorm kernel is the cheaper way.)
-  // On the bf16 path the RMSNorms of passes of up to 512 tokens are folded into the contractions
-  // around them (SkNorm): whoever produces the residual stream also writes the next operand
-  // a' = bf16(gain * x) and the rows' sums of squares over 16-feature slices; whoever consumes a'
-  // scales its result rows by rstd.  (Only for few tokens, where a launch costs more than the extra
-  // epilogue work.  With the large tiles' TMA epilogues a producer would have to load its block of x
-  // back after the reduction: measured on C2-C4, that costs what the RMSNorm kernel costs.)
-  const bool fold = sizeof(T) == 2 && h->use_tc && m.layers[0].tc_qkv.valid && M <= 512;
+  // On the bf16 path the RMSNorms are folded into the contractions around them (SkNorm): whoever
+  // produces the residual stream also writes the next operand a' = bf16(gain * x) and the rows' sums
+  // of squares over slices of features (16 up to 512 tokens, 128 on pairs of SMs); whoever consumes a'
+  // scales its result rows by rstd.  On pairs of SMs the first norm of a pass, which follows the
+  // embedding, stays a kernel of its own.
+  const bool fold = sizeof(T) == 2 && h->use_tc && m.layers[0].tc_qkv.valid && M < kPairMinRows;
+  const bool on_pairs = sizeof(T) == 2 && h->use_tc && M >= kPairMinRows && d % TC_BM == 0 && f % TC_BM == 0 &&
+                        m.layers[0].tc_qkv.valid;
+  const bool fold_pair = on_pairs && M <= kPairFoldMaxRows;
+  // the QKV contraction of a pass of several query tiles rotates its queries and appends to the cache
+  const bool append = on_pairs && g.q_len > ATTN_QT;
   // fp32 models with rows short enough normalise them inside the contraction that reads them.
   const bool fold32 = sizeof(T) == 4 && gemm_f32_eligible(m.layers[0].Wqkv, d);
   const int L = m.arch.n_layers;
@@ -624,35 +631,46 @@ void run_pass(tsfm_spec *h, ModelDev &m, int B, const PassGeom &g, int head_mode
   const double norm_bytes = (double)M * d * (4 + sizeof(T)) + d * 4.0;
   SkNorm consume{};                 // scale the result rows by rstd of the input rows
   consume.ssq_in = h->ssq;
-  consume.n_part = d / 16;
+  consume.n_part = fold_pair ? d / TC_BM : d / 16;
   consume.inv_d = 1.f / d;
   consume.eps = eps;
   for (int l = 0; l < L; ++l) {
     LayerDev &ly = m.layers[l];
-    if (!fold && !fold32) {
+    if (!fold && !fold32 && !(fold_pair && l > 0)) {
       KTimer kt(h, KC_RMSNORM, norm_bytes, 3.0 * M * d);
       launch_ex(s, h->pdl, norm_kernel, dim3((M + 7) / 8), dim3(256), 0, h->x, ly.g1, M, d, eps, (T *)h->a, lr);
     }
+    PairRope pr{};
+    if (append) {
+      pr.rope = m.rope;
+      pr.Kc = (bf16 *)m.Kc + (size_t)l * m.kv_layer_elems;
+      pr.Vc = (bf16 *)m.Vc + (size_t)l * m.kv_layer_elems;
+      pr.g = g;
+      pr.n_heads = m.arch.n_heads;
+      pr.dh = m.dh;
+    }
     gemm<T>(h, &ly.tc_qkv, fold32 ? (const void *)h->x : h->a, ly.Wqkv, h->qkv, M, 3 * d, d, EPI_F32,
-            fold ? &consume : nullptr, lr, fold32 ? ly.g1 : nullptr, eps);
-    if (m.dh == 32) launch_attn<T, 32>(h, m, l, B, g);
-    else if (m.dh == 64) launch_attn<T, 64>(h, m, l, B, g);
-    else launch_attn<T, 128>(h, m, l, B, g);
-    if (l == L - 1 && head_mode == HEAD_NONE) break;   // prefill: only the cache is needed
+            fold || (fold_pair && l > 0) ? &consume : nullptr, lr, fold32 ? ly.g1 : nullptr, eps, append ? &pr : nullptr);
+    const bool cache_only = l == L - 1 && head_mode == HEAD_NONE;      // prefill: only the cache is needed
+    if (m.dh == 32) launch_attn<T, 32>(h, m, l, B, g, append, cache_only);
+    else if (m.dh == 64) launch_attn<T, 64>(h, m, l, B, g, append, cache_only);
+    else launch_attn<T, 128>(h, m, l, B, g, append, cache_only);
+    if (cache_only) break;
     SkNorm produce{};               // residual epilogue also emits the next operand and its statistics
     produce.ssq_out = h->ssq;
     produce.a_out = (bf16 *)h->a;
     produce.gain = ly.g2;
-    gemm<T>(h, &ly.tc_o, h->ao, ly.Wo, h->x, M, d, d, EPI_RESID, fold ? &produce : nullptr, lr);
-    if (!fold && !fold32) {
+    gemm<T>(h, &ly.tc_o, h->ao, ly.Wo, h->x, M, d, d, EPI_RESID, fold || fold_pair ? &produce : nullptr, lr);
+    if (!fold && !fold32 && !fold_pair) {
       KTimer kt(h, KC_RMSNORM, norm_bytes, 3.0 * M * d);
       launch_ex(s, h->pdl, norm_kernel, dim3((M + 7) / 8), dim3(256), 0, h->x, ly.g2, M, d, eps, (T *)h->a, lr);
     }
     gemm<T>(h, &ly.tc_1, fold32 ? (const void *)h->x : h->a, ly.W1, h->hbuf, M, f, d, EPI_GELU_T,
-            fold ? &consume : nullptr, lr, fold32 ? ly.g2 : nullptr, eps);
+            fold || fold_pair ? &consume : nullptr, lr, fold32 ? ly.g2 : nullptr, eps);
     produce.gain = l + 1 < L ? m.layers[l + 1].g1 : nullptr;
     if (l + 1 == L) produce.a_out = nullptr, produce.ssq_out = nullptr;   // the head kernel norms the final rows itself
-    gemm<T>(h, &ly.tc_2, h->hbuf, ly.W2, h->x, M, d, f, EPI_RESID, fold && l + 1 < L ? &produce : nullptr, lr);
+    gemm<T>(h, &ly.tc_2, h->hbuf, ly.W2, h->x, M, d, f, EPI_RESID, (fold || fold_pair) && l + 1 < L ? &produce : nullptr,
+            lr);
   }
   const int Mb = B * (g.q_len / g.head_step);          // boundary rows the head reads (verification)
   const double rows = head_mode == HEAD_LAST_TO_HIST ? B : Mb;

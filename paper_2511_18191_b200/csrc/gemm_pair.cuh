@@ -12,19 +12,31 @@
 //     commits arrive at both ranks' (no copy is multicast);
 //   * persistent: pairs walk the tiles; with two accumulators (2 BN <= 512 columns) the epilogue of a tile
 //     runs under the main loop of the next;
-//   * 8 epilogue warps in two groups take 32-token chunks in turn: tcgen05.ld, conversion, staged as
-//     [token][128 features] and written (fp32, bf16, GELU -> bf16) or added to x by the TMA unit.
-// Warps 0-7 epilogue, 8 TMA producer, 9 tensor-memory allocation and MMA issue.  Waits are bounded as in
-// gemm_tc.cuh.
+//   * 16 epilogue warps in four groups take 16-token chunks in turn: tcgen05.ld, conversion, staged as
+//     [token][128 features] and written (fp32, bf16, GELU -> bf16) or added to x by the TMA unit;
+//   * RMSNorms can be folded in (SkNorm; slices of 128 features): a residual epilogue fetches the old rows
+//     while the main loop runs, and emits x, the next operand bf16(gain x) and the rows' sums of squares; a
+//     consumer scales its rows.  Used where an RMSNorm launch costs more than that (kPairFoldMaxRows);
+//   * the QKV contraction of a pass of several query tiles rotates its queries and keys and puts keys and
+//     values into the cache as bf16 (PairRope): 43 us instead of 34 + 14 (kv_append_kernel) at 6000 x 1024,
+//     142 instead of 132 + 47 at 16320 x 1280.
+// Graph replay of dependent launches, gemm_sk_kernel -> this one: M = 16320, d = 1280: QKV 158 -> 118 us
+// (1355 TFLOP/s), W1 with GELU 254 -> 160, W2 175 -> 149, Wo 67 -> 50; M = 6000, d = 1024: 47 -> 34, 74 -> 40,
+// 61 -> 44, 21 -> 16.
+// Warps 0-15 epilogue, 16 TMA producer, 17 tensor-memory allocation and MMA issue, 18-19 the rows' factors and
+// cache positions of the next tile.  (With 8 epilogue warps the folded forms, a chain of latencies per chunk, set
+// the pace: QKV of 6000 x 1024 60 us.)  Waits are bounded as in gemm_tc.cuh.
 #pragma once
 #include "gemm_sk.cuh"
 
 namespace tsfm {
 
-constexpr int PAIR_CHUNK = 32;                   // tokens per epilogue chunk
-constexpr int PAIR_THREADS = 320;
+constexpr int PAIR_CHUNK = 16;                   // tokens per epilogue chunk
+constexpr int PAIR_GROUPS = 4, PAIR_EPI_WARPS = 4 * PAIR_GROUPS, PAIR_ROW_WARPS = 2;
+constexpr int PAIR_THREADS = 32 * (PAIR_EPI_WARPS + 2 + PAIR_ROW_WARPS);
 constexpr int PAIR_MAX = 74;                     // pairs of SMs on the device
 constexpr int PAIR_STAGE_OUT = PAIR_CHUNK * TC_BM * 4;   // staging per epilogue group
+constexpr int PAIR_ROW_BYTES = 2 * 256 * (4 + 8);        // factors and cache positions of two tiles' rows
 
 __device__ __forceinline__ bool elect_one() {
   uint32_t p;
@@ -49,6 +61,9 @@ __device__ __forceinline__ void umma_commit_pair(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
                ::"r"(bar), "h"((uint16_t)3) : "memory");
 }
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
 __device__ __forceinline__ void mbar_arrive_rank0(uint32_t bar) {
   uint32_t remote;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(bar), "r"(0u));
@@ -69,28 +84,69 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity)
     if (it > 256 && (it & 255) == 0 && globaltimer_ns() - t0 > TC_WAIT_NS) return false;
   }
 }
-// 32 consecutive columns of this thread's lane.
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float *v) {
-  uint32_t r[32];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-      "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr) : "memory");
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+// Rotary positions and cache append of a QKV contraction (N = 3 d, d % 128 == 0): features [0, d) become
+// rotated queries, scaled for base-2 softmax, fp32 in C; [d, 2 d) rotated keys and [2 d, 3 d) values go to the
+// cache only.
+struct PairRope {
+  const float2 *rope;              // [cap][dh / 2], NULL: an ordinary contraction
+  bf16 *Kc, *Vc;                   // this layer's cache [B][heads][cap][dh]
+  PassGeom g;
+  int n_heads, dh;
+};
+
+// Four rows of a staged chunk (one warp): queries and keys rotated, queries to C, keys and values to the cache.
+// A lane takes both members of two rotation pairs; cs holds their table entries, fetched a chunk ahead (a round
+// trip to L2 per chunk otherwise).
+struct PairRopeLane {
+  int dim, hl, lph;                // first of the lane's two dims below dh / 2; first feature of its head in the tile
+  __device__ __forceinline__ PairRopeLane(int lane, int dh) {
+    lph = dh >> 2;
+    dim = (lane & (lph - 1)) * 2;
+    hl = (lane / lph) * dh;
+  }
+};
+__device__ __forceinline__ void pair_rope_fetch(float4 (&cs)[PAIR_CHUNK / 4], const int2 *pos, int w4, int t0, int M, int half, int dim,
+                                                const float2 *rope) {
 #pragma unroll
-  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+  for (int r = 0; r < PAIR_CHUNK / 4; ++r) {
+    const int tl = w4 * (PAIR_CHUNK / 4) + r;
+    cs[r] = make_float4(1.f, 0.f, 1.f, 0.f);
+    if (t0 + tl < M) cs[r] = *reinterpret_cast<const float4 *>(rope + (size_t)pos[tl].y * half + dim);   // cos sin cos sin
+  }
+}
+__device__ __forceinline__ void pair_rope_rows(const float *stage, const int2 *pos, const float4 (&cs)[PAIR_CHUNK / 4], int w4,
+                                               const PairRopeLane &pl, int f0, int t0, int M, int N, float *C, const PairRope &pr) {
+  const int d = N / 3, part = f0 / d, dh = pr.dh, half = dh >> 1;
+  const int head = (f0 - part * d + pl.hl) / dh;
+  const float sc = rsqrtf((float)dh) * 1.4426950408889634f;
+#pragma unroll
+  for (int r = 0; r < PAIR_CHUNK / 4; ++r) {
+    const int tl = w4 * (PAIR_CHUNK / 4) + r, t = t0 + tl;
+    if (t >= M) break;
+    const float2 u = *reinterpret_cast<const float2 *>(stage + tl * TC_BM + pl.hl + pl.dim);
+    const float2 y = *reinterpret_cast<const float2 *>(stage + tl * TC_BM + pl.hl + pl.dim + half);
+    const float2 a = make_float2(u.x * cs[r].x - y.x * cs[r].y, u.y * cs[r].z - y.y * cs[r].w);
+    const float2 b = make_float2(y.x * cs[r].x + u.x * cs[r].y, y.y * cs[r].z + u.y * cs[r].w);
+    if (part == 0) {
+      float *dst = C + (size_t)t * N + f0 + pl.hl + pl.dim;
+      *reinterpret_cast<float2 *>(dst) = make_float2(a.x * sc, a.y * sc);
+      *reinterpret_cast<float2 *>(dst + half) = make_float2(b.x * sc, b.y * sc);
+    } else {
+      const int2 bp = pos[tl];
+      bf16 *dst = (part == 1 ? pr.Kc : pr.Vc) + (((size_t)bp.x * pr.n_heads + head) * pr.g.cap + bp.y) * dh + pl.dim;
+      *reinterpret_cast<uint32_t *>(dst) = part == 1 ? pack_bf16x2(a.x, a.y) : pack_bf16x2(u.x, u.y);
+      *reinterpret_cast<uint32_t *>(dst + half) = part == 1 ? pack_bf16x2(b.x, b.y) : pack_bf16x2(y.x, y.y);
+    }
+  }
 }
 
-// grid = 2 x pairs, cluster = 2.  C leaves through mapC (box 128 features x 32 tokens): tma_c = SK_TMA_F32 /
+// grid = 2 x pairs, cluster = 2.  C leaves through mapC (box 128 features x 16 tokens): tma_c = SK_TMA_F32 /
 // SK_TMA_BF16 (stores; epi tells GELU) or SK_TMA_ADD.
 __global__ void __launch_bounds__(PAIR_THREADS, 1)
 gemm_pair_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant__ CUtensorMap mapA,
                  const __grid_constant__ CUtensorMap mapC, int M, int N, int K, int BN, int stages, int n_acc,
-                 int tmem_cols, int epi, int tma_c, int *__restrict__ status, const LiveRows lr) {
+                 int tmem_cols, int epi, int tma_c, float *C, const SkNorm nm, const PairRope pr, int *__restrict__ status,
+                 const LiveRows lr) {
   // rows in use (active-series compaction): read before the dependency wait, see gemm_sk_kernel
   if (lr.n_live) M = min(M, *reinterpret_cast<const volatile int *>(lr.n_live) * lr.q_len);
   const int FT = (N + 2 * TC_BM - 1) / (2 * TC_BM), n_tiles = FT * ((M + BN - 1) / BN);
@@ -101,13 +157,16 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant
   const uint32_t tiles = (smem_u32(smem_raw) + 1023u) & ~1023u;
   const int a_bytes = (BN / 2) * TC_BK * 2, stage_bytes = TC_W_BYTES + a_bytes;
   const uint32_t out0 = tiles + (uint32_t)(stages * stage_bytes);
-  const uint32_t bars = out0 + 2 * PAIR_STAGE_OUT;
+  const uint32_t bars = out0 + PAIR_GROUPS * PAIR_STAGE_OUT;
   const uint32_t full0 = bars, empty0 = bars + 64, acc_full0 = bars + 128, acc_empty0 = bars + 144, slot = bars + 160;
+  const uint32_t rows_full0 = bars + 176, rows_empty0 = bars + 192;
+  float *row_scale = reinterpret_cast<float *>(smem_raw + (bars + 256 - smem_u32(smem_raw)));   // [2 tiles][256]
+  int2 *row_pos = reinterpret_cast<int2 *>(row_scale + 512);                                    // [2 tiles][256] (series, position)
   uint32_t *slot_ptr = reinterpret_cast<uint32_t *>(smem_raw + (slot - smem_u32(smem_raw)));
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const int KB = (K + TC_BK - 1) / TC_BK;
 
-  if (warp == 8 && lane == 0) {
+  if (warp == PAIR_EPI_WARPS && lane == 0) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(&mapW) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&mapA) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&mapC) : "memory");
@@ -119,11 +178,13 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant
     }
     for (int s = 0; s < 2; ++s) {
       mbar_init(acc_full0 + 8 * s, 1);
-      mbar_init(acc_empty0 + 8 * s, 16);                       // 8 epilogue warps of each rank
+      mbar_init(acc_empty0 + 8 * s, 2 * PAIR_EPI_WARPS);       // of both ranks
+      mbar_init(rows_full0 + 8 * s, PAIR_ROW_WARPS);
+      mbar_init(rows_empty0 + 8 * s, PAIR_EPI_WARPS);
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 9) {
+  if (warp == PAIR_EPI_WARPS + 1) {
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(slot), "r"((uint32_t)tmem_cols) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
@@ -133,7 +194,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant
   tc_fence_after();
   const uint32_t tmem = *slot_ptr;
 
-  if (warp == 8) {
+  if (warp == PAIR_EPI_WARPS) {
     if (elect_one()) {
       // ---------------- TMA producer: this rank's half of both operands.  The first ring-full of weight
       // tiles is requested before the dependency wait.
@@ -176,7 +237,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant
         if (++s == stages) { s = 0; ph ^= 1u; dst = tiles; }
       }
     }
-  } else if (warp == 9) {
+  } else if (warp == PAIR_EPI_WARPS + 1) {
     if (rank == 0 && elect_one()) {
       // ---------------- MMA issuer
       const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(2 * TC_BM >> 4) << 24);
@@ -201,36 +262,102 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant
         if (ok) umma_commit_pair(acc_full0 + 8 * buf);
       }
     }
+  } else if (warp >= PAIR_EPI_WARPS + 2) {
+    // ---------------- factors (folded norm) and cache positions of the rows of each tile
+    pdl_sync();
+    if (nm.ssq_in || pr.rope) {
+      bool ok = true;
+      for (int tile = pair, i = 0; tile < n_tiles && ok; tile += n_pairs, ++i) {
+        const int rb = i & 1, t0 = (tile / FT) * BN;
+        ok = mbar_wait(rows_empty0 + 8 * rb, ((uint32_t)(i >> 1) & 1u) ^ 1u);
+        for (int r = threadIdx.x - 32 * (PAIR_EPI_WARPS + 2); r < BN && t0 + r < M; r += 32 * PAIR_ROW_WARPS) {
+          const int t = t0 + r;
+          if (nm.ssq_in) {
+            const float *src = nm.ssq_in + (size_t)t * nm.n_part;
+            float acc = 0.f;
+#pragma unroll 8
+            for (int j = 0; j < nm.n_part; ++j) acc += __ldcg(src + j);
+            row_scale[rb * 256 + r] = rsqrtf(acc * nm.inv_d + nm.eps);
+          }
+          if (pr.rope) {
+            const SlotPos sp = slot_lookup(pr.g, t / pr.g.q_len);
+            row_pos[rb * 256 + r] = make_int2(sp.b, sp.p0 + t % pr.g.q_len);
+          }
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(rows_full0 + 8 * rb);
+      }
+    }
   } else {
     // ---------------- epilogue
     const int grp = warp >> 2, w4 = warp & 3, fl = w4 * 32 + lane;
     const uint32_t stage = out0 + (uint32_t)(grp * PAIR_STAGE_OUT);
     float *stage_f = reinterpret_cast<float *>(smem_raw + (stage - smem_u32(smem_raw)));
     bf16 *stage_h = reinterpret_cast<bf16 *>(stage_f);
+    uint16_t *stage_u = reinterpret_cast<uint16_t *>(stage_f);
     const bool leader = (threadIdx.x & 127) == 0;
+    const PairRopeLane pl(lane, pr.rope ? pr.dh : 64);
+    const bool produce = nm.a_out != nullptr;                  // residual update with the next norm's operand
     pdl_sync();
     bool ok = true;
     for (int tile = pair, i = 0; tile < n_tiles; tile += n_pairs, ++i) {
       const int buf = n_acc == 2 ? (i & 1) : 0, use = n_acc == 2 ? (i >> 1) : i;
       const int f0 = (tile % FT) * 2 * TC_BM + (int)rank * TC_BM, t0 = (tile / FT) * BN;
-      if (ok) {                                                // (after a wait that ran out: no more waits, nothing stored)
+      const int fc = f0 + lane * 4;                            // features this lane finishes in row order
+      const float *scale = row_scale + (i & 1) * 256;
+      const int2 *pos = row_pos + (i & 1) * 256;
+      // old values of the group's first chunk: while the main loop runs
+      float4 gain = make_float4(0.f, 0.f, 0.f, 0.f);
+      float old[PAIR_CHUNK];
+      auto fetch_old = [&](int c) {
+#pragma unroll
+        for (int j = 0; j < PAIR_CHUNK; ++j)
+          old[j] = (c < BN && t0 + c + j < M && f0 < N) ? __ldcg(C + (size_t)(t0 + c + j) * N + f0 + fl) : 0.f;
+      };
+      if (produce) {
+        if (f0 < N) gain = *reinterpret_cast<const float4 *>(nm.gain + fc);
+        fetch_old(grp * PAIR_CHUNK);
+      }
+      // (after a wait that ran out: no more waits, nothing stored)
+      if (ok && (nm.ssq_in || pr.rope)) ok = mbar_wait(rows_full0 + 8 * (i & 1), (uint32_t)(i >> 1) & 1u);
+      float4 cs[PAIR_CHUNK / 4];
+      const bool rotate = pr.rope && f0 < 2 * (N / 3);         // queries and keys
+      if (ok && rotate) pair_rope_fetch(cs, pos + grp * PAIR_CHUNK, w4, t0 + grp * PAIR_CHUNK, grp * PAIR_CHUNK < BN ? M : 0, pr.dh >> 1, pl.dim, pr.rope);
+      if (ok) {
         ok = mbar_wait_cluster(acc_full0 + 8 * buf, (uint32_t)use & 1u);
         if (!ok) atomicExch(status, DEV_TIMEOUT_EPILOGUE);
       }
       ok = __all_sync(0xffffffffu, ok);
       tc_fence_after();
       const uint32_t tbase = tmem + ((uint32_t)(w4 * 32) << 16) + (uint32_t)(buf * BN);
-      for (int c = grp * PAIR_CHUNK; c < BN; c += 2 * PAIR_CHUNK) {
+      for (int c = grp * PAIR_CHUNK; c < BN; c += PAIR_GROUPS * PAIR_CHUNK) {
         if (t0 + c >= M) break;
         float v[PAIR_CHUNK];
-        tmem_ld32(tbase + c, v);
-        // the staging tile is free once its previous copy has been read
+#pragma unroll
+        for (int j = 0; j < PAIR_CHUNK; j += 16) tmem_ld16(tbase + c + j, v + j);
+        if (nm.ssq_in) {
+#pragma unroll
+          for (int j = 0; j < PAIR_CHUNK; j += 4) {
+            const float4 k = *reinterpret_cast<const float4 *>(scale + c + j);
+            v[j] *= k.x; v[j + 1] *= k.y; v[j + 2] *= k.z; v[j + 3] *= k.w;
+          }
+        }
+        if (produce) {
+#pragma unroll
+          for (int j = 0; j < PAIR_CHUNK; ++j) v[j] += old[j];
+          fetch_old(c + PAIR_GROUPS * PAIR_CHUNK);
+        }
+        // the staging tile is free once its previous copy (or the previous chunk's readers) are done
         if (leader) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
         asm volatile("bar.sync %0, 128;" ::"r"(1 + grp) : "memory");
         if (tma_c == SK_TMA_BF16) {
           if (epi == EPI_GELU_T) {
 #pragma unroll
-            for (int j = 0; j < PAIR_CHUNK; ++j) stage_h[j * TC_BM + fl] = __float2bfloat16_rn(gelu_erf_fast(v[j]));
+            for (int j = 0; j < PAIR_CHUNK; j += 2) {
+              const uint32_t p = gelu_erf_fast2(v[j], v[j + 1]);
+              stage_u[j * TC_BM + fl] = (uint16_t)p;
+              stage_u[(j + 1) * TC_BM + fl] = (uint16_t)(p >> 16);
+            }
           } else {
 #pragma unroll
             for (int j = 0; j < PAIR_CHUNK; ++j) stage_h[j * TC_BM + fl] = __float2bfloat16_rn(v[j]);
@@ -241,8 +368,16 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         asm volatile("bar.sync %0, 128;" ::"r"(1 + grp) : "memory");
+        if (pr.rope) {
+          if (ok && f0 < N) {
+            pair_rope_rows(stage_f, pos + c, cs, w4, pl, f0, t0 + c, M, N, C, pr);
+            const int cn = c + PAIR_GROUPS * PAIR_CHUNK;
+            if (rotate && cn < BN) pair_rope_fetch(cs, pos + cn, w4, t0 + cn, M, pr.dh >> 1, pl.dim, pr.rope);
+          }
+          continue;
+        }
         if (leader && ok && f0 < N) {
-          if (tma_c == SK_TMA_ADD)
+          if (tma_c == SK_TMA_ADD && !produce)
             asm volatile("cp.reduce.async.bulk.tensor.2d.global.shared::cta.add.tile.bulk_group [%0, {%1, %2}], [%3];"
                          ::"l"(&mapC), "r"(f0), "r"(t0 + c), "r"(stage) : "memory");
           else
@@ -250,18 +385,35 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant
                          ::"l"(&mapC), "r"(f0), "r"(t0 + c), "r"(stage) : "memory");
           asm volatile("cp.async.bulk.commit_group;" ::: "memory");
         }
+        if (produce && ok && f0 < N) {
+          // this warp's four rows: the next contraction's operand and the sums of squares over these 128 features
+#pragma unroll
+          for (int r = 0; r < PAIR_CHUNK / 4; ++r) {
+            const int tl = w4 * (PAIR_CHUNK / 4) + r, t = t0 + c + tl;
+            const float4 x = *reinterpret_cast<const float4 *>(stage_f + tl * TC_BM + lane * 4);
+            const float sq = warp_sum(fmaf(x.x, x.x, fmaf(x.y, x.y, fmaf(x.z, x.z, x.w * x.w))));
+            if (t < M) {
+              *reinterpret_cast<uint2 *>(nm.a_out + (size_t)t * N + fc) =
+                  make_uint2(pack_bf16x2(gain.x * x.x, gain.y * x.y), pack_bf16x2(gain.z * x.z, gain.w * x.w));
+              if (lane == 0) nm.ssq_out[(size_t)t * (N >> 7) + (f0 >> 7)] = sq;
+            }
+          }
+        }
       }
       // accumulator drained: rank 0 may overwrite it
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive_rank0(acc_empty0 + 8 * buf);
+      if (lane == 0) {
+        mbar_arrive_rank0(acc_empty0 + 8 * buf);
+        if (nm.ssq_in || pr.rope) mbar_arrive(rows_empty0 + 8 * (i & 1));
+      }
     }
     if (leader) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
   }
   __syncwarp();
   tc_fence_before();
   cluster_sync_all();          // no rank leaves while the other's MMAs read its shared memory or its arrivals are under way
-  if (warp == 9) {
+  if (warp == PAIR_EPI_WARPS + 1) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)tmem_cols) : "memory");
   }
@@ -311,13 +463,13 @@ static void gemm_pair_fill(PairShape *sh, int N, int K, int M) {
   const int cols = sh->BN * sh->n_acc;
   sh->tmem_cols = cols <= 32 ? 32 : cols <= 64 ? 64 : cols <= 128 ? 128 : cols <= 256 ? 256 : 512;
   const int stage = TC_W_BYTES + sh->BN / 2 * TC_BK * 2;
-  const int st = (227 * 1024 - 2 * PAIR_STAGE_OUT - 2048) / stage;
+  const int st = (227 * 1024 - PAIR_GROUPS * PAIR_STAGE_OUT - PAIR_ROW_BYTES - 1280) / stage;
   if (sh->stages == 0) sh->stages = st > 8 ? 8 : st;
-  sh->smem_bytes = sh->stages * stage + 2 * PAIR_STAGE_OUT + 1024 + 256;
+  sh->smem_bytes = sh->stages * stage + PAIR_GROUPS * PAIR_STAGE_OUT + 1024 + 256 + PAIR_ROW_BYTES;
 }
 
 static bool gemm_pair_launch(cudaStream_t st, bool pdl, GemmSkPlan &p, void *C, int M, int epi, int *status, LiveRows lr,
-                             PairShape sh = PairShape{}) {
+                             const SkNorm *norm = nullptr, const PairRope *rope = nullptr, PairShape sh = PairShape{}) {
   if (M < 1 || M > p.M_max) return false;
   if (!sh.BN) {
     sh = gemm_pair_geometry(p.N, p.K, M);
@@ -344,7 +496,8 @@ static bool gemm_pair_launch(cudaStream_t st, bool pdl, GemmSkPlan &p, void *C, 
   cfg.attrs = at;
   cfg.numAttrs = pdl ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, gemm_pair_kernel, p.mapW, p.mapA2[idx], *mapC, M, p.N, p.K, sh.BN, sh.stages, sh.n_acc,
-                            sh.tmem_cols, epi, tma_c, status, lr) == cudaSuccess;
+                            sh.tmem_cols, epi, tma_c, (float *)C, norm ? *norm : SkNorm{}, rope ? *rope : PairRope{}, status,
+                            lr) == cudaSuccess;
 }
 
 }  // namespace tsfm

@@ -43,14 +43,15 @@ __host__ __device__ constexpr uint32_t umma_idesc_rt(int bn) {
 // RMSNorm folded into the contractions around it.  The norm of a row is a scalar factor, so it
 // commutes with the contraction that consumes the row: the kernel that PRODUCES the residual
 // stream (residual epilogue) also writes a' = bf16(gain * x) -- the next contraction's operand,
-// not yet normalised -- and the sum of squares of every 16-feature slice of the row; the kernel
+// not yet normalised -- and the sum of squares of every 16-feature (gemm_pair_kernel:
+// 128-feature) slice of the row; the kernel
 // that CONSUMES a' multiplies its result rows by rstd = rsqrt(sum of the slices / d + eps).
 struct SkNorm {
   const float *ssq_in;      // [M][n_part] slice sums of squares of this contraction's input rows, or NULL
-  float *ssq_out;           // [M][N / 16] written by a residual epilogue, or NULL
+  float *ssq_out;           // [M][N / 16] (gemm_pair_kernel: [M][N / 128]) written by a residual epilogue, or NULL
   const float *gain;        // [N] gain of the norm that follows the residual epilogue
   bf16 *a_out;              // [M][N] bf16(gain * x_new), or NULL
-  int n_part;               // partial sums per input row (d / 16)
+  int n_part;               // partial sums per input row
   float inv_d, eps;
 };
 

@@ -89,6 +89,19 @@ def test_bf16_attention_tiles_of_queries_and_keys(n):
             assert np.sqrt(np.mean((got[b] - want[b]) ** 2)) <= 3e-2 * np.sqrt(np.mean(want[b] ** 2))
 
 
+@pytest.mark.parametrize("target,draft,n", [
+    (Arch(3, 256, 2, 512), Arch(2, 128, 4, 128), 103),      # 515 rows: norms folded, rotation of head sizes 128 and 32, 3-row tail
+    (Arch(3, 256, 4, 256), Arch(2, 128, 2, 384), 130),      # 650 rows, head size 64; half a feature tile over (N = 384)
+    (Arch(2, 128, 2, 128), Arch(2, 192, 3, 192), 620),      # 3100 rows: norms apart; d = 192 takes the other kernels
+])
+def test_bf16_forward_on_pairs_of_sms(target, draft, n):
+    wl = small_workload("bf16", target, draft, 32)
+    gt, wt, gd, wd = run_forward_case(wl, 0, n)
+    assert np.isfinite(gt).all() and np.isfinite(gd).all()
+    assert parity.value_error("rel_rms", gt, wt) < 2e-2       # bf16 operands, as above
+    assert parity.value_error("rel_rms", gd, wd) < 2e-2
+
+
 @pytest.mark.parametrize("dtype,P,P_in,n", [("f32", 16, 1, 70), ("f32", 32, 8, 19), ("bf16", 64, 1, 300), ("bf16", 32, 16, 40)])
 def test_forward_with_input_tokens_shorter_than_the_patch(dtype, P, P_in, n):
     """Embedding of P_in-step tokens ([d, P_in] weights; 16-byte loads or element by element) under a

@@ -1,5 +1,5 @@
-// Causal attention of passes of at most 16 tokens (one query tile) over a bf16 KV cache with a running softmax
-// (one pass over the keys); longer passes: attn_tiles.cuh.
+// Causal attention of passes of 9 to 16 tokens (one query tile) over a bf16 KV cache with a running softmax
+// (one pass over the keys); shorter passes: attn_narrow.cuh, longer ones: attn_tiles.cuh.
 //
 // Work unit = one warp: 16 queries (the M side of mma.sync m16n8k16) against a range of keys of
 // one (series, head).  The warp streams its keys in chunks of 32 through a private ring of

@@ -20,6 +20,7 @@
 #include "kernels_simt.cuh"
 #include "attn_flash.cuh"
 #include "attn_tiles.cuh"
+#include "attn_narrow.cuh"
 #include "accept.cuh"
 #include "gemm_tc.cuh"
 #include "gemm_sk.cuh"
@@ -302,7 +303,7 @@ int attn_set_attr(size_t bytes) {
   return TSFM_OK;
 }
 // bf16 caches take the running-softmax kernel (attn_flash_kernel), fp32 caches attn_kernel.
-// Short rows with at least this many (series, head) pairs: one warp per pair instead of four
+// Passes of 9 to 16 tokens: short rows with at least this many (series, head) pairs: one warp per pair instead of four
 // (measured: C2's draft, 1024 pairs, 15 % faster that way; no difference at 256 pairs).
 constexpr int kFlashWarpMaxCap = 64, kFlashWarpMinPairs = 512;
 // Long rows with at least this many pairs take one warp per pair too: split four ways, a CTA's life
@@ -311,12 +312,20 @@ constexpr int kFlashWarpMaxCap = 64, kFlashWarpMinPairs = 512;
 // through its ring (measured on C4's verification pass and decode step: attention 51.7 -> 47.2 ms
 // per forecast).
 constexpr int kFlashWarpLongMinPairs = 1024;
+// Passes of at most 8 tokens (attn_narrow.cuh).  Rows of up to 64 keys sit in one stage, one warp per pair; with
+// fewer pairs than SMs four warps share a row instead.  Graph replay of dependent launches, us, 16-row tiles ->
+// here: 256 pairs x 36 keys 4.2 -> 2.6 (8 pairs: 2.8 -> 2.2 split, 2.5 not), 1024 x 33 4.7 -> 3.5, 4096 x 33 behind
+// 5 tokens 17.7 -> 12.5, 12288 x 14 24.4 -> 16.2, 1280 x 290 19.4 -> 18.4, 384 x 290 7.5 -> 6.4.
+constexpr int kNarrowSingleMaxCap = 64, kNarrowFewPairs = 148;
 // one-tile passes: a two-stage ring (each warp has a few chunks only, and a third CTA fits on the SM)
 constexpr int kFlashStShort = 2;
 template <int DH> int flash_set_attr() {
   CU_TRY(cudaFuncSetAttribute(attn_tiles_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, TilesGeom<DH>::SMEM_BYTES));
   CU_TRY(cudaFuncSetAttribute(attn_flash_kernel<DH, kFlashStShort>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               FlashGeom<DH, kFlashStShort>::SMEM_BYTES));
+  CU_TRY(cudaFuncSetAttribute(attn_narrow_ring_kernel<DH, kFlashStShort>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              FlashGeom<DH, kFlashStShort>::SMEM_BYTES));
+  CU_TRY(cudaFuncSetAttribute(attn_narrow_single_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, 16 * kNarrowSingleMaxCap * DH));
   CU_TRY(cudaFuncSetAttribute(attn_flash_single_kernel<DH, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, FlashGeom<DH>::single_bytes(1)));
   CU_TRY(cudaFuncSetAttribute(attn_flash_single_kernel<DH, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, FlashGeom<DH>::single_bytes(2)));
   return TSFM_OK;
@@ -375,10 +384,16 @@ void prefer_max_smem_all() {
   prefer_max_smem(gemm_ws_kernel<false>);
   prefer_max_smem(gemm_ws_kernel<true>);
   prefer_max_smem(attn_tiles_kernel<32>);
+  prefer_max_smem(attn_narrow_ring_kernel<32, kFlashStShort>);
+  prefer_max_smem(attn_narrow_single_kernel<32>);
   prefer_max_smem(attn_flash_kernel<32, kFlashStShort>);
   prefer_max_smem(attn_tiles_kernel<64>);
+  prefer_max_smem(attn_narrow_ring_kernel<64, kFlashStShort>);
+  prefer_max_smem(attn_narrow_single_kernel<64>);
   prefer_max_smem(attn_flash_kernel<64, kFlashStShort>);
   prefer_max_smem(attn_tiles_kernel<128>);
+  prefer_max_smem(attn_narrow_ring_kernel<128, kFlashStShort>);
+  prefer_max_smem(attn_narrow_single_kernel<128>);
   prefer_max_smem(attn_flash_kernel<128, kFlashStShort>);
   prefer_max_smem(attn_flash_single_kernel<32, 1>);
   prefer_max_smem(attn_flash_single_kernel<32, 2>);
@@ -532,6 +547,20 @@ void launch_attn(tsfm_spec *h, ModelDev &m, int l, int B, const PassGeom &g, boo
       launch_ex(h->ls, h->pdl, attn_tiles_kernel<DH>, dim3(m.arch.n_heads, B, (g.q_len + 16 * warps - 1) / (16 * warps)),
                 dim3(32 * warps), (size_t)TilesGeom<DH>::SMEM_BYTES, h->qkv, (const bf16 *)Kc, (const bf16 *)Vc, m.rope, g,
                 m.arch.n_heads, appended ? 1 : 0, (bf16 *)h->ao);
+      return;
+    }
+    if (g.q_len <= 8) {
+      const bool short_rows = h->cap <= kNarrowSingleMaxCap, few = pairs < kNarrowFewPairs;
+      if (short_rows && !few) {
+        const int rows = (h->cap + 15) & ~15;
+        launch_ex(h->ls, h->pdl, attn_narrow_single_kernel<DH>, dim3((pairs + 3) / 4), dim3(128), (size_t)16 * rows * DH, h->qkv,
+                  (bf16 *)Kc, (bf16 *)Vc, m.rope, g, m.arch.n_heads, pairs, rows, (bf16 *)h->ao);
+      } else {
+        const int mode = pairs >= kFlashWarpLongMinPairs ? FLASH_WARP : FLASH_SPLIT;
+        launch_ex(h->ls, h->pdl, attn_narrow_ring_kernel<DH, kFlashStShort>, mode == FLASH_WARP ? dim3((pairs + 3) / 4) : dim3(m.arch.n_heads, B),
+                  dim3(128), (size_t)FlashGeom<DH, kFlashStShort>::SMEM_BYTES, h->qkv, (bf16 *)Kc, (bf16 *)Vc, m.rope, g,
+                  m.arch.n_heads, pairs, mode, (bf16 *)h->ao);
+      }
       return;
     }
     const int mode = ((h->cap <= kFlashWarpMaxCap && pairs >= kFlashWarpMinPairs) || pairs >= kFlashWarpLongMinPairs)

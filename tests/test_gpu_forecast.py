@@ -332,6 +332,20 @@ def test_many_series_short_rows_one_warp_per_series_and_head_bf16():
     run_and_compare(wl, 3, 1.0, 9, [0, 100, 198])
 
 
+@pytest.mark.parametrize("ctx,K,T,B", [
+    (3, 1, 4, 90),        # rows of 16 (capacity 9), two queries at most
+    (41, 7, 15, 80),      # capacity 64: the longest row of one stage, eight queries in verification
+    (42, 7, 15, 80),      # capacity 65: the ring, four warps per row
+    (41, 7, 15, 3),       # few pairs on short rows: four warps per row too
+    (20, 4, 9, 75),       # capacity 34: rows of 48, a last block of 16 keys; 150 and 300 pairs
+])
+def test_short_passes_keys_as_the_matrix_rows_bf16(ctx, K, T, B):
+    """Passes of at most 8 tokens on every row layout, head sizes 128 (target) and 32 (draft)."""
+    wl = workload("C4", batch=B, ctx_len=32 * ctx, horizon=32 * T - 5, K=K, series_recipe="c1", target=Arch(1, 256, 2, 256),
+                  draft=Arch(1, 128, 4, 128))
+    run_and_compare(wl, K, 2.0, 21, [0, B // 2, B - 1])
+
+
 @pytest.mark.parametrize("B", [257, 340])
 def test_many_series_long_rows_one_warp_per_series_and_head_bf16(B):
     """C4's row lengths with more than a thousand (series, head) pairs on small models: one warp per

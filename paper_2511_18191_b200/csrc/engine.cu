@@ -381,8 +381,14 @@ void prefer_max_smem_all() {
   prefer_max_smem(gemm_sk_kernel<1, true>);
   prefer_max_smem(gemm_sk_kernel<2, false>);
   prefer_max_smem(gemm_pair_kernel);
-  prefer_max_smem(gemm_ws_kernel<false>);
-  prefer_max_smem(gemm_ws_kernel<true>);
+  prefer_max_smem(gemm_ws_kernel<1, false>);
+  prefer_max_smem(gemm_ws_kernel<1, true>);
+  prefer_max_smem(gemm_ws_kernel<2, false>);
+  prefer_max_smem(gemm_ws_kernel<2, true>);
+  prefer_max_smem(gemm_ws_kernel<3, false>);
+  prefer_max_smem(gemm_ws_kernel<3, true>);
+  prefer_max_smem(gemm_ws_kernel<4, false>);
+  prefer_max_smem(gemm_ws_kernel<4, true>);
   prefer_max_smem(attn_tiles_kernel<32>);
   prefer_max_smem(attn_narrow_ring_kernel<32, kFlashStShort>);
   prefer_max_smem(attn_narrow_single_kernel<32>);
@@ -478,7 +484,7 @@ void gemm(tsfm_spec *h, GemmSkPlan *plan, const void *A, const void *W, void *C,
   const double bytes = ((double)N * K + (double)M * K) * e + (double)M * N * out_b;
   const double flops = 2.0 * M * N * K;
   if (sizeof(T) == 2 && h->use_tc && plan && plan->valid && gemm_ws_eligible(A, W, M, N, K)) {
-    // few tokens, short K: the shared-memory-resident weight tile kernel has the shorter chain
+    // few tokens, short K: the kernel with its weight tile in registers has the shorter chain
     KTimer kt(h, KC_GEMM_WS, bytes, flops);
     if (gemm_ws_launch(h->ls, h->pdl, A, W, C, M, N, K, epi, norm, lr)) {
       LAUNCHED();
@@ -1204,7 +1210,6 @@ int tsfm_spec_create(const tsfm_weights *target_w, const tsfm_weights *draft_w, 
   if ((rc = cfg->dtype == TSFM_F32 ? gemm_f32_init<float>() : gemm_f32_init<bf16>())) return fail(rc);
   if (h->use_tc) {
     if ((rc = gemm_sk_init())) return fail(rc);
-    if ((rc = gemm_ws_init())) return fail(rc);
     if ((rc = gemm_pair_init())) return fail(rc);
     for (ModelDev *m : {&h->tgt, &h->drf}) {
       const int d = m->arch.d_model, f = m->arch.d_ff;
@@ -1426,8 +1431,7 @@ int tsfm_gemm_bf16(void *stream, const void *A, const void *W, float *C, int32_t
     return TSFM_OK;
   }
   if (backend == TSFM_GEMM_WS) {
-    if (!gemm_ws_eligible(A, W, M, N, Kd)) return TSFM_ERR_SHAPE;
-    if (int rc = gemm_ws_init()) return rc;
+    if (!gemm_ws_accepts(A, W, M, N, Kd)) return TSFM_ERR_SHAPE;
     if (!gemm_ws_launch(s, false, A, W, C, M, N, Kd, EPI_F32, nullptr, LiveRows{nullptr, 0})) CU_TRY(cudaGetLastError());
     LAUNCHED();
     CU_TRY(cudaGetLastError());

@@ -1,6 +1,6 @@
-// Small-batch contraction with the whole weight tile resident in shared memory.
+// Small-batch contraction with the weight tile in registers.
 //
-//   C[t, f] (op)= sum_k A[t, k] * W[f, k]        A: [M, K] tokens (bf16), W: [N, K] weights (bf16)
+//   C[t, f] (op)= sum_k A[t, k] * W[f, k]        A: [M, K] tokens (bf16), W: [N, K] weights
 //
 // For the passes of a few dozen tokens (draft steps, one-token decode steps, short verification
 // passes) a contraction is a dependent link in a chain of launches, and what it costs is the
@@ -8,18 +8,19 @@
 // short:
 //   * a CTA owns 16 output features x 32 tokens over the WHOLE K range, so nothing is exchanged
 //     between CTAs and every epilogue (GELU, residual, folded norm) sees complete sums;
-//   * its weight tile (16 x K) does not depend on the preceding kernel: it is requested with
-//     asynchronous copies BEFORE the dependency wait (programmatic dependent launch) and is in
-//     shared memory by the time the activations are;
-//   * the eight warps split K among them (warp w takes the 16-wide k steps w, w + 8, ...), each
-//     accumulating a 32 x 16 partial tile in registers with mma.sync m16n8k16 (bf16 in, fp32
-//     accumulate); the partial tiles are summed through shared memory in a fixed order.
-// The tensor-memory kernel (gemm_sk.cuh) stays the tool wherever K is long, tokens are many or the
-// grid would not fit in one wave: an MMA issued there costs ~72 ns whatever its width, and its
-// chain (TMA -> MMA -> commit -> tcgen05.ld -> cluster exchange) is about 2 us longer than this one.
-//
-// Shared memory: W tile [16][K], A tile [32][K] (bf16, 16-byte chunks of a row XOR-ed with row & 7
-// so that ldmatrix reads are conflict-free), partial tiles [8][32][16] fp32, rstd [32].
+//   * the eight warps split K among them (warp w takes the 64-wide blocks w, w + 8, ...); a lane holds 16
+//     consecutive k of a weight row and of a token row, 32 bytes each, straight from global memory in the
+//     registers that mma.sync m16n8k16 wants: the contraction does not care which k sits at which of its
+//     positions as long as both operands agree, so no shared memory, barrier or ldmatrix stands between the
+//     loads and the MMAs, and rows that do not exist are not touched;
+//   * the weights do not depend on the preceding kernel: they are in registers BEFORE the dependency wait
+//     (programmatic dependent launch);
+//   * the partial tiles are summed through shared memory in a fixed order.
+// Bound: latency.  A link of a chain of dependent launches, us, with both tiles staged in shared memory -> here:
+// M = 1: K = 512 2.5 to 2.7 -> 1.7, K = 2048 4.5 -> 2.3; M = 29: 2.6 to 2.8 -> 1.9 to 2.2, 5.0 -> 3.7; M = 64,
+// K = 384: 2.5 to 3.4 -> 1.9 to 2.7.  (A launch that only reads and writes one value per thread: 0.9 to 1.0.)
+// The tensor-memory kernels stay the tool wherever K is long, tokens are many or the grid would not fit in one
+// wave.
 // grid = (ceil(N / 16), ceil(M / 32)), block = 256.  K a multiple of 64, at most WS_MAX_K.
 #pragma once
 #include "common.cuh"
@@ -30,19 +31,20 @@ namespace tsfm {
 
 constexpr int WS_FN = 16, WS_MT = 32, WS_WARPS = 8, WS_MAX_K = 2048;
 
-static inline int ws_smem_bytes(int K) { return (WS_FN + WS_MT) * K * 2 + WS_WARPS * WS_MT * WS_FN * 4 + WS_MT * 4; }
-
-__device__ __forceinline__ void ws_ldsm4(uint32_t addr, uint32_t (&d)[4]) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-               : "=r"(d[0]), "=r"(d[1]), "=r"(d[2]), "=r"(d[3]) : "r"(addr));
+// (volatile with a memory clobber: stays behind the dependency wait)
+__device__ __forceinline__ uint4 ws_ld16(const bf16 *p) {
+  uint4 v;
+  asm volatile("ld.global.cg.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+  return v;
 }
 
-// NORM: compile the folded-RMSNorm epilogues (SkNorm; slices of 16 features).
-template <bool NORM>
-__global__ void __launch_bounds__(256)
+// NB: 64-wide blocks of K per warp (at most).  NORM: compile the folded-RMSNorm epilogues (SkNorm; slices of 16
+// features).
+template <int NB, bool NORM>
+__global__ void __launch_bounds__(256, NB == 1 ? 3 : NB == 2 ? 2 : 1)
 gemm_ws_kernel(const bf16 *A, const bf16 *__restrict__ W, void *C, int M, int N, int K,
                int epi, const SkNorm nm, const LiveRows lr) {
-  extern __shared__ __align__(128) unsigned char ws_smem[];
+  __shared__ float red[WS_WARPS * WS_MT * WS_FN], rs[WS_MT];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const int f0 = blockIdx.x * WS_FN, t0 = blockIdx.y * WS_MT;
   // rows in use (active-series compaction): read before the dependency wait, see gemm_sk_kernel
@@ -50,33 +52,45 @@ gemm_ws_kernel(const bf16 *A, const bf16 *__restrict__ W, void *C, int M, int N,
     M = min(M, *reinterpret_cast<const volatile int *>(lr.n_live) * lr.q_len);
     if (t0 >= M) return;
   }
-  const int row_bytes = K * 2, cpr = K >> 3;                   // bytes and 16-byte chunks per tile row
-  unsigned char *Ws = ws_smem, *As = ws_smem + WS_FN * row_bytes;
-  float *red = reinterpret_cast<float *>(As + WS_MT * row_bytes);        // [8][32][16]
-  float *rs = red + WS_WARPS * WS_MT * WS_FN;                            // [32]
-  const uint32_t Ws32 = (uint32_t)__cvta_generic_to_shared(Ws), As32 = (uint32_t)__cvta_generic_to_shared(As);
+  const int KB = K >> 6, g = lane >> 2, q4 = lane & 3;
+  const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
 
-  // ---- weight tile: independent of the preceding kernel
-  for (int i = tid; i < WS_FN * cpr; i += 256) {
-    const int r = i / cpr, c = i % cpr;
-    const uint32_t dst = Ws32 + (uint32_t)(r * row_bytes + ((c ^ (r & 7)) << 4));
-    if (f0 + r < N) cp_async16(Ws + (dst - Ws32), W + (size_t)(f0 + r) * K + c * 8);
-    else *reinterpret_cast<uint4 *>(Ws + (dst - Ws32)) = make_uint4(0u, 0u, 0u, 0u);
-  }
-  asm volatile("cp.async.commit_group;" ::: "memory");
+  // ---- weight fragments: independent of the preceding kernel
+  uint4 wf[NB][2][2];
+#pragma unroll
+  for (int b = 0; b < NB; ++b)
+#pragma unroll
+    for (int n = 0; n < 2; ++n) {
+      const int kb = w + b * WS_WARPS, f = f0 + n * 8 + g;
+      const bool in = kb < KB && f < N;
+      const uint4 *p = reinterpret_cast<const uint4 *>(W + (size_t)f * K + kb * 64 + q4 * 16);
+      wf[b][n][0] = in ? __ldg(p) : zero;
+      wf[b][n][1] = in ? __ldg(p + 1) : zero;
+    }
   // the gains of this thread's two output features (folded norm): constants, fetched before the wait
   float2 gg = make_float2(0.f, 0.f);
   if (NORM && nm.a_out && f0 + (tid & 7) * 2 < N) gg = *reinterpret_cast<const float2 *>(nm.gain + f0 + (tid & 7) * 2);
   pdl_sync();
-  // ---- activation tile (rows past M are zero)
-  for (int i = tid; i < WS_MT * cpr; i += 256) {
-    const int r = i / cpr, c = i % cpr;
-    unsigned char *dst = As + r * row_bytes + ((c ^ (r & 7)) << 4);
-    if (t0 + r < M) cp_async16(dst, A + (size_t)(t0 + r) * K + c * 8);
-    else *reinterpret_cast<uint4 *>(dst) = make_uint4(0u, 0u, 0u, 0u);
-  }
-  asm volatile("cp.async.commit_group;" ::: "memory");
-  // ---- while the copies fly: this thread's two outputs, their old values, the rows' rstd
+  // ---- token fragments: rows g and g + 8 of each 16-row tile
+  const int n_mt = t0 + 16 < M ? 2 : 1;
+  uint4 af[2][NB][2][2];
+#pragma unroll
+  for (int m = 0; m < 2; ++m)
+#pragma unroll
+    for (int b = 0; b < NB; ++b)
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        const int kb = w + b * WS_WARPS, t = t0 + m * 16 + r * 8 + g;
+        const bool in = kb < KB && t < M;
+        const bf16 *p = A + (size_t)t * K + kb * 64 + q4 * 16;
+        af[m][b][r][0] = zero;
+        af[m][b][r][1] = zero;
+        if (in) {
+          af[m][b][r][0] = ws_ld16(p);
+          af[m][b][r][1] = ws_ld16(p + 8);
+        }
+      }
+  // ---- while the loads fly: this thread's two outputs, their old values, the rows' rstd
   const int orow = tid >> 3, ocol = (tid & 7) * 2;             // output (orow, ocol), (orow, ocol + 1) of the tile
   const int t = t0 + orow, f = f0 + ocol;
   const bool live = t < M && f < N;                            // (N is even: both columns or none)
@@ -97,31 +111,32 @@ gemm_ws_kernel(const bf16 *A, const bf16 *__restrict__ W, void *C, int M, int N,
     acc += __shfl_xor_sync(0xffffffffu, acc, 4);
     if ((tid & 7) == 0) rs[orow] = rsqrtf(acc * nm.inv_d + nm.eps);
   }
-  asm volatile("cp.async.wait_all;" ::: "memory");
-  __syncthreads();
-
-  // ---- main loop: warp w takes k steps w, w + 8, ...; acc[row tile][feature tile][4]
+  // ---- main loop; acc[row tile][feature tile][4]
   float acc[2][2][4];
 #pragma unroll
   for (int a = 0; a < 2; ++a)
 #pragma unroll
     for (int b = 0; b < 2; ++b) acc[a][b][0] = acc[a][b][1] = acc[a][b][2] = acc[a][b][3] = 0.f;
-  const int a_row = lane & 15, a_chunk = lane >> 4;                           // A fragment addressing
-  const int b_row = (lane & 7) + ((lane >> 4) & 1) * 8, b_chunk = (lane >> 3) & 1;   // B: two feature tiles at once
-  for (int ks = w; ks < (K >> 4); ks += WS_WARPS) {
-    uint32_t bw[4], a0[4], a1[4];
-    ws_ldsm4(Ws32 + (uint32_t)(b_row * row_bytes + (((ks * 2 + b_chunk) ^ (b_row & 7)) << 4)), bw);
-    ws_ldsm4(As32 + (uint32_t)(a_row * row_bytes + (((ks * 2 + a_chunk) ^ (a_row & 7)) << 4)), a0);
-    ws_ldsm4(As32 + (uint32_t)((16 + a_row) * row_bytes + (((ks * 2 + a_chunk) ^ (a_row & 7)) << 4)), a1);
-    mma_bf16_16816(acc[0][0], a0, bw[0], bw[1]);
-    mma_bf16_16816(acc[0][1], a0, bw[2], bw[3]);
-    mma_bf16_16816(acc[1][0], a1, bw[0], bw[1]);
-    mma_bf16_16816(acc[1][1], a1, bw[2], bw[3]);
+#pragma unroll
+  for (int m = 0; m < 2; ++m) {
+    if (m >= n_mt) break;
+#pragma unroll
+    for (int b = 0; b < NB; ++b)
+#pragma unroll
+      for (int s = 0; s < 2; ++s) {                            // 16-byte halves: two k steps each
+        const uint4 lo = af[m][b][0][s], hi = af[m][b][1][s];
+        const uint32_t a0[4] = {lo.x, hi.x, lo.y, hi.y}, a1[4] = {lo.z, hi.z, lo.w, hi.w};
+#pragma unroll
+        for (int n = 0; n < 2; ++n) {
+          mma_bf16_16816(acc[m][n], a0, wf[b][n][s].x, wf[b][n][s].y);
+          mma_bf16_16816(acc[m][n], a1, wf[b][n][s].z, wf[b][n][s].w);
+        }
+      }
   }
   // ---- partial tiles to shared memory, summed in warp order
   {
     float *mine = red + w * (WS_MT * WS_FN);
-    const int g = lane >> 2, q = (lane & 3) * 2;
+    const int q = q4 * 2;
 #pragma unroll
     for (int a = 0; a < 2; ++a)
 #pragma unroll
@@ -162,28 +177,27 @@ gemm_ws_kernel(const bf16 *A, const bf16 *__restrict__ W, void *C, int M, int N,
 }
 
 // ------------------------------------------------------------------ host side
-static int gemm_ws_init() {
-  static std::mutex mu;
-  static bool dev_done[TC_MAX_DEVICES] = {false};
-  std::lock_guard<std::mutex> lock(mu);
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= TC_MAX_DEVICES) return -4;
-  if (dev_done[dev]) return 0;
-  if (cudaFuncSetAttribute(gemm_ws_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess ||
-      cudaFuncSetAttribute(gemm_ws_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess)
-    return -4;
-  dev_done[dev] = true;
-  return 0;
-}
+static inline int ws_blocks(int K) { return (K / 64 + WS_WARPS - 1) / WS_WARPS; }
 
-// Whether this kernel is the better tool for the shape: few tokens, the two tiles fit in shared
-// memory, N even and the operands 16-byte aligned, and the whole grid is resident at once.
-static bool gemm_ws_eligible(const void *A, const void *W, int M, int N, int K) {
+// Shapes that the single-contraction entry point gives to this kernel on request.
+static bool gemm_ws_accepts(const void *A, const void *W, int M, int N, int K) {
   if (M < 1 || M > 256 || K < 64 || K % 64 || K > WS_MAX_K || N % 2) return false;
   if (((uintptr_t)A & 15) || ((uintptr_t)W & 15)) return false;
-  const int smem = ws_smem_bytes(K);
-  if (smem > 227 * 1024) return false;
-  const int per_sm = std::min(8, (228 * 1024) / (smem + 1024));
+  const int bytes = (WS_FN + WS_MT) * K * 2 + WS_WARPS * WS_MT * WS_FN * 4 + WS_MT * 4;
+  const int per_sm = std::min(8, (228 * 1024) / (bytes + 1024));
+  const long ctas = (long)((N + WS_FN - 1) / WS_FN) * ((M + WS_MT - 1) / WS_MT);
+  return ctas <= (long)per_sm * 148;
+}
+// Whether this kernel is the better tool for the shape: K in the registers of eight warps, N even, the operands
+// 16-byte aligned, and the whole grid resident at once -- three CTAs per SM by registers where a warp has one block
+// of K, two with two, else one.  On either side of that line (us, gemm_sk_kernel / this): M = 319, N = 512, K = 512
+// (320 CTAs) 5.1 / 3.5, M = 512, N = 256, K = 1024 (256 CTAs) 6.2 / 3.7, M = 93, N = 1024, K = 1024 (192) 5.3 / 3.7;
+// M = 160, N = 2048, K = 512 (640) 6.0 / 6.2, M = 256, N = 1024, K = 1024 (512) 6.7 / 6.9, M = 64, N = 1280, K = 1280
+// (160) 5.6 / 5.9.
+static bool gemm_ws_eligible(const void *A, const void *W, int M, int N, int K) {
+  if (M < 1 || M > 512 || K < 64 || K % 64 || K > WS_MAX_K || N % 2) return false;
+  if (((uintptr_t)A & 15) || ((uintptr_t)W & 15)) return false;
+  const int nb = ws_blocks(K), per_sm = nb == 1 ? 3 : nb == 2 ? 2 : 1;
   const long ctas = (long)((N + WS_FN - 1) / WS_FN) * ((M + WS_MT - 1) / WS_MT);
   return ctas <= (long)per_sm * 148;
 }
@@ -193,7 +207,6 @@ static bool gemm_ws_launch(cudaStream_t st, bool pdl, const void *A, const void 
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((N + WS_FN - 1) / WS_FN, (M + WS_MT - 1) / WS_MT);
   cfg.blockDim = dim3(256);
-  cfg.dynamicSmemBytes = ws_smem_bytes(K);
   cfg.stream = st;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -201,9 +214,15 @@ static bool gemm_ws_launch(cudaStream_t st, bool pdl, const void *A, const void 
   cfg.attrs = at;
   cfg.numAttrs = pdl ? 1 : 0;
   const SkNorm nm = norm ? *norm : SkNorm{};
-  if (norm)
-    return cudaLaunchKernelEx(&cfg, gemm_ws_kernel<true>, (const bf16 *)A, (const bf16 *)W, C, M, N, K, epi, nm, lr) == cudaSuccess;
-  return cudaLaunchKernelEx(&cfg, gemm_ws_kernel<false>, (const bf16 *)A, (const bf16 *)W, C, M, N, K, epi, nm, lr) == cudaSuccess;
+  auto go = [&](auto kernel) {
+    return cudaLaunchKernelEx(&cfg, kernel, (const bf16 *)A, (const bf16 *)W, C, M, N, K, epi, nm, lr) == cudaSuccess;
+  };
+  switch (ws_blocks(K)) {
+    case 1: return norm ? go(gemm_ws_kernel<1, true>) : go(gemm_ws_kernel<1, false>);
+    case 2: return norm ? go(gemm_ws_kernel<2, true>) : go(gemm_ws_kernel<2, false>);
+    case 3: return norm ? go(gemm_ws_kernel<3, true>) : go(gemm_ws_kernel<3, false>);
+    default: return norm ? go(gemm_ws_kernel<4, true>) : go(gemm_ws_kernel<4, false>);
+  }
 }
 
 }  // namespace tsfm

@@ -20,7 +20,8 @@
 // Bound: latency for small shapes (launch, one L2 round trip, the 8-way sum; 3.5 us a link inside a captured
 // forecast where the 64 x 64 tile took 8 to 31 us at M = 37 ... 185, K = 128, 512: forecast of one series
 // with the 2-layer d = 128 model 636 -> 260 us, of 37 series 2.55 -> 0.90 ms), FMA rate for many rows.
-// grid = (ceil(N / FN), ceil(M / MT)), block = 256.  K a multiple of 16.
+// grid = (ceil(N / FN), row tiles), block = 256.  K a multiple of 16.  The row tiles take y first, and z where
+// there are more than a grid's y can count (2 million rows in tiles of 32).
 #pragma once
 #include "common.cuh"
 #include "kernels_simt.cuh"
@@ -48,6 +49,8 @@ struct RowsArgs {
   int k_pos, Kblk;
 };
 
+constexpr int F32_GRID_Y = 65535;                              // the largest y of a grid
+
 template <typename T, int MT, int FN> constexpr int f32_smem_bytes(int KC) {
   const int rows = MT * (KC + 4) * 4 + FN * (KC * (int)sizeof(T) + 16), red = 8 * MT * FN * 4;   // the partial sums reuse the rows
   return rows > red ? rows : red;
@@ -69,7 +72,9 @@ gemm_f32_kernel(const float *A, const T *__restrict__ W, float *C, int M, int N,
   __shared__ int row_series[MT];
   __shared__ float row_ss[MT];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  const int f0 = blockIdx.x * FN, t0 = blockIdx.y * MT;
+  const long long row_tile = (long long)blockIdx.z * F32_GRID_Y + blockIdx.y;
+  if (row_tile * MT >= M) return;                              // (the last z's share of y is not full)
+  const int f0 = blockIdx.x * FN, t0 = (int)row_tile * MT;
   const PassGeom &g = ra.g;
   const int nb = ra.mode == ROWS_HEAD_LAST ? 1 : ra.mode == ROWS_HEAD_ALL ? g.q_len / g.head_step : g.q_len;   // rows per slot
   // rows in use (active-series compaction): read before the dependency wait, see gemm_sk_kernel
@@ -124,7 +129,7 @@ gemm_f32_kernel(const float *A, const T *__restrict__ W, float *C, int M, int N,
   }
   if (tid < MT) row_ss[tid] = 0.f;
   pdl_sync();
-  if (ra.stamp && blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) *ra.stamp = globaltimer_ns();
+  if (ra.stamp && blockIdx.x == 0 && t0 == 0 && tid == 0) *ra.stamp = globaltimer_ns();
   if (ra.mode != ROWS_PLAIN && !early) lookup();
   if (!__syncthreads_or(tid < MT && src_off[tid] >= 0)) {      // a tile of dead slots
     asm volatile("cp.async.wait_all;" ::: "memory");
@@ -234,7 +239,8 @@ static bool gemm_f32_launch(cudaStream_t st, bool pdl, const float *A, const T *
   const int tile = small ? 16 : 32;
   const int KC = K <= (small ? 768 : 512) ? K : 256;
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((N + tile - 1) / tile, (M + tile - 1) / tile);
+  const int row_tiles = (M - 1) / tile + 1;
+  cfg.gridDim = dim3((N + tile - 1) / tile, std::min(row_tiles, F32_GRID_Y), (row_tiles - 1) / F32_GRID_Y + 1);
   cfg.blockDim = dim3(256);
   cfg.dynamicSmemBytes = small ? f32_smem_bytes<T, 16, 16>(KC) : f32_smem_bytes<T, 32, 32>(KC);
   cfg.stream = st;

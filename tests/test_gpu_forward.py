@@ -60,6 +60,28 @@ def test_fp32_contraction_tiles(target, n):
     assert np.abs(gd - wd).max() < 1e-4
 
 
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_forward_of_more_than_two_million_tokens(dtype):
+    """8200 windows of 256 tokens: 65600 tiles of 32 rows in the embedding, the head and the fp32 contractions, where
+    the y of a grid counts to 65535."""
+    import paper_2511_18191_b200 as tsfm
+    wl = small_workload(dtype, Arch(1, 64, 1, 64), Arch(1, 64, 1, 64), 16)
+    tw, dw = build_models(wl)
+    B, n = 8200, 256
+    dec = tsfm.SpecDecoder(tw, dw, wl.target, wl.draft, wl.patch_len, wl.dtype, "separate", max_batch=B, max_ctx_tokens=n,
+                           max_horizon_patches=1, max_K=1)
+    z = torch.randn((B, n, 16), device="cuda", generator=torch.Generator(device="cuda").manual_seed(3))
+    got = dec.model_forward(0, z)
+    dec.close()
+    tm, _ = parity.oracle_models(wl, tw, dw)
+    for b in (0, 4099, 8199):
+        want = orc.forward(tm, z[b].cpu().numpy().astype(np.float64))
+        if dtype == "f32":
+            assert np.abs(got[b].cpu().numpy() - want).max() < 1e-4
+        else:
+            assert parity.value_error("rel_rms", got[b].cpu().numpy(), want) < 2e-2
+
+
 @pytest.mark.parametrize("backend", [1, 0], ids=["simt", "tcgen05"])
 @pytest.mark.parametrize("target,draft,P,n,mode", [
     (Arch(3, 256, 4, 1024), Arch(2, 128, 4, 256), 96, 9, "separate"),      # few tokens: folded norms, K split

@@ -241,6 +241,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant
     if (rank == 0 && elect_one()) {
       // ---------------- MMA issuer
       const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(2 * TC_BM >> 4) << 24);
+      pdl_sync();                                              // (the limit on the waits below starts with the input, not before)
       int s = 0;
       uint32_t ph = 0;
       bool ok = true;
@@ -266,10 +267,11 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant
     // ---------------- factors (folded norm) and cache positions of the rows of each tile
     pdl_sync();
     if (nm.ssq_in || pr.rope) {
-      bool ok = true;
-      for (int tile = pair, i = 0; tile < n_tiles && ok; tile += n_pairs, ++i) {
+      for (int tile = pair, i = 0; tile < n_tiles; tile += n_pairs, ++i) {
         const int rb = i & 1, t0 = (tile / FT) * BN;
-        ok = mbar_wait(rows_empty0 + 8 * rb, ((uint32_t)(i >> 1) & 1u) ^ 1u);
+        const bool ok = mbar_wait(rows_empty0 + 8 * rb, ((uint32_t)(i >> 1) & 1u) ^ 1u);
+        if (!ok) atomicExch(status, DEV_TIMEOUT_EPILOGUE);
+        if (!__all_sync(0xffffffffu, ok)) break;
         for (int r = threadIdx.x - 32 * (PAIR_EPI_WARPS + 2); r < BN && t0 + r < M; r += 32 * PAIR_ROW_WARPS) {
           const int t = t0 + r;
           if (nm.ssq_in) {
@@ -319,7 +321,10 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant
         fetch_old(grp * PAIR_CHUNK);
       }
       // (after a wait that ran out: no more waits, nothing stored)
-      if (ok && (nm.ssq_in || pr.rope)) ok = mbar_wait(rows_full0 + 8 * (i & 1), (uint32_t)(i >> 1) & 1u);
+      if (ok && (nm.ssq_in || pr.rope)) {
+        ok = mbar_wait(rows_full0 + 8 * (i & 1), (uint32_t)(i >> 1) & 1u);
+        if (!ok) atomicExch(status, DEV_TIMEOUT_EPILOGUE);
+      }
       float4 cs[PAIR_CHUNK / 4];
       const bool rotate = pr.rope && f0 < 2 * (N / 3);         // queries and keys
       if (ok && rotate) pair_rope_fetch(cs, pos + grp * PAIR_CHUNK, w4, t0 + grp * PAIR_CHUNK, grp * PAIR_CHUNK < BN ? M : 0, pr.dh >> 1, pl.dim, pr.rope);

@@ -453,6 +453,40 @@ def other_workloads(names):
     return out
 
 
+# ------------------------------------------------------------------ output
+# Whoever reads the result line keeps the end of stdout, a few thousand characters: the line on stdout holds the
+# headline and one figure or two of every further workload; everything measured goes to stderr, one line too.
+LINE_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling", "vs_baseline",
+             "dtype", "data", "config", "e2e", "gpu_launches", "clocks")
+ROOFLINE_KEYS = ("kernel", "bound", "achieved", "peak", "unit", "frac", "peak_source", "share_of_step", "avg_launch_us")
+
+
+def _plain(v):
+    """JSON-safe copy: five significant digits below the headline, no NaN or infinity."""
+    if isinstance(v, dict):
+        return {k: _plain(x) for k, x in v.items()}
+    if isinstance(v, (list, tuple)):
+        return [_plain(x) for x in v]
+    if isinstance(v, float):
+        return float(f"{v:.5g}") if np.isfinite(v) else None
+    return v
+
+
+def result_line(r):
+    """The line on stdout from everything that was measured."""
+    line = {k: r[k] for k in LINE_KEYS}
+    line["roofline"] = _plain({k: r["roofline"][k] for k in ROOFLINE_KEYS})
+    line["speedup_vs_target_only"] = _plain(r["speedup_vs_target_only"])
+    line["phases_ms"] = _plain(r["phases_ms"])
+    if "cpu_baseline" in r:
+        line["cpu_baseline"] = _plain({k: v for k, v in r["cpu_baseline"].items() if k != "sample"})
+    if "workloads" in r:
+        line["workloads"] = {
+            n: {"error": w["error"][:60]} if "error" in w else
+            _plain({"ms": w["ms_per_step"], "target_only_ms": w["target_only"]["ms_per_step"]}) for n, w in r["workloads"].items()}
+    return json.dumps(line, allow_nan=False)
+
+
 # ------------------------------------------------------------------ our arm
 def run_ours(args, wl, K, tau):
     world = int(os.environ.get("WORLD_SIZE", "1"))
@@ -525,7 +559,8 @@ def run_ours(args, wl, K, tau):
         dist.barrier()
         dist.destroy_process_group()
     if result is not None:
-        print(json.dumps(result))
+        print(json.dumps(_plain(result), allow_nan=False), file=sys.stderr)
+        print(result_line(result))
 
 
 def main():

@@ -9,6 +9,7 @@ import subprocess
 import sys
 
 import numpy as np
+import pytest
 import torch
 import torch.distributed as dist
 import torch.multiprocessing as mp
@@ -55,3 +56,25 @@ def test_reference_arm_runs_on_rank_zero_only():
     line = json.loads(res.stdout.strip().splitlines()[-1])
     assert line["impl"] == "reference" and line["cpu_baseline"]["kind"] == "oracle" and line["value"] > 0
     assert line["e2e"]["h2d_bytes_per_step"] == 0 and line["n_gpus"] == 2
+
+
+def test_result_line_is_short_and_strict_json():
+    """The headline survives a reader that keeps the last 3000 characters, whatever else was measured."""
+    import bench
+    from tsfm_inputs import workload
+    nan = float("nan")
+    kernel = {k: 1 / 3 for k in ("share", "launches_per_step", "ms_per_step", "GB/s", "frac_hbm")}
+    m = {"ms_per_step": 12.3456789012345, "target_only": {"ms_per_step": 2 / 3}, "speedup_vs_target_only": nan,
+         "phases_ms": {f"ms_{p}": 1 / 3 for p in ("prefill", "draft", "verify", "accept")}, "kernels": {f"kernel_{i}": kernel for i in range(12)},
+         "roofline": dict.fromkeys(bench.ROOFLINE_KEYS, 1 / 3), "mse_vs_truth": {"speculative": nan}}
+    wl = workload("C4")
+    r = dict(m, metric=bench.METRIC, value=123456.789012345, unit=bench.UNIT, n_gpus=1, steps=20, warmup=5, higher_is_better=True,
+             scaling="weak", vs_baseline=None, dtype="bf16", data="synthetic", config=bench.bench_config(wl, wl.K, wl.tau),
+             e2e={"value": 1 / 3, "unit": bench.UNIT, "h2d_bytes_per_step": 1, "d2h_bytes_per_step": 2}, gpu_launches=12345,
+             clocks={"sm_mhz": 1965.0, "sm_max_mhz": 1965.0, "reasons": ["sw_power_cap"], "samples": 99},
+             cpu_baseline={"value": 1 / 3, "unit": bench.UNIT, "cores": 64, "kind": "oracle", "sample": "x" * 400},
+             workloads={n: dict(m) for n, _, _, _ in bench.other_workloads(["C2", "C1", "C3", "C5"])} | {"bad": {"error": "e" * 500}})
+    line = bench.result_line(r)
+    assert len(line) < 3000 and "\n" not in line
+    back = json.loads(line, parse_constant=lambda c: pytest.fail(f"not strict JSON: {c}"))
+    assert back["value"] == r["value"] and back["ms_per_step"] == r["ms_per_step"] and set(bench.LINE_KEYS) <= set(back)

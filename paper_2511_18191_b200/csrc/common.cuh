@@ -129,8 +129,9 @@ __device__ __forceinline__ float gelu_erf_fast(float v) {
 
 // Two of them at once, rounded to bf16 (low half: a), for the epilogues of many tokens, whose pace is set by the
 // instructions of this function: packed fp32 arithmetic (two values per instruction), and
-// v Phi(v) = max(v, 0) - |v| erfc(|v| / sqrt(2)) / 2 on both sides, so that nothing is selected.  |v| is bounded by a
-// value whose erfc is 0 in any case: the second term of an infinity is 0 and not inf x 0 (NaN stays NaN).
+// v Phi(v) = max(v, 0) - |v| erfc(|v| / sqrt(2)) / 2 on both sides, so that nothing is selected.  In the second term
+// |v| is bounded by a value whose erfc is 0 in any case: that of an infinity is 0 and not inf x 0.  (Bounding |v| in
+// front of everything instead cost 1 to 3 % of a W1 contraction of 6000 or 16320 tokens; here it is below 1 %.)
 __device__ __forceinline__ uint64_t f32x2(float a, float b) {
   uint64_t r;
   asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
@@ -146,14 +147,8 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
   return r;
 }
-__device__ __forceinline__ float min_nan(float a, float b) {    // NaN if either is
-  float r;
-  asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
-  return r;
-}
 __device__ __forceinline__ uint32_t gelu_erf_fast2(float a, float b) {
-  const float va = min_nan(fabsf(a), 1e18f), vb = min_nan(fabsf(b), 1e18f);
-  const uint64_t v = f32x2(va, vb);
+  const uint64_t v = f32x2(fabsf(a), fabsf(b));
   const uint64_t w = fma2(v, f32x2(0.3275911f * 0.70710678118654752440f, 0.3275911f * 0.70710678118654752440f), f32x2(1.f, 1.f));
   float w0, w1, t0, t1, e0, e1;
   asm("mov.b64 {%0, %1}, %2;" : "=f"(w0), "=f"(w1) : "l"(w));
@@ -174,7 +169,8 @@ __device__ __forceinline__ uint32_t gelu_erf_fast2(float a, float b) {
   const uint64_t he = mul2(mul2(t, p), f32x2(e0, e1));         // erfc / 2
   float h0, h1;
   asm("mov.b64 {%0, %1}, %2;" : "=f"(h0), "=f"(h1) : "l"(he));
-  const __nv_bfloat162 r = __floats2bfloat162_rn(fmaf(-va, h0, fmaxf(a, 0.f)), fmaf(-vb, h1, fmaxf(b, 0.f)));
+  const __nv_bfloat162 r = __floats2bfloat162_rn(fmaf(-fminf(fabsf(a), 1e18f), h0, fmaxf(a, 0.f)),
+                                                  fmaf(-fminf(fabsf(b), 1e18f), h1, fmaxf(b, 0.f)));
   return *reinterpret_cast<const uint32_t *>(&r);
 }
 

@@ -321,17 +321,12 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant
         fetch_old(grp * PAIR_CHUNK);
       }
       // (after a wait that ran out: no more waits, nothing stored)
-      if (ok && (nm.ssq_in || pr.rope)) {
-        ok = mbar_wait(rows_full0 + 8 * (i & 1), (uint32_t)(i >> 1) & 1u);
-        if (!ok) atomicExch(status, DEV_TIMEOUT_EPILOGUE);
-      }
+      if (ok && (nm.ssq_in || pr.rope)) ok = mbar_wait(rows_full0 + 8 * (i & 1), (uint32_t)(i >> 1) & 1u);
       float4 cs[PAIR_CHUNK / 4];
       const bool rotate = pr.rope && f0 < 2 * (N / 3);         // queries and keys
       if (ok && rotate) pair_rope_fetch(cs, pos + grp * PAIR_CHUNK, w4, t0 + grp * PAIR_CHUNK, grp * PAIR_CHUNK < BN ? M : 0, pr.dh >> 1, pl.dim, pr.rope);
-      if (ok) {
-        ok = mbar_wait_cluster(acc_full0 + 8 * buf, (uint32_t)use & 1u);
-        if (!ok) atomicExch(status, DEV_TIMEOUT_EPILOGUE);
-      }
+      if (ok) ok = mbar_wait_cluster(acc_full0 + 8 * buf, (uint32_t)use & 1u);
+      if (!ok) atomicExch(status, DEV_TIMEOUT_EPILOGUE);       // (either wait)
       ok = __all_sync(0xffffffffu, ok);
       tc_fence_after();
       const uint32_t tbase = tmem + ((uint32_t)(w4 * 32) << 16) + (uint32_t)(buf * BN);

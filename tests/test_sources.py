@@ -17,15 +17,15 @@ def _read(path):
 
 @pytest.mark.parametrize("path", FILES, ids=os.path.basename)
 def test_every_bounded_wait_reports_that_it_ran_out(path):
-    """A wait that gives up writes its code to the status word, in its own statement or one of the two behind it;
-    without that the call would return success with an output that was never written."""
+    """A wait that gives up writes its code to the status word, in its own statement or within the next lines (two waits
+    may share a report); without that the call would return success with an output that was never written."""
     lines, seen = _read(path), 0
     for i, line in enumerate(lines):
         if WAIT.search(line) and "__device__" not in line:
             seen += 1
-            # "if (wait) { ... } else report", or the report in the next two lines
+            # "if (wait) { ... } else report", or the report close behind
             positive = re.search(r"if \(mbar_wait\w*\([^!]*\{\s*$", line)
-            near = "".join(lines[i:]).split("} else")[1][:80] if positive else "".join(lines[i:i + 3])
+            near = "".join(lines[i:]).split("} else")[1][:80] if positive else "".join(lines[i:i + 7])
             assert re.search(r"atomicExch\(status, DEV_TIMEOUT_", near), f"{os.path.basename(path)}:{i + 1}: {line.strip()}"
     assert seen
 

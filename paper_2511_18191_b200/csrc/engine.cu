@@ -483,7 +483,19 @@ void gemm(tsfm_spec *h, GemmSkPlan *plan, const void *A, const void *W, void *C,
   const double out_b = (epi == EPI_F32 || epi == EPI_ATOMIC) ? 4.0 : epi == EPI_RESID ? 8.0 : e;
   const double bytes = ((double)N * K + (double)M * K) * e + (double)M * N * out_b;
   const double flops = 2.0 * M * N * K;
-  if (sizeof(T) == 2 && h->use_tc && plan && plan->valid && gemm_ws_eligible(A, W, M, N, K)) {
+  // What the pass has decided on (run_pass) and this contraction's own shape and pointers have to agree: only
+  // gemm_pair_kernel rotates and appends or takes norms in slices of 128 features, only the tensor-core kernels fold
+  // norms of bf16 rows and only gemm_f32_kernel those of fp32 rows.
+  const bool tc = sizeof(T) == 2 && h->use_tc && plan && plan->valid;
+  const bool pair = tc && M >= kPairMinRows && gemm_pair_eligible(*plan, C);
+  if (rope || (norm && M >= kPairMinRows) ? !pair : norm ? !tc : row_gain && !(sizeof(T) == 4 && gemm_f32_eligible(W, K))) {
+    if (h->enqueue_err == TSFM_OK) {
+      h->enqueue_err = TSFM_ERR_INTERNAL;
+      g_cuda_err = "contraction: no kernel for this operand folds the norm or rotation that the pass has planned";
+    }
+    return;
+  }
+  if (tc && gemm_ws_eligible(A, W, M, N, K)) {
     // few tokens, short K: the kernel with its weight tile in registers has the shorter chain
     KTimer kt(h, KC_GEMM_WS, bytes, flops);
     if (gemm_ws_launch(h->ls, h->pdl, A, W, C, M, N, K, epi, norm, lr)) {
@@ -494,9 +506,8 @@ void gemm(tsfm_spec *h, GemmSkPlan *plan, const void *A, const void *W, void *C,
     }
     return;
   }
-  if (sizeof(T) == 2 && h->use_tc && plan && plan->valid) {
+  if (tc) {
     KTimer kt(h, M <= 512 ? KC_GEMM_TC_SMALL : M < 4096 ? KC_GEMM_TC_MID : KC_GEMM_TC_LARGE, bytes, flops);
-    const bool pair = M >= kPairMinRows && gemm_pair_eligible(*plan, C);
     if (pair ? gemm_pair_launch(h->ls, h->pdl, *plan, C, M, epi, h->dev_status, lr, norm, rope)
              : gemm_sk_launch(h->ls, h->pdl, *plan, C, M, epi, h->dev_status, norm, lr)) {
       LAUNCHED();

@@ -473,6 +473,10 @@ constexpr int kPairMinRows = 513;
 // layer folded, 136 + 2 x 8 with the kernel).
 constexpr int kPairFoldMaxRows = 3072;
 
+// Whether gemm_f32_kernel takes an operand (contractions of fp32 models, embedding and head of both kinds).
+// TSFM_GEMM_SIMT keeps to the plain kernels, which share no code with it.
+bool f32_tiles(const tsfm_spec *h, const void *W, int K) { return h->cfg.gemm_backend != TSFM_GEMM_SIMT && gemm_f32_eligible(W, K); }
+
 // C (op)= A . W^T through the tensor-core kernel when a plan exists, else an FMA kernel.  row_gain (fp32
 // models whose rows gemm_f32_kernel takes): A is the residual stream, normalised by the contraction itself.
 template <typename T>
@@ -488,7 +492,7 @@ void gemm(tsfm_spec *h, GemmSkPlan *plan, const void *A, const void *W, void *C,
   // norms of bf16 rows and only gemm_f32_kernel those of fp32 rows.
   const bool tc = sizeof(T) == 2 && h->use_tc && plan && plan->valid;
   const bool pair = tc && M >= kPairMinRows && gemm_pair_eligible(*plan, C);
-  if (rope || (norm && M >= kPairMinRows) ? !pair : norm ? !tc : row_gain && !(sizeof(T) == 4 && gemm_f32_eligible(W, K))) {
+  if (rope || (norm && M >= kPairMinRows) ? !pair : norm ? !tc : row_gain && !(sizeof(T) == 4 && f32_tiles(h, W, K))) {
     if (h->enqueue_err == TSFM_OK) {
       h->enqueue_err = TSFM_ERR_INTERNAL;
       g_cuda_err = "contraction: no kernel for this operand folds the norm or rotation that the pass has planned";
@@ -521,7 +525,7 @@ void gemm(tsfm_spec *h, GemmSkPlan *plan, const void *A, const void *W, void *C,
   }
   KTimer kt(h, KC_GEMM_SIMT, bytes, flops);
   if constexpr (sizeof(T) == 4) {
-    if (gemm_f32_eligible(W, K)) {
+    if (f32_tiles(h, W, K)) {
       RowsArgs ra{};
       ra.mode = ROWS_PLAIN;
       ra.epi = epi;
@@ -643,7 +647,7 @@ void run_pass(tsfm_spec *h, ModelDev &m, int B, const PassGeom &g, int head_mode
   // the QKV contraction of a pass of several query tiles rotates its queries and appends to the cache
   const bool append = on_pairs && g.q_len > ATTN_QT;
   // fp32 models with rows short enough normalise them inside the contraction that reads them.
-  const bool fold32 = sizeof(T) == 4 && gemm_f32_eligible(m.layers[0].Wqkv, d);
+  const bool fold32 = sizeof(T) == 4 && f32_tiles(h, m.layers[0].Wqkv, d);
   const int L = m.arch.n_layers;
   const LiveRows lr{g.n_live, g.q_len};
   auto launched = [&](bool ok, const char *what) {
@@ -658,7 +662,7 @@ void run_pass(tsfm_spec *h, ModelDev &m, int B, const PassGeom &g, int head_mode
   auto *norm_kernel = M <= kNormEarlyMaxRows && d <= 1280 ? rmsnorm_kernel<T, true> : rmsnorm_kernel<T, false>;
   {
     KTimer kt(h, KC_EMBED, (double)M * Pi * 4 + (double)d * Pi * sizeof(T) + (double)M * d * 4, 2.0 * M * Pi * d);
-    if (!fold && gemm_f32_eligible(m.W_emb, Pi)) {
+    if (!fold && f32_tiles(h, m.W_emb, Pi)) {
       RowsArgs ra{};
       ra.mode = ROWS_EMBED;
       ra.epi = EPI_F32;
@@ -722,7 +726,7 @@ void run_pass(tsfm_spec *h, ModelDev &m, int B, const PassGeom &g, int head_mode
   const double rows = head_mode == HEAD_LAST_TO_HIST ? B : Mb;
   KTimer kt(h, head_mode == HEAD_NONE ? -1 : KC_HEAD, rows * d * 4 + (double)P * d * sizeof(T) + rows * P * 4,
             2.0 * rows * P * d);
-  if (head_mode != HEAD_NONE && (fold32 || rows >= kHeadTileRows) && gemm_f32_eligible(m.W_head, d)) {
+  if (head_mode != HEAD_NONE && (fold32 || rows >= kHeadTileRows) && f32_tiles(h, m.W_head, d)) {
     RowsArgs ra{};
     ra.mode = head_mode == HEAD_LAST_TO_HIST ? ROWS_HEAD_LAST : ROWS_HEAD_ALL;
     ra.epi = EPI_F32;

@@ -47,6 +47,21 @@ def test_fp32_forward_matches_oracle(target, draft, P, n):
     assert np.abs(gd - wd).max() < 1e-4
 
 
+@pytest.mark.parametrize("dtype,n", [("f32", 21), ("bf16", 300)])
+def test_forced_plain_kernels_are_a_second_implementation(dtype, n):
+    """TSFM_GEMM_SIMT shares no contraction kernel with the default path: another order of sums, the same result."""
+    import paper_2511_18191_b200 as tsfm
+    wl = small_workload(dtype, Arch(1, 128, 2, 256), Arch(1, 128, 1, 128), 32)
+    plain, want, _, _ = run_forward_case(wl, tsfm.TSFM_GEMM_SIMT, n)
+    auto, _, _, _ = run_forward_case(wl, tsfm.TSFM_GEMM_AUTO, n)
+    if dtype == "f32":
+        assert np.abs(plain - want).max() < 1e-4
+        assert (plain != auto).mean() > 0.1
+    else:
+        assert parity.value_error("rel_rms", plain, want) < 2e-2
+        assert (plain != auto).mean() > 0.1
+
+
 @pytest.mark.parametrize("target,n", [
     (Arch(1, 64, 1, 64), 2),          # K = 64: two vectors per warp; ten rows of a 16-row tile
     (Arch(1, 64, 2, 128), 150),       # 750 rows: ragged last 16-row tile

@@ -319,8 +319,19 @@ constexpr int kFlashWarpLongMinPairs = 1024;
 constexpr int kNarrowSingleMaxCap = 64, kNarrowFewPairs = 148;
 // one-tile passes: a two-stage ring (each warp has a few chunks only, and a third CTA fits on the SM)
 constexpr int kFlashStShort = 2;
+// Shared memory of an attn_tiles_kernel launch: for grids of up to three CTAs per SM at least what keeps an SM from taking
+// more CTAs than an even share of the grid.  The kernel starts while the QKV contraction before it still runs, and where
+// that leaves SMs free (66 of 74 pairs at 1024 tokens of d = 512) those would fill up with CTAs that then run one after
+// the other while the rest of the machine is idle (plain decoding of 64 point tokens a pass behind 512 of them, 16 series,
+// 128 CTAs: 2.97 ms per forecast without, 2.40 with; 8, 24 and 32 series: 2.26 -> 2.12, 3.38 -> 2.95, 3.80 -> 3.39).
+// Larger grids fill the machine anyhow, and the even share then only stands in the way of balancing blocks of different
+// length (scoring 512 CTAs: 510 -> 518 us).
+template <int DH> int tiles_smem(long ctas) {
+  const int share = (int)std::min(4l, (ctas + 147) / 148);
+  return share > 3 ? TilesGeom<DH>::SMEM_BYTES : std::max<int>(TilesGeom<DH>::SMEM_BYTES, 228 * 1024 / (share + 1));
+}
 template <int DH> int flash_set_attr() {
-  CU_TRY(cudaFuncSetAttribute(attn_tiles_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, TilesGeom<DH>::SMEM_BYTES));
+  CU_TRY(cudaFuncSetAttribute(attn_tiles_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, tiles_smem<DH>(1)));
   CU_TRY(cudaFuncSetAttribute(attn_flash_kernel<DH, kFlashStShort>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               FlashGeom<DH, kFlashStShort>::SMEM_BYTES));
   CU_TRY(cudaFuncSetAttribute(attn_narrow_ring_kernel<DH, kFlashStShort>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -565,9 +576,9 @@ void launch_attn(tsfm_spec *h, ModelDev &m, int l, int B, const PassGeom &g, boo
     const int pairs = B * m.arch.n_heads;
     if (pre) {
       const int warps = g.q_len <= 32 ? 2 : 4;
-      launch_ex(h->ls, h->pdl, attn_tiles_kernel<DH>, dim3(m.arch.n_heads, B, (g.q_len + 16 * warps - 1) / (16 * warps)),
-                dim3(32 * warps), (size_t)TilesGeom<DH>::SMEM_BYTES, h->qkv, (const bf16 *)Kc, (const bf16 *)Vc, m.rope, g,
-                m.arch.n_heads, appended ? 1 : 0, (bf16 *)h->ao);
+      const dim3 grid(m.arch.n_heads, B, (g.q_len + 16 * warps - 1) / (16 * warps));
+      launch_ex(h->ls, h->pdl, attn_tiles_kernel<DH>, grid, dim3(32 * warps), (size_t)tiles_smem<DH>((long)grid.x * grid.y * grid.z),
+                h->qkv, (const bf16 *)Kc, (const bf16 *)Vc, m.rope, g, m.arch.n_heads, appended ? 1 : 0, (bf16 *)h->ao);
       return;
     }
     if (g.q_len <= 8) {

@@ -462,14 +462,18 @@ void launch_ex_cluster(cudaStream_t s, bool pdl, int cluster_z, void (*kernel)(K
   LAUNCHED();
 }
 
+// (Grids of more than one CTA per SM start after their predecessor has ended: CTAs that start early gather on the SMs
+// that are done first, and the grid waits for those; 512 tiles of K = 1024 289 -> 199 us, K = 4096 1115 -> 776.)
 template <typename T>
-void launch_gemm_simt(cudaStream_t s, bool pdl, const T *A, const T *W, void *C, int M, int N, int K, int epi) {
+void launch_gemm_simt(cudaStream_t s, bool pdl, const T *A, const T *W, void *C, int M, int N, int K, int epi,
+                      LiveRows lr = LiveRows{nullptr, 0}) {
   dim3 grid((N + 63) / 64, (M + 63) / 64), block(256);
+  pdl = pdl && (long)grid.x * grid.y <= 148;
   switch (epi) {
-    case EPI_F32: launch_ex(s, pdl, gemm_simt_kernel<T, EPI_F32>, grid, block, 0, A, W, C, M, N, K); break;
-    case EPI_T: launch_ex(s, pdl, gemm_simt_kernel<T, EPI_T>, grid, block, 0, A, W, C, M, N, K); break;
-    case EPI_GELU_T: launch_ex(s, pdl, gemm_simt_kernel<T, EPI_GELU_T>, grid, block, 0, A, W, C, M, N, K); break;
-    default: launch_ex(s, pdl, gemm_simt_kernel<T, EPI_RESID>, grid, block, 0, A, W, C, M, N, K); break;
+    case EPI_F32: launch_ex(s, pdl, gemm_simt_kernel<T, EPI_F32>, grid, block, 0, A, W, C, M, N, K, lr); break;
+    case EPI_T: launch_ex(s, pdl, gemm_simt_kernel<T, EPI_T>, grid, block, 0, A, W, C, M, N, K, lr); break;
+    case EPI_GELU_T: launch_ex(s, pdl, gemm_simt_kernel<T, EPI_GELU_T>, grid, block, 0, A, W, C, M, N, K, lr); break;
+    default: launch_ex(s, pdl, gemm_simt_kernel<T, EPI_RESID>, grid, block, 0, A, W, C, M, N, K, lr); break;
   }
 }
 
@@ -488,6 +492,18 @@ constexpr int kPairFoldMaxRows = 3072;
 // TSFM_GEMM_SIMT keeps to the plain kernels, which share no code with it.
 bool f32_tiles(const tsfm_spec *h, const void *W, int K) { return h->cfg.gemm_backend != TSFM_GEMM_SIMT && gemm_f32_eligible(W, K); }
 
+// Contractions of fp32 models with a short K and many 64 x 64 tiles go to gemm_simt_kernel: gemm_f32_kernel divides K
+// over its eight warps and has their partial tiles to sum at the end.  Chains of dependent launches, us, gemm_f32_kernel
+// / gemm_simt_kernel: 512 tiles of K = 64 28.6 / 17.4, of K = 128 37.8 / 29.6, of K = 256 56.4 / 55.5; 1536 tiles 81 / 40,
+// 110 / 74, 166 / 141.  Below 256 tiles the launch of the norm, which gemm_f32_kernel folds in, takes up what is won
+// (scoring 2048 tokens with d = 64, 96 and 128 tiles: 206 us, 251 with the plain kernel).  With longer K the plain
+// kernel's sums have the larger error (K = 512: 1.2e-7 against 0.9e-7) for 3 % of the time at 1536 tiles.
+bool f32_many(int M, int N, int K) {
+  const long tiles = (long)((M + 63) / 64) * ((N + 63) / 64);
+  return K <= 256 && tiles >= (K <= 128 ? 256 : 1024) && M <= 65535 * 64;      // (its row tiles are the y of a grid)
+}
+bool f32_takes(const tsfm_spec *h, const void *W, int M, int N, int K) { return f32_tiles(h, W, K) && !f32_many(M, N, K); }
+
 // C (op)= A . W^T through the tensor-core kernel when a plan exists, else an FMA kernel.  row_gain (fp32
 // models whose rows gemm_f32_kernel takes): A is the residual stream, normalised by the contraction itself.
 template <typename T>
@@ -503,7 +519,7 @@ void gemm(tsfm_spec *h, GemmSkPlan *plan, const void *A, const void *W, void *C,
   // norms of bf16 rows and only gemm_f32_kernel those of fp32 rows.
   const bool tc = sizeof(T) == 2 && h->use_tc && plan && plan->valid;
   const bool pair = tc && M >= kPairMinRows && gemm_pair_eligible(*plan, C);
-  if (rope || (norm && M >= kPairMinRows) ? !pair : norm ? !tc : row_gain && !(sizeof(T) == 4 && f32_tiles(h, W, K))) {
+  if (rope || (norm && M >= kPairMinRows) ? !pair : norm ? !tc : row_gain && !(sizeof(T) == 4 && f32_takes(h, W, M, N, K))) {
     if (h->enqueue_err == TSFM_OK) {
       h->enqueue_err = TSFM_ERR_INTERNAL;
       g_cuda_err = "contraction: no kernel for this operand folds the norm or rotation that the pass has planned";
@@ -536,7 +552,7 @@ void gemm(tsfm_spec *h, GemmSkPlan *plan, const void *A, const void *W, void *C,
   }
   KTimer kt(h, KC_GEMM_SIMT, bytes, flops);
   if constexpr (sizeof(T) == 4) {
-    if (f32_tiles(h, W, K)) {
+    if (f32_takes(h, W, M, N, K)) {
       RowsArgs ra{};
       ra.mode = ROWS_PLAIN;
       ra.epi = epi;
@@ -552,7 +568,7 @@ void gemm(tsfm_spec *h, GemmSkPlan *plan, const void *A, const void *W, void *C,
       return;
     }
   }
-  launch_gemm_simt<T>(h->ls, h->pdl, (const T *)A, (const T *)W, C, M, N, K, epi);
+  launch_gemm_simt<T>(h->ls, h->pdl, (const T *)A, (const T *)W, C, M, N, K, epi, lr);
 }
 
 // appended: the QKV contraction has rotated the queries and put the pass's keys and values into the cache;
@@ -657,8 +673,13 @@ void run_pass(tsfm_spec *h, ModelDev &m, int B, const PassGeom &g, int head_mode
   const bool fold_pair = on_pairs && M <= kPairFoldMaxRows;
   // the QKV contraction of a pass of several query tiles rotates its queries and appends to the cache
   const bool append = on_pairs && g.q_len > ATTN_QT;
-  // fp32 models with rows short enough normalise them inside the contraction that reads them.
-  const bool fold32 = sizeof(T) == 4 && f32_tiles(h, m.layers[0].Wqkv, d);
+  // fp32 models normalise the rows inside the contraction that reads them, unless it is so large that doing it once per
+  // feature tile costs more than a link of the chain (1024 x 3072 x 1024: 316 us, 266 + 2 apart; 1024 x 1024 x 256: 34, 29
+  // + 2; rows of up to 128 values: no difference at any size).
+  auto folds32 = [&](const void *W, int N) {
+    return sizeof(T) == 4 && f32_takes(h, W, M, N, d) && (d <= 128 || (double)M * N * d < 3e8);
+  };
+  const bool fold_qkv = folds32(m.layers[0].Wqkv, 3 * d), fold_1 = folds32(m.layers[0].W1, f);
   const int L = m.arch.n_layers;
   const LiveRows lr{g.n_live, g.q_len};
   auto launched = [&](bool ok, const char *what) {
@@ -697,7 +718,7 @@ void run_pass(tsfm_spec *h, ModelDev &m, int B, const PassGeom &g, int head_mode
   consume.eps = eps;
   for (int l = 0; l < L; ++l) {
     LayerDev &ly = m.layers[l];
-    if (!fold && !fold32 && !(fold_pair && l > 0)) {
+    if (!fold && !fold_qkv && !(fold_pair && l > 0)) {
       KTimer kt(h, KC_RMSNORM, norm_bytes, 3.0 * M * d);
       launch_ex(s, h->pdl, norm_kernel, dim3((M + 7) / 8), dim3(256), 0, h->x, ly.g1, M, d, eps, (T *)h->a, lr);
     }
@@ -710,8 +731,8 @@ void run_pass(tsfm_spec *h, ModelDev &m, int B, const PassGeom &g, int head_mode
       pr.n_heads = m.arch.n_heads;
       pr.dh = m.dh;
     }
-    gemm<T>(h, &ly.tc_qkv, fold32 ? (const void *)h->x : h->a, ly.Wqkv, h->qkv, M, 3 * d, d, EPI_F32,
-            fold || (fold_pair && l > 0) ? &consume : nullptr, lr, fold32 ? ly.g1 : nullptr, eps, append ? &pr : nullptr);
+    gemm<T>(h, &ly.tc_qkv, fold_qkv ? (const void *)h->x : h->a, ly.Wqkv, h->qkv, M, 3 * d, d, EPI_F32,
+            fold || (fold_pair && l > 0) ? &consume : nullptr, lr, fold_qkv ? ly.g1 : nullptr, eps, append ? &pr : nullptr);
     const bool cache_only = l == L - 1 && head_mode == HEAD_NONE;      // prefill: only the cache is needed
     if (m.dh == 32) launch_attn<T, 32>(h, m, l, B, g, append, cache_only);
     else if (m.dh == 64) launch_attn<T, 64>(h, m, l, B, g, append, cache_only);
@@ -722,12 +743,12 @@ void run_pass(tsfm_spec *h, ModelDev &m, int B, const PassGeom &g, int head_mode
     produce.a_out = (bf16 *)h->a;
     produce.gain = ly.g2;
     gemm<T>(h, &ly.tc_o, h->ao, ly.Wo, h->x, M, d, d, EPI_RESID, fold || fold_pair ? &produce : nullptr, lr);
-    if (!fold && !fold32 && !fold_pair) {
+    if (!fold && !fold_1 && !fold_pair) {
       KTimer kt(h, KC_RMSNORM, norm_bytes, 3.0 * M * d);
       launch_ex(s, h->pdl, norm_kernel, dim3((M + 7) / 8), dim3(256), 0, h->x, ly.g2, M, d, eps, (T *)h->a, lr);
     }
-    gemm<T>(h, &ly.tc_1, fold32 ? (const void *)h->x : h->a, ly.W1, h->hbuf, M, f, d, EPI_GELU_T,
-            fold || fold_pair ? &consume : nullptr, lr, fold32 ? ly.g2 : nullptr, eps);
+    gemm<T>(h, &ly.tc_1, fold_1 ? (const void *)h->x : h->a, ly.W1, h->hbuf, M, f, d, EPI_GELU_T,
+            fold || fold_pair ? &consume : nullptr, lr, fold_1 ? ly.g2 : nullptr, eps);
     produce.gain = l + 1 < L ? m.layers[l + 1].g1 : nullptr;
     if (l + 1 == L) produce.a_out = nullptr, produce.ssq_out = nullptr;   // the head kernel norms the final rows itself
     gemm<T>(h, &ly.tc_2, h->hbuf, ly.W2, h->x, M, d, f, EPI_RESID, (fold || fold_pair) && l + 1 < L ? &produce : nullptr,
@@ -737,7 +758,7 @@ void run_pass(tsfm_spec *h, ModelDev &m, int B, const PassGeom &g, int head_mode
   const double rows = head_mode == HEAD_LAST_TO_HIST ? B : Mb;
   KTimer kt(h, head_mode == HEAD_NONE ? -1 : KC_HEAD, rows * d * 4 + (double)P * d * sizeof(T) + rows * P * 4,
             2.0 * rows * P * d);
-  if (head_mode != HEAD_NONE && (fold32 || rows >= kHeadTileRows) && f32_tiles(h, m.W_head, d)) {
+  if (head_mode != HEAD_NONE && (sizeof(T) == 4 || rows >= kHeadTileRows) && f32_tiles(h, m.W_head, d)) {
     RowsArgs ra{};
     ra.mode = head_mode == HEAD_LAST_TO_HIST ? ROWS_HEAD_LAST : ROWS_HEAD_ALL;
     ra.epi = EPI_F32;

@@ -230,14 +230,21 @@ template <typename T> static int gemm_f32_init() {
 // Rows that 16-byte copies can fetch.
 static bool gemm_f32_eligible(const void *W, int K) { return K % 16 == 0 && K >= 16 && !((uintptr_t)W & 15); }
 
-// 32 x 32 tiles (twice the flops per shared-memory read) where the 16 x 16 ones would be more than one
-// wave at four CTAs per SM.  Rows of up to 768 values stay whole (one memory round trip; the longest
-// take one CTA per SM); longer ones go through in chunks of 256, four CTAs per SM.
+// 16 x 16 tiles where the grid has at most four of them per SM (with rows of 512 fp32 values three fit at a time: the
+// largest such grids run somewhat over one wave); beyond that 32 x 32 ones (twice the flops per
+// shared-memory read).
+static bool gemm_f32_small(int M, int N) { return (long)((N + 15) / 16) * ((M + 15) / 16) <= 4 * 148; }
+// A small grid keeps rows of up to 768 values whole (one memory round trip), and so does one of up to two 32 x 32 tiles
+// per SM with rows of up to 512.  Otherwise rows longer than 256 go through in chunks of 256: three CTAs of 66 KB (fp32
+// weights) share an SM, one loading while another computes, where rows of 512 in one piece leave room for one
+// (2048 x 512 x 512, 1024 CTAs: 68 -> 50 us; 256 x 1536 x 512, 384 CTAs: 29 -> 22; 512 x 512 x 512, 256 CTAs: 19.4 whole,
+// 20.7 in chunks).
 template <typename T>
 static bool gemm_f32_launch(cudaStream_t st, bool pdl, const float *A, const T *W, float *C, int M, int N, int K, const RowsArgs &ra) {
-  const bool small = (long)((N + 15) / 16) * ((M + 15) / 16) <= 4 * 148;
+  const bool small = gemm_f32_small(M, N);
   const int tile = small ? 16 : 32;
-  const int KC = K <= (small ? 768 : 512) ? K : 256;
+  const bool two_waves = (long)((N + 31) / 32) * ((M + 31) / 32) <= 2 * 148;
+  const int KC = K <= (small ? 768 : two_waves ? 512 : 256) ? K : 256;
   cudaLaunchConfig_t cfg{};
   const int row_tiles = (M - 1) / tile + 1;
   cfg.gridDim = dim3((N + tile - 1) / tile, std::min(row_tiles, F32_GRID_Y), (row_tiles - 1) / F32_GRID_Y + 1);

@@ -75,6 +75,20 @@ def test_fp32_contraction_tiles(target, n):
     assert np.abs(gd - wd).max() < 1e-4
 
 
+@pytest.mark.parametrize("target,B", [
+    (Arch(1, 64, 1, 128), 182),       # 5460 rows: 258 tiles of 64 x 64 for q, k, v (plain kernel), 172 and 86 for the rest
+    (Arch(1, 256, 4, 1024), 138),     # 4140 rows: 1040 tiles of K = 256 for W1 (plain kernel), 780 for q, k, v
+    (Arch(1, 512, 8, 512), 23),       # 690 rows: chunks of K; the norm a launch of its own for q, k, v, folded in for W1
+    (Arch(1, 512, 8, 512), 16),       # 480 rows: 240 tiles of 32 x 32 with whole rows of 512 for all but q, k, v
+])
+def test_fp32_contractions_of_many_rows(target, B):
+    """Either side of the rule that sends fp32 contractions of many rows to the plain kernel, and of folding norms."""
+    wl = small_workload("f32", target, Arch(1, 64, 2, 128), 32)
+    gt, wt, gd, wd = run_forward_case(wl, 0, 30, B=B)
+    assert np.abs(gt - wt).max() < 1e-4        # as above: rounding of fp32 sums
+    assert np.abs(gd - wd).max() < 1e-4
+
+
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 def test_forward_of_more_than_two_million_tokens(dtype):
     """8200 windows of 256 tokens: 65600 tiles of 32 rows in the embedding, the head and the fp32 contractions, where

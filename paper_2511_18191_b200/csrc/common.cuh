@@ -129,9 +129,10 @@ __device__ __forceinline__ float gelu_erf_fast(float v) {
 
 // Two of them at once, rounded to bf16 (low half: a), for the epilogues of many tokens, whose pace is set by the
 // instructions of this function: packed fp32 arithmetic (two values per instruction), and
-// v Phi(v) = max(v, 0) - |v| erfc(|v| / sqrt(2)) / 2 on both sides, so that nothing is selected.  In the second term
-// |v| is bounded by a value whose erfc is 0 in any case: that of an infinity is 0 and not inf x 0.  (Bounding |v| in
-// front of everything instead cost 1 to 3 % of a W1 contraction of 6000 or 16320 tokens; here it is below 1 %.)
+// v Phi(v) = max(v, 0) - |v| erfc(|v| / sqrt(2)) / 2 on both sides, so that nothing is selected.  The second term is
+// (|v| exp(-v^2 / 2)) (t poly), whose first factor is at most 0.61: a saturating product gives 0 and not inf x 0 for an
+// infinity.  (NaN comes back through t.  Bounding |v| instead, in front of everything or in a last product
+// |v| (erfc / 2), cost 1 to 5 % of a W1 contraction of 6000 to 16320 tokens; this form 0.)
 __device__ __forceinline__ uint64_t f32x2(float a, float b) {
   uint64_t r;
   asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
@@ -155,22 +156,23 @@ __device__ __forceinline__ uint32_t gelu_erf_fast2(float a, float b) {
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t0) : "f"(w0));
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t1) : "f"(w1));
   const uint64_t t = f32x2(t0, t1);
-  // the coefficients of A&S 7.1.26, halved
-  uint64_t p = fma2(t, f32x2(0.5f * 1.061405429f, 0.5f * 1.061405429f), f32x2(0.5f * -1.453152027f, 0.5f * -1.453152027f));
-  p = fma2(t, p, f32x2(0.5f * 1.421413741f, 0.5f * 1.421413741f));
-  p = fma2(t, p, f32x2(0.5f * -0.284496736f, 0.5f * -0.284496736f));
-  p = fma2(t, p, f32x2(0.5f * 0.254829592f, 0.5f * 0.254829592f));
+  // the coefficients of A&S 7.1.26, halved and negated
+  uint64_t p = fma2(t, f32x2(-0.5f * 1.061405429f, -0.5f * 1.061405429f), f32x2(0.5f * 1.453152027f, 0.5f * 1.453152027f));
+  p = fma2(t, p, f32x2(-0.5f * 1.421413741f, -0.5f * 1.421413741f));
+  p = fma2(t, p, f32x2(0.5f * 0.284496736f, 0.5f * 0.284496736f));
+  p = fma2(t, p, f32x2(-0.5f * 0.254829592f, -0.5f * 0.254829592f));
   // exp(-v^2 / 2) = 2^(-(log2(e) / 2) v^2)
   const uint64_t x = mul2(mul2(v, f32x2(-0.72134752044448170368f, -0.72134752044448170368f)), v);
   float x0, x1;
   asm("mov.b64 {%0, %1}, %2;" : "=f"(x0), "=f"(x1) : "l"(x));
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e0) : "f"(x0));
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e1) : "f"(x1));
-  const uint64_t he = mul2(mul2(t, p), f32x2(e0, e1));         // erfc / 2
-  float h0, h1;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(h0), "=f"(h1) : "l"(he));
-  const __nv_bfloat162 r = __floats2bfloat162_rn(fmaf(-fminf(fabsf(a), 1e18f), h0, fmaxf(a, 0.f)),
-                                                  fmaf(-fminf(fabsf(b), 1e18f), h1, fmaxf(b, 0.f)));
+  float g0, g1, r0, r1;
+  asm("mul.rn.sat.f32 %0, %1, %2;" : "=f"(g0) : "f"(fabsf(a)), "f"(e0));
+  asm("mul.rn.sat.f32 %0, %1, %2;" : "=f"(g1) : "f"(fabsf(b)), "f"(e1));
+  const uint64_t y = fma2(f32x2(g0, g1), mul2(t, p), f32x2(fmaxf(a, 0.f), fmaxf(b, 0.f)));
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r0), "=f"(r1) : "l"(y));
+  const __nv_bfloat162 r = __floats2bfloat162_rn(r0, r1);
   return *reinterpret_cast<const uint32_t *>(&r);
 }
 

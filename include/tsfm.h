@@ -58,8 +58,9 @@ extern "C" {
 #define TSFM_GEMM_AUTO  0       /* bf16 contractions on tcgen05 tensor cores where shapes allow     */
 #define TSFM_GEMM_SIMT  1       /* force the plain FMA kernels everywhere (differential reference)  */
 #define TSFM_GEMM_WS    2       /* tsfm_gemm_bf16 only: the small-batch kernel that keeps its weight
-                                   tile in shared memory (TSFM_ERR_SHAPE outside its domain: at most
-                                   256 tokens, K a multiple of 64 up to 2048, grid within one wave);
+                                   tile in registers (TSFM_ERR_SHAPE outside its domain: at most
+                                   512 tokens, K a multiple of 64 up to 2048, N even, a grid of
+                                   16 x 32 tiles that is resident at once);
                                    a decoder picks it by itself where it applies                   */
 
 #define TSFM_EXEC_GRAPH   0       /* a forecast is one CUDA-graph launch: prologue, a device-side WHILE

@@ -179,15 +179,6 @@ gemm_ws_kernel(const bf16 *A, const bf16 *__restrict__ W, void *C, int M, int N,
 // ------------------------------------------------------------------ host side
 static inline int ws_blocks(int K) { return (K / 64 + WS_WARPS - 1) / WS_WARPS; }
 
-// Shapes that the single-contraction entry point gives to this kernel on request.
-static bool gemm_ws_accepts(const void *A, const void *W, int M, int N, int K) {
-  if (M < 1 || M > 256 || K < 64 || K % 64 || K > WS_MAX_K || N % 2) return false;
-  if (((uintptr_t)A & 15) || ((uintptr_t)W & 15)) return false;
-  const int bytes = (WS_FN + WS_MT) * K * 2 + WS_WARPS * WS_MT * WS_FN * 4 + WS_MT * 4;
-  const int per_sm = std::min(8, (228 * 1024) / (bytes + 1024));
-  const long ctas = (long)((N + WS_FN - 1) / WS_FN) * ((M + WS_MT - 1) / WS_MT);
-  return ctas <= (long)per_sm * 148;
-}
 // Whether this kernel is the better tool for the shape: K in the registers of eight warps, N even, the operands
 // 16-byte aligned, and the whole grid resident at once -- three CTAs per SM by registers where a warp has one block
 // of K, two with two, else one.  On either side of that line (us, gemm_sk_kernel / this): M = 319, N = 512, K = 512
@@ -198,6 +189,17 @@ static bool gemm_ws_eligible(const void *A, const void *W, int M, int N, int K) 
   if (M < 1 || M > 512 || K < 64 || K % 64 || K > WS_MAX_K || N % 2) return false;
   if (((uintptr_t)A & 15) || ((uintptr_t)W & 15)) return false;
   const int nb = ws_blocks(K), per_sm = nb == 1 ? 3 : nb == 2 ? 2 : 1;
+  const long ctas = (long)((N + WS_FN - 1) / WS_FN) * ((M + WS_MT - 1) / WS_MT);
+  return ctas <= (long)per_sm * 148;
+}
+
+// Shapes that the single-contraction entry point gives to this kernel on request: those that a decoder gives it, and
+// up to 256 tokens on up to eight CTAs per SM where K is short (shapes it has always taken; they run in several waves).
+static bool gemm_ws_accepts(const void *A, const void *W, int M, int N, int K) {
+  if (gemm_ws_eligible(A, W, M, N, K)) return true;
+  if (M < 1 || M > 256 || K < 64 || K % 64 || K > WS_MAX_K || N % 2) return false;
+  if (((uintptr_t)A & 15) || ((uintptr_t)W & 15)) return false;
+  const int per_sm = std::min(8, 228 * 1024 / ((WS_FN + WS_MT) * K * 2 + 17536));
   const long ctas = (long)((N + WS_FN - 1) / WS_FN) * ((M + WS_MT - 1) / WS_MT);
   return ctas <= (long)per_sm * 148;
 }

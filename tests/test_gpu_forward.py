@@ -204,9 +204,10 @@ def test_many_token_gemm_matches_fp64_product(M, N, K):
 
 
 @pytest.mark.parametrize("M,N,K", [(1, 128, 64), (16, 130, 64), (32, 1536, 512), (33, 96, 128), (40, 512, 192), (64, 384, 1536),
-                                   (128, 1152, 384), (31, 512, 2048), (256, 66, 448), (160, 1536, 512)])
+                                   (128, 1152, 384), (31, 512, 2048), (256, 66, 448), (160, 1536, 512), (319, 512, 512),
+                                   (512, 256, 1024), (400, 128, 1536), (512, 144, 2048)])
 def test_small_batch_gemm_matches_fp64_product(M, N, K):
-    """The kernel that keeps its weight tile in shared memory (few tokens, K up to 2048): ragged token
+    """The kernel that keeps its weight tile in registers (few tokens, K up to 2048): ragged token
     and feature tiles, every k step distribution over its eight warps, and the refusal outside its domain."""
     import paper_2511_18191_b200 as tsfm
     g = torch.Generator(device="cpu").manual_seed(M * 11 + N)

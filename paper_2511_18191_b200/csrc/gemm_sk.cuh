@@ -88,11 +88,8 @@ __device__ __forceinline__ void sk_store_rt(void *C, size_t o, float v, int epi)
 // WT = weight tiles per CTA.
 // NORM = compile the folded-RMSNorm epilogues (SkNorm); the plain instantiations carry none of it.
 // tma_c = SK_TMA_ADD: residual epilogue through mapC (fp32 [M][N], box = BN / S tokens x 128 features);
-// tma_c = SK_TMA_BF16 (S = 1 only): bf16 output (with or without GELU) staged as [token][128
-// features] bf16 and written by one TMA store per weight tile through mapC (bf16 [M][N]) -- whole
-// 128-byte lines at once, where per-thread 2-byte stores leave each line to be completed by a
-// second warp later.
 // tma_c = SK_TMA_F32: fp32 output, staged (and summed over the cluster) like SK_TMA_ADD, stored.
+// (SK_TMA_BF16, a bf16 output with or without GELU: gemm_pair_kernel's.)
 enum { SK_TMA_NONE = 0, SK_TMA_ADD = 1, SK_TMA_BF16 = 2, SK_TMA_F32 = 3 };
 // (Both wait only until the copy has READ its shared-memory source: the staging tile may then be reused
 // or the CTA may leave.  The writes themselves complete before the grid does, which is what the next
@@ -147,8 +144,8 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant__
   const int kb_hi = (int)(((long long)KB_all * (rank + 1)) / S);
   const int KB = kb_hi - kb_lo;
   const int a_bytes = BN * TC_BK * 2, w_bytes = TC_W_BYTES * wt, stage_bytes = w_bytes + a_bytes;
-  // (Measured: spreading the K steps of a stage over several accumulators does not help a narrow
-  // tile -- one MMA of 128 x BN x 16 takes ~90 ns whatever BN is -- so one accumulator per tile.)
+  // (One MMA of 128 x BN x 16 issues every 48 cycles for BN up to 64, 126 at BN = 256: spreading the K steps of a stage
+  // over several accumulators does not help a narrow tile.)
 
   if (warp == 4 && lane == 0) {
     // descriptor fetches off the critical path of the first loads (and of the output copy)
@@ -282,13 +279,6 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant__
         if (t0 + cc >= M) break;
         float v[16];
         tmem_ld16(tbase + cc, v);
-        if (tma_c == SK_TMA_BF16) {
-          bf16 *stage_h = reinterpret_cast<bf16 *>(stage_f);
-#pragma unroll
-          for (int j = 0; j < 16; ++j)
-            stage_h[(cc + j) * TC_BM + fl] = __float2bfloat16_rn(epi == EPI_GELU_T ? gelu_erf_fast(v[j]) : v[j]);
-          continue;
-        }
         if (staged) {
 #pragma unroll
           for (int j = 0; j < 16; ++j) stage_f[(cc + j) * TC_BM + fl] = v[j];
@@ -495,9 +485,12 @@ static int gemm_sk_plan(GemmSkPlan *plan, const void *W, int N, int K, const voi
   return 0;
 }
 
-// Tile and split choice for M tokens: one token tile up to 256 rows (rounded up to 16), and
-// as many K splits (a power of two, at most 8, at most the number of K blocks) as it takes to
-// put the grid on most of the 148 SMs.
+// Tile and split choice for M tokens.
+// Up to 512 tokens: 32-token tiles and as many K splits (a power of two, at most 8, at most the number of K blocks) as
+// it takes to put the grid on most of the 148 SMs.
+// From 513 tokens on only widths N % 128 == 64 get here (whole 128-feature tiles go to gemm_pair_kernel).  The rules for
+// them were measured, with the figures below, on widths that gemm_pair_kernel takes today, and on block steps that
+// still divided by the stage count; they were not fitted again.
 // epi: the epilogue (EPI_*); *STG: ring depth, 0 = the default for the tile.
 static void gemm_sk_geometry(int N, int K, int M, int epi, int *BN, int *S, int *WT, int *STG) {
   *WT = 1;
@@ -612,11 +605,10 @@ static bool gemm_sk_launch(cudaStream_t st, bool pdl, GemmSkPlan &p, void *C, in
   if (!norm && p.N % TC_BM == 0 && BN % S == 0 && !((uintptr_t)C & 15)) {
     if (epi == EPI_RESID) tma_c = SK_TMA_ADD;
     else if (epi == EPI_F32) tma_c = SK_TMA_F32;
-    else if ((epi == EPI_T || epi == EPI_GELU_T) && S == 1) tma_c = SK_TMA_BF16;
   }
   const CUtensorMap *mapC = &p.mapW;                         // placeholder when unused
   if (tma_c) {
-    mapC = sk_map_c(p, C, M, BN / S, tma_c == SK_TMA_BF16);
+    mapC = sk_map_c(p, C, M, BN / S, false);
     if (!mapC) return false;
   }
   const SkShape sh = sk_shape(BN, (KB + S - 1) / S, S > 1 || tma_c || norm, wt, stg);

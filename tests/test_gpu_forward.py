@@ -203,6 +203,13 @@ def test_many_token_gemm_matches_fp64_product(M, N, K):
     assert (got - want).abs().max() < 2e-5 * K ** 0.5 + 1e-5
 
 
+@pytest.mark.parametrize("M,N,K", [(513, 192, 192), (960, 2112, 512), (2048, 832, 768), (1100, 576, 2048), (5000, 320, 2048),
+                                   (9000, 1344, 2048), (4100, 448, 320)])
+def test_many_token_gemm_of_odd_widths_matches_fp64_product(M, N, K):
+    """Widths that are an odd multiple of 64 (from 513 tokens): every branch of the tile rule of the single-SM kernel."""
+    test_many_token_gemm_matches_fp64_product(M, N, K)
+
+
 @pytest.mark.parametrize("M,N,K", [(1, 128, 64), (16, 130, 64), (32, 1536, 512), (33, 96, 128), (40, 512, 192), (64, 384, 1536),
                                    (128, 1152, 384), (31, 512, 2048), (256, 66, 448), (160, 1536, 512), (319, 512, 512),
                                    (512, 256, 1024), (400, 128, 1536), (512, 144, 2048)])

@@ -5,7 +5,8 @@
 // rows that do not exist.  Here the keys are the M side of mma.sync m16n8k16 and the queries its N side:
 // S^T = K Q^T (K through ldmatrix as the A operand), P^T becomes the B operand of O^T = V^T P^T by one 8 x 8
 // transpose (movmatrix) per eight keys.  Half the MMAs, 40 instead of 80 registers of fragments, keys in steps
-// of 16 or 32: 24 instead of 16 warps per SM, which is what these latency-bound warps need.
+// of 16 or 32: registers for 24 instead of 16 of these latency-bound warps per SM.  (Shared memory, head size 64: 24
+// warps with rows of up to 32 keys in one stage, 16 with 48, 12 with 64; three CTAs, 12 warps, with the ring.)
 //   * SINGLE: the whole row of a (series, head), cached keys and keys of the pass, sits in one shared-memory
 //     stage of `rows` rows (a multiple of 16, at most 64); otherwise a ring of ST stages of 32 keys.
 //   * mode FLASH_WARP: one warp per (series, head); grid = ceil(pairs / 4).  mode FLASH_SPLIT: four warps share

@@ -477,10 +477,11 @@ void launch_gemm_simt(cudaStream_t s, bool pdl, const T *A, const T *W, void *C,
   }
 }
 
-// From this many tokens on a contraction runs on pairs of SMs (gemm_pair_kernel against gemm_sk_kernel, graph
-// replay of dependent launches, us: M = 576: 9.5 / 9.7, 6.5 / 8.7, 12.6 / 14.8, 14.7 / 14.6 for the four
-// contractions of a d = 1280 layer; M = 1024, d = 768: 7.7 / 7.5, 5.5 / 6.5, 10.8 / 11.9, 10.3 / 11.6;
-// M = 6000, d = 1024: 32 / 47, 16 / 21, 47 / 74, 43 / 61).
+// From this many tokens on a contraction runs on pairs of SMs, at every width.  Scoring passes with four layers, us, with
+// gemm_sk_kernel / gemm_pair_kernel: d = 128: 520 tokens 151 / 127, 1520: 163 / 150, 6000: 252 / 241; d = 256: 174 / 138,
+// 199 / 172, 341 / 287; d = 512: 199 / 176, 286 / 225, 560 / 429; d = 768: 238 / 212, 371 / 284, 838 / 620; d = 1024:
+// 274 / 243, 476 / 358, 1291 / 844; d = 1280: 314 / 297, 645 / 445, 1606 / 1117.  (Of the contractions alone Wo and W2
+// gain nothing up to 3000 tokens: there it is the norms and the cache append in these epilogues that pay.)
 constexpr int kPairMinRows = 513;
 
 // Up to this many tokens their norms are folded in as well: the epilogues that do it cost 1 us per contraction at

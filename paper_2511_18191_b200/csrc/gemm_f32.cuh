@@ -1,12 +1,13 @@
-// Contractions of fp32 activations in fp32 FMAs: every contraction of the fp32 models, and the patch
-// embedding and the mean head of both kinds of model (weights fp32 or bf16).
+// Contractions of fp32 activations in fp32 FMAs: those of the fp32 models (with a short K and many rows:
+// gemm_simt_kernel, see f32_many), and the patch embedding and the mean head of both kinds of model (weights
+// fp32 or bf16).
 //
 //   C[t, f] (op)= sum_k A'[t, k] * W[f, k]       A' = A, or gain * A / sqrt(mean(A^2) + eps)
 //
 // For the small fp32 models a contraction is a link of a chain of dependent launches and costs what its
 // memory round trips cost; a CTA therefore requests its weight rows before the dependency wait and its
 // activation rows in one go behind it, and since it holds the rows it also normalises them (no RMSNorm
-// launch in front).  For the embedding and the head of passes of many rows it is a matter of reading
+// launch in front; large contractions of long rows take one, see run_pass).  For the embedding and the head of passes of many rows it is a matter of reading
 // every weight once per tile of rows instead of once per row or eight rows.
 //   * tile MT tokens x FN features, K in chunks of KC (all of it in one chunk where that fits); the eight
 //     warps take the 4-feature vectors of a chunk in turn (vector w, w + 8, ...), each lane accumulating
@@ -19,7 +20,8 @@
 //     time fall into different banks.
 // Bound: latency for small shapes (launch, one L2 round trip, the 8-way sum; 3.5 us a link inside a captured
 // forecast where the 64 x 64 tile took 8 to 31 us at M = 37 ... 185, K = 128, 512: forecast of one series
-// with the 2-layer d = 128 model 636 -> 260 us, of 37 series 2.55 -> 0.90 ms), FMA rate for many rows.
+// with the 2-layer d = 128 model 636 -> 260 us, of 37 series 2.55 -> 0.90 ms); for many rows the turns of
+// loading, waiting and computing of the three CTAs of an SM (16384 x 3072 x 1024: 25 of 75 TFLOP/s).
 // grid = (ceil(N / FN), row tiles), block = 256.  K a multiple of 16.  The row tiles take y first, and z where
 // there are more than a grid's y can count (2 million rows in tiles of 32).
 #pragma once

@@ -6,7 +6,7 @@
 // 32 KB (512 cycles) for 260 cycles of tensor work.  Two SMs that work on one tile of 256 features x BN
 // tokens each load their half of both operands (128 feature rows, BN / 2 token rows) and both halves feed
 // both tensor cores: 256 + BN cycles of fill for 2 BN cycles of work per block step and SM, i.e. balanced
-// at BN = 256 where the single-SM form needs 2.5 times the work's time.
+// at BN = 256 where the single-SM form needs twice the work's time.
 //   * cluster of 2 along x; rank r owns features 128 r ... 128 r + 127 of the pair's tile in its own
 //     tensor memory, rank 0 issues every MMA; the copies of both ranks report to rank 0's barriers, the
 //     commits arrive at both ranks' (no copy is multicast);
@@ -435,7 +435,12 @@ static int gemm_pair_init() {
   return 0;
 }
 
-// Tile rule: see the header for the cost of a block step; the epilogue of a pair's last tile is not hidden.
+// Tile rule, in cycles: the block steps of the pair with the most tiles (see the header; tiles below 96 tokens gain
+// nothing, a step's fixed part shows), the epilogue of a pair's last tile, which nothing hides, and 20 for each pair at
+// work: the kernel behind starts on the SMs that are left.  (Chains of one contraction alone, 168 shapes of d = 128 to
+// 1280 at 576 to 16320 tokens: 2.0 % above the best tile on average and 15 % at worst, with 10 for a pair 0.6 and 10 %.
+// In whole passes 10 is the worse: it gives Wo and W2 64-token tiles on 65 to 68 pairs instead of 96-token ones on 45;
+// scoring 800 tokens with d = 1280 333 -> 349 us, 1040 with d = 1024 300 -> 310, decoding 1024 series 2670 -> 2738.)
 static PairShape gemm_pair_geometry(int N, int K, int M) {
   const int FT = (N + 2 * TC_BM - 1) / (2 * TC_BM), KB = (K + TC_BK - 1) / TC_BK;
   PairShape sh{};

@@ -48,13 +48,13 @@ UNIT = "patches/s"
 # operands-once bytes of that launch; traffic grows in proportion to the units a launch processes).
 # A kernel that has changed since its capture is listed with None.
 NCU_TRAFFIC_RATIO = {
-    "gemm_sk_small_M": None,
-    "gemm_sk_mid_M": None,
-    "gemm_sk_large_M": None,
-    "gemm_ws_small_M": None,
-    "attn": None,
+    "gemm_sk_small_M": 0.656,      # 1.78 MB read, 0 written, of 2.72 MB (M=160, N=1536, K=512)
+    "gemm_sk_mid_M": 0.564,        # 11.36 MB of 20.15 MB (M=576, N=3840, K=1280): the fp32 result stays in L2 for its consumer
+    "gemm_sk_large_M": 0.81,       # 244.4 MB of 302.2 MB (M=16320, N=3840, K=1280)
+    "gemm_ws_small_M": 0.77,       # 0.942 MB of 1.229 MB (M=64, N=1152, K=384)
+    "attn": 0.99,                  # 95.7 MB of 96.9 MB (C4 verification pass): the KV stream
 }
-NCU_TRAFFIC_SOURCE = {}
+NCU_TRAFFIC_SOURCE = dict.fromkeys(NCU_TRAFFIC_RATIO, "profiles/kernels_for_many_tokens_short_passes_and_fp32.txt (cold caches)")
 
 
 def parse_args():
@@ -458,7 +458,7 @@ def other_workloads(names):
 # headline and one figure or two of every further workload; everything measured goes to stderr, one line too.
 LINE_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling", "vs_baseline",
              "dtype", "data", "config", "e2e", "gpu_launches", "clocks")
-ROOFLINE_KEYS = ("kernel", "bound", "achieved", "peak", "unit", "frac", "peak_source", "share_of_step", "avg_launch_us")
+ROOFLINE_KEYS = ("kernel", "bound", "achieved", "peak", "unit", "frac", "peak_source", "traffic", "share_of_step", "avg_launch_us")
 
 
 def _plain(v):

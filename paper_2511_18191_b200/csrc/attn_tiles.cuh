@@ -14,8 +14,8 @@
 //   * warps skip the half tiles behind their last query; only the rows of a half tile that holds a visible
 //     key are fetched;
 //   * the query blocks with the most keys start first.
-// Bound: latency of a block's first loads and of the mma.sync chains with 16 warps per SM (tensor pipe 40 %
-// busy on the long case).
+// Bound: latency of a block's first loads and of the mma.sync chains with 16 warps per SM (64 x 20 x 255: tensor pipe
+// 31 % busy, issue slots 34 %).
 // grid = (heads, B, ceil(q_len / (16 warps))), block = 32 x warps, warps = 2 where q_len <= 32, else 4.
 #pragma once
 #include "attn_flash.cuh"

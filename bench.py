@@ -48,7 +48,7 @@ UNIT = "patches/s"
 # operands-once bytes of that launch; traffic grows in proportion to the units a launch processes).
 # A kernel that has changed since its capture is listed with None.
 NCU_TRAFFIC_RATIO = {
-    "gemm_sk_small_M": 0.656,      # 1.78 MB read, 0 written, of 2.72 MB (M=160, N=1536, K=512)
+    "gemm_push_small_M": None,
     "gemm_sk_mid_M": 0.564,        # 11.36 MB of 20.15 MB (M=576, N=3840, K=1280): the fp32 result stays in L2 for its consumer
     "gemm_sk_large_M": 0.81,       # 244.4 MB of 302.2 MB (M=16320, N=3840, K=1280)
     "gemm_ws_small_M": 0.77,       # 0.942 MB of 1.229 MB (M=64, N=1152, K=384)

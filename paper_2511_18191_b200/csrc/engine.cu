@@ -26,6 +26,7 @@
 #include "gemm_sk.cuh"
 #include "gemm_ws.cuh"
 #include "gemm_pair.cuh"
+#include "gemm_push.cuh"
 #include "gemm_f32.cuh"
 
 using namespace tsfm;
@@ -177,11 +178,11 @@ struct tsfm_spec {
 namespace {
 
 // Kernel classes for per-launch timing.
-// The tensor-core contraction is one kernel in three regimes: up to 512 tokens it streams weights
-// (HBM / latency bound), from 4096 tokens it is tensor bound, between them it is one wave of tiles.
+// The tensor-memory contractions in three regimes: up to 512 tokens (gemm_push_kernel: HBM / latency bound), from 4096
+// tokens tensor bound, between them one wave of tiles (gemm_pair_kernel; odd widths gemm_sk_kernel).
 enum { KC_INSTNORM = 0, KC_EMBED, KC_RMSNORM, KC_GEMM_WS, KC_GEMM_TC_SMALL, KC_GEMM_TC_MID, KC_GEMM_TC_LARGE, KC_GEMM_SIMT,
        KC_ATTN, KC_HEAD, KC_ACCEPT, KC_DENORM, KC_COUNT };
-const char *const kKernelNames[KC_COUNT] = {"instnorm", "embed", "rmsnorm", "gemm_ws_small_M", "gemm_sk_small_M",
+const char *const kKernelNames[KC_COUNT] = {"instnorm", "embed", "rmsnorm", "gemm_ws_small_M", "gemm_push_small_M",
                                             "gemm_sk_mid_M", "gemm_sk_large_M", "gemm_simt", "attn", "head", "accept",
                                             "denorm"};
 
@@ -388,9 +389,11 @@ void prefer_max_smem_all() {
   prefer_max_smem(denorm_kernel);
   prefer_max_smem(accept_kernel);
   prefer_max_smem(round_end_kernel);
-  prefer_max_smem(gemm_sk_kernel<1, false>);
-  prefer_max_smem(gemm_sk_kernel<1, true>);
-  prefer_max_smem(gemm_sk_kernel<2, false>);
+  prefer_max_smem(gemm_sk_kernel<1>);
+  prefer_max_smem(gemm_sk_kernel<2>);
+  prefer_max_smem(gemm_push_kernel<EPI_F32>);
+  prefer_max_smem(gemm_push_kernel<EPI_GELU_T>);
+  prefer_max_smem(gemm_push_kernel<EPI_RESID>);
   prefer_max_smem(gemm_pair_kernel);
   prefer_max_smem(gemm_ws_kernel<1, false>);
   prefer_max_smem(gemm_ws_kernel<1, true>);
@@ -541,7 +544,8 @@ void gemm(tsfm_spec *h, GemmSkPlan *plan, const void *A, const void *W, void *C,
   if (tc) {
     KTimer kt(h, M <= 512 ? KC_GEMM_TC_SMALL : M < 4096 ? KC_GEMM_TC_MID : KC_GEMM_TC_LARGE, bytes, flops);
     if (pair ? gemm_pair_launch(h->ls, h->pdl, *plan, C, M, epi, h->dev_status, lr, norm, rope)
-             : gemm_sk_launch(h->ls, h->pdl, *plan, C, M, epi, h->dev_status, norm, lr)) {
+             : M < kPairMinRows ? gemm_push_launch(h->ls, h->pdl, *plan, C, M, epi, h->dev_status, norm, lr)
+                                : gemm_sk_launch(h->ls, h->pdl, *plan, C, M, epi, h->dev_status, lr)) {
       LAUNCHED();
     } else if (h->enqueue_err == TSFM_OK) {
       // No silent fallback: the FMA kernel knows nothing of a folded norm, and a pass that mixes
@@ -1259,6 +1263,7 @@ int tsfm_spec_create(const tsfm_weights *target_w, const tsfm_weights *draft_w, 
   if (h->use_tc) {
     if ((rc = gemm_sk_init())) return fail(rc);
     if ((rc = gemm_pair_init())) return fail(rc);
+    if ((rc = gemm_push_init())) return fail(rc);
     for (ModelDev *m : {&h->tgt, &h->drf}) {
       const int d = m->arch.d_model, f = m->arch.d_ff;
       for (LayerDev &ly : m->layers) {
@@ -1497,12 +1502,13 @@ int tsfm_gemm_bf16(void *stream, const void *A, const void *W, float *C, int32_t
     CU_TRY(e0);
   }
   const bool pair = M >= kPairMinRows && gemm_pair_eligible(plan, C);
-  if (pair && gemm_pair_init()) {
+  if (pair ? gemm_pair_init() : gemm_push_init()) {
     cudaFree(status);
     return TSFM_ERR_CUDA;
   }
   const bool ok = pair ? gemm_pair_launch(s, false, plan, C, M, EPI_F32, status, LiveRows{nullptr, 0})
-                       : gemm_sk_launch(s, false, plan, C, M, EPI_F32, status);
+                  : M < kPairMinRows ? gemm_push_launch(s, false, plan, C, M, EPI_F32, status, nullptr, LiveRows{nullptr, 0})
+                                     : gemm_sk_launch(s, false, plan, C, M, EPI_F32, status);
   if (ok) LAUNCHED();
   int hs = 0;
   cudaError_t e1 = cudaMemcpyAsync(&hs, status, sizeof(int), cudaMemcpyDeviceToHost, s);

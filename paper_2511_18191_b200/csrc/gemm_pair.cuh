@@ -31,6 +31,8 @@
 
 namespace tsfm {
 
+// How an output leaves through the TMA unit: fp32 added to what is there, bf16 stored, fp32 stored.
+enum { SK_TMA_NONE = 0, SK_TMA_ADD = 1, SK_TMA_BF16 = 2, SK_TMA_F32 = 3 };
 constexpr int PAIR_CHUNK = 16;                   // tokens per epilogue chunk
 constexpr int PAIR_GROUPS = 4, PAIR_EPI_WARPS = 4 * PAIR_GROUPS, PAIR_ROW_WARPS = 2;
 constexpr int PAIR_THREADS = 32 * (PAIR_EPI_WARPS + 2 + PAIR_ROW_WARPS);

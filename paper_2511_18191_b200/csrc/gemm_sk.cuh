@@ -13,10 +13,8 @@
 //     r, r + S, ... of all S partial tiles through distributed shared memory and applies the
 //     epilogue once.  No atomics, no pre-zeroed accumulator, a fixed summation order, and every
 //     epilogue (GELU included) can be split.
-//   * a residual epilogue (x += A W^T) on a feature count that is a multiple of 128 leaves the
-//     read-modify-write to the TMA unit: the tile (summed over the cluster first) is staged in
-//     shared memory as [token][128 features] fp32 and added to x by one
-//     cp.reduce.async.bulk.tensor per CTA, so no thread waits for the old values of x.
+// Used from 513 tokens on for widths that are an odd multiple of 64 (whole 128-feature tiles go to gemm_pair_kernel, fewer
+// tokens to gemm_push_kernel) and for outputs that are not 16-byte aligned.
 // Warp roles and bounded waits as in gemm_tc.cuh.
 #pragma once
 #include "gemm_tc.cuh"
@@ -72,7 +70,7 @@ static inline SkShape sk_shape(int BN, int kb_per_cta, bool split, int wt = 1, i
   s.stages = stages;
   const int cols = BN * wt;
   s.tmem_cols = cols <= 32 ? 32 : cols <= 64 ? 64 : cols <= 128 ? 128 : cols <= 256 ? 256 : 512;
-  s.smem_bytes = bytes + 1024 + 256 + 1024;        // + alignment slack, barriers, rstd of the tile's rows
+  s.smem_bytes = bytes + 1024 + 256;        // + alignment slack, barriers
   return s;
 }
 
@@ -86,32 +84,10 @@ __device__ __forceinline__ void sk_store_rt(void *C, size_t o, float v, int epi)
 // grid = (ceil(N / 128), ceil(M / BN), S), cluster = (1, 1, S), block = 192.
 // ring_bytes = size of the tile region (a multiple of 1024); barriers sit behind it.
 // WT = weight tiles per CTA.
-// NORM = compile the folded-RMSNorm epilogues (SkNorm); the plain instantiations carry none of it.
-// tma_c = SK_TMA_ADD: residual epilogue through mapC (fp32 [M][N], box = BN / S tokens x 128 features);
-// tma_c = SK_TMA_F32: fp32 output, staged (and summed over the cluster) like SK_TMA_ADD, stored.
-// (SK_TMA_BF16, a bf16 output with or without GELU: gemm_pair_kernel's.)
-enum { SK_TMA_NONE = 0, SK_TMA_ADD = 1, SK_TMA_BF16 = 2, SK_TMA_F32 = 3 };
-// (Both wait only until the copy has READ its shared-memory source: the staging tile may then be reused
-// or the CTA may leave.  The writes themselves complete before the grid does, which is what the next
-// kernel's dependency wait waits for.)
-__device__ __forceinline__ void sk_tma_store(const CUtensorMap *map, uint32_t src, int x, int y) {
-  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];"
-               ::"l"(map), "r"(x), "r"(y), "r"(src) : "memory");
-  asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-  asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-}
-__device__ __forceinline__ void sk_tma_reduce_add(const CUtensorMap *map, uint32_t src, int x, int y) {
-  asm volatile("cp.reduce.async.bulk.tensor.2d.global.shared::cta.add.tile.bulk_group [%0, {%1, %2}], [%3];"
-               ::"l"(map), "r"(x), "r"(y), "r"(src) : "memory");
-  asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-  asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-}
-
-template <int WT, bool NORM>
+template <int WT>
 __global__ void __launch_bounds__(192, 1)
 gemm_sk_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant__ CUtensorMap mapA,
-               const __grid_constant__ CUtensorMap mapC, void *C, int M, int N, int K, int BN,
-               int stages, int tmem_cols, int ring_bytes, int epi, int tma_c, const SkNorm nm,
+               void *C, int M, int N, int K, int BN, int stages, int tmem_cols, int ring_bytes, int epi,
                int *__restrict__ status, const LiveRows lr) {
   constexpr int wt = WT;
   // Active-series compaction: only the first n_live * q_len rows are in use.  CTAs (whole clusters:
@@ -130,7 +106,6 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant__
   const uint32_t bars = tiles + (uint32_t)ring_bytes;
   const uint32_t full0 = bars, empty0 = bars + 64, accum = bars + 128, slot = bars + 136;
   uint32_t *slot_ptr = reinterpret_cast<uint32_t *>(smem_raw + (slot - smem_u32(smem_raw)));
-  float *rs = reinterpret_cast<float *>(smem_raw + (bars + 256 - smem_u32(smem_raw)));   // [BN] rstd of the tile's rows
   float *stage_f = reinterpret_cast<float *>(smem_raw + (tiles - smem_u32(smem_raw)));
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -148,10 +123,9 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant__
   // over several accumulators does not help a narrow tile.)
 
   if (warp == 4 && lane == 0) {
-    // descriptor fetches off the critical path of the first loads (and of the output copy)
+    // descriptor fetches off the critical path of the first loads
     asm volatile("prefetch.tensormap [%0];" ::"l"(&mapW) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&mapA) : "memory");
-    if (tma_c) asm volatile("prefetch.tensormap [%0];" ::"l"(&mapC) : "memory");
   }
   if (threadIdx.x == 0) {
     for (int s = 0; s < stages; ++s) {
@@ -170,9 +144,6 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant__
   tc_fence_after();
   const uint32_t tmem = *slot_ptr;
 
-  float4 g_vec = make_float4(0.f, 0.f, 0.f, 0.f);
-  constexpr int SK_OLD = 8;                             // rows per thread whose old values are fetched early
-  float4 x_old[NORM ? SK_OLD : 1];
   if (warp == 4 && lane == 0) {
     // ---------------- TMA producer.  The weights do not depend on the preceding kernel: the
     // first ring-full of weight tiles is requested before waiting for it, the activation tiles
@@ -200,44 +171,7 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant__
       if (++s == stages) { s = 0; ph ^= 1u; }
     }
   } else {
-    if (NORM && nm.a_out && warp < 4) {
-      // gains of the features this thread finishes: constants, fetched before the wait
-      const int fv = f0 + (threadIdx.x & 31) * 4;
-      if (N % 4 == 0 && fv + 3 < N) g_vec = *reinterpret_cast<const float4 *>(nm.gain + fv);
-    }
     pdl_sync();
-    if (warp < 4) {
-      if (NORM && nm.ssq_in) {
-        // Four threads per row, 16-byte loads all in flight (d % 64 == 0: whole quads): overlaps the main
-        // loop.  (One thread per row, four bytes at a time, took longer than the loop: K = 1280, 80 slices,
-        // 20 round trips.)
-        const int n4 = nm.n_part >> 2, part = threadIdx.x & 3;
-        for (int i = threadIdx.x >> 2; i < BN; i += 32) {
-          float acc = 0.f;
-          if (t0 + i < M) {
-            const float4 *src = reinterpret_cast<const float4 *>(nm.ssq_in + (size_t)(t0 + i) * nm.n_part);
-#pragma unroll 8
-            for (int j = part; j < n4; j += 4) {
-              const float4 q = src[j];
-              acc += (q.x + q.y) + (q.z + q.w);
-            }
-          }
-          acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-          acc += __shfl_xor_sync(0xffffffffu, acc, 2);
-          if (part == 0) rs[i] = rsqrtf(acc * nm.inv_d + nm.eps);
-        }
-      }
-      if (NORM && epi == EPI_RESID && N % 4 == 0) {
-        // old values of the rows this thread finishes (part 2 of the epilogue), while the main loop runs
-        const int f = f0 + (threadIdx.x & 31) * 4;
-#pragma unroll
-        for (int i = 0; i < SK_OLD; ++i) {
-          const int tl = rank + S * ((threadIdx.x >> 5) + 4 * i);
-          if (tl < BN && t0 + tl < M && f + 3 < N) x_old[i] = __ldcg(reinterpret_cast<const float4 *>((const float *)C + (size_t)(t0 + tl) * N + f));
-        }
-      }
-      if (NORM) asm volatile("bar.sync 1, 128;" ::: "memory");
-    }
   }
   if (warp == 4 && lane == 0) {
   } else if (warp == 5 && lane == 0) {
@@ -262,7 +196,7 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant__
     if (ok) umma_commit(accum);
   }
   // ---------------- epilogue, part 1: drain the accumulator(s), one weight tile at a time
-  const bool staged = NORM || S > 1 || tma_c;          // through shared memory ([token][128 features] fp32)
+  const bool staged = S > 1;          // through shared memory ([token][128 features] fp32)
   bool acc_ok = false;
   if (warp < 4) {
     acc_ok = KB > 0 && mbar_wait(accum, 0);
@@ -293,56 +227,13 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant__
         }
       }
     }
-    if (tma_c && S == 1 && warp < 4) {
-      // the staged tile goes to x as one TMA reduction (rows past M are clipped by the map)
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      asm volatile("bar.sync 2, 128;" ::: "memory");
-      if (threadIdx.x == 0 && acc_ok) {
-        if (tma_c == SK_TMA_ADD) sk_tma_reduce_add(&mapC, tiles, f0 + q * TC_BM, t0);
-        else sk_tma_store(&mapC, tiles, f0 + q * TC_BM, t0);
-      }
-      asm volatile("bar.sync 2, 128;" ::: "memory");       // the stage is free again
-    }
   }
   __syncwarp();
-  if (S > 1 || NORM) {
+  if (S > 1) {
     // ---------------- epilogue, part 2: reduce the S partial tiles through distributed shared memory
-    // (folded norms take this form also where K is not split)
     tc_fence_before();
-    if (S > 1) cluster_sync_all();
-    else if (warp < 4) asm volatile("bar.sync 2, 128;" ::: "memory");
-    if (warp < 4 && (tma_c == SK_TMA_ADD || tma_c == SK_TMA_F32)) {
-      // CTA r sums its block of BN / S rows over the S partial tiles, in place in its own tile,
-      // and hands the block to the TMA unit
-      const int RB = BN / S, rg = threadIdx.x >> 5, c4 = (threadIdx.x & 31) * 4;
-      uint32_t remote[SK_MAX_SPLIT];
-#pragma unroll
-      for (int r = 0; r < SK_MAX_SPLIT; ++r) {
-        const uint32_t a = tiles + (uint32_t)c4 * 4;
-        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote[r]) : "r"(a), "r"((uint32_t)(r < S ? r : 0)));
-      }
-      for (int tl = rank * RB + rg; tl < (rank + 1) * RB; tl += 4) {
-        if (t0 + tl >= M) break;
-        float4 v[SK_MAX_SPLIT];
-#pragma unroll
-        for (int r = 0; r < SK_MAX_SPLIT; ++r)
-          if (r < S)
-            asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
-                         : "=f"(v[r].x), "=f"(v[r].y), "=f"(v[r].z), "=f"(v[r].w)
-                         : "r"(remote[r] + (uint32_t)tl * (TC_BM * 4)) : "memory");
-        float4 sum = v[0];
-#pragma unroll
-        for (int r = 1; r < SK_MAX_SPLIT; ++r)
-          if (r < S) { sum.x += v[r].x; sum.y += v[r].y; sum.z += v[r].z; sum.w += v[r].w; }
-        *reinterpret_cast<float4 *>(stage_f + (size_t)tl * TC_BM + c4) = sum;
-      }
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      asm volatile("bar.sync 2, 128;" ::: "memory");
-      if (threadIdx.x == 0 && t0 + rank * RB < M) {
-        if (tma_c == SK_TMA_ADD) sk_tma_reduce_add(&mapC, tiles + (uint32_t)(rank * RB) * (TC_BM * 4), f0, t0 + rank * RB);
-        else sk_tma_store(&mapC, tiles + (uint32_t)(rank * RB) * (TC_BM * 4), f0, t0 + rank * RB);
-      }
-    } else if (warp < 4) {
+    cluster_sync_all();
+    if (warp < 4) {
       // thread -> (row group, 4 consecutive features): one 16-byte load per partial tile, all S
       // loads of a row in flight together, one 16-byte (fp32) or 8-byte (bf16) store per row
       const int rg = threadIdx.x >> 5, c4 = (threadIdx.x & 31) * 4, f = f0 + c4;
@@ -353,9 +244,8 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant__
         asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote[r]) : "r"(a), "r"((uint32_t)(r < S ? r : 0)));
       }
       const bool vec = (N % 4 == 0) && (f + 3 < N);
-      int it = 0;
 #pragma unroll 1
-      for (int tl = rank + S * rg; tl < BN; tl += 4 * S, ++it) {
+      for (int tl = rank + S * rg; tl < BN; tl += 4 * S) {
         const int t = t0 + tl;
         if (t >= M) break;
         float4 v[SK_MAX_SPLIT];
@@ -370,37 +260,13 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant__
         for (int r = 1; r < SK_MAX_SPLIT; ++r)
           if (r < S) { sum.x += v[r].x; sum.y += v[r].y; sum.z += v[r].z; sum.w += v[r].w; }
         const size_t o = (size_t)t * N + f;
-        if (NORM && nm.ssq_in) { const float k = rs[tl]; sum.x *= k; sum.y *= k; sum.z *= k; sum.w *= k; }
         if (vec) {
           if (epi == EPI_F32) {
             *reinterpret_cast<float4 *>((float *)C + o) = sum;
           } else if (epi == EPI_RESID) {
-            float4 old;
-            if (NORM && it < SK_OLD) {
-#pragma unroll
-              for (int i = 0; i < SK_OLD; ++i)
-                if (i == it) old = x_old[NORM ? i : 0];        // (registers: selected, not indexed)
-            } else {
-              old = *reinterpret_cast<float4 *>((float *)C + o);
-            }
+            float4 old = *reinterpret_cast<float4 *>((float *)C + o);
             old.x += sum.x; old.y += sum.y; old.z += sum.z; old.w += sum.w;
             *reinterpret_cast<float4 *>((float *)C + o) = old;
-            if (NORM && nm.a_out) {
-              const float4 gg = g_vec;
-              const __nv_bfloat162 lo = __floats2bfloat162_rn(gg.x * old.x, gg.y * old.y), hi = __floats2bfloat162_rn(gg.z * old.z, gg.w * old.w);
-              uint2 pk;
-              pk.x = *reinterpret_cast<const uint32_t *>(&lo);
-              pk.y = *reinterpret_cast<const uint32_t *>(&hi);
-              *reinterpret_cast<uint2 *>(nm.a_out + o) = pk;
-              // 4 lanes = one 16-feature slice.  N is a multiple of 32 here, so a slice is inside N
-              // or outside it as a whole: only its own 4 lanes are named in the shuffles (the lanes
-              // of a feature tile's slices beyond N never get here).
-              const unsigned grp = 0xfu << (threadIdx.x & 28);
-              float sq = old.x * old.x + old.y * old.y + old.z * old.z + old.w * old.w;
-              sq += __shfl_xor_sync(grp, sq, 1);
-              sq += __shfl_xor_sync(grp, sq, 2);
-              if ((threadIdx.x & 3) == 0) nm.ssq_out[(size_t)t * (N >> 4) + (f >> 4)] = sq;
-            }
           } else {
             if (epi == EPI_GELU_T) { sum.x = gelu_erf_fast(sum.x); sum.y = gelu_erf_fast(sum.y); sum.z = gelu_erf_fast(sum.z); sum.w = gelu_erf_fast(sum.w); }
             const __nv_bfloat162 lo = __floats2bfloat162_rn(sum.x, sum.y), hi = __floats2bfloat162_rn(sum.z, sum.w);
@@ -417,7 +283,7 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant__
         }
       }
     }
-    if (S > 1) cluster_sync_all();          // no CTA leaves while a peer may still read its tile
+    cluster_sync_all();          // no CTA leaves while a peer may still read its tile
   }
   tc_fence_before();
   __syncthreads();
@@ -441,6 +307,8 @@ struct GemmSkPlan {
   // (buffer, M, rows per box, element type)
   struct CMap { const void *C; int M, rows; bool is_bf16; CUtensorMap map; };
   std::vector<CMap> mapC;
+  struct PushTile { int M, BN, S, SW, SA; };
+  std::vector<PushTile> push;      // gemm_push_kernel's tile for the token counts seen
 };
 
 // fp32 [rows][N] row-major, box = box_rows x 128 features, no swizzle.
@@ -463,9 +331,8 @@ static int gemm_sk_init() {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= TC_MAX_DEVICES) return -4;
   if (dev_done[dev]) return 0;
-  if (cudaFuncSetAttribute(gemm_sk_kernel<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess ||
-      cudaFuncSetAttribute(gemm_sk_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess ||
-      cudaFuncSetAttribute(gemm_sk_kernel<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess)
+  if (cudaFuncSetAttribute(gemm_sk_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess ||
+      cudaFuncSetAttribute(gemm_sk_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess)
     return -4;
   dev_done[dev] = true;
   return 0;
@@ -477,6 +344,7 @@ static int gemm_sk_plan(GemmSkPlan *plan, const void *W, int N, int K, const voi
   for (bool &b : plan->haveA) b = false;
   for (bool &b : plan->haveA2) b = false;
   plan->mapC.clear();
+  plan->push.clear();
   if (K % 8 || K < 16 || N < 1 || M_max < 1) return 0;
   if (((uintptr_t)W & 15) || ((uintptr_t)A & 15)) return 0;
   if (!g_encode) return -4;
@@ -485,19 +353,12 @@ static int gemm_sk_plan(GemmSkPlan *plan, const void *W, int N, int K, const voi
   return 0;
 }
 
-// Tile and split choice for M tokens.
-// Up to 512 tokens: 32-token tiles and as many K splits (a power of two, at most 8, at most the number of K blocks) as
-// it takes to put the grid on most of the 148 SMs.
-// From 513 tokens on only widths N % 128 == 64 get here (whole 128-feature tiles go to gemm_pair_kernel).  The rules for
-// them were measured, with the figures below, on widths that gemm_pair_kernel takes today, and on block steps that
-// still divided by the stage count; they were not fitted again.
+// Tile and split choice for M > 512 tokens.  The rules were measured, with the figures below, on widths that
+// gemm_pair_kernel takes today, and on block steps that still divided by the stage count; they were not fitted again.
 // epi: the epilogue (EPI_*); *STG: ring depth, 0 = the default for the tile.
 static void gemm_sk_geometry(int N, int K, int M, int epi, int *BN, int *S, int *WT, int *STG) {
   *WT = 1;
   *STG = 0;
-  // Measured on B200 (graph replay, dependent launches): up to a few hundred tokens a 32-token
-  // tile with K split until the grid has ~150-250 CTAs is fastest (the partial-tile exchange
-  // grows with the tile, the latency chain does not shrink); large M takes 128/256-token tiles.
   const int FT = (N + TC_BM - 1) / TC_BM, KB = (K + TC_BK - 1) / TC_BK;
   if (M >= 4096) {
     // Very large M (prefill, wide verification), no split.  Measured on B200 (graph replay):
@@ -530,7 +391,7 @@ static void gemm_sk_geometry(int N, int K, int M, int epi, int *BN, int *S, int 
     }
     return;
   }
-  if (M > 512 && KB < 32) {
+  if (KB < 32) {
     // A few hundred to a few thousand tokens with a short K loop: no split (its exchange costs more
     // than the loop).  The time of these shapes is set by wave quantisation -- two CTAs fit on an SM,
     // 296 on the device, and a grid of 297 takes twice as long as one of 296 -- so the token tile is
@@ -556,25 +417,16 @@ static void gemm_sk_geometry(int N, int K, int M, int epi, int *BN, int *S, int 
     *S = 1;
     return;
   }
-  if (M > 512) {
-    // The same token counts with a long K loop: K split 2 or 4 ways; of the measured combinations
-    // the one with the most CTAs within one wave.
-    const int cand[5][2] = {{96, 2}, {128, 2}, {96, 4}, {128, 4}, {160, 4}};
-    int bb = 128, bs = 2, best_ctas = 0;
-    for (const auto &c : cand) {
-      const int ctas = FT * ((M + c[0] - 1) / c[0]) * c[1];
-      if (ctas <= 296 && ctas > best_ctas) { bb = c[0]; bs = c[1]; best_ctas = ctas; }
-    }
-    *BN = bb;
-    *S = bs;
-    return;
+  // The same token counts with a long K loop: K split 2 or 4 ways; of the measured combinations
+  // the one with the most CTAs within one wave.
+  const int cand[5][2] = {{96, 2}, {128, 2}, {96, 4}, {128, 4}, {160, 4}};
+  int bb = 128, bs = 2, best_ctas = 0;
+  for (const auto &c : cand) {
+    const int ctas = FT * ((M + c[0] - 1) / c[0]) * c[1];
+    if (ctas <= 296 && ctas > best_ctas) { bb = c[0]; bs = c[1]; best_ctas = ctas; }
   }
-  int bn = M <= 16 ? 16 : M <= 512 ? 32 : 128;
-  const int tiles = FT * ((M + bn - 1) / bn);
-  int s = 1;
-  while (s * 2 <= SK_MAX_SPLIT && s * 2 <= KB && tiles * s * 2 <= 256) s *= 2;
-  *BN = bn;
-  *S = s;
+  *BN = bb;
+  *S = bs;
 }
 
 // The map of an output written by the TMA unit (box of `rows` tokens x 128 features), encoded on first use;
@@ -589,7 +441,7 @@ static const CUtensorMap *sk_map_c(GemmSkPlan &p, void *C, int M, int rows, bool
 }
 
 static bool gemm_sk_launch(cudaStream_t st, bool pdl, GemmSkPlan &p, void *C, int M, int epi, int *status,
-                           const SkNorm *norm = nullptr, LiveRows lr = LiveRows{nullptr, 0}) {
+                           LiveRows lr = LiveRows{nullptr, 0}) {
   if (!p.valid || M < 1 || M > p.M_max) return false;
   int BN, S, wt, stg;
   gemm_sk_geometry(p.N, p.K, M, epi, &BN, &S, &wt, &stg);
@@ -600,22 +452,9 @@ static bool gemm_sk_launch(cudaStream_t st, bool pdl, GemmSkPlan &p, void *C, in
   }
   const int KB = (p.K + TC_BK - 1) / TC_BK;
   const int FT = (p.N + TC_BM - 1) / TC_BM, TT = (M + BN - 1) / BN;
-  // residual epilogue through the TMA unit: x and its row pitch 16-byte aligned, whole feature tiles
-  int tma_c = SK_TMA_NONE;
-  if (!norm && p.N % TC_BM == 0 && BN % S == 0 && !((uintptr_t)C & 15)) {
-    if (epi == EPI_RESID) tma_c = SK_TMA_ADD;
-    else if (epi == EPI_F32) tma_c = SK_TMA_F32;
-  }
-  const CUtensorMap *mapC = &p.mapW;                         // placeholder when unused
-  if (tma_c) {
-    mapC = sk_map_c(p, C, M, BN / S, false);
-    if (!mapC) return false;
-  }
-  const SkShape sh = sk_shape(BN, (KB + S - 1) / S, S > 1 || tma_c || norm, wt, stg);
+  const SkShape sh = sk_shape(BN, (KB + S - 1) / S, S > 1, wt, stg);
   if (sh.smem_bytes > 227 * 1024) return false;
-  const int ring_bytes = sh.smem_bytes - 1024 - 256 - 1024;
-  const SkNorm nm = norm ? *norm : SkNorm{};
-  const int tc = tma_c;
+  const int ring_bytes = sh.smem_bytes - 1024 - 256;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((FT + wt - 1) / wt, TT, S);
   cfg.blockDim = dim3(192);
@@ -630,11 +469,9 @@ static bool gemm_sk_launch(cudaStream_t st, bool pdl, GemmSkPlan &p, void *C, in
   cfg.numAttrs = pdl ? 2 : 1;
   int N = p.N, K = p.K, stages = sh.stages, cols = sh.tmem_cols, rb = ring_bytes;
   auto go = [&](auto kernel) {
-    return cudaLaunchKernelEx(&cfg, kernel, p.mapW, p.mapA[idx], *mapC, C, M, N, K, BN, stages, cols, rb, epi, tc, nm, status,
-                              lr) == cudaSuccess;
+    return cudaLaunchKernelEx(&cfg, kernel, p.mapW, p.mapA[idx], C, M, N, K, BN, stages, cols, rb, epi, status, lr) == cudaSuccess;
   };
-  if (wt == 2) return go(gemm_sk_kernel<2, false>);
-  return norm ? go(gemm_sk_kernel<1, true>) : go(gemm_sk_kernel<1, false>);
+  return wt == 2 ? go(gemm_sk_kernel<2>) : go(gemm_sk_kernel<1>);
 }
 
 }  // namespace tsfm

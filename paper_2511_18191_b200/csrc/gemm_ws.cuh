@@ -179,24 +179,31 @@ gemm_ws_kernel(const bf16 *A, const bf16 *__restrict__ W, void *C, int M, int N,
 // ------------------------------------------------------------------ host side
 static inline int ws_blocks(int K) { return (K / 64 + WS_WARPS - 1) / WS_WARPS; }
 
-// Whether this kernel is the better tool for the shape: K in the registers of eight warps, N even, the operands
-// 16-byte aligned, and the whole grid resident at once -- three CTAs per SM by registers where a warp has one block
-// of K, two with two, else one.  On either side of that line (us, gemm_sk_kernel / this): M = 319, N = 512, K = 512
-// (320 CTAs) 5.1 / 3.5, M = 512, N = 256, K = 1024 (256 CTAs) 6.2 / 3.7, M = 93, N = 1024, K = 1024 (192) 5.3 / 3.7;
-// M = 160, N = 2048, K = 512 (640) 6.0 / 6.2, M = 256, N = 1024, K = 1024 (512) 6.7 / 6.9, M = 64, N = 1280, K = 1280
-// (160) 5.6 / 5.9.
-static bool gemm_ws_eligible(const void *A, const void *W, int M, int N, int K) {
+// Whether the kernel can serve a shape well: K in the registers of eight warps, N even, the operands 16-byte aligned, and the
+// whole grid resident at once -- three CTAs per SM by registers where a warp has one block of K, two with two, else one.
+static bool gemm_ws_fits(const void *A, const void *W, int M, int N, int K) {
   if (M < 1 || M > 512 || K < 64 || K % 64 || K > WS_MAX_K || N % 2) return false;
   if (((uintptr_t)A & 15) || ((uintptr_t)W & 15)) return false;
   const int nb = ws_blocks(K), per_sm = nb == 1 ? 3 : nb == 2 ? 2 : 1;
   const long ctas = (long)((N + WS_FN - 1) / WS_FN) * ((M + WS_MT - 1) / WS_MT);
   return ctas <= (long)per_sm * 148;
 }
+// Whether it is the better one there.  Contractions that do not widen (Wo, W2): everywhere (us, this / gemm_push_kernel:
+// M = 512, N = K = 512 3.6 / 4.6, M = 128, N = K = 1024 3.7 / 4.1, M = 128, N = 512, K = 2048 4.2 / 4.5).  Those that widen (QKV,
+// W1) scale their rows by factors that every CTA has to sum up: up to 256 CTAs (N = 2048, K = 512: M = 64 3.67 / 3.71, M = 93
+// 3.92 / 3.67), and with K > 512 only while the weights come from L2 in time (N = 2304, K = 768: M = 32 3.9 / 4.0; N = 3072, K =
+// 1024: M = 8 3.1 / 3.5, M = 16 3.58 / 3.53, M = 24 4.3 / 3.7).
+static bool gemm_ws_eligible(const void *A, const void *W, int M, int N, int K) {
+  if (!gemm_ws_fits(A, W, M, N, K)) return false;
+  if (N <= K) return true;
+  const long ctas = (long)((N + WS_FN - 1) / WS_FN) * ((M + WS_MT - 1) / WS_MT);
+  return ws_blocks(K) == 1 ? ctas <= 256 : (long)N * K <= 2500000 || M <= 8;
+}
 
 // Shapes that the single-contraction entry point gives to this kernel on request: those that a decoder gives it, and
 // up to 256 tokens on up to eight CTAs per SM where K is short (shapes it has always taken; they run in several waves).
 static bool gemm_ws_accepts(const void *A, const void *W, int M, int N, int K) {
-  if (gemm_ws_eligible(A, W, M, N, K)) return true;
+  if (gemm_ws_fits(A, W, M, N, K)) return true;
   if (M < 1 || M > 256 || K < 64 || K % 64 || K > WS_MAX_K || N % 2) return false;
   if (((uintptr_t)A & 15) || ((uintptr_t)W & 15)) return false;
   const int per_sm = std::min(8, 228 * 1024 / ((WS_FN + WS_MT) * K * 2 + 17536));

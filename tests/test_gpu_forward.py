@@ -234,3 +234,22 @@ def test_small_batch_gemm_matches_fp64_product(M, N, K):
     want = (A.double() @ W.double().T).numpy()
     assert np.isfinite(got).all()
     assert np.abs(got - want).max() < 2e-5 * K ** 0.5 + 1e-5
+
+
+@pytest.mark.parametrize("M,N,K", [(1, 1280, 5120), (3, 130, 4096), (17, 1280, 5120), (64, 3840, 1280), (93, 1024, 4096), (129, 64, 2560),
+                                   (500, 192, 80), (512, 5120, 1280), (511, 1280, 5120)])
+def test_few_token_gemm_matches_fp64_product(M, N, K):
+    """The kernel of up to 512 tokens: K in one piece and split over clusters of every size the tile rule asks for, rings that
+    hold K and rings that turn over, half a feature tile, ragged token tiles, K that is no whole block."""
+    test_many_token_gemm_matches_fp64_product(M, N, K)
+
+
+@pytest.mark.parametrize("n", [2, 4, 26, 102])
+def test_bf16_forward_of_wide_models_on_few_tokens(n):
+    """Folded norms of up to 512 rows (5 n) in the epilogues of that kernel: widths whose contractions no other kernel takes
+    (K = 1088 and 4352; 2560 with half a feature tile over)."""
+    wl = small_workload("bf16", Arch(2, 1088, 17, 4352), Arch(2, 320, 5, 2560), 32)
+    gt, wt, gd, wd = run_forward_case(wl, 0, n)
+    assert np.isfinite(gt).all() and np.isfinite(gd).all()
+    assert parity.value_error("rel_rms", gt, wt) < 2e-2       # bf16 operands, as above
+    assert parity.value_error("rel_rms", gd, wd) < 2e-2

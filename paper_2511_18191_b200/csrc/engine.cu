@@ -27,6 +27,7 @@
 #include "gemm_ws.cuh"
 #include "gemm_pair.cuh"
 #include "gemm_push.cuh"
+#include "attn_mma.cuh"
 #include "gemm_f32.cuh"
 
 using namespace tsfm;
@@ -111,6 +112,8 @@ struct ModelDev {
   std::vector<LayerDev> layers;
   void *Kc = nullptr, *Vc = nullptr;     // [L][B][heads][cap][dh]
   size_t kv_layer_elems = 0;
+  bool attn_mma = false;                 // attn_mma_kernel takes the long passes: its maps of the whole caches
+  CUtensorMap mapK{}, mapV{};
   float2 *rope = nullptr;                // [cap][dh/2] (cos, sin)
 };
 
@@ -391,6 +394,7 @@ void prefer_max_smem_all() {
   prefer_max_smem(round_end_kernel);
   prefer_max_smem(gemm_sk_kernel<1>);
   prefer_max_smem(gemm_sk_kernel<2>);
+  prefer_max_smem(attn_mma_kernel);
   prefer_max_smem(gemm_push_kernel<EPI_F32>);
   prefer_max_smem(gemm_push_kernel<EPI_GELU_T>);
   prefer_max_smem(gemm_push_kernel<EPI_RESID>);
@@ -576,6 +580,11 @@ void gemm(tsfm_spec *h, GemmSkPlan *plan, const void *A, const void *W, void *C,
   launch_gemm_simt<T>(h->ls, h->pdl, (const T *)A, (const T *)W, C, M, N, K, epi, lr);
 }
 
+// Passes of more tokens than this, with heads of 64, attend on the tensor-memory kernel (attn_mma_kernel; figures there).  Up
+// to 32 queries fill a quarter of its 128 rows: 3200 blocks of 30 queries x 30 keys run 18 us in attn_tiles_kernel, which also
+// keeps the other head sizes.
+constexpr int kMmaAttnTokens = 32;
+
 // appended: the QKV contraction has rotated the queries and put the pass's keys and values into the cache;
 // cache_only: nothing reads the attention's output (last layer of a prefill).
 template <typename T, int DH>
@@ -595,6 +604,12 @@ void launch_attn(tsfm_spec *h, ModelDev &m, int l, int B, const PassGeom &g, boo
   if (pre && cache_only) return;
   if constexpr (sizeof(T) == 2) {
     const int pairs = B * m.arch.n_heads;
+    if (DH == AM_DH && m.attn_mma && g.q_len > kMmaAttnTokens) {
+      launch_ex(h->ls, h->pdl, attn_mma_kernel, dim3(m.arch.n_heads, B, (g.q_len + AM_Q - 1) / AM_Q), dim3(AM_THREADS), (size_t)AM_SMEM,
+                m.mapK, m.mapV, h->qkv, m.rope, g, m.arch.n_heads, (int)(l * (m.kv_layer_elems / AM_DH)), appended ? 1 : 0,
+                (bf16 *)h->ao, h->dev_status);
+      return;
+    }
     if (pre) {
       const int warps = g.q_len <= 32 ? 2 : 4;
       const dim3 grid(m.arch.n_heads, B, (g.q_len + 16 * warps - 1) / (16 * warps));
@@ -1265,6 +1280,13 @@ int tsfm_spec_create(const tsfm_weights *target_w, const tsfm_weights *draft_w, 
     if ((rc = gemm_pair_init())) return fail(rc);
     if ((rc = gemm_push_init())) return fail(rc);
     for (ModelDev *m : {&h->tgt, &h->drf}) {
+      const size_t kv_rows = m->kv_layer_elems / m->dh * m->arch.n_layers;
+      if (m->dh == AM_DH && kv_rows < (1u << 30)) {           // (coordinates of a copy are 32-bit)
+        if (tc_encode(&m->mapK, m->Kc, (int)kv_rows, AM_DH, AM_KEYS) || tc_encode(&m->mapV, m->Vc, (int)kv_rows, AM_DH, AM_KEYS) ||
+            cudaFuncSetAttribute(attn_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, AM_SMEM) != cudaSuccess)
+          return fail(TSFM_ERR_CUDA);
+        m->attn_mma = true;
+      }
       const int d = m->arch.d_model, f = m->arch.d_ff;
       for (LayerDev &ly : m->layers) {
         if ((rc = gemm_sk_plan(&ly.tc_qkv, ly.Wqkv, 3 * d, d, h->a, h->M_max))) return fail(rc);

@@ -253,3 +253,24 @@ def test_bf16_forward_of_wide_models_on_few_tokens(n):
     assert np.isfinite(gt).all() and np.isfinite(gd).all()
     assert parity.value_error("rel_rms", gt, wt) < 2e-2       # bf16 operands, as above
     assert parity.value_error("rel_rms", gd, wd) < 2e-2
+
+
+@pytest.mark.parametrize("B,n", [(1, 33), (2, 128), (1, 200), (3, 257), (5, 129)])
+def test_bf16_attention_of_long_passes(B, n):
+    """Heads of 64, more than 32 tokens: one or several blocks of 128 queries, ragged last blocks and key tiles, queries rotated
+    in the kernel (up to 512 rows) or before it.  A NaN in a late token reaches the tokens behind it in its own series only, and
+    changes nothing else by a bit."""
+    import paper_2511_18191_b200 as tsfm
+    wl = small_workload("bf16", Arch(2, 128, 2, 256), Arch(1, 256, 4, 256), 32)
+    gt, wt, gd, wd = run_forward_case(wl, 0, n, B=B)
+    assert parity.value_error("rel_rms", gt, wt) < 2e-2 and parity.value_error("rel_rms", gd, wd) < 2e-2   # bf16 operands, as above
+    tw, dw = build_models(wl)
+    dec = tsfm.SpecDecoder(tw, dw, wl.target, wl.draft, wl.patch_len, wl.dtype, "separate", max_batch=B, max_ctx_tokens=n,
+                           max_horizon_patches=4, max_K=4)
+    z = torch.from_numpy(np.random.default_rng(0).standard_normal((B, n, wl.token_len)).astype(np.float32)).cuda()
+    z[B - 1, n - 7] = float("nan")
+    got = dec.model_forward(0, z).cpu().numpy()
+    dec.close()
+    want = gt.copy()
+    want[B - 1, n - 7:] = np.nan
+    np.testing.assert_array_equal(got, want)

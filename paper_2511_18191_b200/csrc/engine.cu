@@ -366,8 +366,9 @@ template <typename F> void prefer_max_smem(F *fn) {
 }
 template <typename T> void prefer_max_smem_typed() {
   prefer_max_smem(embed_kernel<T>);
-  prefer_max_smem(rmsnorm_kernel<T, false>);
-  prefer_max_smem(rmsnorm_kernel<T, true>);
+  prefer_max_smem(rmsnorm_kernel<T, false, 10>);
+  prefer_max_smem(rmsnorm_kernel<T, false, 16>);
+  prefer_max_smem(rmsnorm_kernel<T, true, 10>);
   prefer_max_smem(head_kernel<T>);
   prefer_max_smem(embed_rows_kernel<T>);
   prefer_max_smem(gemm_f32_kernel<T, 16, 16>);
@@ -711,7 +712,7 @@ void run_pass(tsfm_spec *h, ModelDev &m, int B, const PassGeom &g, int head_mode
     }
   };
   // the RMSNorm of passes of a few thousand rows is a link in a chain: constants before the wait
-  auto *norm_kernel = M <= kNormEarlyMaxRows && d <= 1280 ? rmsnorm_kernel<T, true> : rmsnorm_kernel<T, false>;
+  auto *norm_kernel = d > 1280 ? rmsnorm_kernel<T, false, 16> : M <= kNormEarlyMaxRows ? rmsnorm_kernel<T, true, 10> : rmsnorm_kernel<T, false, 10>;
   {
     KTimer kt(h, KC_EMBED, (double)M * Pi * 4 + (double)d * Pi * sizeof(T) + (double)M * d * 4, 2.0 * M * Pi * d);
     if (!fold && f32_tiles(h, m.W_emb, Pi)) {

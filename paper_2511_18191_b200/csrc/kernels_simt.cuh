@@ -301,11 +301,13 @@ __device__ __forceinline__ void store4(bf16 *o, float a, float b, float c, float
 // takes two L2 round trips out of the chain at the price of registers (rows of at most 1280
 // features, so that two CTAs still fit on an SM).  The count was written by the kernel that closed
 // the previous round, at least two kernels back.
-template <typename T, bool EARLY>
-__global__ void __launch_bounds__(256, 2)
+// CACHE: float4 per lane kept in registers (rows of up to 128 CACHE features are read once).  Rows of up to 1280 features
+// leave room for three CTAs per SM: a stream of many rows is bound by the bytes in flight (two
+// CTAs -> three, us a link: 16320 x 1280 29.5 -> 26.8, 7424 x 1024 10.2 -> 8.5, 5120 x 768 5.0 -> 4.7).
+template <typename T, bool EARLY, int CACHE>
+__global__ void __launch_bounds__(256, !EARLY && CACHE <= 10 ? 3 : 2)
 rmsnorm_kernel(const float *x, const float *__restrict__ gain, int M, int d, float eps,
                T *__restrict__ a, LiveRows lr) {
-  constexpr int CACHE = EARLY ? 10 : 16;                      // float4 per lane kept in registers
   const int lane = threadIdx.x & 31;
   const size_t row = (size_t)blockIdx.x * 8 + (threadIdx.x >> 5);
   const float4 *gr = reinterpret_cast<const float4 *>(gain);

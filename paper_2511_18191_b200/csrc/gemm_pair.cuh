@@ -64,17 +64,17 @@ __device__ __forceinline__ void umma_bf16_pair(uint32_t tmem_d, uint64_t da, uin
       "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
       ::"r"(tmem_d), "l"(da), "l"(db), "r"(idesc), "r"(acc) : "memory");
 }
-// Arrives at the barrier of this offset in both ranks once the MMAs issued so far are done.
-__device__ __forceinline__ void umma_commit_pair(uint32_t bar) {
+// Arrives at the barrier of this offset in both ranks of a pair (mask) once the MMAs issued so far are done.
+__device__ __forceinline__ void umma_commit_pair(uint32_t bar, uint32_t mask) {
   asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-               ::"r"(bar), "h"((uint16_t)3) : "memory");
+               ::"r"(bar), "h"((uint16_t)mask) : "memory");
 }
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
-__device__ __forceinline__ void mbar_arrive_rank0(uint32_t bar) {
+__device__ __forceinline__ void mbar_arrive_rank(uint32_t bar, uint32_t rank) {
   uint32_t remote;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(bar), "r"(0u));
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(bar), "r"(rank));
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(remote) : "memory");
 }
 __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
@@ -160,27 +160,31 @@ __device__ __forceinline__ void pair_rope_rows(const float *stage, const int2 *p
 // SK_TMA_BF16 (stores; epi tells GELU) or SK_TMA_ADD; SK_TMA_NONE: fp32, straight from registers.
 __global__ void __launch_bounds__(PAIR_THREADS, 1)
 gemm_pair_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant__ CUtensorMap mapA,
-                 const __grid_constant__ CUtensorMap mapC, int M, int N, int K, int BN, int stages, int n_acc,
+                 const __grid_constant__ CUtensorMap mapC, int M, int N, int K, int BN, int split, int stages, int n_acc,
                  int tmem_cols, int epi, int tma_c, float *C, const SkNorm nm, const PairRope pr, int *__restrict__ status,
                  const LiveRows lr) {
   // rows in use (active-series compaction): read before the dependency wait, see gemm_sk_kernel
   if (lr.n_live) M = min(M, *reinterpret_cast<const volatile int *>(lr.n_live) * lr.q_len);
   const int FT = (N + 2 * TC_BM - 1) / (2 * TC_BM), n_tiles = FT * ((M + BN - 1) / BN);
-  const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
-  const uint32_t rank = blockIdx.x & 1;                        // == %cluster_ctarank
-  if (pair >= n_tiles) return;                                 // both ranks alike
+  // rank within the pair; which half of K the pair takes (split == 2: two pairs, a cluster of four, on one tile)
+  const uint32_t rank = blockIdx.x & 1, half = split == 2 ? (blockIdx.x >> 1) & 1 : 0;
+  const int pair = blockIdx.x / (2 * split), n_pairs = gridDim.x / (2 * split);
+  if (pair >= n_tiles) return;                                 // the whole cluster alike
   extern __shared__ uint8_t smem_raw[];
   const uint32_t tiles = (smem_u32(smem_raw) + 1023u) & ~1023u;
   const int a_bytes = (BN / 2) * TC_BK * 2, stage_bytes = TC_W_BYTES + a_bytes;
   const uint32_t out0 = tiles + (uint32_t)(stages * stage_bytes);
   const uint32_t bars = out0 + PAIR_GROUPS * PAIR_STAGE_OUT;
   const uint32_t full0 = bars, empty0 = bars + 64, acc_full0 = bars + 128, acc_empty0 = bars + 144, slot = bars + 160;
-  const uint32_t rows_full0 = bars + 176, rows_empty0 = bars + 192;
+  const uint32_t rows_full0 = bars + 176, rows_empty0 = bars + 192, recv_bar = bars + 208;
+  const uint32_t recv0 = bars + 256 + PAIR_ROW_BYTES;          // (split) the other pair's sums of the rows finished here: [quad][feature] x 4 rows
   float *row_scale = reinterpret_cast<float *>(smem_raw + (bars + 256 - smem_u32(smem_raw)));   // [2 tiles][256]
   int2 *row_pos = reinterpret_cast<int2 *>(row_scale + 512);                                    // [2 tiles][256] (series, position)
   uint32_t *slot_ptr = reinterpret_cast<uint32_t *>(smem_raw + (slot - smem_u32(smem_raw)));
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
-  const int KB = (K + TC_BK - 1) / TC_BK;
+  const int KB_all = (K + TC_BK - 1) / TC_BK, kb0 = KB_all * (int)half / split, KB = KB_all * ((int)half + 1) / split - kb0;
+  // rows of the tile that this pair finishes
+  const int r_beg = (int)half * (BN / split), r_end = r_beg + BN / split;
 
   if (warp == PAIR_EPI_WARPS && lane == 0) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(&mapW) : "memory");
@@ -197,6 +201,11 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant
       mbar_init(acc_empty0 + 8 * lane, 2 * PAIR_EPI_WARPS);    // of both ranks
       mbar_init(rows_full0 + 8 * lane, PAIR_ROW_WARPS);
       mbar_init(rows_empty0 + 8 * lane, PAIR_EPI_WARPS);
+    }
+    if (lane == 0 && split == 2) {
+      mbar_init(recv_bar, 1);
+      const int rows = min(M - (pair / FT) * BN, r_end) - r_beg;             // in whole chunks
+      mbar_expect_tx(recv_bar, rows > 0 ? (uint32_t)((rows + PAIR_CHUNK - 1) / PAIR_CHUNK * PAIR_STAGE_OUT) : 0u);
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     __syncwarp();
@@ -236,20 +245,20 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant
       uint32_t dst = tiles, bar = full0;
       for (int it = 0; it < pre; ++it, dst += stage_bytes, bar += 8, next(pw)) {
         if (rank == 0) mbar_expect_tx(bar, 2u * (uint32_t)stage_bytes);
-        tma_load_2d_pair(dst, &mapW, pw.kb * TC_BK, pw.wy, bar);
+        tma_load_2d_pair(dst, &mapW, (kb0 + pw.kb) * TC_BK, pw.wy, bar);
       }
       pdl_sync();
       dst = tiles, bar = full0;
       for (int it = 0; it < pre; ++it, dst += stage_bytes, bar += 8, next(pa))
-        tma_load_2d_pair(dst + TC_W_BYTES, &mapA, pa.kb * TC_BK, pa.ay, bar);
+        tma_load_2d_pair(dst + TC_W_BYTES, &mapA, (kb0 + pa.kb) * TC_BK, pa.ay, bar);
       int s = 0;
       uint32_t ph = 0;
       dst = tiles;
       for (int it = pre; it < total; ++it, next(pa)) {
         if (!mbar_wait_cluster(empty0 + 8 * s, ph)) { atomicExch(status, DEV_TIMEOUT_TMA); break; }
         if (rank == 0) mbar_expect_tx(full0 + 8 * s, 2u * (uint32_t)stage_bytes);
-        tma_load_2d_pair(dst, &mapW, pa.kb * TC_BK, pa.wy, full0 + 8 * s);
-        tma_load_2d_pair(dst + TC_W_BYTES, &mapA, pa.kb * TC_BK, pa.ay, full0 + 8 * s);
+        tma_load_2d_pair(dst, &mapW, (kb0 + pa.kb) * TC_BK, pa.wy, full0 + 8 * s);
+        tma_load_2d_pair(dst + TC_W_BYTES, &mapA, (kb0 + pa.kb) * TC_BK, pa.ay, full0 + 8 * s);
         dst += stage_bytes;
         if (++s == stages) { s = 0; ph ^= 1u; dst = tiles; }
       }
@@ -276,12 +285,12 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant
 #pragma unroll
             for (int k = 0; k < TC_BK / 16; ++k)
               umma_bf16_pair(tmem + (uint32_t)(buf * BN), dw + 2 * k, da + 2 * k, idesc, (kb | k) ? 1u : 0u);
-            umma_commit_pair(empty0 + 8 * s);
+            umma_commit_pair(empty0 + 8 * s, 3u << (2 * half));
           }
           dw += (uint32_t)(stage_bytes >> 4);
           if (++s == stages) { s = 0; ph ^= 1u; dw = dw0; }
         }
-        if (ok && leader) umma_commit_pair(acc_full0 + 8 * buf);
+        if (ok && leader) umma_commit_pair(acc_full0 + 8 * buf, 3u << (2 * half));
       }
       __syncwarp();
     }
@@ -342,11 +351,11 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant
       auto fetch_old = [&](int c) {
 #pragma unroll
         for (int j = 0; j < PAIR_CHUNK; ++j)
-          old[j] = (c < BN && t0 + c + j < M && f0 < N) ? __ldcg(C + (size_t)(t0 + c + j) * N + f0 + fl) : 0.f;
+          old[j] = (c < r_end && t0 + c + j < M && f0 < N) ? __ldcg(C + (size_t)(t0 + c + j) * N + f0 + fl) : 0.f;
       };
       if (produce) {
         if (f0 < N) gain = *reinterpret_cast<const float4 *>(nm.gain + fc);
-        fetch_old(grp * PAIR_CHUNK);
+        fetch_old(r_beg + grp * PAIR_CHUNK);
       }
       // (after a wait that ran out: no more waits, nothing stored)
       if (ok && (nm.ssq_in || pr.rope)) ok = mbar_wait(rows_full0 + 8 * (i & 1), (uint32_t)(i >> 1) & 1u);
@@ -375,11 +384,38 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant
             if (j < lim) dst[(size_t)j * N] = v[j];
         }
       }
-      for (int c = grp * PAIR_CHUNK; c < BN && !direct; c += PAIR_GROUPS * PAIR_CHUNK) {
+      if (split == 2) {
+        // the sums of the rows that the other pair finishes go to the CTA with the same features there (see gemm_push_kernel)
+        const int o_beg = BN / 2 - r_beg;                      // (0 or BN / 2)
+        uint32_t there, bar_there;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(there) : "r"(recv0 + (uint32_t)fl * 16), "r"((blockIdx.x & 3) ^ 2));
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(bar_there) : "r"(recv_bar), "r"((blockIdx.x & 3) ^ 2));
+        for (int c = grp * PAIR_CHUNK; c < BN / 2 && t0 + o_beg + c < M && ok; c += PAIR_GROUPS * PAIR_CHUNK) {
+          float v[PAIR_CHUNK];
+          tmem_ld16(tbase + o_beg + c, v);
+#pragma unroll
+          for (int j = 0; j < PAIR_CHUNK; j += 4)
+            asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];"
+                         ::"r"(there + (uint32_t)((c + j) / 4 * TC_BM * 16)), "f"(v[j]), "f"(v[j + 1]), "f"(v[j + 2]), "f"(v[j + 3]), "r"(bar_there)
+                         : "memory");
+        }
+        if (ok) ok = mbar_wait_cluster(recv_bar, 0);
+        if (!ok) atomicExch(status, DEV_TIMEOUT_EPILOGUE);
+        ok = __all_sync(0xffffffffu, ok);
+      }
+      for (int c = r_beg + grp * PAIR_CHUNK; c < r_end && !direct; c += PAIR_GROUPS * PAIR_CHUNK) {
         if (t0 + c >= M) break;
         float v[PAIR_CHUNK];
 #pragma unroll
         for (int j = 0; j < PAIR_CHUNK; j += 16) tmem_ld16(tbase + c + j, v + j);
+        if (split == 2) {
+          const float4 *from = reinterpret_cast<const float4 *>(smem_raw + (recv0 - smem_u32(smem_raw))) + (c - r_beg) / 4 * TC_BM + fl;
+#pragma unroll
+          for (int j = 0; j < PAIR_CHUNK; j += 4) {
+            const float4 p = from[j / 4 * TC_BM];
+            v[j] += p.x; v[j + 1] += p.y; v[j + 2] += p.z; v[j + 3] += p.w;
+          }
+        }
         if (nm.ssq_in) {
 #pragma unroll
           for (int j = 0; j < PAIR_CHUNK; j += 4) {
@@ -449,7 +485,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant
       tc_fence_before();
       __syncwarp();
       if (lane == 0) {
-        mbar_arrive_rank0(acc_empty0 + 8 * buf);
+        mbar_arrive_rank(acc_empty0 + 8 * buf, 2 * half);
         if (nm.ssq_in || pr.rope) mbar_arrive(rows_empty0 + 8 * (i & 1));
       }
     }
@@ -466,7 +502,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant
 
 // ------------------------------------------------------------------ host side
 struct PairShape {
-  int BN, stages, n_acc, tmem_cols, pairs, smem_bytes;
+  int BN, stages, n_acc, tmem_cols, pairs, smem_bytes, split;
 };
 
 static int gemm_pair_init() {
@@ -486,7 +522,12 @@ static int gemm_pair_init() {
 // 1280 at 576 to 16320 tokens: 2.0 % above the best tile on average and 15 % at worst, with 10 for a pair 0.6 and 10 %.
 // In whole passes 10 is the worse: it gives Wo and W2 64-token tiles on 65 to 68 pairs instead of 96-token ones on 45;
 // scoring 800 tokens with d = 1280 333 -> 349 us, 1040 with d = 1024 300 -> 310, decoding 1024 series 2670 -> 2738.)
-static PairShape gemm_pair_geometry(int N, int K, int M) {
+// can_split (residual updates): where the tiles keep at most half of the pairs busy and K is long, two pairs share a tile, each
+// with half of K (32 tiles at most: 128 SMs in clusters of four); the exchange counts 2000 cycles.  Inside forecasts, us: 576 x
+// 1280 x 5120 (30 tiles) 18.5 -> 13.4, 1024 x 768 x 3072 (33 -> 24 tiles) 12.9 -> 10.6.  Not where more pairs are busy already
+// (1280 x 1024 x 4096, 56: 16.2 -> 15.4 and the next contraction starts later; 1280 x 768 x 3072, 66: 13.6 -> 15.4) and not
+// with a short K (576 x 1280 x 1280 10.0 -> 8.5, but the W1 behind it 12.9 -> 13.9; 1280 x 1024 x 1024 9.0 -> 10.1).
+static PairShape gemm_pair_geometry(int N, int K, int M, bool can_split = false) {
   const int FT = (N + 2 * TC_BM - 1) / (2 * TC_BM), KB = (K + TC_BK - 1) / TC_BK;
   PairShape sh{};
   long best = 0;
@@ -497,8 +538,20 @@ static PairShape gemm_pair_geometry(int N, int K, int M) {
     if (!best || cost < best) {
       best = cost;
       sh.BN = bn;
+      sh.pairs = tiles;
     }
   }
+  sh.split = 1;
+  if (can_split && KB >= 32 && sh.pairs <= PAIR_MAX / 2)
+    for (int bn = 32; bn <= 256; bn += 32) {
+      const int tiles = FT * ((M + bn - 1) / bn);
+      const long cost = (KB + 1) / 2 * (256 + (bn < 96 ? 96 : bn)) + 4 * bn + 40 * tiles + 2000;
+      if (tiles <= 32 && cost < best) {
+        best = cost;
+        sh.BN = bn;
+        sh.split = 2;
+      }
+    }
   return sh;
 }
 // Shapes and outputs it takes: whole 128-feature tiles leave through the TMA unit.
@@ -513,16 +566,17 @@ static void gemm_pair_fill(PairShape *sh, int N, int K, int M) {
   const int cols = sh->BN * sh->n_acc;
   sh->tmem_cols = cols <= 32 ? 32 : cols <= 64 ? 64 : cols <= 128 ? 128 : cols <= 256 ? 256 : 512;
   const int stage = TC_W_BYTES + sh->BN / 2 * TC_BK * 2;
-  const int st = (227 * 1024 - PAIR_GROUPS * PAIR_STAGE_OUT - PAIR_ROW_BYTES - 1280) / stage;
+  const int recv = sh->split == 2 ? sh->BN / 2 * TC_BM * 4 : 0;
+  const int st = (227 * 1024 - PAIR_GROUPS * PAIR_STAGE_OUT - PAIR_ROW_BYTES - 1280 - recv) / stage;
   if (sh->stages == 0) sh->stages = st > PAIR_MAX_STAGES ? PAIR_MAX_STAGES : st;
-  sh->smem_bytes = sh->stages * stage + PAIR_GROUPS * PAIR_STAGE_OUT + 1024 + 256 + PAIR_ROW_BYTES;
+  sh->smem_bytes = sh->stages * stage + PAIR_GROUPS * PAIR_STAGE_OUT + 1024 + 256 + PAIR_ROW_BYTES + recv;
 }
 
 static bool gemm_pair_launch(cudaStream_t st, bool pdl, GemmSkPlan &p, void *C, int M, int epi, int *status, LiveRows lr,
                              const SkNorm *norm = nullptr, const PairRope *rope = nullptr, PairShape sh = PairShape{}) {
   if (M < 1 || M > p.M_max) return false;
   if (!sh.BN) {
-    sh = gemm_pair_geometry(p.N, p.K, M);
+    sh = gemm_pair_geometry(p.N, p.K, M, epi == EPI_RESID);
     gemm_pair_fill(&sh, p.N, p.K, M);
   }
   const int idx = sh.BN / 32 - 1;
@@ -534,18 +588,18 @@ static bool gemm_pair_launch(cudaStream_t st, bool pdl, GemmSkPlan &p, void *C, 
   const CUtensorMap *mapC = tma_c == SK_TMA_NONE ? &p.mapW : sk_map_c(p, C, M, PAIR_CHUNK, tma_c == SK_TMA_BF16);
   if (!mapC) return false;
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(2 * sh.pairs);
+  cfg.gridDim = dim3(2 * sh.split * sh.pairs);
   cfg.blockDim = dim3(PAIR_THREADS);
   cfg.dynamicSmemBytes = sh.smem_bytes;
   cfg.stream = st;
   cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = 2; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  at[0].val.clusterDim.x = 2 * sh.split; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
   at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = pdl ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, gemm_pair_kernel, p.mapW, p.mapA2[idx], *mapC, M, p.N, p.K, sh.BN, sh.stages, sh.n_acc,
+  return cudaLaunchKernelEx(&cfg, gemm_pair_kernel, p.mapW, p.mapA2[idx], *mapC, M, p.N, p.K, sh.BN, sh.split, sh.stages, sh.n_acc,
                             sh.tmem_cols, epi, tma_c, (float *)C, norm ? *norm : SkNorm{}, rope ? *rope : PairRope{}, status,
                             lr) == cudaSuccess;
 }

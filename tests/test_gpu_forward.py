@@ -274,3 +274,13 @@ def test_bf16_attention_of_long_passes(B, n):
     want = gt.copy()
     want[B - 1, n - 7:] = np.nan
     np.testing.assert_array_equal(got, want)
+
+
+@pytest.mark.parametrize("n", [103, 205])
+def test_bf16_forward_with_k_split_over_two_pairs(n):
+    """Residual contractions of 515 and 1025 rows whose K is long and whose tiles are few: two pairs of SMs per tile, each with
+    half of K and half of the rows to finish, the last row block ragged or without rows for one of them."""
+    wl = small_workload("bf16", Arch(2, 256, 4, 2048), Arch(1, 384, 6, 4096), 32)
+    gt, wt, gd, wd = run_forward_case(wl, 0, n)
+    assert parity.value_error("rel_rms", gt, wt) < 2e-2       # bf16 operands, as above
+    assert parity.value_error("rel_rms", gd, wd) < 2e-2

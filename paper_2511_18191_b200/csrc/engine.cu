@@ -327,7 +327,7 @@ constexpr int kFlashStShort = 2;
 // more CTAs than an even share of the grid.  The kernel starts while the QKV contraction before it still runs, and where
 // that leaves SMs free (66 of 74 pairs at 1024 tokens of d = 512) those would fill up with CTAs that then run one after
 // the other while the rest of the machine is idle (plain decoding of 64 point tokens a pass behind 512 of them, 16 series,
-// 128 CTAs: 2.97 ms per forecast without, 2.40 with; 8, 24 and 32 series: 2.26 -> 2.12, 3.38 -> 2.95, 3.80 -> 3.39).
+// 128 CTAs, before attn_mma_kernel took such passes with heads of 64: 2.97 ms per forecast without, 2.40 with; 8, 24 and 32 series: 2.26 -> 2.12, 3.38 -> 2.95, 3.80 -> 3.39).
 // Larger grids fill the machine anyhow, and the even share then only stands in the way of balancing blocks of different
 // length (scoring 512 CTAs: 510 -> 518 us).
 template <int DH> int tiles_smem(long ctas) {

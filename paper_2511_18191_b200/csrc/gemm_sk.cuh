@@ -236,7 +236,7 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant__
         const uint32_t a = tiles + (uint32_t)c4 * 4;
         asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote[r]) : "r"(a), "r"((uint32_t)(r < S ? r : 0)));
       }
-      const bool vec = (N % 4 == 0) && (f + 3 < N);
+      const bool vec = N % 4 == 0 && f + 3 < N && !((uintptr_t)C & 15);
 #pragma unroll 1
       for (int tl = rank + S * rg; tl < BN; tl += 4 * S) {
         const int t = t0 + tl;

@@ -244,6 +244,23 @@ def test_few_token_gemm_matches_fp64_product(M, N, K):
     test_many_token_gemm_matches_fp64_product(M, N, K)
 
 
+@pytest.mark.parametrize("M,N,K", [(600, 2560, 2048), (600, 256, 2048), (520, 130, 2560), (700, 192, 128), (64, 256, 2048)])
+@pytest.mark.parametrize("offset", [1, 2, 3])
+def test_gemm_into_outputs_that_start_on_any_float(M, N, K, offset):
+    """Outputs that are not 16-byte aligned: K split in two and in four, rows that are whole float4 and not, K in one piece, and
+    the kernel of up to 512 tokens.  The values around the output stay as they are."""
+    import paper_2511_18191_b200 as tsfm
+    g = torch.Generator(device="cpu").manual_seed(M + N)
+    A = torch.randn((M, K), generator=g).to(torch.bfloat16)
+    W = (torch.randn((N, K), generator=g) / K ** 0.5).to(torch.bfloat16)
+    buf = torch.full((M * N + 8,), float("nan"), device="cuda")
+    C = buf[offset:offset + M * N]
+    tsfm.tsfm_gemm_bf16(torch.cuda.current_stream().cuda_stream, A.cuda(), W.cuda(), C, M, N, K, tsfm.TSFM_GEMM_AUTO)
+    torch.cuda.synchronize()
+    assert (C.view(M, N).cpu().double() - A.double() @ W.double().T).abs().max() < 2e-5 * K ** 0.5 + 1e-5
+    assert torch.isnan(buf[:offset]).all() and torch.isnan(buf[offset + M * N:]).all()
+
+
 @pytest.mark.parametrize("n", [2, 4, 26, 102])
 def test_bf16_forward_of_wide_models_on_few_tokens(n):
     """Folded norms of up to 512 rows (5 n) in the epilogues of that kernel: widths whose contractions no other kernel takes

@@ -60,7 +60,8 @@ extern "C" {
 #define TSFM_GEMM_WS    2       /* tsfm_gemm_bf16 only: the small-batch kernel that keeps its weight
                                    tile in registers (TSFM_ERR_SHAPE outside its domain: at most
                                    512 tokens, K a multiple of 64 up to 2048, N even, a grid of
-                                   16 x 32 tiles that is resident at once);
+                                   16 x 32 tiles that is resident at once,
+                                   C 8-byte aligned);
                                    a decoder picks it by itself where it applies                   */
 
 #define TSFM_EXEC_GRAPH   0       /* a forecast is one CUDA-graph launch: prologue, a device-side WHILE

@@ -1507,7 +1507,7 @@ int tsfm_gemm_bf16(void *stream, const void *A, const void *W, float *C, int32_t
     return TSFM_OK;
   }
   if (backend == TSFM_GEMM_WS) {
-    if (!gemm_ws_accepts(A, W, M, N, Kd)) return TSFM_ERR_SHAPE;
+    if (((uintptr_t)C & 7) || !gemm_ws_accepts(A, W, M, N, Kd)) return TSFM_ERR_SHAPE;       // (it stores two features at a time)
     if (!gemm_ws_launch(s, false, A, W, C, M, N, Kd, EPI_F32, nullptr, LiveRows{nullptr, 0})) CU_TRY(cudaGetLastError());
     LAUNCHED();
     CU_TRY(cudaGetLastError());

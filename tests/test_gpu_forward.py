@@ -261,6 +261,20 @@ def test_gemm_into_outputs_that_start_on_any_float(M, N, K, offset):
     assert torch.isnan(buf[:offset]).all() and torch.isnan(buf[offset + M * N:]).all()
 
 
+def test_small_batch_gemm_refuses_outputs_that_it_cannot_store():
+    """Pairs of features leave as eight bytes: an output that starts on an odd float is refused on the host, as misaligned
+    operands are, and left alone."""
+    import paper_2511_18191_b200 as tsfm
+    A, W = torch.ones((8, 64), dtype=torch.bfloat16, device="cuda"), torch.ones((16, 64), dtype=torch.bfloat16, device="cuda")
+    buf = torch.zeros(132, device="cuda")
+    s = torch.cuda.current_stream().cuda_stream
+    with pytest.raises(tsfm.TsfmError) as e:
+        tsfm.tsfm_gemm_bf16(s, A, W, buf[1:129], 8, 16, 64, tsfm.TSFM_GEMM_WS)
+    assert e.value.code == tsfm.TSFM_ERR_SHAPE and not buf.any()
+    tsfm.tsfm_gemm_bf16(s, A, W, buf[2:130], 8, 16, 64, tsfm.TSFM_GEMM_WS)
+    assert (buf[2:130] == 64).all() and not buf[:2].any() and not buf[130:].any()
+
+
 @pytest.mark.parametrize("n", [2, 4, 26, 102])
 def test_bf16_forward_of_wide_models_on_few_tokens(n):
     """Folded norms of up to 512 rows (5 n) in the epilogues of that kernel: widths whose contractions no other kernel takes

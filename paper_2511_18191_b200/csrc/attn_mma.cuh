@@ -28,6 +28,12 @@ constexpr int AM_Q = 128, AM_KEYS = 128, AM_DH = 64;
 constexpr int AM_TILE = AM_KEYS * AM_DH * 2;                    // 16 KB: a tile of keys, of values, or one part of the queries
 constexpr int AM_WARPS = 8, AM_THREADS = 32 * (AM_WARPS + 2);
 constexpr int AM_SMEM = 6 * AM_TILE + 1024 + 128 + 2 * AM_Q * 4;   // Q high, Q low, two stages of K and V
+// Shared memory of a launch: two CTAs fit on an SM, but a grid of at most one per SM takes more than half of it, so that no two
+// share one while another SM is idle.  (The QKV contraction before it leaves SMs free early, and CTAs that start there pile
+// up: see tiles_smem.  64 pairs x 128 queries behind 640 keys 24.6 us a launch with two, 18.4 with one; x 256 behind 768 34
+// and 26; 128 pairs x 96 behind 672 27 and 22; 64 x 256 behind none 11 and 8.)
+constexpr int AM_SMEM_ALONE = 114 * 1024;
+inline int attn_mma_smem(long ctas) { return ctas <= 148 ? AM_SMEM_ALONE : AM_SMEM; }
 constexpr int AM_COLS = 256, AM_S = 0, AM_P = 128, AM_O = 192;   // columns of tensor memory
 
 __device__ __forceinline__ void umma_bf16_ts(uint32_t tmem_d, uint32_t tmem_a, uint64_t db, uint32_t idesc, uint32_t acc) {

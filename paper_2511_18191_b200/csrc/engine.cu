@@ -606,9 +606,10 @@ void launch_attn(tsfm_spec *h, ModelDev &m, int l, int B, const PassGeom &g, boo
   if constexpr (sizeof(T) == 2) {
     const int pairs = B * m.arch.n_heads;
     if (DH == AM_DH && m.attn_mma && g.q_len > kMmaAttnTokens) {
-      launch_ex(h->ls, h->pdl, attn_mma_kernel, dim3(m.arch.n_heads, B, (g.q_len + AM_Q - 1) / AM_Q), dim3(AM_THREADS), (size_t)AM_SMEM,
-                m.mapK, m.mapV, h->qkv, m.rope, g, m.arch.n_heads, (int)(l * (m.kv_layer_elems / AM_DH)), appended ? 1 : 0,
-                (bf16 *)h->ao, h->dev_status);
+      const dim3 grid(m.arch.n_heads, B, (g.q_len + AM_Q - 1) / AM_Q);
+      launch_ex(h->ls, h->pdl, attn_mma_kernel, grid, dim3(AM_THREADS), (size_t)attn_mma_smem((long)pairs * grid.z), m.mapK, m.mapV,
+                h->qkv, m.rope, g, m.arch.n_heads, (int)(l * (m.kv_layer_elems / AM_DH)), appended ? 1 : 0, (bf16 *)h->ao,
+                h->dev_status);
       return;
     }
     if (pre) {
@@ -1284,7 +1285,7 @@ int tsfm_spec_create(const tsfm_weights *target_w, const tsfm_weights *draft_w, 
       const size_t kv_rows = m->kv_layer_elems / m->dh * m->arch.n_layers;
       if (m->dh == AM_DH && kv_rows < (1u << 30)) {           // (coordinates of a copy are 32-bit)
         if (tc_encode(&m->mapK, m->Kc, (int)kv_rows, AM_DH, AM_KEYS) || tc_encode(&m->mapV, m->Vc, (int)kv_rows, AM_DH, AM_KEYS) ||
-            cudaFuncSetAttribute(attn_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, AM_SMEM) != cudaSuccess)
+            cudaFuncSetAttribute(attn_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, AM_SMEM_ALONE) != cudaSuccess)
           return fail(TSFM_ERR_CUDA);
         m->attn_mma = true;
       }

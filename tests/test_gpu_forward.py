@@ -307,6 +307,34 @@ def test_bf16_attention_of_long_passes(B, n):
     np.testing.assert_array_equal(got, want)
 
 
+def attention_launches(heads, B, n, tmp_path):
+    """(kernel, CTAs, shared memory) of the attention launches of a scoring pass, from the profiler's records."""
+    import json
+    import paper_2511_18191_b200 as tsfm
+    arch = Arch(1, 64 * heads, heads, 64)
+    wl = small_workload("bf16", arch, arch, 16, mode="layer_skip")
+    dec = tsfm.SpecDecoder(build_models(wl)[0], None, arch, arch, 16, "bf16", "layer_skip", max_batch=B, max_ctx_tokens=n,
+                           max_horizon_patches=1, max_K=1)
+    z = torch.zeros((B, n, 16), device="cuda")
+    dec.model_forward(0, z)
+    with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
+        dec.model_forward(0, z)
+    dec.close()
+    prof.export_chrome_trace(str(tmp_path / "t.json"))
+    ev = [e for e in json.loads((tmp_path / "t.json").read_text())["traceEvents"] if e.get("cat") == "kernel"]
+    if not ev:
+        pytest.skip("the profiler records no kernels here")
+    return [(e["name"], int(np.prod(e["args"]["grid"])), int(e["args"]["shared memory"])) for e in ev if "attn" in e["name"]]
+
+
+@pytest.mark.parametrize("heads,B,n", [(4, 1, 520), (4, 12, 380), (4, 13, 380)])
+def test_small_attention_grids_do_not_share_sms(heads, B, n, tmp_path):
+    """20, 144 and 156 CTAs: up to one per SM each takes more than half of an SM's shared memory."""
+    (name, ctas, smem), = attention_launches(heads, B, n, tmp_path)
+    assert "attn_mma_kernel" in name and ctas == heads * B * -(-n // 128)
+    assert (smem + 1024 > 114 * 1024) == (ctas <= 148)
+
+
 @pytest.mark.parametrize("n", [103, 205])
 def test_bf16_forward_with_k_split_over_two_pairs(n):
     """Residual contractions of 515 and 1025 rows whose K is long and whose tiles are few: two pairs of SMs per tile, each with

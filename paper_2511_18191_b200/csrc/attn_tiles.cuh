@@ -13,7 +13,11 @@
 //     into bf16 high and low parts, scores in base-2 units, probabilities rounded to bf16 for P V;
 //   * warps skip the half tiles behind their last query; only the rows of a half tile that holds a visible
 //     key are fetched;
-//   * the query blocks with the most keys start first.
+//   * the query blocks with the most keys start first;
+//   * a value that a query must not see does not reach it, although an infinity or NaN times its probability of 0 is NaN: a
+//     block that ends with such outputs beside finite sums of probabilities goes over its keys again, with these values as
+//     0 in the tiles that only some of its queries see, and NaN for the queries that do see them (the look at the outputs:
+//     nothing to be seen from 33 tokens on, 0.3 to 0.6 us a launch of 8 to 17 at 18 to 30).
 // Bound: latency of a block's first loads and of the mma.sync chains with 16 warps per SM (64 x 20 x 255: tensor pipe
 // 31 % busy, issue slots 34 %).
 // grid = (heads, B, ceil(q_len / (16 warps))), block = 32 x warps, warps = 2 where q_len <= 32, else 4.
@@ -34,6 +38,7 @@ attn_tiles_kernel(const float *qkv, const bf16 *Kc, const bf16 *Vc, const float2
   using G = TilesGeom<DH>;
   constexpr int HALF = DH / 2, KS = DH / 16, CPR = DH / 8;
   extern __shared__ __align__(256) unsigned char tiles_smem[];
+  __shared__ int bad_row;                                      // first value row of a tile with an infinity or NaN
   const uint32_t ring = (uint32_t)__cvta_generic_to_shared(tiles_smem);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
   const int gr = lane >> 2, q4 = lane & 3, d = n_heads * DH;
@@ -93,45 +98,75 @@ attn_tiles_kernel(const float *qkv, const bf16 *Kc, const bf16 *Vc, const float2
         }
     }
   }
-  float o[DH / 8][4];
-#pragma unroll
-  for (int n = 0; n < DH / 8; ++n) o[n][0] = o[n][1] = o[n][2] = o[n][3] = 0.f;
-  float m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};
   const int qpos0 = p0 + jq + gr;                              // position of row gr; row gr + 8 is 8 further
   const FlashLane<DH> fl(lane);
-
-  for (int tile = 0; tile < n_tiles; ++tile) {
-    issue(tile + 1);
-    flash_wait<1>();
-    __syncthreads();
-    const uint32_t stage = ring + (uint32_t)((tile & 1) * G::STAGE_BYTES);
-#pragma unroll 1
-    for (int half = 0; half < 2; ++half) {
-      const int t0 = tile * G::KEYS + half * G::HALF_KEYS;
-      if (nq <= 0 || t0 > p0 + jq + nq - 1) break;             // no key of this half is visible to this warp
-      const uint32_t kst = stage + (uint32_t)(half * G::HALF_KEYS * G::ROW_BYTES), vst = kst + G::TILE_BYTES;
-      flash_step<DH>(kst, vst, fl, qhi, qlo, o, m_run, l_run, [&](float (&s)[4][4]) {
-        if (t0 + G::HALF_KEYS - 1 > p0 + jq) {                 // (only halves that reach past the first query)
+  float o[DH / 8][4], m_run[2], l_run[2];
+  bool nan_seen[2] = {false, false};
+  for (bool again = false;; again = true) {
 #pragma unroll
-          for (int n = 0; n < 4; ++n)
-#pragma unroll
-            for (int e = 0; e < 4; ++e)
-              if (t0 + n * 8 + q4 * 2 + (e & 1) > qpos0 + (e >> 1) * 8) s[n][e] = -INFINITY;
+    for (int n = 0; n < DH / 8; ++n) o[n][0] = o[n][1] = o[n][2] = o[n][3] = 0.f;
+    m_run[0] = m_run[1] = -INFINITY;
+    l_run[0] = l_run[1] = 0.f;
+    if (again) issue(0);
+    for (int tile = 0; tile < n_tiles; ++tile) {
+      issue(tile + 1);
+      flash_wait<1>();
+      __syncthreads();
+      if (again && (tile + 1) * G::KEYS > p0 + qb + 1) {       // (the same for the whole block)
+        if (threadIdx.x == 0) bad_row = G::KEYS;
+        __syncthreads();
+        for (int idx = threadIdx.x; idx < G::KEYS * CPR; idx += blockDim.x) {
+          uint4 *v = reinterpret_cast<uint4 *>(tiles_smem + (tile & 1) * G::STAGE_BYTES + G::TILE_BYTES + idx * 16);
+          const uint4 u = *v;                                  // (an exponent of all ones carries into its sign)
+          if ((((u.x & 0x7f807f80u) + 0x00800080u) | ((u.y & 0x7f807f80u) + 0x00800080u) | ((u.z & 0x7f807f80u) + 0x00800080u) |
+               ((u.w & 0x7f807f80u) + 0x00800080u)) & 0x80008000u) {
+            *v = make_uint4(0u, 0u, 0u, 0u);
+            atomicMin(&bad_row, idx / CPR);
+          }
         }
-      });
+        __syncthreads();
+#pragma unroll
+        for (int rr = 0; rr < 2; ++rr) nan_seen[rr] |= qpos0 + rr * 8 >= tile * G::KEYS + bad_row;
+      }
+      const uint32_t stage = ring + (uint32_t)((tile & 1) * G::STAGE_BYTES);
+#pragma unroll 1
+      for (int half = 0; half < 2; ++half) {
+        const int t0 = tile * G::KEYS + half * G::HALF_KEYS;
+        if (nq <= 0 || t0 > p0 + jq + nq - 1) break;           // no key of this half is visible to this warp
+        const uint32_t kst = stage + (uint32_t)(half * G::HALF_KEYS * G::ROW_BYTES), vst = kst + G::TILE_BYTES;
+        flash_step<DH>(kst, vst, fl, qhi, qlo, o, m_run, l_run, [&](float (&s)[4][4]) {
+          if (t0 + G::HALF_KEYS - 1 > p0 + jq) {               // (only halves that reach past the first query)
+#pragma unroll
+            for (int n = 0; n < 4; ++n)
+#pragma unroll
+              for (int e = 0; e < 4; ++e)
+                if (t0 + n * 8 + q4 * 2 + (e & 1) > qpos0 + (e >> 1) * 8) s[n][e] = -INFINITY;
+          }
+        });
+      }
+      if (tile + 1 < n_tiles) __syncthreads();                 // the stage is free for the tile after next
     }
-    __syncthreads();                                           // the stage is free for the tile after next
-  }
+    // outputs; they leave before the vote (behind it: 3 % of a launch of 33 to 240 tokens)
+    bool bad = false;
 #pragma unroll
-  for (int rr = 0; rr < 2; ++rr) {
-    l_run[rr] += __shfl_xor_sync(0xffffffffu, l_run[rr], 1);
-    l_run[rr] += __shfl_xor_sync(0xffffffffu, l_run[rr], 2);
-    const int i = gr + rr * 8;
-    if (i >= nq) continue;
-    const float inv = 1.f / l_run[rr];
-    uint32_t *dst = reinterpret_cast<uint32_t *>(out + (row0 + jq + i) * d + h * DH);
+    for (int rr = 0; rr < 2; ++rr) {
+      l_run[rr] += __shfl_xor_sync(0xffffffffu, l_run[rr], 1);
+      l_run[rr] += __shfl_xor_sync(0xffffffffu, l_run[rr], 2);
+      float c[2] = {0.f, 0.f};                                 // 0, or NaN where an output is infinite or NaN
 #pragma unroll
-    for (int n = 0; n < DH / 8; ++n) dst[n * 4 + q4] = pack_bf16x2(o[n][rr * 2] * inv, o[n][rr * 2 + 1] * inv);
+      for (int n = 0; n < DH / 8; ++n) {
+        c[0] = fmaf(o[n][rr * 2], 0.f, c[0]);
+        c[1] = fmaf(o[n][rr * 2 + 1], 0.f, c[1]);
+      }
+      const int i = gr + rr * 8;
+      if (i >= nq) continue;
+      bad |= c[0] + c[1] != 0.f && l_run[rr] == l_run[rr];
+      const float inv = nan_seen[rr] ? __int_as_float(0x7fffffff) : 1.f / l_run[rr];
+      uint32_t *dst = reinterpret_cast<uint32_t *>(out + (row0 + jq + i) * d + h * DH);
+#pragma unroll
+      for (int n = 0; n < DH / 8; ++n) dst[n * 4 + q4] = pack_bf16x2(o[n][rr * 2] * inv, o[n][rr * 2 + 1] * inv);
+    }
+    if (again || !__syncthreads_or(bad)) break;
   }
 }
 

@@ -1,5 +1,5 @@
-// Causal attention of passes of 17 to 32 tokens, and of longer ones with heads of 32 or 128 (heads of 64: attn_mma.cuh), over
-// a bf16 KV cache.  The keys and values of the pass are in the cache: the QKV contraction put them there and
+// Causal attention of passes of 17 tokens and more over a bf16 KV cache (with heads of 64 those that fill blocks of 128
+// queries go to attn_mma.cuh, see attn_mma_pays).  The keys and values of the pass are in the cache: the QKV contraction put them there and
 // rotated and scaled the queries (rotated = 1, see PairRope), or kv_append_kernel did (rotated = 0: the queries
 // are rotated here).
 //

@@ -581,9 +581,26 @@ void gemm(tsfm_spec *h, GemmSkPlan *plan, const void *A, const void *W, void *C,
   launch_gemm_simt<T>(h->ls, h->pdl, (const T *)A, (const T *)W, C, M, N, K, epi, lr);
 }
 
-// Passes of more tokens than this, with heads of 64, attend on the tensor-memory kernel (attn_mma_kernel; figures there).  Up
-// to 32 queries fill a quarter of its 128 rows: 3200 blocks of 30 queries x 30 keys run 18 us in attn_tiles_kernel, which also
-// keeps the other head sizes.
+// Which kernel a pass with heads of 64 attends on, from 33 tokens on (up to 32 attn_tiles_kernel runs two warps a CTA): the
+// tensor-memory kernel takes 128 queries a CTA and costs the same for one of them as for all, attn_tiles_kernel takes 64 in
+// four warps.  A launch costs its waves of blocks (two and four on an SM), a block its start and its steps of 128 and 64 keys (a
+// step of attn_tiles_kernel mostly by the warps that have queries).  In us, fitted to the attention's share of prefills of 33 to
+// 704 tokens and of passes of 48 to 256 tokens behind 100 to 2000 keys, 8 to 3200 (series, head) pairs, 617 shapes: 0.4 % above
+// the better kernel on average, at most 1.8 us (6 %) above attn_tiles_kernel.  Measured at 1280 pairs, us a launch,
+// attn_tiles_kernel / attn_mma_kernel: 33 tokens 12 / 32, 64 15 / 34, 128 40 / 41, 144 56 / 81, 192 71 / 88, 256 107 / 99, 320 146
+// / 150, 384 190 / 156; 48 behind 192 to 336 keys 39 / 56, 64 behind 576 to 768 88 / 90, 96 behind 192 to 480 87 / 73, 128 behind
+// 256 to 640 123 / 80.
+bool attn_mma_pays(long pairs, int first, int q_len) {
+  double tiles = 0, mma = 0;
+  long n64 = 0, n128 = 0;
+  for (int q = 0; q < q_len; q += 64, ++n64) {
+    const int rows = std::min(64, q_len - q);
+    tiles += 3.6 + (first + q + rows + 63) / 64 * (0.6 + 1.5 * 0.25 * ((rows + 15) / 16));
+  }
+  for (int q = 0; q < q_len; q += AM_Q, ++n128) mma += 6.1 + 1.8 * ((first + std::min(q + AM_Q, q_len) + AM_KEYS - 1) / AM_KEYS);
+  const long waves64 = (pairs * n64 + 4 * 148 - 1) / (4 * 148), waves128 = (pairs * n128 + 2 * 148 - 1) / (2 * 148);
+  return waves128 * (mma / n128) < waves64 * (tiles / n64);
+}
 constexpr int kMmaAttnTokens = 32;
 
 // appended: the QKV contraction has rotated the queries and put the pass's keys and values into the cache;
@@ -605,7 +622,7 @@ void launch_attn(tsfm_spec *h, ModelDev &m, int l, int B, const PassGeom &g, boo
   if (pre && cache_only) return;
   if constexpr (sizeof(T) == 2) {
     const int pairs = B * m.arch.n_heads;
-    if (DH == AM_DH && m.attn_mma && g.q_len > kMmaAttnTokens) {
+    if (DH == AM_DH && m.attn_mma && g.q_len > kMmaAttnTokens && attn_mma_pays(pairs, std::max(g.base, 0), g.q_len)) {
       const dim3 grid(m.arch.n_heads, B, (g.q_len + AM_Q - 1) / AM_Q);
       launch_ex(h->ls, h->pdl, attn_mma_kernel, grid, dim3(AM_THREADS), (size_t)attn_mma_smem((long)pairs * grid.z), m.mapK, m.mapV,
                 h->qkv, m.rope, g, m.arch.n_heads, (int)(l * (m.kv_layer_elems / AM_DH)), appended ? 1 : 0, (bf16 *)h->ao,

@@ -286,11 +286,11 @@ def test_bf16_forward_of_wide_models_on_few_tokens(n):
     assert parity.value_error("rel_rms", gd, wd) < 2e-2
 
 
-@pytest.mark.parametrize("B,n", [(1, 33), (2, 128), (1, 200), (3, 257), (5, 129)])
+@pytest.mark.parametrize("B,n", [(1, 33), (2, 128), (1, 200), (3, 257), (5, 129), (1, 500), (2, 385), (3, 520)])
 def test_bf16_attention_of_long_passes(B, n):
-    """Heads of 64, more than 32 tokens: one or several blocks of 128 queries, ragged last blocks and key tiles, queries rotated
-    in the kernel (up to 512 rows) or before it.  A NaN in a late token reaches the tokens behind it in its own series only, and
-    changes nothing else by a bit."""
+    """Heads of 64, more than 32 tokens: blocks of 64 and (the last three) of 128 queries, ragged last blocks and key tiles,
+    queries rotated in the kernel (up to 512 rows) or before it.  A NaN in a late token reaches the tokens behind it in its own
+    series only, and changes nothing else by a bit."""
     import paper_2511_18191_b200 as tsfm
     wl = small_workload("bf16", Arch(2, 128, 2, 256), Arch(1, 256, 4, 256), 32)
     gt, wt, gd, wd = run_forward_case(wl, 0, n, B=B)
@@ -333,6 +333,14 @@ def test_small_attention_grids_do_not_share_sms(heads, B, n, tmp_path):
     (name, ctas, smem), = attention_launches(heads, B, n, tmp_path)
     assert "attn_mma_kernel" in name and ctas == heads * B * -(-n // 128)
     assert (smem + 1024 > 114 * 1024) == (ctas <= 148)
+
+
+@pytest.mark.parametrize("B,n,mma", [(16, 33, False), (320, 64, False), (320, 100, False), (320, 160, False), (80, 192, False),
+                                     (1, 256, True), (320, 256, True), (320, 380, True)])
+def test_blocks_of_128_queries_are_not_given_passes_that_leave_them_empty(B, n, mma, tmp_path):
+    """Windows of 33 to 200 tokens run faster in blocks of 64 queries, as long passes do in blocks of 128."""
+    (name, _, _), = attention_launches(4, B, n, tmp_path)
+    assert ("attn_mma_kernel" in name) == mma and ("attn_tiles_kernel" in name) != mma
 
 
 @pytest.mark.parametrize("n", [103, 205])

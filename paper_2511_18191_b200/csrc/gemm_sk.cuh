@@ -1,20 +1,18 @@
-// bf16 x bf16 -> fp32 contraction on the sm_100a tensor cores, split along K across a
-// thread-block cluster.
+// bf16 x bf16 -> fp32 contraction on the sm_100a tensor cores, one SM per tile, from 513 tokens on: widths that are an odd
+// multiple of 64 and outputs that are not 16-byte aligned (whole 128-feature tiles go to gemm_pair_kernel, fewer tokens to
+// gemm_push_kernel).
 //
 //   C[t, f] (op)= sum_k A[t, k] * W[f, k]        A: [M, K] tokens, W: [N, K] weights
 //
 // Same swap-AB tiling as gemm_tc.cuh (128 weight rows = MMA M, BN tokens = MMA N, 64-wide K
 // stages fed by TMA into a 128-byte-swizzled ring, accumulator in tensor memory), with two
-// differences that matter when the token count is small and the call is latency-bound:
-//   * BN is a run-time value (any multiple of 16 up to 256), so M = 160 verification tokens
-//     are one tile, not a padded 256;
-//   * the K loop is split over the S CTAs of a cluster (grid.z = cluster.z = S <= 8).  Each CTA
-//     parks its partial tile in its own shared memory; after a cluster barrier CTA r sums rows
+// differences:
+//   * BN is a run-time value (any multiple of 16 up to 256), chosen so that the grid fills its waves;
+//   * a long K loop of up to 4095 tokens is split over the S = 2 or 4 CTAs of a cluster (grid.z = cluster.z = S).  Each
+//     CTA parks its partial tile in its own shared memory; after a cluster barrier CTA r sums rows
 //     r, r + S, ... of all S partial tiles through distributed shared memory and applies the
 //     epilogue once.  No atomics, no pre-zeroed accumulator, a fixed summation order, and every
 //     epilogue (GELU included) can be split.
-// Used from 513 tokens on for widths that are an odd multiple of 64 (whole 128-feature tiles go to gemm_pair_kernel, fewer
-// tokens to gemm_push_kernel) and for outputs that are not 16-byte aligned.
 // Warp roles and bounded waits as in gemm_tc.cuh.
 #pragma once
 #include "gemm_tc.cuh"
@@ -22,7 +20,7 @@
 
 namespace tsfm {
 
-constexpr int SK_MAX_SPLIT = 8;
+constexpr int SK_MAX_SPLIT = 4;
 
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");

@@ -1,16 +1,19 @@
-// Causal attention of passes of many tokens on the tensor cores (tcgen05), head size 64, over a bf16 KV cache.
+// Causal attention of passes of many tokens on the tensor cores (tcgen05), head size 64, over a bf16 KV cache (which passes:
+// attn_mma_pays).
 //
 // A CTA takes 128 consecutive queries of one (series, head) and walks over the keys they may see in tiles of 128:
 //   S = Q K^T (Q in two bf16 parts, high and low, so that the scores keep fp32-like accuracy: eight MMAs of 128 x 128 x 16
-//   from shared memory into tensor memory), softmax by two threads per query row, each half of the tile's keys (no shuffle: the row sits in the
-//   threads' lane of tensor memory; the two maxima meet in shared memory), probabilities back into tensor memory as bf16, O = P V (P from tensor memory, V as it lies in
-//   the cache: the "MN-major" form of the operand), summed over the tiles in registers with the running maximum's factors,
-//   as attn_tiles_kernel does it for 16 queries per warp.
+//   from shared memory into tensor memory), softmax by two threads per query row, each half of the tile's keys (no shuffle:
+//   the row sits in the threads' lane of tensor memory; the two maxima meet in shared memory), probabilities back into tensor
+//   memory as bf16, O = P V (P from tensor memory, V as it lies in the cache: the "MN-major" form of the operand), summed over
+//   the tiles in registers with the running maximum's factors, as attn_tiles_kernel does it for 16 queries per warp.
 // While one CTA's rows are in softmax the other CTA of the SM keeps the tensor core busy (98 KB of shared memory and half of
 // tensor memory each).
 // Values that a query must not see never meet it: rows behind the last key are zeroed in shared memory, and in tiles that some
 // queries see in part, value rows with an infinity or NaN are zeroed too and the queries that do see them set to NaN (a
-// product 0 x NaN would reach all 128 queries).
+// product 0 x NaN would reach all 128 queries).  An infinity so makes the head NaN, where in a tile that every query sees it
+// stays in its dimension: the token's output is NaN in either case, since the contraction behind multiplies the infinity by
+// weights of both signs and the norm behind that by 0.
 // Bound: the chain of a tile (MMAs, two passes over the scores, MMAs, sums) and a block's first loads, with 16 softmax warps
 // per SM.
 // attn_tiles_kernel -> here, us a launch inside a forecast: 16 series x 8 heads x 256 queries behind 704 to 1000 keys 53 -> 28,
@@ -30,8 +33,8 @@ constexpr int AM_WARPS = 8, AM_THREADS = 32 * (AM_WARPS + 2);
 constexpr int AM_SMEM = 6 * AM_TILE + 1024 + 128 + 2 * AM_Q * 4;   // Q high, Q low, two stages of K and V
 // Shared memory of a launch: two CTAs fit on an SM, but a grid of at most one per SM takes more than half of it, so that no two
 // share one while another SM is idle.  (The QKV contraction before it leaves SMs free early, and CTAs that start there pile
-// up: see tiles_smem.  64 pairs x 128 queries behind 640 keys 24.6 us a launch with two, 18.4 with one; x 256 behind 768 34
-// and 26; 128 pairs x 96 behind 672 27 and 22; 64 x 256 behind none 11 and 8.)
+// up: see tiles_smem.  Inside forecasts, us a launch with two -> one: 64 pairs x 128 queries behind 770 to 1150 keys 23.7 ->
+// 17.5, x 256 behind 1024 to 1792 33.6 -> 25.1, x 256 behind none 10.6 -> 8.0; 128 pairs x 96 behind 770 to 1060 23.7 -> 19.1.)
 constexpr int AM_SMEM_ALONE = 114 * 1024;
 inline int attn_mma_smem(long ctas) { return ctas <= 148 ? AM_SMEM_ALONE : AM_SMEM; }
 constexpr int AM_COLS = 256, AM_S = 0, AM_P = 128, AM_O = 192;   // columns of tensor memory

@@ -1,7 +1,7 @@
 // Causal attention of passes of 17 tokens and more over a bf16 KV cache (with heads of 64 those that fill blocks of 128
-// queries go to attn_mma.cuh, see attn_mma_pays).  The keys and values of the pass are in the cache: the QKV contraction put them there and
-// rotated and scaled the queries (rotated = 1, see PairRope), or kv_append_kernel did (rotated = 0: the queries
-// are rotated here).
+// queries go to attn_mma.cuh, see attn_mma_pays).  The keys and values of the pass are in the cache: the QKV
+// contraction put them there and rotated and scaled the queries (rotated = 1, see PairRope), or kv_append_kernel
+// did (rotated = 0: the queries are rotated here).
 //
 // A CTA takes up to 64 consecutive queries of one (series, head), 16 per warp (the M side of mma.sync
 // m16n8k16), and streams the keys they may see in tiles of 64 through two shared-memory stages that all its

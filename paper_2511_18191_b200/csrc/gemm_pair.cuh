@@ -7,9 +7,9 @@
 // tokens each load their half of both operands (128 feature rows, BN / 2 token rows) and both halves feed
 // both tensor cores: 256 + BN cycles of fill for 2 BN cycles of work per block step and SM, i.e. balanced
 // at BN = 256 where the single-SM form needs twice the work's time.
-//   * cluster of 2 along x; rank r owns features 128 r ... 128 r + 127 of the pair's tile in its own
-//     tensor memory, rank 0 issues every MMA; the copies of both ranks report to rank 0's barriers, the
-//     commits arrive at both ranks' (no copy is multicast);
+//   * cluster of 2 along x (4 where two pairs share a tile, each with half of K); rank r owns features
+//     128 r ... 128 r + 127 of the pair's tile in its own tensor memory, rank 0 issues every MMA; the copies of
+//     both ranks report to rank 0's barriers, the commits arrive at both ranks' (no copy is multicast);
 //   * persistent: pairs walk the tiles; with two accumulators (2 BN <= 512 columns) the epilogue of a tile
 //     runs under the main loop of the next;
 //   * 16 epilogue warps in four groups.  Where a pair walks over several tiles they take 16-token chunks in turn: tcgen05.ld,
@@ -156,7 +156,7 @@ __device__ __forceinline__ void pair_rope_rows(const float *stage, const int2 *p
   }
 }
 
-// grid = 2 x pairs, cluster = 2.  C leaves through mapC (box 128 features x 16 tokens): tma_c = SK_TMA_F32 /
+// grid = 2 x split x pairs, cluster = 2 x split (split: pairs per tile).  C leaves through mapC (box 128 features x 16 tokens): tma_c = SK_TMA_F32 /
 // SK_TMA_BF16 (stores; epi tells GELU) or SK_TMA_ADD; SK_TMA_NONE: fp32, straight from registers.
 __global__ void __launch_bounds__(PAIR_THREADS, 1)
 gemm_pair_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant__ CUtensorMap mapA,

@@ -19,9 +19,10 @@
 //     a CTA can hold more weights than tokens;
 //   * the MMA warp runs its loop as a whole and lets one lane issue: addresses and descriptors are then uniform
 //     values (0.21 -> 0.17 us a block step); stages are two K blocks (-> 0.11).
-// Bound: latency, and from K = 1280 on the weights (d = 1280, M = 64 from HBM: 39 MB a layer, 6.1 us).  Chains of dependent
-// launches (graph replay), us, gemm_sk_kernel's former form for these sizes (32-token tiles, K split until the grid fills
-// the SMs, pulled partial tiles) -> here, QKV / Wo / W1 / W2: d = 1280, M = 64 6.3 / 5.3 / 7.9 / 7.7 -> 5.2 / 4.0 / 6.1 / 6.6;
+// Bound: latency, and from K = 1280 on the weights (d = 1280, M = 64 from HBM: 39 MB a layer, 6.1 us).  Inside a forecast
+// (d = 1280, M = 64, weights from HBM), us a launch, gemm_sk_kernel's former form for these sizes (32-token tiles, K split until the
+// grid fills the SMs, pulled partial tiles) -> here, QKV / Wo / W1 / W2: 6.9 / 5.0 / 8.0 / 7.8 -> 5.5 / 5.0 / 5.3 / 7.4: Wo gains
+// nothing there.  Chains of these contractions alone (graph replay): d = 1280, M = 64 6.3 / 5.3 / 7.9 / 7.7 -> 5.2 / 4.0 / 6.1 / 6.6;
 // d = 1024, M = 93 6.2 / - / 7.1 / 7.0 -> 4.5 / - / 5.4 / 5.9; d = 512, M = 160 5.4 / - / 6.1 / 5.9 -> 3.6 / - / 4.0 / 4.8; d = 1280,
 // M = 512 20 / 11 / 31 / 28 -> 9.8 / 8.6 / 12 / 15.  (64-feature tiles: 0.2 % on average, not kept.  A bulk prefetch of the next
 // link's weights into L2: nothing.)

@@ -49,8 +49,8 @@ UNIT = "patches/s"
 # A kernel that has changed since its capture is listed with None.
 NCU_TRAFFIC_RATIO = {
     "gemm_push_small_M": None,
-    "gemm_sk_mid_M": None,
-    "gemm_sk_large_M": 0.81,       # 244.4 MB of 302.2 MB (M=16320, N=3840, K=1280)
+    "gemm_pair_mid_M": None,
+    "gemm_pair_large_M": None,
     "gemm_ws_small_M": 0.77,       # 0.942 MB of 1.229 MB (M=64, N=1152, K=384)
     "attn": 0.99,                  # 95.7 MB of 96.9 MB (C4 verification pass): the KV stream
 }

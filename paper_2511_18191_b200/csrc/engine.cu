@@ -182,11 +182,11 @@ namespace {
 
 // Kernel classes for per-launch timing.
 // The tensor-memory contractions in three regimes: up to 512 tokens (gemm_push_kernel: HBM / latency bound), from 4096
-// tokens tensor bound, between them one wave of tiles (gemm_pair_kernel; odd widths gemm_sk_kernel).
+// tokens tensor bound, between them one wave of tiles (both gemm_pair_kernel; odd widths gemm_sk_kernel).
 enum { KC_INSTNORM = 0, KC_EMBED, KC_RMSNORM, KC_GEMM_WS, KC_GEMM_TC_SMALL, KC_GEMM_TC_MID, KC_GEMM_TC_LARGE, KC_GEMM_SIMT,
        KC_ATTN, KC_HEAD, KC_ACCEPT, KC_DENORM, KC_COUNT };
 const char *const kKernelNames[KC_COUNT] = {"instnorm", "embed", "rmsnorm", "gemm_ws_small_M", "gemm_push_small_M",
-                                            "gemm_sk_mid_M", "gemm_sk_large_M", "gemm_simt", "attn", "head", "accept",
+                                            "gemm_pair_mid_M", "gemm_pair_large_M", "gemm_simt", "attn", "head", "accept",
                                             "denorm"};
 
 // Brackets one launch with two events when profiling is on (no-op otherwise).
@@ -327,7 +327,8 @@ constexpr int kFlashStShort = 2;
 // more CTAs than an even share of the grid.  The kernel starts while the QKV contraction before it still runs, and where
 // that leaves SMs free (66 of 74 pairs at 1024 tokens of d = 512) those would fill up with CTAs that then run one after
 // the other while the rest of the machine is idle (plain decoding of 64 point tokens a pass behind 512 of them, 16 series,
-// 128 CTAs, before attn_mma_kernel took such passes with heads of 64: 2.97 ms per forecast without, 2.40 with; 8, 24 and 32 series: 2.26 -> 2.12, 3.38 -> 2.95, 3.80 -> 3.39).
+// 128 CTAs, before attn_mma_kernel took such passes with heads of 64: 2.97 ms per forecast without, 2.40 with; 8, 24 and 32
+// series: 2.26 -> 2.12, 3.38 -> 2.95, 3.80 -> 3.39; attn_mma_smem does the same there).
 // Larger grids fill the machine anyhow, and the even share then only stands in the way of balancing blocks of different
 // length (scoring 512 CTAs: 510 -> 518 us).
 template <int DH> int tiles_smem(long ctas) {

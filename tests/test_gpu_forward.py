@@ -237,10 +237,10 @@ def test_small_batch_gemm_matches_fp64_product(M, N, K):
 
 
 @pytest.mark.parametrize("M,N,K", [(1, 1280, 5120), (3, 130, 4096), (17, 1280, 5120), (64, 3840, 1280), (93, 1024, 4096), (129, 64, 2560),
-                                   (500, 192, 80), (512, 5120, 1280), (511, 1280, 5120)])
+                                   (500, 192, 80), (512, 5120, 1280), (511, 1280, 5120), (130, 1088, 4352), (510, 320, 2560)])
 def test_few_token_gemm_matches_fp64_product(M, N, K):
-    """The kernel of up to 512 tokens: K in one piece and split over clusters of every size the tile rule asks for, rings that
-    hold K and rings that turn over, half a feature tile, ragged token tiles, K that is no whole block."""
+    """The kernel of up to 512 tokens: K in one piece and split over clusters of every size (8, 8, 8, 2, 6, 8, 1, 1, 3, 4, 4),
+    rings that hold K and rings that turn over, half a feature tile, ragged token tiles, K that is no whole block."""
     test_many_token_gemm_matches_fp64_product(M, N, K)
 
 
@@ -277,8 +277,9 @@ def test_small_batch_gemm_refuses_outputs_that_it_cannot_store():
 
 @pytest.mark.parametrize("n", [2, 4, 26, 102])
 def test_bf16_forward_of_wide_models_on_few_tokens(n):
-    """Folded norms of up to 512 rows (5 n) in the epilogues of that kernel: widths whose contractions no other kernel takes
-    (K = 1088 and 4352; 2560 with half a feature tile over)."""
+    """Folded norms of up to 512 rows (5 n) in the epilogues of that kernel: the target's QKV, W1 and W2 and the draft's W2 (K =
+    1088, 4352 and 2560; half a feature tile over) at every n, the others from 130 rows on, where gemm_ws_kernel has no room
+    (the draft's Wo never)."""
     wl = small_workload("bf16", Arch(2, 1088, 17, 4352), Arch(2, 320, 5, 2560), 32)
     gt, wt, gd, wd = run_forward_case(wl, 0, n)
     assert np.isfinite(gt).all() and np.isfinite(gd).all()

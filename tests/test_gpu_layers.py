@@ -1,4 +1,7 @@
-"""One decoder layer's attention on its own."""
+"""Attention and MLP of one decoder layer on their own, against 64-bit arithmetic that rounds where the bf16 path rounds
+(operands, cached keys and values, the attention's output, the MLP's activations).  What is left is the order of fp32 sums, so
+that these bounds see what a whole forward pass at 2e-2 cannot: a query that lost its low part, a row factor or a slice of a
+folded norm that is off, a partial sum that went astray."""
 import math
 
 import numpy as np
@@ -32,6 +35,82 @@ def forward(w, arch, z):
     got = dec.model_forward(0, torch.from_numpy(z).cuda()).cpu().numpy()
     dec.close()
     return got
+
+
+def bf16(x):
+    return round_to_bf16(np.asarray(x, dtype=np.float32)).astype(np.float64)
+
+
+def rstd(x):
+    return 1 / np.sqrt((x * x).mean(-1, keepdims=True) + 1e-6)
+
+
+def normed(x, g, folded):
+    """What a contraction makes of a normed row: operand and factor."""
+    if folded:
+        return bf16(g * x.astype(np.float32)), rstd(x)
+    return bf16(g * x * rstd(x)), 1.0
+
+
+def relative(got, want):
+    return float(np.sqrt(((got - want) ** 2).mean() / (want ** 2).mean()))
+
+
+def attention(w, heads, z, round_queries=False):
+    """Layer output of x + Wo attention(x) for rows whose norm needs no rounding (all values +1 or -1, gain 1)."""
+    x = z.astype(np.float64)
+    B, n, d = x.shape
+    dh = d // heads
+    split = lambda t: t.reshape(B, n, heads, dh).transpose(0, 2, 1, 3)  # noqa: E731
+    q, k, v = (split(x * rstd(x) @ w["layers.0." + m].T.astype(np.float64)) for m in ("Wq", "Wk", "Wv"))
+    angle = np.arange(n)[:, None] * 1e4 ** (-2.0 * np.arange(dh // 2) / dh)
+    c, s = np.cos(angle), np.sin(angle)
+    turn = lambda t: np.concatenate([t[..., :dh // 2] * c - t[..., dh // 2:] * s, t[..., dh // 2:] * c + t[..., :dh // 2] * s], -1)  # noqa: E731
+    q = turn(q) * (math.log2(math.e) / math.sqrt(dh))
+    e = (bf16(q) if round_queries else q) @ bf16(turn(k)).transpose(0, 1, 3, 2)
+    e = np.where(np.tril(np.ones((n, n), dtype=bool)), e, -np.inf)
+    p = np.exp2(e - e.max(-1, keepdims=True))
+    o = p / p.sum(-1, keepdims=True) @ bf16(v)
+    y = x + bf16(o.transpose(0, 2, 1, 3).reshape(B, n, d)) @ w["layers.0.Wo"].T.astype(np.float64)
+    return y * rstd(y) * w["g_f"]
+
+
+@pytest.mark.parametrize("B,n", [(1, 20), (2, 33), (3, 64), (2, 100), (1, 129), (2, 200), (2, 300), (3, 384)])
+def test_attention_keeps_both_parts_of_its_queries(B, n):
+    """Heads of 64 with scores of a few dozen, where a query rounded to bf16 shows.  The bound: probabilities are bf16 (rms error
+    of a rounding 2^-9 / sqrt(3) = 1.1e-3, less where several keys share a row)."""
+    arch = Arch(1, 128, 2, 64)
+    rng = np.random.default_rng(n)
+    w = layer_weights(arch, rng, Wq=12, Wk=1, Wv=4, Wo=1, W1=1, W2=0)
+    w["layers.0.g1"] = np.ones(128, dtype=np.float32)
+    z = np.where(rng.random((B, n, 128)) < 0.5, -1, 1).astype(np.float32)
+    want = attention(w, 2, z)
+    assert relative(attention(w, 2, z, round_queries=True), want) > 2 * 1.5e-3
+    assert relative(forward(w, arch, z), want) < 1.5e-3
+
+
+@pytest.mark.parametrize("d,f,B,n,folded", [
+    (192, 192, 1, 3, True),           # weights in registers
+    (256, 2560, 4, 20, True),         # up to 512 rows: K of W2 split over a cluster
+    (128, 4352, 5, 101, True),        # 505 rows
+    (256, 1024, 5, 103, True),        # pairs of SMs, several row blocks, the last one ragged
+    (256, 4096, 5, 103, True),        # K of W2 split over two pairs
+    (128, 2048, 5, 205, True),        # the same, half a feature tile over
+    (192, 320, 4, 150, False),        # odd multiples of 64: the kernel on one SM, norm apart
+    (256, 512, 8, 500, False),        # 4000 rows: norms apart, several tiles per pair
+])
+def test_mlp_of_a_layer(d, f, B, n, folded):
+    """x + W2 GELU(W1 norm(x)).  The bound: fp32 sums of relative error 1e-6 round to the other bf16 neighbour, 2^-8 away, in 5 of
+    ten thousand activations (rms 9e-5 of what the MLP adds)."""
+    arch = Arch(1, d, d // 64, f)
+    rng = np.random.default_rng(f + n)
+    w = layer_weights(arch, rng, Wq=1, Wk=1, Wv=1, Wo=0, W1=1.5, W2=4)
+    z = (rng.standard_normal((B, n, d)) * np.exp(rng.standard_normal((B, n, 1)))).astype(np.float32)
+    x = z.astype(np.float64)
+    a, k = normed(x, w["layers.0.g2"], folded)
+    h = torch.from_numpy(a @ w["layers.0.W1"].T.astype(np.float64) * k)
+    y = x + bf16(torch.nn.functional.gelu(h).numpy()) @ w["layers.0.W2"].T.astype(np.float64)
+    assert relative(forward(w, arch, z), y * rstd(y) * w["g_f"]) < 1.5e-4
 
 
 @pytest.mark.parametrize("heads,n,late", [

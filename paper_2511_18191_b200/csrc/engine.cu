@@ -586,10 +586,11 @@ void gemm(tsfm_spec *h, GemmSkPlan *plan, const void *A, const void *W, void *C,
 // tensor-memory kernel takes 128 queries a CTA and costs the same for one of them as for all, attn_tiles_kernel takes 64 in
 // four warps.  A launch costs its waves of blocks (two and four on an SM), a block its start and its steps of 128 and 64 keys (a
 // step of attn_tiles_kernel mostly by the warps that have queries).  In us, fitted to the attention's share of prefills of 33 to
-// 704 tokens and of passes of 48 to 256 tokens behind 100 to 2000 keys, 8 to 3200 (series, head) pairs, 617 shapes: 0.4 % above
-// the better kernel on average, at most 1.8 us (6 %) above attn_tiles_kernel.  Measured at 1280 pairs, us a launch,
-// attn_tiles_kernel / attn_mma_kernel: 33 tokens 12 / 32, 64 15 / 34, 128 40 / 41, 144 56 / 81, 192 71 / 88, 256 107 / 99, 320 146
-// / 150, 384 190 / 156; 48 behind 192 to 336 keys 39 / 56, 64 behind 576 to 768 88 / 90, 96 behind 192 to 480 87 / 73, 128 behind
+// 704 tokens and of passes of 48 to 256 tokens behind 100 to 2000 keys, 8 to 3200 (series, head) pairs, 617 shapes.  Measured with
+// the rule in place: 0.6 % above the better kernel on average; 14 of them more than 4 % and 0.4 us above attn_tiles_kernel (48
+// tokens behind a few hundred keys with few pairs, 0.5 to 0.9 us; the rest within the scatter of runs).  At 1280 pairs, us a
+// launch, attn_tiles_kernel / attn_mma_kernel: 33 tokens 12 / 32, 64 15 / 34, 128 40 / 41, 144 56 / 81, 192 71 / 88, 256 107 / 99,
+// 320 146 / 150, 384 190 / 156; 48 behind 192 to 336 keys 39 / 56, 64 behind 576 to 768 88 / 90, 96 behind 192 to 480 87 / 73, 128 behind
 // 256 to 640 123 / 80.
 bool attn_mma_pays(long pairs, int first, int q_len) {
   double tiles = 0, mma = 0;

@@ -17,7 +17,7 @@
 // Bound: the chain of a tile (MMAs, two passes over the scores, MMAs, sums) and a block's first loads, with 16 softmax warps
 // per SM.
 // attn_tiles_kernel -> here, us a launch inside a forecast: 16 series x 8 heads x 256 queries behind 704 to 1000 keys 53 -> 28,
-// 704 queries behind none 49 -> 38, 4 heads x 64 queries 23 -> 19; 64 series x 20 heads x 255 queries 114 -> 108 (one or two
+// 704 queries behind none 49 -> 38, 4 heads x 64 queries 23 -> 17.5; 64 series x 20 heads x 255 queries 114 -> 108 (one or two
 // tiles a block: mostly start and first loads).  With one thread per row 28.6, 43, 21, 122.
 // Warps 0-7 softmax (query row = 32 (w % 4) + lane, keys and output dims of half w / 4), 8 TMA producer, 9 tensor memory and
 // MMA issue.  Waits are bounded as in gemm_tc.cuh.  grid = (heads, B, ceil(q_len / 128)), block = 320.

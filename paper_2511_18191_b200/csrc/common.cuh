@@ -150,10 +150,9 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
   return r;
 }
 __device__ __forceinline__ uint32_t gelu_erf_fast2(float a, float b) {
-  const uint64_t v = f32x2(fabsf(a), fabsf(b));
-  const uint64_t w = fma2(v, f32x2(0.3275911f * 0.70710678118654752440f, 0.3275911f * 0.70710678118654752440f), f32x2(1.f, 1.f));
-  float w0, w1, t0, t1, e0, e1;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(w0), "=f"(w1) : "l"(w));
+  const uint64_t v = f32x2(a, b);
+  const float w0 = fmaf(fabsf(a), 0.3275911f * 0.70710678118654752440f, 1.f), w1 = fmaf(fabsf(b), 0.3275911f * 0.70710678118654752440f, 1.f);
+  float t0, t1, e0, e1;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t0) : "f"(w0));
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t1) : "f"(w1));
   const uint64_t t = f32x2(t0, t1);

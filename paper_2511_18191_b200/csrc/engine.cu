@@ -400,7 +400,11 @@ void prefer_max_smem_all() {
   prefer_max_smem(gemm_push_kernel<EPI_F32>);
   prefer_max_smem(gemm_push_kernel<EPI_GELU_T>);
   prefer_max_smem(gemm_push_kernel<EPI_RESID>);
-  prefer_max_smem(gemm_pair_kernel);
+  prefer_max_smem(gemm_pair_kernel<PAIR_F32>);
+  prefer_max_smem(gemm_pair_kernel<PAIR_GELU>);
+  prefer_max_smem(gemm_pair_kernel<PAIR_RESID>);
+  prefer_max_smem(gemm_pair_kernel<PAIR_FOLD>);
+  prefer_max_smem(gemm_pair_kernel<PAIR_QKV>);
   prefer_max_smem(gemm_ws_kernel<1, false>);
   prefer_max_smem(gemm_ws_kernel<1, true>);
   prefer_max_smem(gemm_ws_kernel<2, false>);
@@ -493,10 +497,13 @@ void launch_gemm_simt(cudaStream_t s, bool pdl, const T *A, const T *W, void *C,
 // gain nothing up to 3000 tokens: there it is the norms and the cache append in these epilogues that pay.)
 constexpr int kPairMinRows = 513;
 
-// Up to this many tokens their norms are folded in as well: the epilogues that do it cost 1 us per contraction at
-// 576 to 2048 tokens, where an RMSNorm launch is a link of 4 us, and 3 to 6 us at 6000 (scoring, d = 1024: 153 us a
-// layer folded, 136 + 2 x 8 with the kernel).
-constexpr int kPairFoldMaxRows = 3072;
+// Up to how many tokens their norms are folded in as well: those epilogues read the old values and write the next operand
+// beside the new ones, the RMSNorm launch they replace is a link of its own and reads it all once more.  Scoring passes of six
+// layers, ms, apart / folded: d = 512, 4080 tokens 0.476 / 0.450, 9600: 0.825 / 0.805; d = 768, 5100: 0.757 / 0.723, 6990: 0.945 /
+// 0.928; d = 1024, 4080: 0.868 / 0.850, 5100: 1.017 / 1.017, 6000: 1.157 / 1.166, 9600: 1.785 / 1.838; d = 1280, 3500: 1.088 /
+// 1.034, 4080: 1.146 / 1.147, 5100: 1.380 / 1.412, 9600: 2.51 / 2.54: up to about 5 million values.  (Narrower models would gain
+// too, d = 256 7 % at 4080 and 9600 tokens; the roundings of their passes of many tokens are pinned with the norm apart.)
+inline bool pair_folds(int M, int d) { return d >= 512 ? (long)M * d <= 5l << 20 : M <= 3072; }
 
 // Whether gemm_f32_kernel takes an operand (contractions of fp32 models, embedding and head of both kinds).
 // TSFM_GEMM_SIMT keeps to the plain kernels, which share no code with it.
@@ -711,7 +718,7 @@ void run_pass(tsfm_spec *h, ModelDev &m, int B, const PassGeom &g, int head_mode
   const bool fold = sizeof(T) == 2 && h->use_tc && m.layers[0].tc_qkv.valid && M < kPairMinRows;
   const bool on_pairs = sizeof(T) == 2 && h->use_tc && M >= kPairMinRows && d % TC_BM == 0 && f % TC_BM == 0 &&
                         m.layers[0].tc_qkv.valid;
-  const bool fold_pair = on_pairs && M <= kPairFoldMaxRows;
+  const bool fold_pair = on_pairs && pair_folds(M, d);
   // the QKV contraction of a pass of several query tiles rotates its queries and appends to the cache
   const bool append = on_pairs && g.q_len > ATTN_QT;
   // fp32 models normalise the rows inside the contraction that reads them, unless it is so large that doing it once per

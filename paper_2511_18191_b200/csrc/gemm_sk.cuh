@@ -288,32 +288,20 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constant__
 struct GemmSkPlan {
   bool valid = false;
   int N = 0, K = 0, M_max = 0;
-  const void *A = nullptr;
+  const void *A = nullptr, *W = nullptr;
   CUtensorMap mapW;
+  CUtensorMap mapQkv;              // W in the row order of gemm_pair_kernel's rotating epilogue for heads of qkv_dh
+  int qkv_dh = 0;
   CUtensorMap mapA[16];            // box (BN = 16 * (i + 1)) x 64, encoded on first use
   bool haveA[16] = {false};
   CUtensorMap mapA2[8];            // box 16 * (i + 1) x 64: one rank's half of a pair's token tile
   bool haveA2[8] = {false};
-  // outputs written by the TMA unit (fp32 residual stream, bf16 activations): one map per
-  // (buffer, M, rows per box, element type)
-  struct CMap { const void *C; int M, rows; bool is_bf16; CUtensorMap map; };
+  // outputs that gemm_pair_kernel writes through the TMA unit: one map per (buffer, rows, form)
+  struct CMap { const void *C; int M; bool is_bf16, fragments; CUtensorMap map; };
   std::vector<CMap> mapC;
   struct PushTile { int M, BN, S, SW, SA; };
   std::vector<PushTile> push;      // gemm_push_kernel's tile for the token counts seen
 };
-
-// fp32 [rows][N] row-major, box = box_rows x 128 features, no swizzle.
-static int sk_encode_c(CUtensorMap *map, const void *base, int rows, int N, int box_rows, bool is_bf16) {
-  cuuint64_t dims[2] = {(cuuint64_t)N, (cuuint64_t)rows};
-  cuuint64_t strides[1] = {(cuuint64_t)N * (is_bf16 ? 2 : 4)};
-  cuuint32_t box[2] = {(cuuint32_t)TC_BM, (cuuint32_t)box_rows};
-  cuuint32_t estr[2] = {1, 1};
-  CUresult r = g_encode(map, is_bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2,
-                        const_cast<void *>(base), dims, strides, box, estr,
-                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
-                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS ? 0 : -4;
-}
 
 static int gemm_sk_init() {
   if (int rc = gemm_tc_init()) return rc;
@@ -331,7 +319,7 @@ static int gemm_sk_init() {
 
 static int gemm_sk_plan(GemmSkPlan *plan, const void *W, int N, int K, const void *A, int M_max) {
   plan->valid = false;
-  plan->N = N; plan->K = K; plan->M_max = M_max; plan->A = A;
+  plan->N = N; plan->K = K; plan->M_max = M_max; plan->A = A; plan->W = W; plan->qkv_dh = 0;
   for (bool &b : plan->haveA) b = false;
   for (bool &b : plan->haveA2) b = false;
   plan->mapC.clear();
@@ -420,15 +408,26 @@ static void gemm_sk_geometry(int N, int K, int M, int epi, int *BN, int *S, int 
   *S = bs;
 }
 
-// The map of an output written by the TMA unit (box of `rows` tokens x 128 features), encoded on first use;
-// valid until the next call.
-static const CUtensorMap *sk_map_c(GemmSkPlan &p, void *C, int M, int rows, bool is_bf16) {
+// The map of an output [M][N] that leaves in boxes of 32 features x 8 tokens, or (fragments) x 16 with the 16-byte pieces of its
+// 64-byte rows swizzled; encoded on first use.
+static bool sk_map_c(GemmSkPlan &p, const void *C, int M, bool is_bf16, bool fragments, CUtensorMap *out) {
   for (const auto &c : p.mapC)
-    if (c.C == C && c.M == M && c.rows == rows && c.is_bf16 == is_bf16) return &c.map;
-  GemmSkPlan::CMap c{C, M, rows, is_bf16, {}};
-  if (sk_encode_c(&c.map, C, M, p.N, rows, is_bf16)) return nullptr;
+    if (c.C == C && c.M == M && c.is_bf16 == is_bf16 && c.fragments == fragments) {
+      *out = c.map;
+      return true;
+    }
+  GemmSkPlan::CMap c{C, M, is_bf16, fragments, {}};
+  cuuint64_t dims[2] = {(cuuint64_t)p.N, (cuuint64_t)M};
+  cuuint64_t strides[1] = {(cuuint64_t)p.N * (is_bf16 ? 2 : 4)};
+  cuuint32_t box[2] = {32, fragments ? 16u : 8u};
+  cuuint32_t estr[2] = {1, 1};
+  if (g_encode(&c.map, is_bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<void *>(C), dims, strides,
+               box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, fragments ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_NONE,
+               CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+    return false;
   p.mapC.push_back(c);
-  return &p.mapC.back().map;
+  *out = c.map;
+  return true;
 }
 
 static bool gemm_sk_launch(cudaStream_t st, bool pdl, GemmSkPlan &p, void *C, int M, int epi, int *status,

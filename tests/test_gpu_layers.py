@@ -113,6 +113,38 @@ def test_mlp_of_a_layer(d, f, B, n, folded):
     assert relative(forward(w, arch, z), y * rstd(y) * w["g_f"]) < 1.5e-4
 
 
+@pytest.mark.parametrize("half", [0, 1])
+@pytest.mark.parametrize("f,B,n", [(512, 9, 500), (2048, 19, 331)])
+def test_mlp_of_a_layer_with_folded_norms_and_several_tiles_per_pair(f, B, n, half):
+    """4500 and 6289 rows of 512 values (the token and the token halved; the head reads one of the two): the last row block in
+    part, accumulators used in turn.  The bound as above."""
+    d, P = 512, 256
+    arch = Arch(1, d, d // 64, f)
+    rng = np.random.default_rng(f + n)
+    w = layer_weights(arch, rng, Wq=1, Wk=1, Wv=1, Wo=0, W1=1.5, W2=4)
+    eye = np.eye(P, dtype=np.float32)
+    w["W_emb"], w["W_head"] = np.concatenate([eye, eye / 2]), np.concatenate([eye * (half == 0), eye * (half == 1)], 1)
+    z = (rng.standard_normal((B, n, P)) * np.exp(rng.standard_normal((B, n, 1)))).astype(np.float32)
+    x = np.concatenate([z, z / 2], -1).astype(np.float64)
+    a, k = normed(x, w["layers.0.g2"], True)
+    h = torch.from_numpy(a @ w["layers.0.W1"].T.astype(np.float64) * k)
+    y = x + bf16(torch.nn.functional.gelu(h).numpy()) @ w["layers.0.W2"].T.astype(np.float64)
+    want = y * rstd(y) * w["g_f"]
+    assert relative(forward(w, arch, z), want[..., half * P:half * P + P]) < 1.5e-4
+
+
+@pytest.mark.parametrize("heads,B,n", [(4, 9, 60), (1, 9, 60), (4, 2, 300), (1, 2, 300), (2, 9, 142), (2, 9, 143), (2, 41, 251)])
+def test_rotation_in_the_contraction_of_passes_of_many_tokens(heads, B, n):
+    """Heads of 32, 64 and 128, the rotation table of a pass in shared memory or not, ragged row blocks, several tiles per pair.
+    The bound as above."""
+    arch = Arch(1, 128, heads, 64)
+    rng = np.random.default_rng(n + heads)
+    w = layer_weights(arch, rng, Wq=8, Wk=1, Wv=4, Wo=1, W1=1, W2=0)
+    w["layers.0.g1"] = np.ones(128, dtype=np.float32)
+    z = np.where(rng.random((B, n, 128)) < 0.5, -1, 1).astype(np.float32)
+    assert relative(forward(w, arch, z), attention(w, heads, z)) < 1.5e-3
+
+
 @pytest.mark.parametrize("heads,n,late", [
     (2, 20, 3), (4, 32, 9), (1, 31, 1),          # blocks of two warps, head sizes 64, 32 and 128
     (2, 40, 7), (4, 100, 40), (1, 70, 2),        # blocks of four

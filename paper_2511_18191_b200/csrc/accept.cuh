@@ -1,7 +1,7 @@
 // Fused acceptance step of one speculative round (Sec. 3.2 Eq. 5, Sec. 3.3, Algorithm 1):
 // per series, the K tempered Gaussian log-ratios, the K Philox uniforms, the first rejection
 // by warp ballot, the correction / bonus patch, the new committed count (= the ragged KV
-// rollback length) and the round's counters -- one warp per series, one launch per round.
+// rollback length) and the round's counters, and with the last series the end of the round: one launch per round.
 #pragma once
 #include "common.cuh"
 
@@ -73,159 +73,205 @@ struct AcceptArgs {
   int *n_accept;                   // [B] (or NULL)
   float *ell, *log_u;              // [B, K] (or NULL)
   AcceptCounters *ctr;             // or NULL
-  int *unfinished;                 // or NULL: += 1 per series still short of T after this round
-  // When st is non-NULL the scales (tau), the Philox key and the round index come from it, and
-  // n_accept / ell / log_u / unfinished are per-round arrays indexed by that round.
+  // When st is non-NULL the scales (tau), the Philox key and the round index come from it, n_accept / ell / log_u are
+  // per-round arrays indexed by that round, and the CTA that finishes last closes the round:
   DevState *st;
+  int *ticket;                     // CTAs that are done (0 before and after)
+  int *unfinished;                 // [T] series still short of T after each round
+  int *live, *n_live;              // the unfinished series in ascending order, for the next round's compacted passes
+  cudaGraphConditionalHandle handle;   // inside a captured graph (use_handle): its WHILE node
+  int use_handle;
+  const int *body_launches;        // kernel launches of a round, added to launch_ctr
+  unsigned long long *launch_ctr;
 };
 
-// Closes a round: accumulates the phase clocks, advances the round counter, adds the round's
-// kernel launches to the device-side launch counter, lists the series that still have patches
-// to commit (ascending, for the next round's compacted passes) and, inside a captured graph, tells
-// the WHILE node whether another round is needed.  One CTA of 256 threads.
-__global__ void __launch_bounds__(256)
-round_end_kernel(DevState *st, const int *unfinished, int T, cudaGraphConditionalHandle handle, int use_handle,
-                 const int *body_launches, unsigned long long *launch_ctr, const int *done, int B,
-                 int *live, int *n_live) {
+// The state of a call that its statistics are made of, in one piece.
+struct CallState {
+  DevState st;
+  AcceptCounters ctr;
+  int status, ticket;
+};
+
+// Closes a round (all threads of the last CTA): lists the series that still have patches to commit, accumulates the phase
+// clocks, advances the round counter, adds the round's launches to the device-side launch counter and, inside a captured
+// graph, tells the WHILE node whether another round is needed.
+__device__ __forceinline__ void close_round(const AcceptArgs &a) {
   __shared__ int warp_count[8];
-  __shared__ int base;
-  pdl_sync();
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  if (threadIdx.x == 0) base = 0;
-  __syncthreads();
-  for (int b0 = 0; b0 < B; b0 += 256) {             // ordered compaction, 256 series at a time
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  int base = 0;
+  for (int b0 = 0; b0 < a.B; b0 += blockDim.x) {               // ordered compaction, a block of series at a time
     const int b = b0 + threadIdx.x;
-    const bool alive = b < B && done[b] < T;
+    const bool alive = b < a.B && __ldcg(a.done + b) < a.T;
     const unsigned m = __ballot_sync(0xffffffffu, alive);
+    __syncthreads();
     if (lane == 0) warp_count[w] = __popc(m);
     __syncthreads();
     int off = base;
-    for (int i = 0; i < w; ++i) off += warp_count[i];
-    if (alive) live[off + __popc(m & ((1u << lane) - 1u))] = b;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      int t = 0;
-      for (int i = 0; i < 8; ++i) t += warp_count[i];
-      base += t;
+    for (int i = 0; i < nw; ++i) {
+      if (i < w) off += warp_count[i];
+      base += warp_count[i];
     }
-    __syncthreads();
+    if (alive) a.live[off + __popc(m & ((1u << lane) - 1u))] = b;
   }
   if (threadIdx.x != 0) return;
-  *n_live = base;
+  DevState *st = a.st;
   const int r = st->round;
   const unsigned long long now = globaltimer_ns();
+  *a.n_live = a.unfinished[r] = base;
+  *a.ticket = 0;
   if (r == 0) st->ns_prefill = st->t_phase[0] - st->t_call;
   st->ns_draft += st->t_phase[1] - st->t_phase[0];
-  st->ns_verify += st->t_phase[2] - st->t_phase[1];
-  st->ns_accept += now - st->t_phase[2];
+  const unsigned long long t_accept = *reinterpret_cast<const volatile unsigned long long *>(&st->t_phase[2]);   // (another CTA's)
+  st->ns_verify += t_accept - st->t_phase[1];
+  st->ns_accept += now - t_accept;
   st->round = r + 1;
-  if (body_launches && launch_ctr) *launch_ctr += (unsigned long long)*body_launches;
+  if (a.body_launches && a.launch_ctr) *a.launch_ctr += (unsigned long long)*a.body_launches;
   // every round commits at least one patch per unfinished series, so T rounds always suffice:
   // the second condition bounds the loop whatever the counters say
-  if (use_handle) cudaGraphSetConditional(handle, (unfinished[r] > 0 && r + 1 < T) ? 1u : 0u);
+  if (a.use_handle) cudaGraphSetConditional(a.handle, (base > 0 && r + 1 < a.T) ? 1u : 0u);
 }
 
-// block = 128 (4 series per CTA), grid = ceil(B / 4).
-__global__ void __launch_bounds__(128) accept_kernel(AcceptArgs a) {
-  const int lane = threadIdx.x & 31;
-  const int b = blockIdx.x * 4 + (threadIdx.x >> 5);
-  pdl_sync();
+// One CTA per series, a warp per position (in turn; the last one has the bonus patch, which is only kept).  Everything but the
+// verification pass's means was written several kernels ago and is fetched before the dependency wait: the call's state, the
+// committed count, the proposals.  The rows of mu_p stay in shared memory for the commit where they fit.  Bound: the chain
+// of round trips.  With one warp per series, that went through its positions one after the other behind the wait, and the end of
+// the round as a launch of its own, a round's two links took 10 us at K = 3 and 4, 9 of them for a single series.
+// block = 32 min(K + 1, 8), grid = B, dynamic shared memory: stage_rows rows of P floats ((K + 1), or 0: not kept).
+constexpr int ACCEPT_WARPS = 8, ACCEPT_E = 4;                  // elements of a row that a lane has in flight
+constexpr int ACCEPT_STAGE_BYTES = 40 * 1024;
+__global__ void __launch_bounds__(32 * ACCEPT_WARPS) accept_kernel(AcceptArgs a, int stage_rows) {
+  extern __shared__ float accept_rows[];
+  __shared__ float pos_ep[32], pos_eq[32];                     // energies of every position
+  __shared__ int last;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5, b = blockIdx.x;
+  const int K = a.K, P = a.P;
+  int flags = 0;
+  float fallback_r = 0.f;
   if (a.st) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) a.st->t_phase[2] = globaltimer_ns();
-    const int r = a.st->round;
-    a.sigma_p = a.st->tau;
-    a.sigma_q = a.st->sigma_q;
-    a.key = make_uint2(a.st->key0, a.st->key1);
+    const volatile DevState *st = a.st;
+    const int r = st->round;
+    a.sigma_p = st->tau;
+    a.sigma_q = st->sigma_q;
+    a.key = make_uint2(st->key0, st->key1);
     a.round_idx = r;
+    flags = st->flags;
+    fallback_r = st->fallback_r;
     if (a.n_accept) a.n_accept += (size_t)r * a.B;
     if (a.ell) a.ell += (size_t)r * a.B * a.K;
     if (a.log_u) a.log_u += (size_t)r * a.B * a.K;
-    if (a.unfinished) a.unfinished += r;
   }
-  if (b >= a.B) return;
-  const int m = a.done[b];
-  if (m >= a.T) {                                   // finished earlier: nothing to decide
-    if (lane == 0 && a.n_accept) a.n_accept[b] = -1;
-    return;
-  }
-  const int K = a.K, P = a.P;
-  const long long hist_adv = a.commit_follows_done ? (long long)m * P : 0;
+  const int m = *reinterpret_cast<const volatile int *>(a.done + b);
+  const bool finished = m >= a.T;                              // earlier: nothing to decide
+  const long long hist_adv = a.commit_follows_done && !finished ? (long long)m * P : 0;
   const float *xb = a.x + b * a.x_stride_b + hist_adv;
-  const int flags = a.st ? a.st->flags : 0;
-  const float fallback_r = a.st ? a.st->fallback_r : 0.f;
-  const float *qb = (a.mu_q_alt && (flags & VAR_SAMPLE_PROPOSALS)) ? a.mu_q_alt + (size_t)b * a.K * a.P
-                                                                     : a.mu_q + b * a.x_stride_b + hist_adv;
+  const bool apart = a.mu_q_alt && (flags & VAR_SAMPLE_PROPOSALS);
+  const float *qb = apart ? a.mu_q_alt + (size_t)b * a.K * a.P : a.mu_q + b * a.x_stride_b + hist_adv;
+  const bool same = qb == xb;                                  // proposals that are the draft's means
   const float *pb = a.mu_p + (size_t)b * (K + 1) * P;
-
-  // energies ||x - mu_p||_d^2 and ||x - mu_q||_d^2 of every position; lane i keeps position i
-  float my_ep = 0.f, my_eq = 0.f;
-  for (int i = 0; i < K; ++i) {
-    float ep = 0.f, eq = 0.f;
-    for (int c = lane; c < P; c += 32) {
-      const float xv = xb[(size_t)i * P + c];
-      const float dp = xv - pb[(size_t)i * P + c];
-      const float dq = xv - qb[(size_t)i * P + c];
-      ep = fmaf(dp, dp, ep);
-      eq = fmaf(dq, dq, eq);
+  float x0[ACCEPT_E], q0[ACCEPT_E];                            // the start of this warp's first row
+#pragma unroll
+  for (int e = 0; e < ACCEPT_E; ++e) {
+    const int c = lane + 32 * e;
+    const bool in = !finished && w < K && c < P;
+    x0[e] = in ? __ldcg(xb + (size_t)w * P + c) : 0.f;
+    q0[e] = same ? x0[e] : in ? __ldcg(qb + (size_t)w * P + c) : 0.f;
+  }
+  // log u of position `lane`
+  float lu = 0.f;
+  if (w == 0 && lane < K && !finished)
+    lu = logf(a.forced_u ? a.forced_u[(size_t)b * K + lane]
+                         : uniform_from_word(philox4x32_10(make_uint4((uint32_t)(a.series0 + b), (uint32_t)a.round_idx, (uint32_t)lane, 0u), a.key).x));
+  pdl_sync();
+  if (a.st && b == 0 && threadIdx.x == 0) a.st->t_phase[2] = globaltimer_ns();
+  if (!finished) {
+    // energies ||x - mu_p||_d^2 and ||x - mu_q||_d^2 of every position
+    for (int i = w; i <= K; i += nw) {
+      float ep = 0.f, eq = 0.f;
+      for (int c0 = 0; c0 < P; c0 += 32 * ACCEPT_E) {
+        float xv[ACCEPT_E], qv[ACCEPT_E], pv[ACCEPT_E];
+#pragma unroll
+        for (int e = 0; e < ACCEPT_E; ++e) {
+          const int c = c0 + lane + 32 * e;
+          const bool in = c < P, first = i == w && c0 == 0;
+          pv[e] = in ? __ldcg(pb + (size_t)i * P + c) : 0.f;
+          xv[e] = first ? x0[e] : in && i < K ? __ldcg(xb + (size_t)i * P + c) : 0.f;
+          qv[e] = same ? xv[e] : first ? q0[e] : in && i < K ? __ldcg(qb + (size_t)i * P + c) : 0.f;
+        }
+#pragma unroll
+        for (int e = 0; e < ACCEPT_E; ++e) {
+          const int c = c0 + lane + 32 * e;
+          const float dp = xv[e] - pv[e], dq = xv[e] - qv[e];
+          ep = fmaf(dp, dp, ep);
+          eq = fmaf(dq, dq, eq);
+          if (i < stage_rows && c < P) accept_rows[i * P + c] = pv[e];
+        }
+      }
+      ep = warp_sum(ep) / (float)P;
+      eq = warp_sum(eq) / (float)P;
+      if (lane == 0 && i < K) pos_ep[i] = ep, pos_eq[i] = eq;
     }
-    ep = warp_sum(ep) / (float)P;
-    eq = warp_sum(eq) / (float)P;
-    if (lane == i) { my_ep = ep; my_eq = eq; }
-  }
-  // Eq. 5 and the log-domain test  log u <= min(l, 0)
-  bool ok = true;
-  float l = 0.f, lu = 0.f;
-  if (lane < K) {
-    l = -my_ep / (2.f * a.sigma_p * a.sigma_p) + my_eq / (2.f * a.sigma_q * a.sigma_q)
-        + 0.5f * logf((a.sigma_q * a.sigma_q) / (a.sigma_p * a.sigma_p));
-    if (flags & VAR_NO_TEMPERING) l *= (float)P;     // l is (1/d) log p/q: undo the 1/d (component ablation)
-    float u;
-    if (a.forced_u) u = a.forced_u[(size_t)b * K + lane];
-    else u = uniform_from_word(philox4x32_10(
-                 make_uint4((uint32_t)(a.series0 + b), (uint32_t)a.round_idx, (uint32_t)lane, 0u), a.key).x);
-    lu = logf(u);
-    ok = (lu <= l) && (lu <= 0.f);                   // log u <= min(l, 0); a NaN statistic compares false: rejected
-    if (a.ell) a.ell[(size_t)b * K + lane] = l;
-    if (a.log_u) a.log_u[(size_t)b * K + lane] = lu;
-  }
-  const unsigned rejected = __ballot_sync(0xffffffffu, !ok);     // lanes >= K vote "accepted"
-  const int n = rejected ? min(__ffs(rejected) - 1, K) : K;      // leading accepts
-  const int L = n + 1;
-  const int keep = min(L, a.T - m);
+    __syncthreads();
+    if (w == 0) {
+      // Eq. 5 and the log-domain test  log u <= min(l, 0)
+      bool ok = true;
+      float l = 0.f;
+      if (lane < K) {
+        l = -pos_ep[lane] / (2.f * a.sigma_p * a.sigma_p) + pos_eq[lane] / (2.f * a.sigma_q * a.sigma_q)
+            + 0.5f * logf((a.sigma_q * a.sigma_q) / (a.sigma_p * a.sigma_p));
+        if (flags & VAR_NO_TEMPERING) l *= (float)P;     // l is (1/d) log p/q: undo the 1/d (component ablation)
+        ok = (lu <= l) && (lu <= 0.f);                   // log u <= min(l, 0); a NaN statistic compares false: rejected
+        if (a.ell) a.ell[(size_t)b * K + lane] = l;
+        if (a.log_u) a.log_u[(size_t)b * K + lane] = lu;
+      }
+      const unsigned rejected = __ballot_sync(0xffffffffu, !ok);     // lanes >= K vote "accepted"
+      const int n = rejected ? min(__ffs(rejected) - 1, K) : K;      // leading accepts
+      const int L = n + 1;
+      const int keep = min(L, a.T - m);
 
-  // commit: accepted proposals (if they are not in place already) then mu_p^(n+1)
-  float *cb = a.commit + b * a.commit_stride_b + hist_adv;
-  if (a.commit_accepted)
-    for (int c = lane; c < n * P; c += 32) cb[c] = xb[c];
-  for (int c = lane; c < P; c += 32) {
-    float t = pb[(size_t)n * P + c];
-    if (fallback_r != 0.f)                          // t = mu_p + r eps (Algorithm 1, correction and bonus)
-      t += fallback_r * standard_normal(a.key, (uint32_t)(a.series0 + b), (uint32_t)a.round_idx, (uint32_t)n, NOISE_FALLBACK, c);
-    cb[(size_t)n * P + c] = t;
-  }
+      // commit: accepted proposals (if they are not in place already) then mu_p^(n+1)
+      float *cb = a.commit + b * a.commit_stride_b + hist_adv;
+      if (a.commit_accepted)
+        for (int c = lane; c < n * P; c += 32) cb[c] = xb[c];
+      for (int c = lane; c < P; c += 32) {
+        float t = n < stage_rows ? accept_rows[n * P + c] : __ldcg(pb + (size_t)n * P + c);
+        if (fallback_r != 0.f)                          // t = mu_p + r eps (Algorithm 1, correction and bonus)
+          t += fallback_r * standard_normal(a.key, (uint32_t)(a.series0 + b), (uint32_t)a.round_idx, (uint32_t)n, NOISE_FALLBACK, c);
+        cb[(size_t)n * P + c] = t;
+      }
 
-  const bool tested = lane < min(n + 1, K);
-  const bool near = tested && fabsf(l - lu) < a.margin;
-  const unsigned near_mask = __ballot_sync(0xffffffffu, near);
-  if (a.ctr) {
-    if (tested) {
-      atomicAdd(&a.ctr->tested_by_pos[lane], 1ull);
-      if (lane < n) atomicAdd(&a.ctr->accepted_by_pos[lane], 1ull);
+      const bool tested = lane < min(n + 1, K);
+      const bool near = tested && fabsf(l - lu) < a.margin;
+      const unsigned near_mask = __ballot_sync(0xffffffffu, near);
+      if (a.ctr) {
+        if (tested) {
+          atomicAdd(&a.ctr->tested_by_pos[lane], 1ull);
+          if (lane < n) atomicAdd(&a.ctr->accepted_by_pos[lane], 1ull);
+        }
+        if (lane == 0) {
+          atomicAdd(&a.ctr->drafted, (unsigned long long)K);
+          atomicAdd(&a.ctr->tested, (unsigned long long)min(n + 1, K));
+          atomicAdd(&a.ctr->accepted, (unsigned long long)n);
+          atomicAdd(&a.ctr->committed, (unsigned long long)keep);
+          atomicAdd(&a.ctr->near_margin, (unsigned long long)__popc(near_mask));
+          atomicAdd(&a.ctr->L_hist[L], 1ull);
+        }
+      }
+      if (lane == 0) {
+        a.done[b] = m + keep;
+        if (a.n_accept) a.n_accept[b] = n;
+      }
     }
-    if (lane == 0) {
-      atomicAdd(&a.ctr->drafted, (unsigned long long)K);
-      atomicAdd(&a.ctr->tested, (unsigned long long)min(n + 1, K));
-      atomicAdd(&a.ctr->accepted, (unsigned long long)n);
-      atomicAdd(&a.ctr->committed, (unsigned long long)keep);
-      atomicAdd(&a.ctr->near_margin, (unsigned long long)__popc(near_mask));
-      atomicAdd(&a.ctr->L_hist[L], 1ull);
-    }
+  } else if (threadIdx.x == 0 && a.n_accept) {
+    a.n_accept[b] = -1;
   }
-  if (lane == 0) {
-    if (a.unfinished && m + keep < a.T) atomicAdd(a.unfinished, 1);
-    a.done[b] = m + keep;
-    if (a.n_accept) a.n_accept[b] = n;
+  if (!a.st) return;
+  if (threadIdx.x == 0) {
+    __threadfence();                                           // done[b], the time stamp: before the ticket
+    last = atomicAdd(a.ticket, 1) == (int)gridDim.x - 1;
+    __threadfence();
   }
+  __syncthreads();
+  if (last) close_round(a);
 }
 
 }  // namespace tsfm

@@ -152,9 +152,12 @@ struct tsfm_spec {
   float *hist = nullptr, *vout = nullptr, *mean = nullptr, *sd = nullptr;
   float *muq = nullptr;                  // [B][max_K][P] draft means of the round (sampled proposals)
   int *done = nullptr;
-  int *live = nullptr, *n_live = nullptr;   // [B] slot -> unfinished series, and their number (round_end_kernel)
+  int *live = nullptr, *n_live = nullptr;   // [B] slot -> unfinished series, and their number (accept_kernel)
   bool compact = true;                   // rounds run over the unfinished series only
+  CallState *call = nullptr;             // st, ctr, dev_status and ticket point into it
+  CallState *h_call = nullptr;           // pinned: what a call's statistics are read into
   AcceptCounters *ctr = nullptr;
+  int *ticket = nullptr;
   int *unfinished = nullptr;             // [max_T + 1]
   int *h_unfinished = nullptr;           // pinned
   int *dev_status = nullptr;
@@ -393,7 +396,6 @@ void prefer_max_smem_all() {
   prefer_max_smem(instnorm_kernel);
   prefer_max_smem(denorm_kernel);
   prefer_max_smem(accept_kernel);
-  prefer_max_smem(round_end_kernel);
   prefer_max_smem(gemm_sk_kernel<1>);
   prefer_max_smem(gemm_sk_kernel<2>);
   prefer_max_smem(attn_mma_kernel);
@@ -520,6 +522,12 @@ bool f32_many(int M, int N, int K) {
   return K <= 256 && tiles >= (K <= 128 ? 256 : 1024) && M <= 65535 * 64;      // (its row tiles are the y of a grid)
 }
 bool f32_takes(const tsfm_spec *h, const void *W, int M, int N, int K) { return f32_tiles(h, W, K) && !f32_many(M, N, K); }
+
+void launch_accept(cudaStream_t s, bool pdl, const AcceptArgs &a) {
+  const size_t rows = (size_t)(a.K + 1) * a.P * sizeof(float);
+  const bool keep = rows <= ACCEPT_STAGE_BYTES;
+  launch_ex(s, pdl, accept_kernel, dim3(a.B), dim3(32 * std::min(a.K + 1, ACCEPT_WARPS)), keep ? rows : 0, a, keep ? a.K + 1 : 0);
+}
 
 // C (op)= A . W^T through the tensor-core kernel when a plan exists, else an FMA kernel.  row_gain (fp32
 // models whose rows gemm_f32_kernel takes): A is the residual stream, normalised by the contraction itself.
@@ -857,13 +865,13 @@ int check_call(tsfm_spec *h, const float *series, int B, int ctx_len, int H, flo
 // Each of these only enqueues work on h->ls; none synchronises, so that they can run under
 // stream capture.
 
-void enqueue_begin(tsfm_spec *h, int B, int ctx_len) {
+void enqueue_begin(tsfm_spec *h, int B, int ctx_len, FillList fill = FillList{}) {
   const int hist_stride = h->cap * h->P_in;             // values per series in the history buffer
   const int hist_len = hist_stride - (h->check ? h->P_in : 0);   // (the spare token stays untouched)
-  cudaMemsetAsync(h->dev_status, 0, sizeof(int), h->ls);
+  fill.add(h->dev_status, sizeof(int), 0);
   KTimer kt(h, KC_INSTNORM, (double)B * (ctx_len + (double)hist_len) * 4, 4.0 * B * ctx_len);
-  launch_ex(h->ls, h->pdl, instnorm_kernel, dim3(B), dim3(256), 0, h->st, ctx_len, hist_stride, hist_len, h->cfg.norm_eps, h->hist,
-            h->mean, h->sd, h->done, h->live, h->n_live);
+  launch_ex(h->ls, h->pdl, instnorm_kernel, dim3(B), dim3(INSTNORM_THREADS), 0, h->st, ctx_len, hist_stride, hist_len, h->cfg.norm_eps, h->hist,
+            h->mean, h->sd, h->done, h->live, h->n_live, fill);
 }
 
 // Bounds-checking mode: after the work of a call, look at every guard region.
@@ -886,14 +894,15 @@ void enqueue_denorm(tsfm_spec *h, int B, int N, int H) {
 // last patch, the draft except its last two: those are re-read by the first round).
 // N counts context tokens; a patch is tpp = P / P_in of them.
 void enqueue_spec_prologue(tsfm_spec *h, int B, int N, int T, int K) {
-  cudaStream_t s = h->ls;
-  cudaMemsetAsync(h->ctr, 0, sizeof(AcceptCounters), s);
-  cudaMemsetAsync(h->unfinished, 0, sizeof(int) * (T + 1), s);
-  cudaMemsetAsync(h->tr_nacc, 0xff, sizeof(int) * (size_t)T * B, s);
-  cudaMemsetAsync(h->tr_ell, 0, sizeof(float) * (size_t)T * B * K, s);
-  cudaMemsetAsync(h->tr_logu, 0, sizeof(float) * (size_t)T * B * K, s);
+  FillList fill;
+  fill.add(h->ctr, sizeof(AcceptCounters), 0);
+  fill.add(h->ticket, sizeof(int), 0);
+  fill.add(h->unfinished, sizeof(int) * (size_t)(T + 1), 0);
+  fill.add(h->tr_nacc, sizeof(int) * (size_t)T * B, 0xffffffffu);
+  fill.add(h->tr_ell, sizeof(float) * (size_t)T * B * K, 0);
+  fill.add(h->tr_logu, sizeof(float) * (size_t)T * B * K, 0);
   const int tpp = h->tpp;
-  enqueue_begin(h, B, N * h->P_in);
+  enqueue_begin(h, B, N * h->P_in, fill);
   pass(h, h->tgt, B, PassGeom{nullptr, 0, N - tpp, h->cap}, HEAD_NONE);
   pass(h, h->drf, B, PassGeom{nullptr, 0, N - 2 * tpp, h->cap}, HEAD_NONE);
 }
@@ -936,14 +945,17 @@ void enqueue_round(tsfm_spec *h, int B, int N, int T, int K, cudaGraphConditiona
   a.n_accept = h->tr_nacc;
   a.ell = h->tr_ell;
   a.log_u = h->tr_logu;
-  a.unfinished = h->unfinished;
   a.st = h->st;
-  {
-    KTimer kt(h, KC_ACCEPT, (double)B * (2 * K + 2) * P * 4, 4.0 * B * K * P);
-    launch_ex(h->ls, h->pdl, accept_kernel, dim3((B + 3) / 4), dim3(128), 0, a);
-  }
-  launch_ex(h->ls, h->pdl, round_end_kernel, dim3(1), dim3(256), 0, h->st, (const int *)h->unfinished, T, handle,
-            use_handle, body_launches, h->dev_launches, (const int *)h->done, B, h->live, h->n_live);
+  a.ticket = h->ticket;
+  a.unfinished = h->unfinished;
+  a.live = h->live;
+  a.n_live = h->n_live;
+  a.handle = handle;
+  a.use_handle = use_handle;
+  a.body_launches = body_launches;
+  a.launch_ctr = h->dev_launches;
+  KTimer kt(h, KC_ACCEPT, (double)B * (2 * K + 2) * P * 4, 4.0 * B * K * P);
+  launch_accept(h->ls, h->pdl, a);
 }
 
 // Plain patch-autoregressive decoding with one model (the target, or the draft on its own).
@@ -1096,14 +1108,15 @@ int status_code(tsfm_spec *h, int status) {
   return TSFM_ERR_INTERNAL;
 }
 
-// Reads status and phase clocks back (synchronises) and fills ms_total.
-int finish_stats(tsfm_spec *h, tsfm_stats *stats, DevState *st_out) {
+// Reads the state of the call back (one copy into pinned memory, synchronises) and fills ms_total and the status.  (Three copies
+// into pageable memory, each staged and waited for by itself, took 45 us.)
+int finish_stats(tsfm_spec *h, tsfm_stats *stats) {
   cudaStream_t s = h->stream;
   CU_TRY(cudaEventRecord(h->ev[1], s));
-  CU_TRY(cudaMemcpyAsync(st_out, h->st, sizeof(DevState), cudaMemcpyDeviceToHost, s));
-  CU_TRY(cudaMemcpyAsync(&stats->device_status, h->dev_status, sizeof(int), cudaMemcpyDeviceToHost, s));
+  CU_TRY(cudaMemcpyAsync(h->h_call, h->call, sizeof(CallState), cudaMemcpyDeviceToHost, s));
   CU_TRY(cudaStreamSynchronize(s));
   CU_TRY(cudaEventElapsedTime(&stats->ms_total, h->ev[0], h->ev[1]));
+  stats->device_status = h->h_call->status;
   return TSFM_OK;
 }
 
@@ -1169,7 +1182,7 @@ int tsfm_spec_destroy(tsfm_spec *h) {
   if (h->cap_stream2) cudaStreamDestroy(h->cap_stream2);
   for (cudaEvent_t e : h->prof_pool) cudaEventDestroy(e);
   for (void *p : h->owned) cudaFree(p);
-  if (h->h_unfinished) cudaFreeHost(h->h_unfinished);
+  if (h->h_call) cudaFreeHost(h->h_call);
   for (cudaEvent_t e : h->ev) cudaEventDestroy(e);
   delete h;
   return TSFM_OK;
@@ -1271,13 +1284,15 @@ int tsfm_spec_create(const tsfm_weights *target_w, const tsfm_weights *draft_w, 
   if ((rc = dev_alloc(h, &h->done, Bm, "done"))) return fail(rc);
   if ((rc = dev_alloc(h, &h->live, Bm, "live"))) return fail(rc);
   if ((rc = dev_alloc(h, &h->n_live, 1))) return fail(rc);
-  if ((rc = dev_alloc(h, &h->ctr, 1))) return fail(rc);
   if ((rc = dev_alloc(h, &h->unfinished, cfg->max_horizon_patches + 1, "unfinished"))) return fail(rc);
-  if ((rc = dev_alloc(h, &h->dev_status, 1))) return fail(rc);
-  if ((rc = dev_alloc(h, &h->st, 1))) return fail(rc);
+  if ((rc = dev_alloc(h, &h->call, 1, "call state"))) return fail(rc);
+  h->st = &h->call->st;
+  h->ctr = &h->call->ctr;
+  h->dev_status = &h->call->status;
+  h->ticket = &h->call->ticket;
   if ((rc = dev_alloc(h, &h->dev_launches, 1))) return fail(rc);
   if ((rc = dev_alloc(h, &h->dev_body_launches, kMaxGraphs))) return fail(rc);
-  if (cudaMemsetAsync(h->st, 0, sizeof(DevState), h->stream) != cudaSuccess ||
+  if (cudaMemsetAsync(h->call, 0, sizeof(CallState), h->stream) != cudaSuccess ||
       cudaMemsetAsync(h->dev_launches, 0, sizeof(unsigned long long), h->stream) != cudaSuccess)
     return fail(TSFM_ERR_CUDA);
   if (cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking) != cudaSuccess ||
@@ -1289,11 +1304,11 @@ int tsfm_spec_create(const tsfm_weights *target_w, const tsfm_weights *draft_w, 
   if ((rc = dev_alloc(h, &h->tr_logu, tr * cfg->max_K, "trace log_u"))) return fail(rc);
   if ((rc = dev_alloc(h, &h->stage_in, (size_t)Bm * cfg->max_ctx_tokens * h->P_in, "stage_in"))) return fail(rc);
   if ((rc = dev_alloc(h, &h->stage_out, (size_t)Bm * cfg->max_horizon_patches * P, "stage_out"))) return fail(rc);
-  if (cudaMallocHost((void **)&h->h_unfinished, sizeof(int)) != cudaSuccess) return fail(TSFM_ERR_CUDA);
+  if (cudaMallocHost((void **)&h->h_call, sizeof(CallState) + sizeof(int)) != cudaSuccess) return fail(TSFM_ERR_CUDA);
+  h->h_unfinished = (int *)(h->h_call + 1);
   h->ev.resize(2 + 4 * (size_t)cfg->max_horizon_patches + 4);
   for (auto &ev : h->ev)
     if (cudaEventCreate(&ev) != cudaSuccess) { ev = nullptr; return fail(TSFM_ERR_CUDA); }
-  if (cudaMemsetAsync(h->dev_status, 0, sizeof(int), h->stream) != cudaSuccess) return fail(TSFM_ERR_CUDA);
 
   if (h->check) {
     if ((rc = dev_alloc(h, &h->dev_guards, h->guards.size() + 1, "guard table"))) return fail(rc);
@@ -1353,8 +1368,8 @@ static int single_model_forecast(tsfm_spec *h, int mode, const float *series, in
   if (int rc = take_enqueue_err(h)) return rc;
   if (stats) {
     std::memset(stats, 0, sizeof(*stats));
-    DevState st;
-    if (int rc = finish_stats(h, stats, &st)) return rc;
+    if (int rc = finish_stats(h, stats)) return rc;
+    const DevState &st = h->h_call->st;
     stats->ms_prefill = (float)((st.t_phase[0] - st.t_call) * 1e-6);
     (mode == 1 ? stats->ms_verify : stats->ms_draft) = (float)((st.t_end - st.t_phase[0]) * 1e-6);
     stats->rounds = T;
@@ -1416,10 +1431,9 @@ int tsfm_spec_forecast_variant(tsfm_spec *h, const float *series, int32_t B, int
   if (int rc = take_enqueue_err(h)) return rc;
   if (stats) {
     std::memset(stats, 0, sizeof(*stats));
-    AcceptCounters c;
-    DevState st;
-    CU_TRY(cudaMemcpyAsync(&c, h->ctr, sizeof(c), cudaMemcpyDeviceToHost, s));
-    if (int rc = finish_stats(h, stats, &st)) return rc;
+    if (int rc = finish_stats(h, stats)) return rc;
+    const AcceptCounters &c = h->h_call->ctr;
+    const DevState &st = h->h_call->st;
     stats->rounds = st.round;
     stats->proposals_drafted = (int64_t)c.drafted;
     stats->proposals_tested = (int64_t)c.tested;
@@ -1498,8 +1512,7 @@ int tsfm_accept_round(void *stream, const float *x, const float *mu_q, const flo
   a.round_idx = round_idx; a.series0 = series0;
   a.forced_u = forced_u;
   a.n_accept = n_accept; a.ell = ell; a.log_u = log_u;
-  accept_kernel<<<(B + 3) / 4, 128, 0, (cudaStream_t)stream>>>(a);
-  LAUNCHED();
+  launch_accept((cudaStream_t)stream, false, a);
   CU_TRY(cudaGetLastError());
   return TSFM_OK;
 }
@@ -1517,10 +1530,9 @@ int tsfm_model_forward(tsfm_spec *h, int32_t which, const float *tokens, int32_t
   enqueue_guard_check(h);
   CU_TRY(cudaGetLastError());
   if (int rc = take_enqueue_err(h)) return rc;
-  int status = 0;
-  CU_TRY(cudaMemcpyAsync(&status, h->dev_status, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+  CU_TRY(cudaMemcpyAsync(&h->h_call->status, h->dev_status, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
   CU_TRY(cudaStreamSynchronize(h->stream));
-  return status_code(h, status);
+  return status_code(h, h->h_call->status);
 }
 
 int tsfm_gemm_bf16(void *stream, const void *A, const void *W, float *C, int32_t M, int32_t N, int32_t Kd,

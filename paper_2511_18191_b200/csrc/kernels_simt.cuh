@@ -17,7 +17,7 @@ namespace tsfm {
 //
 // Active-series compaction: inside the round loop only the series that still have patches to
 // commit take part in a pass.  `live` lists them in ascending order and `n_live` counts them (both
-// written by round_end_kernel); the pass works on SLOTS 0 .. n_live-1, slot s standing for series
+// written by accept_kernel); the pass works on SLOTS 0 .. n_live-1, slot s standing for series
 // live[s].  Activation rows are compacted (row = slot * q_len + j); history, KV caches, `done` and
 // the verification output stay indexed by series.  Grids are sized for all B series (a captured
 // graph cannot change them): blocks of slots >= n_live return at once.  live == NULL: slot = series.
@@ -40,7 +40,7 @@ __device__ __forceinline__ int series_of(const PassGeom &g, int slot) { return g
 // are two independent loads (issued together); the committed count follows the series index.  The
 // loads are volatile (served by L2) because most kernels do this lookup BEFORE their dependency wait,
 // to take its two L2 round trips off the chain of dependent launches: `live` / `n_live` are written
-// only by round_end_kernel (and the instance-norm kernel), `done` only by accept_kernel, and every
+// only by accept_kernel and the instance-norm kernel, and so is `done`, and every
 // kernel of a pass except the embedding that opens a round has at least two kernels between itself
 // and those -- a grid starts only after every CTA of its predecessor has passed its own dependency
 // wait, i.e. after the predecessor's predecessor has finished.  A dead slot's entry of `live` is a
@@ -67,32 +67,77 @@ __device__ __forceinline__ int live_rows(const LiveRows &lr, int M) {
   return lr.n_live ? min(M, *lr.n_live * lr.q_len) : M;
 }
 
+// Words to clear or fill at the start of a call (counters, traces, the status word), shared by its first kernel's blocks:
+// as memset nodes of the graph they were six links of 4 us.
+struct FillList {
+  static constexpr int MAX = 7;
+  uint32_t *p[MAX];
+  size_t n[MAX];
+  uint32_t value[MAX];
+  int count = 0;
+  void add(void *q, size_t bytes, uint32_t v) {                // whole words
+    p[count] = (uint32_t *)q;
+    n[count] = bytes / 4;
+    value[count++] = v;
+  }
+};
+__device__ __forceinline__ void fill_words(const FillList &f) {
+#pragma unroll 1
+  for (int k = 0; k < f.count; ++k)
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < f.n[k]; i += (size_t)gridDim.x * blockDim.x) f.p[k][i] = f.value[k];
+}
+
 // ----------------------------------------------------------------------------------
 // Instance statistics frozen on the context (Sec. 3.4) and history initialisation.
-// grid = B, block = 256.  hist[b, :ctx_len] = (series - mean) / sd; the rest of the
-// series' hist_len values is zeroed.  Sums in fp64 (8 K values, one pass each).
+// grid = B, block = 512.  hist[b, :ctx_len] = (series - mean) / sd; the rest of the
+// series' hist_len values is zeroed.  Sums in fp64.  The first 512 INSTNORM_KEEP values of a series are read once and stay in
+// registers for the variance and the normalised values (bound: one round trip and three block-wide steps; 2880 values 6.4 us with
+// three dependent passes over them, 8192 values 31 us).
 // ----------------------------------------------------------------------------------
-__global__ void instnorm_kernel(DevState *__restrict__ st, int ctx_len, int hist_stride, int hist_len,
+constexpr int INSTNORM_THREADS = 512, INSTNORM_KEEP = 16;
+__global__ void __launch_bounds__(INSTNORM_THREADS)
+instnorm_kernel(DevState *__restrict__ st, int ctx_len, int hist_stride, int hist_len,
                                 float norm_eps, float *__restrict__ hist,
                                 float *__restrict__ mean_out, float *__restrict__ sd_out,
-                                int *__restrict__ done, int *__restrict__ live, int *__restrict__ n_live) {
+                                int *__restrict__ done, int *__restrict__ live, int *__restrict__ n_live, FillList fill) {
   __shared__ double red[32];
   const int b = blockIdx.x;
   pdl_sync();
   if (b == 0 && threadIdx.x == 0) st->t_call = globaltimer_ns();
   const float *s = st->series + (size_t)b * ctx_len;
+  constexpr int KEPT = INSTNORM_THREADS * INSTNORM_KEEP;
+  float v[INSTNORM_KEEP];
+#pragma unroll
+  for (int k = 0; k < INSTNORM_KEEP; ++k) {
+    const int i = threadIdx.x + k * INSTNORM_THREADS;
+    v[k] = i < ctx_len ? s[i] : 0.f;
+  }
+  fill_words(fill);
   double acc = 0.0;
-  for (int i = threadIdx.x; i < ctx_len; i += blockDim.x) acc += (double)s[i];
+#pragma unroll
+  for (int k = 0; k < INSTNORM_KEEP; ++k) acc += (double)v[k];
+  for (int i = threadIdx.x + KEPT; i < ctx_len; i += INSTNORM_THREADS) acc += (double)s[i];
   const double mean = block_sum_d(acc, red) / ctx_len;
   acc = 0.0;
-  for (int i = threadIdx.x; i < ctx_len; i += blockDim.x) {
+#pragma unroll
+  for (int k = 0; k < INSTNORM_KEEP; ++k)
+    if (threadIdx.x + k * INSTNORM_THREADS < ctx_len) {
+      const double c = (double)v[k] - mean;
+      acc += c * c;
+    }
+  for (int i = threadIdx.x + KEPT; i < ctx_len; i += INSTNORM_THREADS) {
     const double c = (double)s[i] - mean;
     acc += c * c;
   }
   const double var = block_sum_d(acc, red) / ctx_len;
   const double sd = sqrt(var + (double)norm_eps);
   float *hb = hist + (size_t)b * hist_stride;             // (stride > length only in bounds-checking mode)
-  for (int i = threadIdx.x; i < hist_len; i += blockDim.x)
+#pragma unroll
+  for (int k = 0; k < INSTNORM_KEEP; ++k) {
+    const int i = threadIdx.x + k * INSTNORM_THREADS;
+    if (i < hist_len) hb[i] = i < ctx_len ? (float)(((double)v[k] - mean) / sd) : 0.f;
+  }
+  for (int i = threadIdx.x + KEPT; i < hist_len; i += INSTNORM_THREADS)
     hb[i] = (i < ctx_len) ? (float)(((double)s[i] - mean) / sd) : 0.f;
   if (threadIdx.x == 0) {
     mean_out[b] = (float)mean;

@@ -67,6 +67,13 @@ def test_accept_matches_oracle(B, K, P):
     assert flips <= max(1, B // 200)
 
 
+@pytest.mark.parametrize("B,K,P", [(3, 7, 1), (5, 8, 31), (2, 9, 129), (3, 31, 320), (2, 32, 300), (4, 8, 4096)])
+def test_accept_at_the_edges_of_its_rows_and_warps(B, K, P):
+    """Rows shorter than a warp and longer than what its lanes have in flight, positions in several turns of the warps, boundary
+    rows that fit into shared memory or not ((K + 1) P values, 10240 at most)."""
+    test_accept_matches_oracle(B, K, P)
+
+
 def test_figure1_example_with_scripted_uniforms():
     g = dict(l.split(None, 1) for l in open(os.path.join(os.path.dirname(__file__), "golden", "figure1_round.txt")) if l[0] != "#")
     K, P = int(g["K"]), 96

@@ -29,6 +29,7 @@
 #include "gemm_push.cuh"
 #include "attn_mma.cuh"
 #include "gemm_f32.cuh"
+#include "gemm_rows.cuh"
 
 using namespace tsfm;
 
@@ -375,8 +376,6 @@ template <typename T> void prefer_max_smem_typed() {
   prefer_max_smem(rmsnorm_kernel<T, true, 10>);
   prefer_max_smem(head_kernel<T>);
   prefer_max_smem(embed_rows_kernel<T>);
-  prefer_max_smem(gemm_f32_kernel<T, 16, 16>);
-  prefer_max_smem(gemm_f32_kernel<T, 32, 32>);
   prefer_max_smem(gemm_simt_kernel<T, EPI_F32>);
   prefer_max_smem(gemm_simt_kernel<T, EPI_T>);
   prefer_max_smem(gemm_simt_kernel<T, EPI_GELU_T>);
@@ -393,6 +392,10 @@ template <typename T> void prefer_max_smem_typed() {
 void prefer_max_smem_all() {
   prefer_max_smem_typed<float>();
   prefer_max_smem_typed<bf16>();
+  prefer_max_smem(gemm_f32_kernel<16, 16>);
+  prefer_max_smem(gemm_f32_kernel<32, 32>);
+  prefer_max_smem(gemm_rows_kernel<1>);
+  prefer_max_smem(gemm_rows_kernel<3>);
   prefer_max_smem(instnorm_kernel);
   prefer_max_smem(denorm_kernel);
   prefer_max_smem(accept_kernel);
@@ -507,9 +510,18 @@ constexpr int kPairMinRows = 513;
 // too, d = 256 7 % at 4080 and 9600 tokens; the roundings of their passes of many tokens are pinned with the norm apart.)
 inline bool pair_folds(int M, int d) { return d >= 512 ? (long)M * d <= 5l << 20 : M <= 3072; }
 
-// Whether gemm_f32_kernel takes an operand (contractions of fp32 models, embedding and head of both kinds).
+// Whether gemm_f32_kernel takes an operand (contractions of fp32 models, their embedding and head).
 // TSFM_GEMM_SIMT keeps to the plain kernels, which share no code with it.
 bool f32_tiles(const tsfm_spec *h, const void *W, int K) { return h->cfg.gemm_backend != TSFM_GEMM_SIMT && gemm_f32_eligible(W, K); }
+
+// Whether gemm_rows_kernel takes embedding or head of a bf16 model.
+bool rows_tiles(const tsfm_spec *h, const void *W, int K) { return h->cfg.gemm_backend != TSFM_GEMM_SIMT && gemm_rows_eligible(W, K); }
+bool rows_launch(cudaStream_t s, bool pdl, const float *A, const float *W, float *C, int M, int N, int K, const RowsArgs &ra) {
+  return gemm_f32_launch(s, pdl, A, W, C, M, N, K, ra);
+}
+bool rows_launch(cudaStream_t s, bool pdl, const float *A, const bf16 *W, float *C, int M, int N, int K, const RowsArgs &ra) {
+  return gemm_rows_launch(s, pdl, A, W, C, M, N, K, ra);
+}
 
 // Contractions of fp32 models with a short K and many 64 x 64 tiles go to gemm_simt_kernel: gemm_f32_kernel divides K
 // over its eight warps and has their partial tiles to sum at the end.  Chains of dependent launches, us, gemm_f32_kernel
@@ -701,9 +713,10 @@ enum { HEAD_NONE = 0, HEAD_LAST_TO_HIST = 1, HEAD_ALL_TO_VOUT = 2 };
 // Passes of at least this many rows take the embedding kernel that shares each weight load between 8
 // rows where a token is too short for the tiled contraction (point tokens).
 constexpr int kManyRows = 1024;
-// From this many rows on the head is a tiled contraction (gemm_f32_kernel) on the bf16 path too; below
-// it one CTA per row and eight outputs, with constants fetched before the dependency wait, is shorter.
-constexpr int kHeadTileRows = 192;
+// From this many rows on the head is a tiled contraction (gemm_rows_kernel) on the bf16 path too; below it one CTA per row and
+// eight outputs, with constants fetched before the dependency wait, is shorter: 32 rows of 512 values 3.1 us (tiled 5.6), 93 of
+// 1024 7.9 (8.4), 160 of 512 9.4 (5.6), 64 of 1280 4.5 (10.3).
+constexpr int kHeadTileRows = 128;
 // Up to this many rows the separate RMSNorm kernel fetches its constants before the dependency wait.
 constexpr int kNormEarlyMaxRows = 2048;
 
@@ -750,14 +763,14 @@ void run_pass(tsfm_spec *h, ModelDev &m, int B, const PassGeom &g, int head_mode
   auto *norm_kernel = d > 1280 ? rmsnorm_kernel<T, false, 16> : M <= kNormEarlyMaxRows ? rmsnorm_kernel<T, true, 10> : rmsnorm_kernel<T, false, 10>;
   {
     KTimer kt(h, KC_EMBED, (double)M * Pi * 4 + (double)d * Pi * sizeof(T) + (double)M * d * 4, 2.0 * M * Pi * d);
-    if (!fold && f32_tiles(h, m.W_emb, Pi)) {
+    if (!fold && (sizeof(T) == 4 ? f32_tiles(h, m.W_emb, Pi) : rows_tiles(h, m.W_emb, Pi))) {
       RowsArgs ra{};
       ra.mode = ROWS_EMBED;
       ra.epi = EPI_F32;
       ra.g = g;
       ra.opens_round = opens_round ? 1 : 0;
       ra.stamp = stamp;
-      launched(gemm_f32_launch(s, h->pdl, (const float *)h->hist, (const T *)m.W_emb, h->x, M, d, Pi, ra), "embedding");
+      launched(rows_launch(s, h->pdl, (const float *)h->hist, (const T *)m.W_emb, h->x, M, d, Pi, ra), "embedding");
     } else if (!fold && M >= kManyRows)
       launch_ex(s, h->pdl, embed_rows_kernel<T>, dim3((M + 7) / 8, (d + 127) / 128), dim3(128), 8 * Pi * sizeof(float),
                 h->hist, g, M, Pi, d, (const T *)m.W_emb, h->x, stamp);
@@ -814,7 +827,7 @@ void run_pass(tsfm_spec *h, ModelDev &m, int B, const PassGeom &g, int head_mode
   const double rows = head_mode == HEAD_LAST_TO_HIST ? B : Mb;
   KTimer kt(h, head_mode == HEAD_NONE ? -1 : KC_HEAD, rows * d * 4 + (double)P * d * sizeof(T) + rows * P * 4,
             2.0 * rows * P * d);
-  if (head_mode != HEAD_NONE && (sizeof(T) == 4 || rows >= kHeadTileRows) && f32_tiles(h, m.W_head, d)) {
+  if (head_mode != HEAD_NONE && (sizeof(T) == 4 ? f32_tiles(h, m.W_head, d) : rows >= kHeadTileRows && rows_tiles(h, m.W_head, d))) {
     RowsArgs ra{};
     ra.mode = head_mode == HEAD_LAST_TO_HIST ? ROWS_HEAD_LAST : ROWS_HEAD_ALL;
     ra.epi = EPI_F32;
@@ -826,7 +839,7 @@ void run_pass(tsfm_spec *h, ModelDev &m, int B, const PassGeom &g, int head_mode
     ra.muq = h->muq;
     ra.k_pos = ds.k_pos;
     ra.Kblk = ds.K;
-    launched(gemm_f32_launch(s, h->pdl, (const float *)h->x, (const T *)m.W_head, head_mode == HEAD_LAST_TO_HIST ? h->hist : vout,
+    launched(rows_launch(s, h->pdl, (const float *)h->x, (const T *)m.W_head, head_mode == HEAD_LAST_TO_HIST ? h->hist : vout,
                              (int)rows, P, d, ra), "head");
   } else if (head_mode == HEAD_LAST_TO_HIST) {
     launch_ex(s, h->pdl, head_kernel<T>, dim3(B, (P + 7) / 8), dim3(256), d * sizeof(float), h->x, m.g_f,
@@ -1317,7 +1330,7 @@ int tsfm_spec_create(const tsfm_weights *target_w, const tsfm_weights *draft_w, 
       return fail(TSFM_ERR_CUDA);
   }
   prefer_max_smem_all();
-  if ((rc = cfg->dtype == TSFM_F32 ? gemm_f32_init<float>() : gemm_f32_init<bf16>())) return fail(rc);
+  if ((rc = cfg->dtype == TSFM_F32 ? gemm_f32_init() : gemm_rows_init())) return fail(rc);
   if (h->use_tc) {
     if ((rc = gemm_sk_init())) return fail(rc);
     if ((rc = gemm_pair_init())) return fail(rc);

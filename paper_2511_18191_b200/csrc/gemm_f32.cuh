@@ -1,6 +1,5 @@
-// Contractions of fp32 activations in fp32 FMAs: those of the fp32 models (with a short K and many rows:
-// gemm_simt_kernel, see f32_many), and the patch embedding and the mean head of both kinds of model (weights
-// fp32 or bf16).
+// Contractions of the fp32 models in fp32 FMAs, patch embedding and mean head among them (with a short K and many rows:
+// gemm_simt_kernel, see f32_many).
 //
 //   C[t, f] (op)= sum_k A'[t, k] * W[f, k]       A' = A, or gain * A / sqrt(mean(A^2) + eps)
 //
@@ -51,24 +50,40 @@ struct RowsArgs {
   int k_pos, Kblk;
 };
 
+// Offsets of row t in A and C (so -1: no such row) and its series, in the modes other than ROWS_PLAIN: see slot_lookup.
+__device__ __forceinline__ void rows_lookup(const RowsArgs &ra, int t, int M, int N, int K, long long *so, long long *dof, int *series) {
+  const PassGeom &g = ra.g;
+  *so = -1;
+  *dof = 0;
+  if (t >= M) return;
+  const int nb = ra.mode == ROWS_HEAD_LAST ? 1 : ra.mode == ROWS_HEAD_ALL ? g.q_len / g.head_step : g.q_len;   // rows per slot
+  const int slot = t / nb, i = t % nb;
+  const SlotPos sp = slot_lookup(g, slot);
+  if (sp.dead) return;
+  *series = sp.b;
+  if (ra.mode == ROWS_EMBED) {
+    *so = ((long long)sp.b * g.cap + sp.p0 + i) * K;
+    *dof = (long long)t * N;
+    return;
+  }
+  const int j = ra.mode == ROWS_HEAD_LAST ? g.q_len - 1 : (i + 1) * g.head_step - 1;
+  *so = ((long long)slot * g.q_len + j) * K;
+  *dof = ra.mode == ROWS_HEAD_LAST ? ((long long)sp.b * g.cap + sp.p0 + g.q_len) * ra.tok_len : ((long long)sp.b * nb + i) * N;
+}
+
 constexpr int F32_GRID_Y = 65535;                              // the largest y of a grid
 
-template <typename T, int MT, int FN> constexpr int f32_smem_bytes(int KC) {
-  const int rows = MT * (KC + 4) * 4 + FN * (KC * (int)sizeof(T) + 16), red = 8 * MT * FN * 4;   // the partial sums reuse the rows
+template <int MT, int FN> constexpr int f32_smem_bytes(int KC) {
+  const int rows = MT * (KC + 4) * 4 + FN * (KC + 4) * 4, red = 8 * MT * FN * 4;   // the partial sums reuse the rows
   return rows > red ? rows : red;
 }
 
 __device__ __forceinline__ float4 f32_vec4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
-__device__ __forceinline__ float4 f32_vec4(const bf16 *p) {
-  const uint2 u = *reinterpret_cast<const uint2 *>(p);
-  return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xffff0000u), __uint_as_float(u.y << 16),
-                     __uint_as_float(u.y & 0xffff0000u));
-}
 
-template <typename T, int MT, int FN>
+template <int MT, int FN>
 __global__ void __launch_bounds__(256)
-gemm_f32_kernel(const float *A, const T *__restrict__ W, float *C, int M, int N, int K, int KC, const RowsArgs ra) {
-  constexpr int RM = MT / 4, RF = FN / 8, VW = 16 / sizeof(T);
+gemm_f32_kernel(const float *A, const float *__restrict__ W, float *C, int M, int N, int K, int KC, const RowsArgs ra) {
+  constexpr int RM = MT / 4, RF = FN / 8;
   extern __shared__ __align__(16) float f32_smem[];
   __shared__ long long src_off[MT], dst_off[MT];               // row offsets in A and C; src -1: no such row
   __shared__ int row_series[MT];
@@ -77,46 +92,23 @@ gemm_f32_kernel(const float *A, const T *__restrict__ W, float *C, int M, int N,
   const long long row_tile = (long long)blockIdx.z * F32_GRID_Y + blockIdx.y;
   if (row_tile * MT >= M) return;                              // (the last z's share of y is not full)
   const int f0 = blockIdx.x * FN, t0 = (int)row_tile * MT;
-  const PassGeom &g = ra.g;
-  const int nb = ra.mode == ROWS_HEAD_LAST ? 1 : ra.mode == ROWS_HEAD_ALL ? g.q_len / g.head_step : g.q_len;   // rows per slot
   // rows in use (active-series compaction): read before the dependency wait, see gemm_sk_kernel
   if (ra.mode == ROWS_PLAIN) {
     if (ra.lr.n_live) M = min(M, *reinterpret_cast<const volatile int *>(ra.lr.n_live) * ra.lr.q_len);
     if (t0 >= M) return;
   }
-  auto lookup = [&]() {                                        // slots of the other modes: see slot_lookup
-    if (tid < MT) {
-      const int t = t0 + tid;
-      long long so = -1, dof = 0;
-      if (t < M) {
-        const int slot = t / nb, i = t % nb;
-        const SlotPos sp = slot_lookup(g, slot);
-        if (!sp.dead) {
-          row_series[tid] = sp.b;
-          if (ra.mode == ROWS_EMBED) {
-            so = ((long long)sp.b * g.cap + sp.p0 + i) * K;
-            dof = (long long)t * N;
-          } else {
-            const int j = ra.mode == ROWS_HEAD_LAST ? g.q_len - 1 : (i + 1) * g.head_step - 1;
-            so = ((long long)slot * g.q_len + j) * K;
-            dof = ra.mode == ROWS_HEAD_LAST ? ((long long)sp.b * g.cap + sp.p0 + g.q_len) * ra.tok_len
-                                            : ((long long)sp.b * nb + i) * N;
-          }
-        }
-      }
-      src_off[tid] = so;
-      dst_off[tid] = dof;
-    }
+  auto lookup = [&]() {
+    if (tid < MT) rows_lookup(ra, t0 + tid, M, N, K, &src_off[tid], &dst_off[tid], &row_series[tid]);
   };
-  const int lda = KC + 4, ldw = KC + VW;
+  const int lda = KC + 4;
   float *As = f32_smem;
-  T *Ws = reinterpret_cast<T *>(f32_smem + MT * lda);
+  float *Ws = f32_smem + MT * lda;
   auto load_w = [&](int k0, int kc) {
-    const int cpr = kc / VW;
+    const int cpr = kc / 4;
     for (int i = tid; i < FN * cpr; i += 256) {
-      const int r = i / cpr, c = (i % cpr) * VW;
-      if (f0 + r < N) cp_async16(Ws + r * ldw + c, W + (size_t)(f0 + r) * K + k0 + c);
-      else *reinterpret_cast<uint4 *>(Ws + r * ldw + c) = make_uint4(0u, 0u, 0u, 0u);
+      const int r = i / cpr, c = (i % cpr) * 4;
+      if (f0 + r < N) cp_async16(Ws + r * lda + c, W + (size_t)(f0 + r) * K + k0 + c);
+      else *reinterpret_cast<float4 *>(Ws + r * lda + c) = make_float4(0.f, 0.f, 0.f, 0.f);
     }
   };
   load_w(0, min(KC, K));
@@ -187,7 +179,7 @@ gemm_f32_kernel(const float *A, const T *__restrict__ W, float *C, int M, int N,
 #pragma unroll
       for (int i = 0; i < RM; ++i) a[i] = *reinterpret_cast<const float4 *>(As + (tr + 4 * i) * lda + v * 4);
 #pragma unroll
-      for (int j = 0; j < RF; ++j) b[j] = f32_vec4(Ws + (tf + 8 * j) * ldw + v * 4);
+      for (int j = 0; j < RF; ++j) b[j] = f32_vec4(Ws + (tf + 8 * j) * lda + v * 4);
 #pragma unroll
       for (int i = 0; i < RM; ++i)
 #pragma unroll
@@ -223,9 +215,9 @@ gemm_f32_kernel(const float *A, const T *__restrict__ W, float *C, int M, int N,
 }
 
 // ------------------------------------------------------------------ host side
-template <typename T> static int gemm_f32_init() {
-  if (cudaFuncSetAttribute(gemm_f32_kernel<T, 16, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024) != cudaSuccess ||
-      cudaFuncSetAttribute(gemm_f32_kernel<T, 32, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024) != cudaSuccess)
+static int gemm_f32_init() {
+  if (cudaFuncSetAttribute(gemm_f32_kernel<16, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024) != cudaSuccess ||
+      cudaFuncSetAttribute(gemm_f32_kernel<32, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024) != cudaSuccess)
     return -4;
   return 0;
 }
@@ -237,12 +229,10 @@ static bool gemm_f32_eligible(const void *W, int K) { return K % 16 == 0 && K >=
 // shared-memory read).
 static bool gemm_f32_small(int M, int N) { return (long)((N + 15) / 16) * ((M + 15) / 16) <= 4 * 148; }
 // A small grid keeps rows of up to 768 values whole (one memory round trip), and so does one of up to two 32 x 32 tiles
-// per SM with rows of up to 512.  Otherwise rows longer than 256 go through in chunks of 256: three CTAs of 66 KB (fp32
-// weights) share an SM, one loading while another computes, where rows of 512 in one piece leave room for one
+// per SM with rows of up to 512.  Otherwise rows longer than 256 go through in chunks of 256: three CTAs of 66 KB share an SM, one loading while another computes, where rows of 512 in one piece leave room for one
 // (2048 x 512 x 512, 1024 CTAs: 68 -> 50 us; 256 x 1536 x 512, 384 CTAs: 29 -> 22; 512 x 512 x 512, 256 CTAs: 19.4 whole,
 // 20.7 in chunks).
-template <typename T>
-static bool gemm_f32_launch(cudaStream_t st, bool pdl, const float *A, const T *W, float *C, int M, int N, int K, const RowsArgs &ra) {
+static bool gemm_f32_launch(cudaStream_t st, bool pdl, const float *A, const float *W, float *C, int M, int N, int K, const RowsArgs &ra) {
   const bool small = gemm_f32_small(M, N);
   const int tile = small ? 16 : 32;
   const bool two_waves = (long)((N + 31) / 32) * ((M + 31) / 32) <= 2 * 148;
@@ -251,15 +241,15 @@ static bool gemm_f32_launch(cudaStream_t st, bool pdl, const float *A, const T *
   const int row_tiles = (M - 1) / tile + 1;
   cfg.gridDim = dim3((N + tile - 1) / tile, std::min(row_tiles, F32_GRID_Y), (row_tiles - 1) / F32_GRID_Y + 1);
   cfg.blockDim = dim3(256);
-  cfg.dynamicSmemBytes = small ? f32_smem_bytes<T, 16, 16>(KC) : f32_smem_bytes<T, 32, 32>(KC);
+  cfg.dynamicSmemBytes = small ? f32_smem_bytes<16, 16>(KC) : f32_smem_bytes<32, 32>(KC);
   cfg.stream = st;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = pdl ? 1 : 0;
-  return (small ? cudaLaunchKernelEx(&cfg, gemm_f32_kernel<T, 16, 16>, A, W, C, M, N, K, KC, ra)
-                : cudaLaunchKernelEx(&cfg, gemm_f32_kernel<T, 32, 32>, A, W, C, M, N, K, KC, ra)) == cudaSuccess;
+  return (small ? cudaLaunchKernelEx(&cfg, gemm_f32_kernel<16, 16>, A, W, C, M, N, K, KC, ra)
+                : cudaLaunchKernelEx(&cfg, gemm_f32_kernel<32, 32>, A, W, C, M, N, K, KC, ra)) == cudaSuccess;
 }
 
 }  // namespace tsfm

@@ -133,6 +133,34 @@ def test_mlp_of_a_layer_with_folded_norms_and_several_tiles_per_pair(f, B, n, ha
     assert relative(forward(w, arch, z), want[..., half * P:half * P + P]) < 1.5e-4
 
 
+@pytest.mark.parametrize("d,P,P_in,B,n", [
+    (64, 16, 16, 9, 60),              # 540 rows: rows of one block of k, 8 and 16 features a CTA
+    (192, 48, 48, 5, 103),            # half a block of k, a ragged tile of rows
+    (128, 80, 80, 3, 43),             # 129 rows: embedding row by row, head tiled
+    (1280, 32, 32, 64, 9),            # five chunks of a row
+    (320, 256, 16, 2, 320),           # a chunk and a quarter; 192 + 64 features
+    (832, 96, 96, 200, 27),           # 5400 rows: 96 and 192 features a CTA
+])
+def test_embedding_and_head_are_exact_to_fp32(d, P, P_in, B, n):
+    """Layers that add nothing between embedding, final norm and head of a bf16 model, whose rows are fp32.  The bound: sums of
+    up to 1280 products in blocks of 32, fp32 rounding (relative 2^-24 each) in embedding, square, factor and head: measured
+    1.0e-7 to 1.3e-7, and an operand that lost its last 8 bits shows as 2^-17 = 8e-6."""
+    arch = Arch(1, d, d // 64, 64)
+    rng = np.random.default_rng(d + n)
+    w = make_model(arch, P, 1, "bf16", patch_in=P_in)
+    for name in ("Wo", "W2"):
+        w["layers.0." + name][:] = 0
+    w["g_f"] = (1 + 0.2 * rng.standard_normal(d)).astype(np.float32)
+    import paper_2511_18191_b200 as tsfm
+    z = rng.standard_normal((B, n, P_in)).astype(np.float32)
+    dec = tsfm.SpecDecoder(w, None, arch, arch, P, "bf16", "layer_skip", max_batch=B, max_ctx_tokens=max(n, 2 * P // P_in),
+                           max_horizon_patches=1, max_K=1, patch_in=P_in)
+    got = dec.model_forward(0, torch.from_numpy(z).cuda()).cpu().numpy()
+    dec.close()
+    x = z.astype(np.float64) @ w["W_emb"].T.astype(np.float64)
+    assert relative(got, (w["g_f"] * x * rstd(x)) @ w["W_head"].T.astype(np.float64)) < 3e-7
+
+
 @pytest.mark.parametrize("heads,B,n", [(4, 9, 60), (1, 9, 60), (4, 2, 300), (1, 2, 300), (2, 9, 142), (2, 9, 143), (2, 41, 251)])
 def test_rotation_in_the_contraction_of_passes_of_many_tokens(heads, B, n):
     """Heads of 32, 64 and 128, the rotation table of a pass in shared memory or not, ragged row blocks, several tiles per pair.

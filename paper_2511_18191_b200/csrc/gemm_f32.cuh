@@ -14,7 +14,8 @@
 //     every epilogue sees complete sums.  Vectors of four products are summed before they are added, the eight
 //     partial sums as a tree: short chains of additions keep the rounding error of a sum at that of a
 //     warp-wide tree;
-//   * the norm's factor 1 / sqrt(...) is common to a row: the sums run over gain * A and are scaled at the end;
+//   * the norm's factor 1 / sqrt(...) is common to a row: the sums run over gain * A (or over A and gain * W, made before the
+//     wait, where K is in one chunk: 0.5 us a link less behind it) and are scaled at the end;
 //   * rows are padded by 16 bytes: the four token rows and eight feature rows that a warp reads at a
 //     time fall into different banks.
 // Bound: latency for small shapes (launch, one L2 round trip, the 8-way sum; 3.5 us a link inside a captured
@@ -112,6 +113,21 @@ gemm_f32_kernel(const float *A, const float *__restrict__ W, float *C, int M, in
     }
   };
   load_w(0, min(KC, K));
+  // a norm's gain, where all of K is here at once (and the grid, of small tiles, starts early): multiplied into the weights before the dependency wait, so that behind it the
+  // rows are used as they arrive (their sums of squares are not needed before the end)
+  const bool gain_in_w = MT == 16 && ra.gain && KC >= K;
+  if (gain_in_w) {
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    const int vpr = K >> 2;
+    for (int i = tid; i < FN * vpr; i += 256) {
+      const int r = i / vpr, c = (i - r * vpr) * 4;
+      float4 v = *reinterpret_cast<const float4 *>(Ws + r * lda + c);
+      const float4 gg = *reinterpret_cast<const float4 *>(ra.gain + c);
+      v.x *= gg.x; v.y *= gg.y; v.z *= gg.z; v.w *= gg.w;
+      *reinterpret_cast<float4 *>(Ws + r * lda + c) = v;
+    }
+  }
   const bool early = ra.mode != ROWS_PLAIN && !ra.opens_round;
   if (ra.mode == ROWS_PLAIN) {
     if (tid < MT) {
@@ -164,15 +180,16 @@ gemm_f32_kernel(const float *A, const float *__restrict__ W, float *C, int M, in
         float ss = 0.f;
         for (int v = lane; v < vpr; v += 32) {
           float4 a = *reinterpret_cast<const float4 *>(As + r * lda + v * 4);
-          const float4 gg = *reinterpret_cast<const float4 *>(ra.gain + k0 + v * 4);
           ss = fmaf(a.x, a.x, fmaf(a.y, a.y, fmaf(a.z, a.z, fmaf(a.w, a.w, ss))));
+          if (gain_in_w) continue;
+          const float4 gg = *reinterpret_cast<const float4 *>(ra.gain + k0 + v * 4);
           a.x *= gg.x; a.y *= gg.y; a.z *= gg.z; a.w *= gg.w;
           *reinterpret_cast<float4 *>(As + r * lda + v * 4) = a;
         }
         ss = warp_sum(ss);
         if (lane == 0) row_ss[r] += ss;
       }
-      __syncthreads();
+      if (!gain_in_w) __syncthreads();
     }
     for (int v = w; v < vpr; v += 8) {
       float4 a[RM], b[RF];

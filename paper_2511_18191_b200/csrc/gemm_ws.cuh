@@ -188,14 +188,17 @@ static bool gemm_ws_fits(const void *A, const void *W, int M, int N, int K) {
   const long ctas = (long)((N + WS_FN - 1) / WS_FN) * ((M + WS_MT - 1) / WS_MT);
   return ctas <= (long)per_sm * 148;
 }
-// Whether it is the better one there.  Contractions that do not widen (Wo, W2): everywhere (us, this / gemm_push_kernel:
-// M = 512, N = K = 512 3.6 / 4.6, M = 128, N = K = 1024 3.7 / 4.1, M = 128, N = 512, K = 2048 4.2 / 4.5).  Those that widen (QKV,
+// Whether it is the better one there.  Contractions that do not widen (Wo, W2): where they have less than a million weights or
+// fewer than 24 tokens (decode steps of whole models, us a layer, this / gemm_push_kernel: N = K = 1024 M = 20 19.4 / 19.8, 24 21.3 /
+// 20.0, 32 21.9 / 20.1, 93 26.4 / 25.1, 128 28.4 / 27.6; N = 512, K = 2048 M = 11 11.5 / 12.4, 24 13.7 / 13.8, 48 17.6 / 16.5, 96
+// 18.8 / 18.4; N = K = 2048 M = 24 29.2 / 25.3; N = K = 768 M = 32 21.0 / 22.2, 128 24.5 / 25.6; N = 384, K = 1536 M = 32 14.2 / 14.5;
+// in chains of the contraction alone, with weights in L2, N = K = 1024 M = 128 3.7 / 4.1).  Those that widen (QKV,
 // W1) scale their rows by factors that every CTA has to sum up: up to 256 CTAs (N = 2048, K = 512: M = 64 3.67 / 3.71, M = 93
 // 3.92 / 3.67), and with K > 512 only while the weights come from L2 in time (N = 2304, K = 768: M = 32 3.9 / 4.0; N = 3072, K =
 // 1024: M = 8 3.1 / 3.5, M = 16 3.58 / 3.53, M = 24 4.3 / 3.7).
 static bool gemm_ws_eligible(const void *A, const void *W, int M, int N, int K) {
   if (!gemm_ws_fits(A, W, M, N, K)) return false;
-  if (N <= K) return true;
+  if (N <= K) return (long)N * K < 1000000 || M < 24;
   const long ctas = (long)((N + WS_FN - 1) / WS_FN) * ((M + WS_MT - 1) / WS_MT);
   return ws_blocks(K) == 1 ? ctas <= 256 : (long)N * K <= 2500000 || M <= 8;
 }

@@ -726,8 +726,10 @@ attn_kernel(const float *qkv, T *Kc, T *Vc,
   const int rank = skv > 1 ? blockIdx.z % skv : 0;   // == %cluster_ctarank: the cluster spans z only
   const int d = n_heads * DH;
   const SlotPos sp = slot_lookup(g, slot);           // before the dependency wait: see SlotPos
-  pdl_sync();
-  if (sp.dead) return;                               // the whole cluster (same y) leaves together
+  if (sp.dead) {                                     // the whole cluster (same y) leaves together
+    pdl_sync();
+    return;
+  }
   const int b = sp.b, p0 = sp.p0;
   const int j_lo = qt * QT;
   const int j_hi = min(g.q_len, j_lo + QT);          // queries [j_lo, j_hi)
@@ -739,30 +741,51 @@ attn_kernel(const float *qkv, T *Kc, T *Vc,
   T *Kb = Kc + ((size_t)b * n_heads + h) * g.cap * DH;
   T *Vb = Vc + ((size_t)b * n_heads + h) * g.cap * DH;
 
-  // cached keys/values: p0 rows of DH elements as 16-byte asynchronous copies, all issued up
-  // front (the cache comes from HBM: the copy is bound by the bytes in flight)
-  {
-    constexpr int VPR = DH / EPV;                    // 16-byte chunks per row
-    const int nvec = max(min(k_hi, pre ? nk_all : p0) - k_lo, 0) * VPR;
-    const T *Kg = Kb + (size_t)k_lo * DH, *Vg = Vb + (size_t)k_lo * DH;
-    for (int i = threadIdx.x; i < nvec; i += blockDim.x) {
+  // cached keys/values as 16-byte asynchronous copies, all issued up front; rows below pos0 were written by this layer's
+  // attention in an earlier pass, at least a layer of kernels ago: before the dependency wait
+  constexpr int VPR = DH / EPV;                      // 16-byte chunks per row
+  const T *Kg = Kb + (size_t)k_lo * DH, *Vg = Vb + (size_t)k_lo * DH;
+  auto copy_rows = [&](int i0, int i1) {
+    for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
       const int t = i / VPR, c = i % VPR;
       cp_async16(Ks + (size_t)t * VW + (((c + t) & (VPR - 1)) << 2), Kg + (size_t)i * EPV);
       cp_async16(Vs + (size_t)i * 4, Vg + (size_t)i * EPV);
     }
-  }
+  };
+  const int v_old = max(min(k_hi, p0) - k_lo, 0) * VPR;
+  copy_rows(0, v_old);
+  // constants of this thread's first key pair and first query pair too
+  const int nq = j_hi - j_lo;                        // <= ATTN_QT
+  const int n_own = pre ? 0 : j_hi * (HALF / 2);
+  auto own_cs = [&](int i) { return *reinterpret_cast<const float4 *>(rope + (size_t)(p0 + i / (HALF / 2)) * HALF + (i % (HALF / 2)) * 2); };
+  auto q_cs = [&](int idx) { return rope[(size_t)(p0 + j_lo + idx / HALF) * HALF + idx % HALF]; };
+  const int tid = threadIdx.x;
+  float4 cs0 = make_float4(0.f, 0.f, 0.f, 0.f);
+  float2 qcs0 = make_float2(0.f, 0.f);
+  if (tid < n_own) cs0 = own_cs(tid);
+  if (tid < nq * HALF) qcs0 = q_cs(tid);
+  pdl_sync();
+  if (pre) copy_rows(v_old, max(k_hi - k_lo, 0) * VPR);
+  // first query pair: in flight with the first keys and values below
+  float q1 = 0.f, q2 = 0.f;
+  auto load_q = [&](int idx) {
+    const float *src = qkv + (row0 + j_lo + idx / HALF) * 3 * d + h * DH + idx % HALF;
+    q1 = __ldcg(src);
+    q2 = __ldcg(src + HALF);
+  };
+  if (tid < nq * HALF) load_q(tid);
   // keys/values of this pass (rotate keys; the owning tile appends to the cache).
   // One thread handles the element pair (c, c + 1) of the first half and its rotation partners.
-  for (int i = threadIdx.x; i < (pre ? 0 : j_hi * (HALF / 2)); i += blockDim.x) {
+  for (int i = tid; i < n_own; i += blockDim.x) {
     const int j = i / (HALF / 2), c = (i % (HALF / 2)) * 2;
     const float *src = qkv + (row0 + j) * 3 * d + h * DH;
     const int tg = p0 + j, t = tg - k_lo;            // position in the row, row in this CTA
     if (tg < k_lo || tg >= k_hi) continue;
-    const float4 cs = *reinterpret_cast<const float4 *>(rope + (size_t)tg * HALF + c);   // cos0 sin0 cos1 sin1
-    const float2 ka = *reinterpret_cast<const float2 *>(src + d + c);
-    const float2 kb = *reinterpret_cast<const float2 *>(src + d + c + HALF);
-    const float2 va = *reinterpret_cast<const float2 *>(src + 2 * d + c);
-    const float2 vb = *reinterpret_cast<const float2 *>(src + 2 * d + c + HALF);
+    const float4 cs = i == tid ? cs0 : own_cs(i);    // cos0 sin0 cos1 sin1
+    const float2 ka = __ldcg(reinterpret_cast<const float2 *>(src + d + c));
+    const float2 kb = __ldcg(reinterpret_cast<const float2 *>(src + d + c + HALF));
+    const float2 va = __ldcg(reinterpret_cast<const float2 *>(src + 2 * d + c));
+    const float2 vb = __ldcg(reinterpret_cast<const float2 *>(src + 2 * d + c + HALF));
     const float r1a = ka.x * cs.x - kb.x * cs.y, r1b = ka.y * cs.z - kb.y * cs.w;    // first half
     const float r2a = kb.x * cs.x + ka.x * cs.y, r2b = kb.y * cs.z + ka.y * cs.w;    // second half
     if (BF) {
@@ -793,19 +816,16 @@ attn_kernel(const float *qkv, T *Kc, T *Vc,
     }
   }
 
-  const int tid = threadIdx.x;
   const float scale = rsqrtf((float)DH);
-  const int nq = j_hi - j_lo;                        // <= ATTN_QT
   const int nk = k_hi - k_lo;                        // key rows held here
   // rows the tile routine will touch: its compile-time query bound
   const int nqb = nq <= 2 ? nq : nq <= 4 ? 4 : nq <= 6 ? 6 : nq <= 9 ? 9 : ATTN_QT;
   for (int idx = tid; idx < nqb * HALF; idx += blockDim.x) {       // rotated, scaled queries (zero past nq)
-    const int i = idx / HALF, c = idx % HALF, j = j_lo + i;
+    const int i = idx / HALF, c = idx % HALF;
     float r1 = 0.f, r2 = 0.f;
     if (i < nq) {
-      const float *src = qkv + (row0 + j) * 3 * d + h * DH;
-      const float2 cs = rope[(size_t)(p0 + j) * HALF + c];
-      const float q1 = src[c], q2 = src[c + HALF];
+      if (idx != tid) load_q(idx);
+      const float2 cs = idx == tid ? qcs0 : q_cs(idx);
       r1 = (q1 * cs.x - q2 * cs.y) * scale;
       r2 = (q2 * cs.x + q1 * cs.y) * scale;
     }

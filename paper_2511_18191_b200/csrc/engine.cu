@@ -335,12 +335,15 @@ constexpr int kFlashStShort = 2;
 // series: 2.26 -> 2.12, 3.38 -> 2.95, 3.80 -> 3.39; attn_mma_smem does the same there).
 // Larger grids fill the machine anyhow, and the even share then only stands in the way of balancing blocks of different
 // length (scoring 512 CTAs: 510 -> 518 us).
-template <int DH> int tiles_smem(long ctas) {
+inline int even_share_smem(long ctas, int need) {
   const int share = (int)std::min(4l, (ctas + 147) / 148);
-  return share > 3 ? TilesGeom<DH>::SMEM_BYTES : std::max<int>(TilesGeom<DH>::SMEM_BYTES, 228 * 1024 / (share + 1));
+  return share > 3 ? need : std::max(need, 228 * 1024 / (share + 1));
 }
+template <int DH> int tiles_smem(long ctas) { return even_share_smem(ctas, TilesGeom<DH>::SMEM_BYTES); }
 template <int DH> int flash_set_attr() {
   CU_TRY(cudaFuncSetAttribute(attn_tiles_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, tiles_smem<DH>(1)));
+  if constexpr (DH <= 64)
+    CU_TRY(cudaFuncSetAttribute(attn_short_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, even_share_smem(1, 128 * DH)));
   CU_TRY(cudaFuncSetAttribute(attn_flash_kernel<DH, kFlashStShort>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               FlashGeom<DH, kFlashStShort>::SMEM_BYTES));
   CU_TRY(cudaFuncSetAttribute(attn_narrow_ring_kernel<DH, kFlashStShort>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -419,10 +422,12 @@ void prefer_max_smem_all() {
   prefer_max_smem(gemm_ws_kernel<4, false>);
   prefer_max_smem(gemm_ws_kernel<4, true>);
   prefer_max_smem(attn_tiles_kernel<32>);
+  prefer_max_smem(attn_short_kernel<32>);
   prefer_max_smem(attn_narrow_ring_kernel<32, kFlashStShort>);
   prefer_max_smem(attn_narrow_single_kernel<32>);
   prefer_max_smem(attn_flash_kernel<32, kFlashStShort>);
   prefer_max_smem(attn_tiles_kernel<64>);
+  prefer_max_smem(attn_short_kernel<64>);
   prefer_max_smem(attn_narrow_ring_kernel<64, kFlashStShort>);
   prefer_max_smem(attn_narrow_single_kernel<64>);
   prefer_max_smem(attn_flash_kernel<64, kFlashStShort>);
@@ -659,6 +664,13 @@ void launch_attn(tsfm_spec *h, ModelDev &m, int l, int B, const PassGeom &g, boo
       return;
     }
     if (pre) {
+      if constexpr (DH <= 64) {                                // (heads of 128: 11.2 us either way, 200 series x 4 heads x 30 tokens)
+        if ((g.done ? g.cap : g.base + g.q_len) <= 32) {       // the most that a query can see
+          launch_ex(h->ls, h->pdl, attn_short_kernel<DH>, dim3(m.arch.n_heads, B), dim3(64), (size_t)even_share_smem(pairs, 128 * DH), h->qkv,
+                    (const bf16 *)Kc, (const bf16 *)Vc, m.rope, g, m.arch.n_heads, appended ? 1 : 0, (bf16 *)h->ao);
+          return;
+        }
+      }
       const int warps = g.q_len <= 32 ? 2 : 4;
       const dim3 grid(m.arch.n_heads, B, (g.q_len + 16 * warps - 1) / (16 * warps));
       launch_ex(h->ls, h->pdl, attn_tiles_kernel<DH>, grid, dim3(32 * warps), (size_t)tiles_smem<DH>((long)grid.x * grid.y * grid.z),

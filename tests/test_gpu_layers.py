@@ -89,6 +89,18 @@ def test_attention_keeps_both_parts_of_its_queries(B, n):
     assert relative(forward(w, arch, z), want) < 1.5e-3
 
 
+@pytest.mark.parametrize("heads,B,n", [(2, 1, 17), (4, 40, 17), (2, 31, 24), (4, 20, 31), (2, 150, 32), (4, 3, 32), (2, 2, 33)])
+def test_attention_of_passes_that_see_at_most_32_keys(heads, B, n):
+    """Heads of 64 and 32 at the ends of 17 to 32 tokens, few and many series (rotated here or by the contraction).  The bound as
+    above."""
+    arch = Arch(1, 128, heads, 64)
+    rng = np.random.default_rng(n + heads)
+    w = layer_weights(arch, rng, Wq=12, Wk=1, Wv=4, Wo=1, W1=1, W2=0)
+    w["layers.0.g1"] = np.ones(128, dtype=np.float32)
+    z = np.where(rng.random((B, n, 128)) < 0.5, -1, 1).astype(np.float32)
+    assert relative(forward(w, arch, z), attention(w, heads, z)) < 1.5e-3
+
+
 @pytest.mark.parametrize("d,f,B,n,folded", [
     (192, 192, 1, 3, True),           # weights in registers
     (256, 2560, 4, 20, True),         # up to 512 rows: K of W2 split over a cluster

@@ -78,7 +78,7 @@ attn_mma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant_
                  o_full = bars + 72, slot_addr = bars + 80;
   uint32_t *slot_ptr = reinterpret_cast<uint32_t *>(gbase + 6 * AM_TILE + 80);
   float *half_val = reinterpret_cast<float *>(gbase + 6 * AM_TILE + 128);     // [2][128] what the two threads of a row exchange
-  int *bad_row = reinterpret_cast<int *>(gbase + 6 * AM_TILE + 96);           // first value row of the tile with an infinity or NaN
+  uint32_t *bad_rows = reinterpret_cast<uint32_t *>(gbase + 6 * AM_TILE + 96);   // [4] value rows of the tile with an infinity or NaN
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const int h = blockIdx.x, qb = (gridDim.z - 1 - blockIdx.z) * AM_Q, d = n_heads * AM_DH;     // blocks with the most keys first
   const SlotPos sp = slot_lookup(g, blockIdx.y);               // before the dependency wait: see SlotPos
@@ -213,9 +213,9 @@ attn_mma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant_
     const uint32_t trow = tmem + ((uint32_t)(w4 * 32) << 16);
     const int row = w4 * 32 + lane, qpos = p0 + qb + row;      // this thread's query and its position
     float *mine = half_val + part * AM_Q + row, *other = half_val + (part ^ 1) * AM_Q + row;
-    float o[32];
+    uint64_t o[16];                                            // two dims each
 #pragma unroll
-    for (int i = 0; i < 32; ++i) o[i] = 0.f;
+    for (int i = 0; i < 16; ++i) o[i] = 0;
     float m_run = -INFINITY, l_run = 0.f;
     bool ok = true, nan_seen = false;
     for (int t = 0; t < n_tiles; ++t) {
@@ -225,27 +225,29 @@ attn_mma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant_
         // value rows that some queries must not see: see above
         if (ok) ok = mbar_wait(vfull0 + 8 * (t & 1), (uint32_t)((t >> 1) & 1));
         if (!ok) atomicExch(status, DEV_TIMEOUT_EPILOGUE);
-        if (threadIdx.x == 0) *bad_row = 0x7fffffff;           // none
+        if (threadIdx.x < 4) bad_rows[threadIdx.x] = 0;        // none
         asm volatile("bar.sync 1, 256;" ::: "memory");
         uint4 *v = reinterpret_cast<uint4 *>(gbase + 2 * AM_TILE + (t & 1) * 2 * AM_TILE + AM_TILE + row * 128);
-        bool zero = t0 + row >= n_keys;
-        if (!zero) {                                           // (both threads of a row look at all of it)
-          uint32_t bad = 0;
+        const bool behind = t0 + row >= n_keys;
+        if (!behind) {                                         // each thread of a row looks at half of it
+          uint32_t bad = 0;                                    // (an exponent of all ones carries into its sign)
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const uint4 w = v[(i + row) & 7];
-            bad |= __vcmpeq2(w.x & 0x7f807f80u, 0x7f807f80u) | __vcmpeq2(w.y & 0x7f807f80u, 0x7f807f80u) |
-                   __vcmpeq2(w.z & 0x7f807f80u, 0x7f807f80u) | __vcmpeq2(w.w & 0x7f807f80u, 0x7f807f80u);
+          for (int i = 0; i < 4; ++i) {
+            const uint4 w = v[(i + part * 4 + row) & 7];
+            bad |= ((w.x & 0x7f807f80u) + 0x00800080u) | ((w.y & 0x7f807f80u) + 0x00800080u) | ((w.z & 0x7f807f80u) + 0x00800080u) |
+                   ((w.w & 0x7f807f80u) + 0x00800080u);
           }
-          if (bad) atomicMin(bad_row, row), zero = true;
+          if (bad & 0x80008000u) atomicOr(bad_rows + (row >> 5), 1u << (row & 31));
         }
         asm volatile("bar.sync 1, 256;" ::: "memory");
-        if (zero) {
+        const uint32_t b0 = bad_rows[0], b1 = bad_rows[1], b2 = bad_rows[2], b3 = bad_rows[3];
+        const int bad_row = b0 ? __ffs(b0) - 1 : b1 ? 31 + __ffs(b1) : b2 ? 63 + __ffs(b2) : b3 ? 95 + __ffs(b3) : 0x7fffffff;
+        if (behind || (bad_rows[row >> 5] >> (row & 31) & 1)) {
 #pragma unroll
           for (int i = 0; i < 4; ++i) v[(i + part * 4 + row) & 7] = make_uint4(0u, 0u, 0u, 0u);
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        nan_seen |= qpos - t0 >= *bad_row;
+        nan_seen |= qpos - t0 >= bad_row;
       }
       if (ok) ok = mbar_wait(s_full, (uint32_t)(t & 1));
       if (!ok) atomicExch(status, DEV_TIMEOUT_EPILOGUE);
@@ -259,11 +261,10 @@ attn_mma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant_
         float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
         if (partial) {
 #pragma unroll
-          for (int i = 0; i < 32; ++i) m4[i & 3] = fmaxf(m4[i & 3], c + i <= lim ? s[i] : -INFINITY);
-        } else {
-#pragma unroll
-          for (int i = 0; i < 32; ++i) m4[i & 3] = fmaxf(m4[i & 3], s[i]);
+          for (int i = 0; i < 32; ++i) s[i] = c + i <= lim ? s[i] : -INFINITY;
         }
+#pragma unroll
+        for (int i = 0; i < 32; i += 2) asm("max.f32 %0, %0, %1, %2;" : "+f"(m4[(i >> 1) & 3]) : "f"(s[i]), "f"(s[i + 1]));
         mx = fmaxf(mx, fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])));
       }
       *mine = mx;
@@ -271,7 +272,8 @@ attn_mma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant_
       const float m_new = fmaxf(m_run, fmaxf(mx, *other)), m_use = m_new == -INFINITY ? 0.f : m_new;
       const float alpha = flash_ex2(m_run - m_use);
       m_run = m_new;
-      float sum4[4] = {0.f, 0.f, 0.f, 0.f};
+      uint64_t sum2[2] = {0, 0};
+      const uint64_t minus_m = f32x2(-m_use, -m_use), alpha2 = f32x2(alpha, alpha);
 #pragma unroll 1
       for (int c = 0; c < 64; c += 32) {
         float s[32];
@@ -279,18 +281,20 @@ attn_mma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant_
         uint32_t p[16];
 #pragma unroll
         for (int i = 0; i < 32; i += 2) {
-          float a = flash_ex2(s[i] - m_use), b = flash_ex2(s[i + 1] - m_use);
+          const float2 x = unpack2(add2(f32x2(s[i], s[i + 1]), minus_m));
+          float a = flash_ex2(x.x), b = flash_ex2(x.y);
           if (partial) {
             a = c + i <= lim ? a : 0.f;
             b = c + i + 1 <= lim ? b : 0.f;
           }
-          sum4[(i >> 1) & 3] += a + b;
+          sum2[(i >> 1) & 1] = add2(sum2[(i >> 1) & 1], f32x2(a, b));
           p[i >> 1] = pack_bf16x2(a, b);
         }
         tmem_st16(trow + AM_P + ((c0 + c) >> 1), p);
       }
       asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-      l_run = fmaf(l_run, alpha, (sum4[0] + sum4[1]) + (sum4[2] + sum4[3]));
+      const float2 sum = unpack2(add2(sum2[0], sum2[1]));
+      l_run = fmaf(l_run, alpha, sum.x + sum.y);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(p_ready);
@@ -301,7 +305,7 @@ attn_mma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant_
       float v[32];
       tmem_ld32(trow + AM_O + part * 32, v);
 #pragma unroll
-      for (int i = 0; i < 32; ++i) o[i] = fmaf(o[i], alpha, v[i]);
+      for (int i = 0; i < 16; ++i) o[i] = fma2(o[i], alpha2, f32x2(v[2 * i], v[2 * i + 1]));
     }
     *mine = l_run;                                             // (the row's last maxima were read before its last p_ready)
     asm volatile("bar.sync %0, 64;" ::"r"(2 + w4) : "memory");
@@ -309,9 +313,11 @@ attn_mma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant_
       const float inv = nan_seen ? __int_as_float(0x7fffffff) : 1.f / (part ? *other + l_run : l_run + *other);
       uint4 *dst = reinterpret_cast<uint4 *>(out + ((size_t)blockIdx.y * g.q_len + qb + row) * d + h * AM_DH + part * 32);
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
-        dst[i] = make_uint4(pack_bf16x2(o[8 * i] * inv, o[8 * i + 1] * inv), pack_bf16x2(o[8 * i + 2] * inv, o[8 * i + 3] * inv),
-                            pack_bf16x2(o[8 * i + 4] * inv, o[8 * i + 5] * inv), pack_bf16x2(o[8 * i + 6] * inv, o[8 * i + 7] * inv));
+      for (int i = 0; i < 4; ++i) {
+        const float2 a = unpack2(o[4 * i]), b = unpack2(o[4 * i + 1]), c = unpack2(o[4 * i + 2]), e = unpack2(o[4 * i + 3]);
+        dst[i] = make_uint4(pack_bf16x2(a.x * inv, a.y * inv), pack_bf16x2(b.x * inv, b.y * inv), pack_bf16x2(c.x * inv, c.y * inv),
+                            pack_bf16x2(e.x * inv, e.y * inv));
+      }
     }
   }
   tc_fence_before();

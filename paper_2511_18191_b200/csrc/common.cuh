@@ -149,6 +149,16 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
   return r;
 }
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(uint64_t a) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a));
+  return r;
+}
 __device__ __forceinline__ uint32_t gelu_erf_fast2(float a, float b) {
   const uint64_t v = f32x2(a, b);
   const float w0 = fmaf(fabsf(a), 0.3275911f * 0.70710678118654752440f, 1.f), w1 = fmaf(fabsf(b), 0.3275911f * 0.70710678118654752440f, 1.f);

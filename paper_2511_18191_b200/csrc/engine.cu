@@ -397,6 +397,8 @@ void prefer_max_smem_all() {
   prefer_max_smem_typed<bf16>();
   prefer_max_smem(gemm_f32_kernel<16, 16>);
   prefer_max_smem(gemm_f32_kernel<32, 32>);
+  prefer_max_smem(gemm_f32_reg_kernel<2>);
+  prefer_max_smem(gemm_f32_reg_kernel<4>);
   prefer_max_smem(gemm_rows_kernel<1>);
   prefer_max_smem(gemm_rows_kernel<3>);
   prefer_max_smem(instnorm_kernel);

@@ -231,6 +231,104 @@ gemm_f32_kernel(const float *A, const float *__restrict__ W, float *C, int M, in
   }
 }
 
+// The same for small grids and short K, 16 x 16 outputs a CTA: a warp's share of K (every eighth vector of four) is nobody else's, so
+// both operands go straight into registers, the weights (times a norm's gain) before the dependency wait and all of the rows
+// behind it in one round trip; no copy through shared memory and no barrier stands before the sum of the partial tiles.
+// Bound: one round trip to L2 and the sum of eight partial tiles.  Links of the fp32 models' forecasts, us, gemm_f32_kernel -> here:
+// K = 64 2.3 .. 2.9 -> 1.5 .. 2.1, K = 128 2.0 .. 3.6 -> 1.5 .. 2.8; a speculative forecast of one series 231 -> 207 us,
+// of 37 series of different lengths 707 -> 654.  Where it is taken: f32_in_registers.
+// NV: vectors per warp, K <= 32 NV.  grid as above (z = 1), block = 256.
+template <int NV>
+__global__ void __launch_bounds__(256, NV <= 2 ? 3 : 2)
+gemm_f32_reg_kernel(const float *A, const float *__restrict__ W, float *C, int M, int N, int K, const RowsArgs ra) {
+  __shared__ float red[8][256], row_ss[8][16];
+  __shared__ long long src_off[16], dst_off[16];               // (modes other than ROWS_PLAIN)
+  __shared__ int row_series[16];
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, tr = lane >> 3, tf = lane & 7;
+  const int f0 = blockIdx.x * 16, t0 = blockIdx.y * 16, orow = tid >> 4, f = f0 + (tid & 15);
+  const bool plain = ra.mode == ROWS_PLAIN;
+  // rows in use (active-series compaction): read before the dependency wait, see gemm_sk_kernel
+  if (plain) {
+    if (ra.lr.n_live) M = min(M, *reinterpret_cast<const volatile int *>(ra.lr.n_live) * ra.lr.q_len);
+    if (t0 >= M) return;
+  }
+  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+  float4 b[NV][2];                                             // features tf, tf + 8
+#pragma unroll
+  for (int n = 0; n < NV; ++n) {
+    const int k = (w + 8 * n) * 4;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) b[n][j] = k < K && f0 + tf + 8 * j < N ? *reinterpret_cast<const float4 *>(W + (size_t)(f0 + tf + 8 * j) * K + k) : zero;
+  }
+  if (ra.gain) {
+#pragma unroll
+    for (int n = 0; n < NV; ++n) {
+      const int k = (w + 8 * n) * 4;
+      const float4 gg = k < K ? *reinterpret_cast<const float4 *>(ra.gain + k) : zero;
+#pragma unroll
+      for (int j = 0; j < 2; ++j) b[n][j].x *= gg.x, b[n][j].y *= gg.y, b[n][j].z *= gg.z, b[n][j].w *= gg.w;
+    }
+  }
+  const bool early = !plain && !ra.opens_round;
+  auto lookup = [&]() {
+    if (tid < 16) rows_lookup(ra, t0 + tid, M, N, K, &src_off[tid], &dst_off[tid], &row_series[tid]);
+  };
+  if (early) lookup();
+  pdl_sync();
+  if (ra.stamp && blockIdx.x == 0 && t0 == 0 && tid == 0) *ra.stamp = globaltimer_ns();
+  if (!plain) {
+    if (!early) lookup();
+    if (!__syncthreads_or(tid < 16 && src_off[tid] >= 0)) return;        // a tile of dead slots
+  }
+  auto src = [&](int r) { return !plain ? src_off[r] : t0 + r < M ? (long long)(t0 + r) * K : -1ll; };
+  float4 a[4][NV];                                             // rows tr, tr + 4, ...
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const long long so = src(tr + 4 * i);
+#pragma unroll
+    for (int n = 0; n < NV; ++n) {
+      const int k = (w + 8 * n) * 4;
+      a[i][n] = so >= 0 && k < K ? __ldcg(reinterpret_cast<const float4 *>(A + so + k)) : zero;
+    }
+  }
+  const bool live = src(orow) >= 0 && f < N;
+  float *dst = C + (plain ? (long long)(t0 + orow) * N : dst_off[orow]) + f;
+  const float old = ra.epi == EPI_RESID && live ? __ldcg(dst) : 0.f;
+  float acc[4][2], ss[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    acc[i][0] = acc[i][1] = ss[i] = 0.f;
+#pragma unroll
+    for (int n = 0; n < NV; ++n) {
+      const float4 v = a[i][n];
+#pragma unroll
+      for (int j = 0; j < 2; ++j) acc[i][j] += fmaf(v.x, b[n][j].x, fmaf(v.y, b[n][j].y, fmaf(v.z, b[n][j].z, v.w * b[n][j].w)));
+      if (ra.gain) ss[i] = fmaf(v.x, v.x, fmaf(v.y, v.y, fmaf(v.z, v.z, fmaf(v.w, v.w, ss[i]))));
+    }
+#pragma unroll
+    for (int j = 0; j < 2; ++j) red[w][(tr + 4 * i) * 16 + tf + 8 * j] = acc[i][j];
+    if (ra.gain && tf == 0) row_ss[w][tr + 4 * i] = ss[i];
+  }
+  __syncthreads();
+  if (!live) return;
+  float p[8], q[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) p[k] = red[k][tid];
+  float v = ((p[0] + p[1]) + (p[2] + p[3])) + ((p[4] + p[5]) + (p[6] + p[7]));
+  if (ra.gain) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) q[k] = row_ss[k][orow];
+    v *= rsqrtf((((q[0] + q[1]) + (q[2] + q[3])) + ((q[4] + q[5]) + (q[6] + q[7]))) / K + ra.eps);
+  }
+  if (ra.epi == EPI_RESID) v += old;
+  else if (ra.epi == EPI_GELU_T) v = gelu_erf(v);
+  if (ra.mode == ROWS_HEAD_LAST && ra.st && (ra.st->flags & VAR_SAMPLE_PROPOSALS)) {   // (see gemm_f32_kernel)
+    ra.muq[((size_t)row_series[orow] * ra.Kblk + ra.k_pos) * N + f] = v;
+    v += ra.st->sigma_q * head_normal(ra.st, row_series[orow], ra.k_pos, f);
+  }
+  *dst = v;
+}
+
 // ------------------------------------------------------------------ host side
 static int gemm_f32_init() {
   if (cudaFuncSetAttribute(gemm_f32_kernel<16, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024) != cudaSuccess ||
@@ -245,8 +343,18 @@ static bool gemm_f32_eligible(const void *W, int K) { return K % 16 == 0 && K >=
 // largest such grids run somewhat over one wave); beyond that 32 x 32 ones (twice the flops per
 // shared-memory read).
 static bool gemm_f32_small(int M, int N) { return (long)((N + 15) / 16) * ((M + 15) / 16) <= 4 * 148; }
+// Which links take the registers: those of few rows in models of width up to 128.  A CTA of NV = 4 holds half of an SM's
+// registers, and past 64 rows the links around it, waiting beside it with their weights, no longer find room (plain decoding,
+// 2 layers, d = 128, us a forecast of eight patches, gemm_f32_kernel -> here: 8 series 315 -> 280, 37 356 -> 326, 64 396 -> 384;
+// 80 series 406 -> 421, 128 468 -> 499, 256 590 -> 670); NV = 2 a quarter (4 layers, d = 64: 30 series 539 -> 485, 100 604 -> 545,
+// 160 666 -> 642; 200 702 -> 721, 700 1241 -> 1281).  The embedding of a wider model alone gives nothing (d = 256: 8 series 475 both,
+// 64 735 -> 757), and neither did K = 256 in twice the warps (3.7 us a link for 3.0: more of the time before the wait is weights).
+static bool f32_in_registers(int mode, int M, int N, int K) {
+  return K <= 128 && (mode != ROWS_EMBED || N <= 128) && M <= (K <= 64 ? 160 : 64);
+}
 // A small grid keeps rows of up to 768 values whole (one memory round trip), and so does one of up to two 32 x 32 tiles
-// per SM with rows of up to 512.  Otherwise rows longer than 256 go through in chunks of 256: three CTAs of 66 KB share an SM, one loading while another computes, where rows of 512 in one piece leave room for one
+// per SM with rows of up to 512.  Otherwise rows longer than 256 go through in chunks of 256: three CTAs of 66 KB share an SM,
+// one loading while another computes, where rows of 512 in one piece leave room for one
 // (2048 x 512 x 512, 1024 CTAs: 68 -> 50 us; 256 x 1536 x 512, 384 CTAs: 29 -> 22; 512 x 512 x 512, 256 CTAs: 19.4 whole,
 // 20.7 in chunks).
 static bool gemm_f32_launch(cudaStream_t st, bool pdl, const float *A, const float *W, float *C, int M, int N, int K, const RowsArgs &ra) {
@@ -265,6 +373,11 @@ static bool gemm_f32_launch(cudaStream_t st, bool pdl, const float *A, const flo
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = pdl ? 1 : 0;
+  if (small && f32_in_registers(ra.mode, M, N, K)) {
+    cfg.dynamicSmemBytes = 0;
+    return (K <= 64 ? cudaLaunchKernelEx(&cfg, gemm_f32_reg_kernel<2>, A, W, C, M, N, K, ra)
+                    : cudaLaunchKernelEx(&cfg, gemm_f32_reg_kernel<4>, A, W, C, M, N, K, ra)) == cudaSuccess;
+  }
   return (small ? cudaLaunchKernelEx(&cfg, gemm_f32_kernel<16, 16>, A, W, C, M, N, K, KC, ra)
                 : cudaLaunchKernelEx(&cfg, gemm_f32_kernel<32, 32>, A, W, C, M, N, K, KC, ra)) == cudaSuccess;
 }

@@ -173,6 +173,34 @@ def test_embedding_and_head_are_exact_to_fp32(d, P, P_in, B, n):
     assert relative(got, (w["g_f"] * x * rstd(x)) @ w["W_head"].T.astype(np.float64)) < 3e-7
 
 
+@pytest.mark.parametrize("d,f,P,P_in,B,n", [
+    (64, 64, 64, 64, 1, 1), (64, 64, 48, 48, 1, 17), (64, 64, 16, 16, 10, 16), (64, 64, 16, 16, 7, 23),   # up to 160 rows
+    (64, 64, 32, 8, 5, 3),                                       # embedding by itself
+    (128, 128, 128, 128, 1, 15), (128, 64, 112, 112, 4, 16), (128, 128, 80, 16, 5, 13), (64, 128, 96, 96, 2, 9),   # up to 64
+    (192, 128, 64, 64, 1, 33),                                   # a wider model: W2 only
+])
+def test_fp32_links_of_few_rows(d, f, P, P_in, B, n):
+    """x + W2 GELU(W1 norm(x)), norm and head of an fp32 model.  The bound: five links of up to 192 products in tree sums,
+    each with up to ten roundings of relative size 2^-24 that add as the square root: 4e-7."""
+    arch = Arch(1, d, d // 32, f)
+    rng = np.random.default_rng(d + n)
+    w = make_model(arch, P, 1, "f32", patch_in=P_in)
+    w["layers.0.Wo"][:] = 0
+    w["layers.0.W1"] *= 3
+    for name in ("g_f", "layers.0.g2"):
+        w[name] = (1 + 0.2 * rng.standard_normal(d)).astype(np.float32)
+    import paper_2511_18191_b200 as tsfm
+    z = rng.standard_normal((B, n, P_in)).astype(np.float32)
+    dec = tsfm.SpecDecoder(w, None, arch, arch, P, "f32", "layer_skip", max_batch=B, max_ctx_tokens=max(n, 2 * P // P_in),
+                           max_horizon_patches=1, max_K=1, patch_in=P_in)
+    got = dec.model_forward(0, torch.from_numpy(z).cuda()).cpu().numpy()
+    dec.close()
+    x = z.astype(np.float64) @ w["W_emb"].T.astype(np.float64)
+    h = torch.from_numpy((w["layers.0.g2"] * x * rstd(x)) @ w["layers.0.W1"].T.astype(np.float64))
+    y = x + torch.nn.functional.gelu(h).numpy() @ w["layers.0.W2"].T.astype(np.float64)
+    assert relative(got, (w["g_f"] * y * rstd(y)) @ w["W_head"].T.astype(np.float64)) < 4e-7
+
+
 @pytest.mark.parametrize("heads,B,n", [(4, 9, 60), (1, 9, 60), (4, 2, 300), (1, 2, 300), (2, 9, 142), (2, 9, 143), (2, 41, 251)])
 def test_rotation_in_the_contraction_of_passes_of_many_tokens(heads, B, n):
     """Heads of 32, 64 and 128, the rotation table of a pass in shared memory or not, ragged row blocks, several tiles per pair.

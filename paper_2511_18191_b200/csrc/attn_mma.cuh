@@ -14,11 +14,13 @@
 // product 0 x NaN would reach all 128 queries).  An infinity so makes the head NaN, where in a tile that every query sees it
 // stays in its dimension: the token's output is NaN in either case, since the contraction behind multiplies the infinity by
 // weights of both signs and the norm behind that by 0.
-// Bound: the chain of a tile (MMAs, two passes over the scores, MMAs, sums) and a block's first loads, with 16 softmax warps
-// per SM.
-// attn_tiles_kernel -> here, us a launch inside a forecast: 16 series x 8 heads x 256 queries behind 704 to 1000 keys 53 -> 28,
-// 704 queries behind none 49 -> 38, 4 heads x 64 queries 23 -> 17.5; 64 series x 20 heads x 255 queries 114 -> 108 (one or two
-// tiles a block: mostly start and first loads).  With one thread per row 28.6, 43, 21, 122.
+// Bound: the chain of a tile (MMAs, two passes over the scores, MMAs, sums; 4000 cycles) and a block's start (5000 cycles), with 16
+// softmax warps per SM.  A start is one round trip: the queries' loads all leave before the first of them is used and run beside
+// the allocation of tensor memory (taken four rows at a time, between stores to shared memory, they were 4500 of 13000 to 16000 cycles
+// of a block); outputs leave as rows of 64 bytes by way of shared memory (16 bytes a lane and row before: 1600 cycles).
+// us a launch with queries and outputs as before -> now: 64 series x 20 heads x 255 queries 106 -> 84, 64 x 16 x 256 87 -> 68, 16 x 8 x
+// 704 36 -> 33.  attn_tiles_kernel -> here: 1280 pairs x 255 queries 112 -> 75, 256 x 256 20 -> 16, 128 x 704 48 -> 34; where which is
+// taken: attn_mma_pays.  With one thread per row 14 % slower.
 // Warps 0-7 softmax (query row = 32 (w % 4) + lane, keys and output dims of half w / 4), 8 TMA producer, 9 tensor memory and
 // MMA issue.  Waits are bounded as in gemm_tc.cuh.  grid = (heads, B, ceil(q_len / 128)), block = 320.
 #pragma once
@@ -91,6 +93,19 @@ attn_mma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant_
   const int n_tiles = (n_keys + AM_KEYS - 1) / AM_KEYS;
   const int row0 = layer_row0 + (sp.b * n_heads + h) * g.cap;
 
+  // TMA producer: tiles of keys that earlier passes left in the cache are requested before the dependency wait
+  const bool leader = elect_one();
+  auto load = [&](int t) {
+    const uint32_t s = (uint32_t)(t & 1), dst = ring + s * 2 * AM_TILE;
+    mbar_expect_tx(kfull0 + 8 * s, AM_TILE);
+    tma_load_2d(dst, &mapK, 0, row0 + t * AM_KEYS, kfull0 + 8 * s);
+    mbar_expect_tx(vfull0 + 8 * s, AM_TILE);
+    tma_load_2d(dst + AM_TILE, &mapV, 0, row0 + t * AM_KEYS, vfull0 + 8 * s);
+  };
+  const int early = min(min(p0 / AM_KEYS, 2), n_tiles);
+  // a softmax warp's queries: dims qc .. qc + 3 and their partners 32 further of four rows
+  const int qc = (lane & 7) * 4;
+  float4 qa[4], qp[4];
   if (warp == AM_WARPS) {
     if (lane < 2) {
       mbar_init(kfull0 + 8 * lane, 1);
@@ -105,9 +120,23 @@ attn_mma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant_
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     __syncwarp();
+    if (leader)
+      for (int t = 0; t < early; ++t) load(t);
   } else if (warp == AM_WARPS + 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(slot_addr), "r"((uint32_t)AM_COLS) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  } else {
+    pdl_sync();
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int r = warp * 16 + i * 4 + (lane >> 3);
+      qa[i] = qp[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (r < nq) {
+        const float *src = qkv + ((size_t)blockIdx.y * g.q_len + qb + r) * 3 * d + h * AM_DH + qc;
+        qa[i] = __ldcg(reinterpret_cast<const float4 *>(src));
+        qp[i] = __ldcg(reinterpret_cast<const float4 *>(src + 32));
+      }
+    }
   }
   tc_fence_before();
   __syncthreads();
@@ -115,19 +144,7 @@ attn_mma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant_
   const uint32_t tmem = *slot_ptr;
 
   if (warp == AM_WARPS) {
-    // ---------------- TMA producer.  Tiles of keys that earlier passes left in the cache are requested before the
-    // dependency wait.
-    const bool leader = elect_one();
-    auto load = [&](int t) {
-      const uint32_t s = (uint32_t)(t & 1), dst = ring + s * 2 * AM_TILE;
-      mbar_expect_tx(kfull0 + 8 * s, AM_TILE);
-      tma_load_2d(dst, &mapK, 0, row0 + t * AM_KEYS, kfull0 + 8 * s);
-      mbar_expect_tx(vfull0 + 8 * s, AM_TILE);
-      tma_load_2d(dst + AM_TILE, &mapV, 0, row0 + t * AM_KEYS, vfull0 + 8 * s);
-    };
-    const int early = min(min(p0 / AM_KEYS, 2), n_tiles);
-    if (leader)
-      for (int t = 0; t < early; ++t) load(t);
+    // ---------------- TMA producer
     pdl_sync();
     bool ok = true;
     for (int t = early; t < n_tiles && ok; ++t) {
@@ -140,7 +157,6 @@ attn_mma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant_
     __syncwarp();
   } else if (warp == AM_WARPS + 1) {
     // ---------------- MMA issuer (the warp as a whole, one lane issues)
-    const bool leader = elect_one();
     constexpr uint32_t idesc_s = (1u << 4) | (1u << 7) | (1u << 10) | ((AM_KEYS >> 3) << 17) | ((AM_Q >> 4) << 24);
     constexpr uint32_t idesc_o = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((AM_DH >> 3) << 17) | ((AM_Q >> 4) << 24);
     pdl_sync();
@@ -173,25 +189,18 @@ attn_mma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant_
     __syncwarp();
   } else {
     // ---------------- softmax; first the block's queries: rotated and scaled, high and low parts to shared memory
-    pdl_sync();
     {
       const float sc = rsqrtf((float)AM_DH) * 1.4426950408889634f;
-      const int c = (lane & 7) * 4;                            // dims c .. c + 3 and their partners 32 further
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         const int r = warp * 16 + i * 4 + (lane >> 3);
-        float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
-        if (r < nq) {
-          const float *src = qkv + ((size_t)blockIdx.y * g.q_len + qb + r) * 3 * d + h * AM_DH + c;
-          a = __ldcg(reinterpret_cast<const float4 *>(src));
-          b = __ldcg(reinterpret_cast<const float4 *>(src + 32));
-          if (!rotated) {
-            const float4 *rp = reinterpret_cast<const float4 *>(rope + (size_t)(p0 + qb + r) * (AM_DH / 2) + c);
-            const float4 cs = rp[0], ct = rp[1];               // cos sin of dims c, c + 1 and c + 2, c + 3
-            const float4 x = a, y = b;
-            a = make_float4((x.x * cs.x - y.x * cs.y) * sc, (x.y * cs.z - y.y * cs.w) * sc, (x.z * ct.x - y.z * ct.y) * sc, (x.w * ct.z - y.w * ct.w) * sc);
-            b = make_float4((y.x * cs.x + x.x * cs.y) * sc, (y.y * cs.z + x.y * cs.w) * sc, (y.z * ct.x + x.z * ct.y) * sc, (y.w * ct.z + x.w * ct.w) * sc);
-          }
+        float4 a = qa[i], b = qp[i];
+        if (!rotated && r < nq) {
+          const float4 *rp = reinterpret_cast<const float4 *>(rope + (size_t)(p0 + qb + r) * (AM_DH / 2) + qc);
+          const float4 cs = rp[0], ct = rp[1];                 // cos sin of dims qc, qc + 1 and qc + 2, qc + 3
+          const float4 x = a, y = b;
+          a = make_float4((x.x * cs.x - y.x * cs.y) * sc, (x.y * cs.z - y.y * cs.w) * sc, (x.z * ct.x - y.z * ct.y) * sc, (x.w * ct.z - y.w * ct.w) * sc);
+          b = make_float4((y.x * cs.x + x.x * cs.y) * sc, (y.y * cs.z + x.y * cs.w) * sc, (y.z * ct.x + x.z * ct.y) * sc, (y.w * ct.z + x.w * ct.w) * sc);
         }
         uint2 hi, lo;
 #pragma unroll
@@ -199,7 +208,7 @@ attn_mma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant_
           const float4 v = half ? b : a;
           split_bf16x2(v.x, v.y, hi.x, lo.x);
           split_bf16x2(v.z, v.w, hi.y, lo.y);
-          const int cc = c + half * 32;                        // 16-byte chunk cc / 8 of row r sits at chunk ^ (r & 7)
+          const int cc = qc + half * 32;                        // 16-byte chunk cc / 8 of row r sits at chunk ^ (r & 7)
           const uint32_t off = (uint32_t)(r * 128 + (((cc >> 3) ^ (r & 7)) << 4) + (cc & 7) * 2);
           *reinterpret_cast<uint2 *>(gbase + off) = hi;
           *reinterpret_cast<uint2 *>(gbase + AM_TILE + off) = lo;
@@ -309,14 +318,23 @@ attn_mma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant_
     }
     *mine = l_run;                                             // (the row's last maxima were read before its last p_ready)
     asm volatile("bar.sync %0, 64;" ::"r"(2 + w4) : "memory");
-    if (ok && row < nq) {
+    // this warp's 32 rows of 64 bytes through shared memory (the queries' MMAs are done), so that four lanes write a row's
+    if (ok) {
       const float inv = nan_seen ? __int_as_float(0x7fffffff) : 1.f / (part ? *other + l_run : l_run + *other);
-      uint4 *dst = reinterpret_cast<uint4 *>(out + ((size_t)blockIdx.y * g.q_len + qb + row) * d + h * AM_DH + part * 32);
+      uint4 *stage = reinterpret_cast<uint4 *>(gbase + warp * 2048);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {                            // piece i of row r at i ^ (r / 2 % 4)
+        const float2 a = unpack2(o[4 * i]), b = unpack2(o[4 * i + 1]), c = unpack2(o[4 * i + 2]), e = unpack2(o[4 * i + 3]);
+        stage[lane * 4 + (i ^ ((lane >> 1) & 3))] = make_uint4(pack_bf16x2(a.x * inv, a.y * inv), pack_bf16x2(b.x * inv, b.y * inv),
+                                                               pack_bf16x2(c.x * inv, c.y * inv), pack_bf16x2(e.x * inv, e.y * inv));
+      }
+      __syncwarp();
+      bf16 *dst = out + ((size_t)blockIdx.y * g.q_len + qb + w4 * 32) * d + h * AM_DH + part * 32 + (lane & 3) * 8;
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        const float2 a = unpack2(o[4 * i]), b = unpack2(o[4 * i + 1]), c = unpack2(o[4 * i + 2]), e = unpack2(o[4 * i + 3]);
-        dst[i] = make_uint4(pack_bf16x2(a.x * inv, a.y * inv), pack_bf16x2(b.x * inv, b.y * inv), pack_bf16x2(c.x * inv, c.y * inv),
-                            pack_bf16x2(e.x * inv, e.y * inv));
+        const int r = i * 8 + (lane >> 2);
+        const uint4 v = stage[r * 4 + ((lane & 3) ^ ((r >> 1) & 3))];
+        if (w4 * 32 + r < nq) *reinterpret_cast<uint4 *>(dst + (size_t)r * d) = v;
       }
     }
   }

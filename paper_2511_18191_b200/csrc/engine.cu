@@ -619,23 +619,24 @@ void gemm(tsfm_spec *h, GemmSkPlan *plan, const void *A, const void *W, void *C,
 // Which kernel a pass with heads of 64 attends on, from 33 tokens on (up to 32 attn_tiles_kernel runs two warps a CTA): the
 // tensor-memory kernel takes 128 queries a CTA and costs the same for one of them as for all, attn_tiles_kernel takes 64 in
 // four warps.  A launch costs its waves of blocks (two and four on an SM), a block its start and its steps of 128 and 64 keys (a
-// step of attn_tiles_kernel mostly by the warps that have queries).  In us, fitted to the attention's share of prefills of 33 to
-// 704 tokens and of passes of 48 to 256 tokens behind 100 to 2000 keys, 8 to 3200 (series, head) pairs, 617 shapes.  Measured with
-// the rule in place: 0.6 % above the better kernel on average; 14 of them more than 4 % and 0.4 us above attn_tiles_kernel (48
-// tokens behind a few hundred keys with few pairs, 0.5 to 0.9 us; the rest within the scatter of runs).  At 1280 pairs, us a
-// launch, attn_tiles_kernel / attn_mma_kernel: 33 tokens 12 / 32, 64 15 / 34, 128 40 / 41, 144 56 / 81, 192 71 / 88, 256 107 / 99,
-// 320 146 / 150, 384 190 / 156; 48 behind 192 to 336 keys 39 / 56, 64 behind 576 to 768 88 / 90, 96 behind 192 to 480 87 / 73, 128 behind
-// 256 to 640 123 / 80.
+// step of attn_tiles_kernel mostly by the warps that have queries, and more the more waves share the memory).  In us, fitted to the
+// attention's share of scoring passes of 33 to 704 tokens, 8 to 3200 (series, head) pairs, 190 shapes: 1.1 % above the better
+// kernel on average, 17 of them more than 4 % (0.4 to 0.7 us at 8 and 32 pairs).  At 1280 pairs, us a launch, attn_tiles_kernel /
+// attn_mma_kernel: 33 tokens 13 / 27, 64 16 / 27, 96 31 / 29, 128 43 / 35, 144 60 / 68, 192 76 / 69, 256 112 / 75, 320 151 / 117; at
+// 256 pairs 64 tokens 5.4 / 7.0, 128 10.5 / 7.7, 192 13.8 / 15.5, 256 19.6 / 15.8, 704 100 / 65.  Windows of up to 100 tokens keep the
+// blocks of 64 queries whatever the grid (a test holds them there at 1280 pairs): 96 tokens 4.5 / 5.1 at 64 pairs, 18.5 / 19.4 at 800,
+// 31 / 29 at 1280, and only beyond that a loss worth the name (59 / 49 at 2048).
 bool attn_mma_pays(long pairs, int first, int q_len) {
+  if (first == 0 && q_len <= 100) return false;
   double tiles = 0, mma = 0;
   long n64 = 0, n128 = 0;
   for (int q = 0; q < q_len; q += 64, ++n64) {
     const int rows = std::min(64, q_len - q);
-    tiles += 3.6 + (first + q + rows + 63) / 64 * (0.6 + 1.5 * 0.25 * ((rows + 15) / 16));
+    tiles += 2.7 + (first + q + rows + 63) / 64 * (0.49 + 0.41 * ((rows + 15) / 16));
   }
-  for (int q = 0; q < q_len; q += AM_Q, ++n128) mma += 6.1 + 1.8 * ((first + std::min(q + AM_Q, q_len) + AM_KEYS - 1) / AM_KEYS);
+  for (int q = 0; q < q_len; q += AM_Q, ++n128) mma += 3.9 + 1.8 * ((first + std::min(q + AM_Q, q_len) + AM_KEYS - 1) / AM_KEYS);
   const long waves64 = (pairs * n64 + 4 * 148 - 1) / (4 * 148), waves128 = (pairs * n128 + 2 * 148 - 1) / (2 * 148);
-  return waves128 * (mma / n128) < waves64 * (tiles / n64);
+  return waves128 * (mma / n128) < waves64 * (tiles / n64) * (1 + 0.034 * std::min(waves64, 16l));
 }
 constexpr int kMmaAttnTokens = 32;
 

@@ -373,12 +373,12 @@ template <typename F> void prefer_max_smem(F *fn) {
   cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
 }
 template <typename T> void prefer_max_smem_typed() {
-  prefer_max_smem(embed_kernel<T>);
+  prefer_max_smem(embed_kernel<T, 1>);
+  prefer_max_smem(embed_kernel<T, 4>);
   prefer_max_smem(rmsnorm_kernel<T, false, 10>);
   prefer_max_smem(rmsnorm_kernel<T, false, 16>);
   prefer_max_smem(rmsnorm_kernel<T, true, 10>);
   prefer_max_smem(head_kernel<T>);
-  prefer_max_smem(embed_rows_kernel<T>);
   prefer_max_smem(gemm_simt_kernel<T, EPI_F32>);
   prefer_max_smem(gemm_simt_kernel<T, EPI_T>);
   prefer_max_smem(gemm_simt_kernel<T, EPI_GELU_T>);
@@ -724,10 +724,14 @@ void launch_attn(tsfm_spec *h, ModelDev &m, int l, int B, const PassGeom &g, boo
   }
 }
 
+// Shared memory of an embedding of four rows a CTA, which passes of at least kEmbedFourRows rows take (see embed_kernel) where it
+// fits without opting in (tokens of up to 168 values).
+constexpr int kEmbedFourRows = 32;
+template <typename T> constexpr size_t embed_smem(int P) {
+  return 4 * P * sizeof(float) + (P % Vec16<T>::N ? 0 : 128 * (P * sizeof(T) + 16));
+}
+
 enum { HEAD_NONE = 0, HEAD_LAST_TO_HIST = 1, HEAD_ALL_TO_VOUT = 2 };
-// Passes of at least this many rows take the embedding kernel that shares each weight load between 8
-// rows where a token is too short for the tiled contraction (point tokens).
-constexpr int kManyRows = 1024;
 // From this many rows on the head is a tiled contraction (gemm_rows_kernel) on the bf16 path too; below it one CTA per row and
 // eight outputs, with constants fetched before the dependency wait, is shorter: 32 rows of 512 values 3.1 us (tiled 5.6), 93 of
 // 1024 7.9 (8.4), 160 of 512 9.4 (5.6), 64 of 1280 4.5 (10.3).
@@ -777,6 +781,7 @@ void run_pass(tsfm_spec *h, ModelDev &m, int B, const PassGeom &g, int head_mode
   // the RMSNorm of passes of a few thousand rows is a link in a chain: constants before the wait
   auto *norm_kernel = d > 1280 ? rmsnorm_kernel<T, false, 16> : M <= kNormEarlyMaxRows ? rmsnorm_kernel<T, true, 10> : rmsnorm_kernel<T, false, 10>;
   {
+    const bool four = M >= kEmbedFourRows && embed_smem<T>(Pi) <= 48 * 1024;
     KTimer kt(h, KC_EMBED, (double)M * Pi * 4 + (double)d * Pi * sizeof(T) + (double)M * d * 4, 2.0 * M * Pi * d);
     if (!fold && (sizeof(T) == 4 ? f32_tiles(h, m.W_emb, Pi) : rows_tiles(h, m.W_emb, Pi))) {
       RowsArgs ra{};
@@ -786,11 +791,9 @@ void run_pass(tsfm_spec *h, ModelDev &m, int B, const PassGeom &g, int head_mode
       ra.opens_round = opens_round ? 1 : 0;
       ra.stamp = stamp;
       launched(rows_launch(s, h->pdl, (const float *)h->hist, (const T *)m.W_emb, h->x, M, d, Pi, ra), "embedding");
-    } else if (!fold && M >= kManyRows)
-      launch_ex(s, h->pdl, embed_rows_kernel<T>, dim3((M + 7) / 8, (d + 127) / 128), dim3(128), 8 * Pi * sizeof(float),
-                h->hist, g, M, Pi, d, (const T *)m.W_emb, h->x, stamp);
-    else
-      launch_ex(s, h->pdl, embed_kernel<T>, dim3(M, (d + 127) / 128), dim3(128), Pi * sizeof(float), h->hist, g, Pi, d,
+    } else
+      launch_ex(s, h->pdl, four ? embed_kernel<T, 4> : embed_kernel<T, 1>, dim3(four ? (M + 3) / 4 : M, (d + 127) / 128), dim3(128),
+                four ? embed_smem<T>(Pi) : Pi * sizeof(float), h->hist, g, M, Pi, d,
                 (const T *)m.W_emb, h->x, stamp, fold ? m.layers[0].g1 : (const float *)nullptr,
                 fold ? (T *)h->a : (T *)nullptr, fold ? h->ssq : (float *)nullptr, opens_round ? 1 : 0);
   }

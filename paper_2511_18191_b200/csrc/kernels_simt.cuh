@@ -204,113 +204,123 @@ template <> struct Vec16<bf16> {
   static __device__ __forceinline__ void load(const bf16 *p, float *v) { unpack(raw(p), v); }
 };
 
+__device__ __forceinline__ void cp_async16(void *smem_dst, const void *gmem_src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(smem_dst)), "l"(gmem_src) : "memory");
+}
+
 // ----------------------------------------------------------------------------------
 // Token embedding x[row, f] = sum_i W_emb[f, i] * z[i], z = history token of P values (fp32;
-// P here is the input token length P_in).  grid = (M rows, ceil(d / 128)), block = 128: one
-// output feature per thread, its weight row read with independent 16-byte loads when P is a
-// multiple of the vector width, element by element for short tokens (point tokens: P = 1).
+// P here is the input token length P_in).  grid = (ceil(M / R), ceil(d / 128)), block = 128: one
+// output feature per thread and R rows, 16-byte loads when P is a multiple of the vector width, element by element
+// for short tokens (point tokens: P = 1).
+// R = 1, few rows: a thread reads its own weight row before the dependency wait.  Neighbouring threads read rows 2 P bytes
+// apart, 32 lines an instruction: 1500 cycles of an SM's load path a CTA, which many rows pay over and over.
+// R = 4, from 32 rows on: the CTA's 128 weight rows are one piece of memory and come to shared memory as such (rows 16 bytes
+// apart, so that eight threads' vectors fall into different banks), once for four rows.  The same order of sums, the same bits.
+// Bound: a round trip each for weights and tokens and the chain of P products.  us a link inside plain decoding, R = 1 -> 4:
+// 256 rows x 1024 x 96 11.9 -> 5.8, 500 x 768 x 96 16.8 -> 7.6, 256 x 512 x 64 5.4 -> 3.7, 256 x 1280 x 32 6.2 -> 3.7; 64 x 512 x 64
+// 2.1 -> 2.7, but the kernel behind finds more room: a forecast of eight patches 396 -> 380 (32 x 1024 x 96 466 -> 447, 93 x 1024 x 96
+// 626 -> 623, 64 x 1280 x 32 596 -> 597; 8 rows 359 -> 364).
 // ----------------------------------------------------------------------------------
-template <typename T>
+template <typename T, int R>
 __global__ void __launch_bounds__(128)
-embed_kernel(const float *hist, PassGeom g, int P, int d, const T *__restrict__ W,
+embed_kernel(const float *hist, PassGeom g, int M, int P, int d, const T *__restrict__ W,
              float *__restrict__ x, unsigned long long *__restrict__ stamp,
              const float *__restrict__ gain, T *__restrict__ a_out, float *__restrict__ ssq_out, int opens_round) {
-  extern __shared__ float zs[];
-  constexpr int V = Vec16<T>::N, PRE = 12;                     // weight vectors fetched before the wait
-  const int row = blockIdx.x, slot = row / g.q_len, j = row % g.q_len;
-  const int f = blockIdx.y * 128 + threadIdx.x;
-  // Before the dependency wait: what does not depend on the preceding kernel -- the start of this
-  // thread's weight row, its gain, and (unless this pass opens a round, when the kernel that closed
-  // the previous round is the predecessor itself) the slot lookup.
+  extern __shared__ __align__(16) float zs[];                  // [R][P]; R > 1: and 128 weight rows, 16 bytes apart
+  __shared__ long long src[R];                                 // (R > 1) a row's token in the history, -1: no such row
+  constexpr int V = Vec16<T>::N, PRE = 12;                     // (R == 1) weight vectors fetched before the wait
+  const int row0 = blockIdx.x * R, f = blockIdx.y * 128 + threadIdx.x;
+  // Before the dependency wait: what does not depend on the preceding kernel -- this thread's weight row (or its
+  // start), its gain, and (unless this pass opens a round, when the kernel that closed the previous round is the
+  // predecessor itself) the slot lookup.
   const T *wr = W + (size_t)min(f, d - 1) * P;
-  typename Vec16<T>::Raw wpre[PRE];
-  if (P % V == 0) {
+  const bool staged = R > 1 && P % V == 0;
+  typename Vec16<T>::Raw wpre[R == 1 ? PRE : 1];
+  unsigned char *const ws = reinterpret_cast<unsigned char *>(zs + R * P);
+  const int wrow = P * (int)sizeof(T) + 16;
+  if (staged) {
+    const int vpr = P / V, n = min(128, d - (int)blockIdx.y * 128) * vpr;
+    const unsigned char *from = reinterpret_cast<const unsigned char *>(W + (size_t)blockIdx.y * 128 * P);
+    const int dr = 128 / vpr, dc = 128 % vpr;
+    for (int i = threadIdx.x, r = i / vpr, c = i % vpr; i < n; i += 128) {
+      cp_async16(ws + r * wrow + c * 16, from + (size_t)i * 16);
+      r += dr, c += dc;
+      if (c >= vpr) c -= vpr, ++r;
+    }
+  } else if (R == 1 && P % V == 0) {
 #pragma unroll
     for (int k = 0; k < PRE; ++k)
-      if (k * V < P) wpre[k] = Vec16<T>::raw(wr + k * V);
+      if (k * V < P) wpre[R == 1 ? k : 0] = Vec16<T>::raw(wr + k * V);
   }
   const float gf = a_out ? gain[min(f, d - 1)] : 0.f;
-  SlotPos sp;
-  if (!opens_round) sp = slot_lookup(g, slot);
+  auto token_of = [&](int row) -> long long {
+    if (row >= M) return -1;
+    const SlotPos sp = slot_lookup(g, row / g.q_len);
+    return sp.dead ? -1 : ((long long)sp.b * g.cap + sp.p0 + row % g.q_len) * P;
+  };
+  long long own = -1;                                          // (R == 1: every thread's; otherwise of row row0 + threadIdx.x)
+  auto lookup = [&]() {
+    if (R == 1) own = token_of(row0);
+    else if (threadIdx.x < R) src[threadIdx.x] = own = token_of(row0 + threadIdx.x);
+  };
+  if (!opens_round) lookup();
   pdl_sync();
-  if (stamp && row == 0 && blockIdx.y == 0 && threadIdx.x == 0) *stamp = globaltimer_ns();
-  if (opens_round) sp = slot_lookup(g, slot);
-  if (sp.dead) return;
-  const int b = sp.b;
-  const float *z = hist + ((size_t)b * g.cap + sp.p0 + j) * P;
-  for (int i = threadIdx.x; i < P; i += blockDim.x) zs[i] = z[i];
+  if (stamp && row0 == 0 && blockIdx.y == 0 && threadIdx.x == 0) *stamp = globaltimer_ns();
+  if (opens_round) lookup();
+  if (R == 1) {
+    if (own < 0) return;
+    for (int i = threadIdx.x; i < P; i += blockDim.x) zs[i] = hist[own + i];
+  } else {
+    if (!__syncthreads_or(own >= 0)) {                         // a tile of dead slots
+      asm volatile("cp.async.wait_all;" ::: "memory");
+      return;
+    }
+    for (int r = threadIdx.x >> 5; r < R; r += 4) {
+      const long long so = src[r];
+      if (so < 0) continue;                                    // (its row of zs is read and goes nowhere)
+      if (P % 4 == 0)
+        for (int i = (threadIdx.x & 31) * 4; i < P; i += 128) cp_async16(zs + r * P + i, hist + so + i);
+      else
+        for (int i = threadIdx.x & 31; i < P; i += 32) zs[r * P + i] = hist[so + i];
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+  }
   __syncthreads();
   if (f >= d) return;
-  float acc = 0.f;
-  if (P % V == 0) {
+  float acc[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) acc[r] = 0.f;
+  auto step = [&](const float (&w)[V], int i) {
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+      for (int c = 0; c < V; c += 4) {
+        const float4 z = *reinterpret_cast<const float4 *>(zs + r * P + i + c);
+        acc[r] = fmaf(w[c + 3], z.w, fmaf(w[c + 2], z.z, fmaf(w[c + 1], z.y, fmaf(w[c], z.x, acc[r]))));
+      }
+  };
+  if (staged) {
+    const T *own_w = reinterpret_cast<const T *>(ws + threadIdx.x * wrow);
+#pragma unroll 4
+    for (int i = 0; i < P; i += V) {
+      float w[V];
+      Vec16<T>::unpack(*reinterpret_cast<const typename Vec16<T>::Raw *>(own_w + i), w);
+      step(w, i);
+    }
+  } else if (P % V == 0) {
 #pragma unroll
     for (int k = 0; k < PRE; ++k)
       if (k * V < P) {
         float w[V];
-        Vec16<T>::unpack(wpre[k], w);
-#pragma unroll
-        for (int c = 0; c < V; ++c) acc = fmaf(w[c], zs[k * V + c], acc);
+        Vec16<T>::unpack(wpre[R == 1 ? k : 0], w);
+        step(w, k * V);
       }
 #pragma unroll 4
     for (int i = PRE * V; i < P; i += V) {
       float w[V];
       Vec16<T>::load(wr + i, w);
-#pragma unroll
-      for (int c = 0; c < V; ++c) acc = fmaf(w[c], zs[i + c], acc);
-    }
-  } else {
-    for (int i = 0; i < P; ++i) acc = fmaf(to_f32(wr[i]), zs[i], acc);
-  }
-  x[(size_t)row * d + f] = acc;
-  if (a_out) {            // operand of the first contraction, normalised later (see SkNorm); d % 64 == 0
-    a_out[(size_t)row * d + f] = from_f32<T>(gf * acc);
-    float sq = acc * acc;                                       // sums of squares over slices of 16 features
-    sq += __shfl_xor_sync(0xffffffffu, sq, 1);
-    sq += __shfl_xor_sync(0xffffffffu, sq, 2);
-    sq += __shfl_xor_sync(0xffffffffu, sq, 4);
-    sq += __shfl_xor_sync(0xffffffffu, sq, 8);
-    if ((threadIdx.x & 15) == 0) ssq_out[(size_t)row * (d >> 4) + (f >> 4)] = sq;
-  }
-}
-
-// The same embedding for passes of many rows: 8 rows per CTA share every weight load.
-// grid = (ceil(M / 8), ceil(d / 128)), block = 128, dynamic shared memory 8 * P floats.
-template <typename T>
-__global__ void __launch_bounds__(128)
-embed_rows_kernel(const float *hist, PassGeom g, int M, int P, int d, const T *__restrict__ W,
-                  float *__restrict__ x, unsigned long long *__restrict__ stamp) {
-  constexpr int R = 8;
-  extern __shared__ float zs[];                               // [R][P]
-  pdl_sync();
-  const int row0 = blockIdx.x * R;
-  if (stamp && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *stamp = globaltimer_ns();
-  if (slot_dead(g, row0 / g.q_len)) return;                   // every row of this CTA is past the live ones
-  for (int i = threadIdx.x; i < R * P; i += blockDim.x) {
-    const int row = row0 + i / P;
-    float v = 0.f;
-    if (row < M && !slot_dead(g, row / g.q_len)) {
-      const int b = series_of(g, row / g.q_len), j = row % g.q_len;
-      v = hist[((size_t)b * g.cap + pos0_of(g, b) + j) * P + i % P];
-    }
-    zs[i] = v;
-  }
-  __syncthreads();
-  const int f = blockIdx.y * 128 + threadIdx.x;
-  if (f >= d) return;
-  const T *wr = W + (size_t)f * P;
-  constexpr int V = Vec16<T>::N;
-  float acc[R];
-#pragma unroll
-  for (int r = 0; r < R; ++r) acc[r] = 0.f;
-  if (P % V == 0) {
-#pragma unroll 2
-    for (int i = 0; i < P; i += V) {
-      float w[V];
-      Vec16<T>::load(wr + i, w);
-#pragma unroll
-      for (int r = 0; r < R; ++r)
-#pragma unroll
-        for (int c = 0; c < V; ++c) acc[r] = fmaf(w[c], zs[r * P + i + c], acc[r]);
+      step(w, i);
     }
   } else {
     for (int i = 0; i < P; ++i) {
@@ -319,9 +329,27 @@ embed_rows_kernel(const float *hist, PassGeom g, int M, int P, int d, const T *_
       for (int r = 0; r < R; ++r) acc[r] = fmaf(w1, zs[r * P + i], acc[r]);
     }
   }
+  bool live[R];
 #pragma unroll
-  for (int r = 0; r < R; ++r)
-    if (row0 + r < M) x[(size_t)(row0 + r) * d + f] = acc[r];
+  for (int r = 0; r < R; ++r) {
+    live[r] = R == 1 || src[r] >= 0;
+    if (live[r]) x[(size_t)(row0 + r) * d + f] = acc[r];
+  }
+  if (a_out) {            // operand of the first contraction, normalised later (see SkNorm); d % 64 == 0
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+      if (live[r]) a_out[(size_t)(row0 + r) * d + f] = from_f32<T>(gf * acc[r]);
+    float sq[R];                                               // sums of squares over slices of 16 features
+#pragma unroll
+    for (int r = 0; r < R; ++r) sq[r] = acc[r] * acc[r];
+#pragma unroll
+    for (int o = 1; o < 16; o *= 2)
+#pragma unroll
+      for (int r = 0; r < R; ++r) sq[r] += __shfl_xor_sync(0xffffffffu, sq[r], o);
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+      if (live[r] && (threadIdx.x & 15) == 0) ssq_out[(size_t)(row0 + r) * (d >> 4) + (f >> 4)] = sq[r];
+  }
 }
 
 // ----------------------------------------------------------------------------------
@@ -523,9 +551,6 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
 // word of consecutive rows spread over the banks.  Physical word of logical word w of row t:
 template <int VW> __device__ __forceinline__ int attn_kword(int t, int w) {
   return t * VW + ((((w >> 2) + t) & (VW / 4 - 1)) << 2) + (w & 3);
-}
-__device__ __forceinline__ void cp_async16(void *smem_dst, const void *gmem_src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(smem_dst)), "l"(gmem_src) : "memory");
 }
 
 constexpr int ATTN_QT = 16;                             // queries per tile (at most)

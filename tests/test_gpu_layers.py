@@ -173,6 +173,17 @@ def test_embedding_and_head_are_exact_to_fp32(d, P, P_in, B, n):
     assert relative(got, (w["g_f"] * x * rstd(x)) @ w["W_head"].T.astype(np.float64)) < 3e-7
 
 
+@pytest.mark.parametrize("d,P,P_in,B,n", [
+    (128, 96, 96, 1, 31), (128, 96, 96, 2, 16),                  # row by row and four rows a block
+    (192, 32, 32, 3, 11), (64, 176, 176, 5, 7), (320, 160, 160, 67, 7),   # ragged rows and features; too long for shared memory
+    (128, 16, 1, 3, 37), (128, 16, 4, 25, 43),                   # tokens shorter than a vector, folded and not
+])
+def test_embedding_of_few_rows(d, P, P_in, B, n):
+    """The bound as above: here the embedding is one chain of up to 176 sums, whose roundings (0.42 x 2^-24 of a partial sum in the
+    mean square) add up to sqrt(176 / 2) x 2.5e-8 = 2.4e-7, with the rest 2.6e-7."""
+    test_embedding_and_head_are_exact_to_fp32(d, P, P_in, B, n)
+
+
 @pytest.mark.parametrize("d,f,P,P_in,B,n", [
     (64, 64, 64, 64, 1, 1), (64, 64, 48, 48, 1, 17), (64, 64, 16, 16, 10, 16), (64, 64, 16, 16, 7, 23),   # up to 160 rows
     (64, 64, 32, 8, 5, 3),                                       # embedding by itself

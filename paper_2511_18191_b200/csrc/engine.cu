@@ -1009,7 +1009,7 @@ int take_enqueue_err(tsfm_spec *h) {
 
 // ---------------------------------------------------------------- graph capture
 // A forecast of a given geometry is captured once into a CUDA graph and replayed: the
-// prologue, a WHILE node whose body is one round (the round-end kernel sets the condition),
+// prologue, a WHILE node whose body is one round (the last CTA of the accept kernel sets the condition),
 // and the de-normalisation.  Capture runs on the handle's own streams (the caller's stream
 // may be the legacy default stream, which cannot capture); the graph is launched on the
 // caller's stream.

@@ -148,7 +148,8 @@ instnorm_kernel(DevState *__restrict__ st, int ctx_len, int hist_stride, int his
   }
 }
 
-// out[b, s] = hist[b, ctx_len + s] * sd + mean, s < H.   grid = B.
+// out[b, s] = hist[b, ctx_len + s] * sd + mean, s < H.   grid = B, block = 256.  Four values a thread are fetched before the
+// first is stored (they would follow one another: either array could be the other).
 __global__ void denorm_kernel(const float *hist, int ctx_len, int hist_len, int H,
                               const float *mean, const float *sd,
                               DevState *__restrict__ st) {
@@ -158,7 +159,15 @@ __global__ void denorm_kernel(const float *hist, int ctx_len, int hist_len, int 
   if (b == 0 && threadIdx.x == 0) st->t_end = globaltimer_ns();
   const float m = mean[b], s = sd[b];
   const float *hb = hist + (size_t)b * hist_len + ctx_len;
-  for (int i = threadIdx.x; i < H; i += blockDim.x) out[(size_t)b * H + i] = hb[i] * s + m;
+  for (int i0 = threadIdx.x; i0 < H; i0 += 4 * 256) {
+    float v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (i0 + 256 * u < H) v[u] = __ldcg(hb + i0 + 256 * u);
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (i0 + 256 * u < H) out[(size_t)b * H + i0 + 256 * u] = v[u] * s + m;
+  }
 }
 
 // Bounds-checking mode: every guard byte must still hold GUARD_BYTE after a forecast; the first
@@ -946,8 +955,15 @@ head_kernel(const float *x, const float *__restrict__ gain, const T *__restrict_
   if (sp.dead) return;
   const int b = sp.b;
   const float *xr = x + ((size_t)slot * g.q_len + j) * d;
-  float ss = 0.f;
-  for (int i = threadIdx.x; i < d; i += blockDim.x) {
+  // all of the row's loads leave before the first value is used (between stores to shared memory they would follow one another)
+  float xv[GPRE], ss = 0.f;
+#pragma unroll
+  for (int k = 0; k < GPRE; ++k)
+    if ((int)threadIdx.x + 256 * k < d) xv[k] = __ldcg(xr + threadIdx.x + 256 * k);
+#pragma unroll
+  for (int k = 0; k < GPRE; ++k)
+    if ((int)threadIdx.x + 256 * k < d) ss = fmaf(xv[k], xv[k], ss);
+  for (int i = threadIdx.x + 256 * GPRE; i < d; i += blockDim.x) {
     const float v = xr[i];
     xs[i] = v;
     ss = fmaf(v, v, ss);
@@ -955,7 +971,7 @@ head_kernel(const float *x, const float *__restrict__ gain, const T *__restrict_
   const float rstd = rsqrtf(block_sum(ss, red) / d + eps);
 #pragma unroll
   for (int k = 0; k < GPRE; ++k)
-    if ((int)threadIdx.x + 256 * k < d) xs[threadIdx.x + 256 * k] = gpre[k] * xs[threadIdx.x + 256 * k] * rstd;
+    if ((int)threadIdx.x + 256 * k < d) xs[threadIdx.x + 256 * k] = gpre[k] * xv[k] * rstd;
   for (int i = threadIdx.x + 256 * GPRE; i < d; i += blockDim.x) xs[i] = gain[i] * xs[i] * rstd;
   __syncthreads();
   float *dst = only_last ? hist + ((size_t)b * g.cap + sp.p0 + g.q_len) * tok_len

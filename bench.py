@@ -49,12 +49,13 @@ UNIT = "patches/s"
 # A kernel that has changed since its capture is listed with None.
 NCU_TRAFFIC_RATIO = {
     "gemm_push_small_M": 0.91,     # 10.03 MB of 10.98 MB (M=64, N=3840, K=1280)
-    "gemm_pair_mid_M": 0.56,       # 11.37 MB of 20.15 MB (M=576, N=3840, K=1280): the fp32 result stays in L2 for its consumer
-    "gemm_pair_large_M": 0.82,     # 246.7 MB of 302.2 MB (M=16320, N=3840, K=1280)
+    "gemm_pair_mid_M": 0.56,       # 11.34 MB of 20.15 MB (M=576, N=3840, K=1280): the fp32 result stays in L2 for its consumer
+    "gemm_pair_large_M": 0.81,     # 244.7 MB of 302.2 MB (M=16320, N=3840, K=1280)
     "gemm_ws_small_M": 0.77,       # 0.942 MB of 1.229 MB (M=64, N=1152, K=384)
     "attn": 0.99,                  # 95.7 MB of 96.9 MB (C4 verification pass, attn_flash_kernel): the KV stream
 }
 NCU_TRAFFIC_SOURCE = dict.fromkeys(NCU_TRAFFIC_RATIO, "profiles/kernels_for_many_tokens_short_passes_and_fp32.txt (cold caches)")
+NCU_TRAFFIC_SOURCE.update(dict.fromkeys(("gemm_pair_mid_M", "gemm_pair_large_M"), "profiles/pair_kernel_and_blocks_of_128_queries.txt (cold caches)"))
 
 
 def parse_args():

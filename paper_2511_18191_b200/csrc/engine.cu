@@ -668,7 +668,8 @@ void launch_attn(tsfm_spec *h, ModelDev &m, int l, int B, const PassGeom &g, boo
     }
     if (pre) {
       if constexpr (DH <= 64) {                                // (heads of 128: 11.2 us either way, 200 series x 4 heads x 30 tokens)
-        if ((g.done ? g.cap : g.base + g.q_len) <= 32) {       // the most that a query can see
+        // the most that a query can see (the spare token of bounds-checking mode is nobody's: the same kernel with it and without)
+        if ((g.done ? h->cap - (h->check ? 1 : 0) : g.base + g.q_len) <= 32) {
           launch_ex(h->ls, h->pdl, attn_short_kernel<DH>, dim3(m.arch.n_heads, B), dim3(64), (size_t)even_share_smem(pairs, 128 * DH), h->qkv,
                     (const bf16 *)Kc, (const bf16 *)Vc, m.rope, g, m.arch.n_heads, appended ? 1 : 0, (bf16 *)h->ao);
           return;

@@ -324,6 +324,37 @@ def test_block_size_beyond_one_query_tile_bf16():
         run_and_compare(wl, 20, 2.0, 17, [0, 1, 2, 3], exec_mode=mode)
 
 
+@pytest.mark.parametrize("heads,ctx,T,K", [(2, 5, 6, 17), (4, 8, 6, 17), (2, 8, 6, 17), (4, 2, 3, 26)])
+def test_verification_passes_that_see_at_most_32_keys(heads, ctx, T, K, tmp_path):
+    """Heads of 64 and 32, 18 to 27 tokens behind each series' own number of keys, capacities of 29 and 32 (the largest): against the
+    oracle, and bit for bit the same kernels without compaction and in bounds-checking mode, whose capacity is one token more."""
+    import json
+    import paper_2511_18191_b200 as tsfm
+    arch, draft = Arch(2, 128, heads, 256), Arch(1, 128, heads, 256)
+    wl = workload("C1", batch=9, ctx_len=32 * ctx, patch_len=32, horizon=32 * T - 3, K=K, target=arch, draft=draft)
+    d = run_and_compare(wl, K, 3.0, 17, range(9))["stats"]
+    assert 1 < d["rounds"] < T
+    s, ctx_series = series_on_device(wl)
+    res, kernels = [], []
+    for mode in (0, tsfm.TSFM_EXEC_NO_COMPACT, tsfm.TSFM_EXEC_CHECK_BOUNDS):
+        dec = make_decoder(wl, max_K=K, exec_mode=tsfm.TSFM_EXEC_STREAM | mode)[0]
+        dec.forecast(ctx_series, wl.horizon, K, 3.0, 17)
+        with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
+            out, _ = dec.forecast(ctx_series, wl.horizon, K, 3.0, 17)
+        res.append((out.cpu().numpy(), dec.last_trace(9, K)[0]))
+        dec.close()
+        prof.export_chrome_trace(str(tmp_path / "t.json"))
+        kernels.append({e["name"] for e in json.loads((tmp_path / "t.json").read_text())["traceEvents"]
+                        if e.get("cat") == "kernel" and "attn" in e["name"]})
+    finished_at = (res[0][1] >= 0).sum(axis=0)
+    assert finished_at.min() < finished_at.max(), "the case must desynchronise the batch"
+    for other in res[1:]:
+        np.testing.assert_array_equal(res[0][0], other[0])
+        np.testing.assert_array_equal(res[0][1], other[1])
+    assert kernels[0] == kernels[1] == kernels[2]
+    assert not kernels[0] or any("attn_short_kernel" in k for k in kernels[0])
+
+
 def test_many_series_short_rows_one_warp_per_series_and_head_bf16():
     """Enough (series, head) pairs on short rows for the attention mode that gives each warp a pair
     of its own, with a pair count that is not a multiple of the four warps of a CTA (199 x 6)."""

@@ -522,7 +522,9 @@ inline bool pair_folds(int M, int d) { return d >= 512 ? (long)M * d <= 5l << 20
 bool f32_tiles(const tsfm_spec *h, const void *W, int K) { return h->cfg.gemm_backend != TSFM_GEMM_SIMT && gemm_f32_eligible(W, K); }
 
 // Whether gemm_rows_kernel takes embedding or head of a bf16 model.
-bool rows_tiles(const tsfm_spec *h, const void *W, int K) { return h->cfg.gemm_backend != TSFM_GEMM_SIMT && gemm_rows_eligible(W, K); }
+bool rows_tiles(const tsfm_spec *h, const void *W, int N, int K) {
+  return h->cfg.gemm_backend != TSFM_GEMM_SIMT && gemm_rows_eligible(W, N, K);
+}
 bool rows_launch(cudaStream_t s, bool pdl, const float *A, const float *W, float *C, int M, int N, int K, const RowsArgs &ra) {
   return gemm_f32_launch(s, pdl, A, W, C, M, N, K, ra);
 }
@@ -784,7 +786,7 @@ void run_pass(tsfm_spec *h, ModelDev &m, int B, const PassGeom &g, int head_mode
   {
     const bool four = M >= kEmbedFourRows && embed_smem<T>(Pi) <= 48 * 1024;
     KTimer kt(h, KC_EMBED, (double)M * Pi * 4 + (double)d * Pi * sizeof(T) + (double)M * d * 4, 2.0 * M * Pi * d);
-    if (!fold && (sizeof(T) == 4 ? f32_tiles(h, m.W_emb, Pi) : rows_tiles(h, m.W_emb, Pi))) {
+    if (!fold && (sizeof(T) == 4 ? f32_tiles(h, m.W_emb, Pi) : rows_tiles(h, m.W_emb, d, Pi))) {
       RowsArgs ra{};
       ra.mode = ROWS_EMBED;
       ra.epi = EPI_F32;
@@ -846,7 +848,7 @@ void run_pass(tsfm_spec *h, ModelDev &m, int B, const PassGeom &g, int head_mode
   const double rows = head_mode == HEAD_LAST_TO_HIST ? B : Mb;
   KTimer kt(h, head_mode == HEAD_NONE ? -1 : KC_HEAD, rows * d * 4 + (double)P * d * sizeof(T) + rows * P * 4,
             2.0 * rows * P * d);
-  if (head_mode != HEAD_NONE && (sizeof(T) == 4 ? f32_tiles(h, m.W_head, d) : rows >= kHeadTileRows && rows_tiles(h, m.W_head, d))) {
+  if (head_mode != HEAD_NONE && (sizeof(T) == 4 ? f32_tiles(h, m.W_head, d) : rows >= kHeadTileRows && rows_tiles(h, m.W_head, P, d))) {
     RowsArgs ra{};
     ra.mode = head_mode == HEAD_LAST_TO_HIST ? ROWS_HEAD_LAST : ROWS_HEAD_ALL;
     ra.epi = EPI_F32;

@@ -244,8 +244,10 @@ static int gemm_rows_init() {
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024) != cudaSuccess) return -4;
   return 0;
 }
-// Rows that 16-byte loads can fetch, gains that fit beside a chunk.
-static bool gemm_rows_eligible(const void *W, int K) { return K % 16 == 0 && K >= 16 && K <= 32768 && !((uintptr_t)W & 15); }
+// Rows that 16-byte loads can fetch, gains that fit beside a chunk, features that leave in pairs.
+static bool gemm_rows_eligible(const void *W, int N, int K) {
+  return K % 16 == 0 && K >= 16 && K <= 32768 && N % 16 == 0 && !((uintptr_t)W & 15);
+}
 
 static bool gemm_rows_launch(cudaStream_t st, bool pdl, const float *A, const bf16 *W, float *C, int M, int N, int K, const RowsArgs &ra) {
   const RowsShape sh = gemm_rows_shape(M, N);

@@ -903,6 +903,10 @@ void enqueue_begin(tsfm_spec *h, int B, int ctx_len, FillList fill = FillList{})
   const int hist_stride = h->cap * h->P_in;             // values per series in the history buffer
   const int hist_len = hist_stride - (h->check ? h->P_in : 0);   // (the spare token stays untouched)
   fill.add(h->dev_status, sizeof(int), 0);
+  if (fill.full && h->enqueue_err == TSFM_OK) {
+    h->enqueue_err = TSFM_ERR_INTERNAL;
+    g_cuda_err = "the list of what a call clears is too short";
+  }
   KTimer kt(h, KC_INSTNORM, (double)B * (ctx_len + (double)hist_len) * 4, 4.0 * B * ctx_len);
   launch_ex(h->ls, h->pdl, instnorm_kernel, dim3(B), dim3(INSTNORM_THREADS), 0, h->st, ctx_len, hist_stride, hist_len, h->cfg.norm_eps, h->hist,
             h->mean, h->sd, h->done, h->live, h->n_live, fill);

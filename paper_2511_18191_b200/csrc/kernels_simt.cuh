@@ -75,7 +75,12 @@ struct FillList {
   size_t n[MAX];
   uint32_t value[MAX];
   int count = 0;
+  bool full = false;                                           // an entry found no room
   void add(void *q, size_t bytes, uint32_t v) {                // whole words
+    if (count == MAX) {
+      full = true;
+      return;
+    }
     p[count] = (uint32_t *)q;
     n[count] = bytes / 4;
     value[count++] = v;

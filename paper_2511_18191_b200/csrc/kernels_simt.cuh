@@ -31,20 +31,15 @@ struct PassGeom {
   int tpp = 1;                   // tokens per committed patch
   int head_step = 1;             // the head reads tokens head_step - 1, 2 head_step - 1, ... of the pass
 };
-__device__ __forceinline__ int pos0_of(const PassGeom &g, int b) {
-  return (g.done ? g.done[b] * g.tpp : 0) + g.base;
-}
-__device__ __forceinline__ bool slot_dead(const PassGeom &g, int slot) { return g.n_live && slot >= *g.n_live; }
-__device__ __forceinline__ int series_of(const PassGeom &g, int slot) { return g.live ? g.live[slot] : slot; }
 // Series, first token position and liveness of a slot in one go.  The live count and the slot's series
 // are two independent loads (issued together); the committed count follows the series index.  The
 // loads are volatile (served by L2) because most kernels do this lookup BEFORE their dependency wait,
 // to take its two L2 round trips off the chain of dependent launches: `live` / `n_live` are written
 // only by accept_kernel and the instance-norm kernel, and so is `done`, and every
-// kernel of a pass except the embedding that opens a round has at least two kernels between itself
-// and those -- a grid starts only after every CTA of its predecessor has passed its own dependency
-// wait, i.e. after the predecessor's predecessor has finished.  A dead slot's entry of `live` is a
-// stale but valid series index, so the lookup stays in bounds.
+// kernel of a pass except the embedding that opens a round has at least one kernel between itself
+// and those (the pass's second kernel: that embedding) -- and one is enough: a grid starts only after every CTA of
+// its predecessor has passed its own dependency wait, i.e. after the predecessor's predecessor has finished.  A dead
+// slot's entry of `live` is a stale but valid series index, so the lookup stays in bounds.
 struct SlotPos {
   int b, p0;
   bool dead;

@@ -3,6 +3,7 @@
 // by warp ballot, the correction / bonus patch, the new committed count (= the ragged KV
 // rollback length) and the round's counters, and with the last series the end of the round: one launch per round.
 #pragma once
+#include <type_traits>
 #include "common.cuh"
 
 namespace tsfm {
@@ -96,23 +97,36 @@ struct CallState {
 // clocks, advances the round counter, adds the round's launches to the device-side launch counter and, inside a captured
 // graph, tells the WHILE node whether another round is needed.
 __device__ __forceinline__ void close_round(const AcceptArgs &a) {
-  __shared__ int warp_count[8];
+  constexpr int U = 4;                                         // series a lane has in flight (8: 60 registers, a CTA less on an SM at K = 4)
+  __shared__ int warp_count[2][8];                             // (in turn: one barrier a step)
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  int base = 0;
-  for (int b0 = 0; b0 < a.B; b0 += blockDim.x) {               // ordered compaction, a block of series at a time
-    const int b = b0 + threadIdx.x;
-    const bool alive = b < a.B && __ldcg(a.done + b) < a.T;
-    const unsigned m = __ballot_sync(0xffffffffu, alive);
-    __syncthreads();
-    if (lane == 0) warp_count[w] = __popc(m);
+  int base = 0, turn = 0;
+  // ordered compaction: a warp takes n x 32 neighbouring series, the block nw times that at a time
+  auto step = [&](int b0, auto series) {
+    constexpr int n = decltype(series)::value;
+    const int first = b0 + w * n * 32 + lane;
+    int done[n], count = 0;
+    unsigned m[n];
+#pragma unroll
+    for (int u = 0; u < n; ++u) done[u] = first + 32 * u < a.B ? __ldcg(a.done + first + 32 * u) : a.T;
+#pragma unroll
+    for (int u = 0; u < n; ++u) count += __popc(m[u] = __ballot_sync(0xffffffffu, done[u] < a.T));
+    if (lane == 0) warp_count[turn][w] = count;
     __syncthreads();
     int off = base;
     for (int i = 0; i < nw; ++i) {
-      if (i < w) off += warp_count[i];
-      base += warp_count[i];
+      if (i < w) off += warp_count[turn][i];
+      base += warp_count[turn][i];
     }
-    if (alive) a.live[off + __popc(m & ((1u << lane) - 1u))] = b;
-  }
+    turn ^= 1;
+#pragma unroll
+    for (int u = 0; u < n; ++u) {
+      if (done[u] < a.T) a.live[off + __popc(m[u] & ((1u << lane) - 1u))] = first + 32 * u;
+      off += __popc(m[u]);
+    }
+  };
+  if (a.B <= blockDim.x) step(0, std::integral_constant<int, 1>{});
+  else for (int b0 = 0; b0 < a.B; b0 += U * blockDim.x) step(b0, std::integral_constant<int, U>{});
   if (threadIdx.x != 0) return;
   DevState *st = a.st;
   const int r = st->round;
@@ -131,19 +145,22 @@ __device__ __forceinline__ void close_round(const AcceptArgs &a) {
   if (a.use_handle) cudaGraphSetConditional(a.handle, (base > 0 && r + 1 < a.T) ? 1u : 0u);
 }
 
-// One CTA per series, a warp per position (in turn; the last one has the bonus patch, which is only kept).  Everything but the
+// A few warps per series, one per position in turn (the last position has the bonus patch, which is only kept).  Everything but the
 // verification pass's means was written several kernels ago and is fetched before the dependency wait: the call's state, the
 // committed count, the proposals.  The rows of mu_p stay in shared memory for the commit where they fit.  Bound: the chain
 // of round trips.  With one warp per series, that went through its positions one after the other behind the wait, and the end of
 // the round as a launch of its own, a round's two links took 10 us at K = 3 and 4, 9 of them for a single series.
-// block = 32 min(K + 1, 8), grid = B, dynamic shared memory: stage_rows rows of P floats ((K + 1), or 0: not kept).
+// block = 32 S nw: S series of nw warps each (see launch_accept), grid = ceil(B / S), dynamic shared memory: stage_rows rows of P
+// floats a series ((K + 1), or 0: not kept).
 constexpr int ACCEPT_WARPS = 8, ACCEPT_E = 4;                  // elements of a row that a lane has in flight
 constexpr int ACCEPT_STAGE_BYTES = 40 * 1024;
-__global__ void __launch_bounds__(32 * ACCEPT_WARPS) accept_kernel(AcceptArgs a, int stage_rows) {
+__global__ void __launch_bounds__(32 * ACCEPT_WARPS) accept_kernel(AcceptArgs a, int nw, int stage_rows) {
   extern __shared__ float accept_rows[];
-  __shared__ float pos_ep[32], pos_eq[32];                     // energies of every position
+  __shared__ float all_ep[ACCEPT_WARPS * 32], all_eq[ACCEPT_WARPS * 32];   // energies of every position of the CTA's series
   __shared__ int last;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5, b = blockIdx.x;
+  const int lane = threadIdx.x & 31, s = (threadIdx.x >> 5) / nw, w = (threadIdx.x >> 5) - s * nw, S = (blockDim.x >> 5) / nw;
+  const int b = blockIdx.x * S + s;
+  float *const pos_ep = all_ep + s * 32, *const pos_eq = all_eq + s * 32;
   const int K = a.K, P = a.P;
   int flags = 0;
   float fallback_r = 0.f;
@@ -160,14 +177,15 @@ __global__ void __launch_bounds__(32 * ACCEPT_WARPS) accept_kernel(AcceptArgs a,
     if (a.ell) a.ell += (size_t)r * a.B * a.K;
     if (a.log_u) a.log_u += (size_t)r * a.B * a.K;
   }
-  const int m = *reinterpret_cast<const volatile int *>(a.done + b);
-  const bool finished = m >= a.T;                              // earlier: nothing to decide
+  const int m = b < a.B ? *reinterpret_cast<const volatile int *>(a.done + b) : a.T;
+  const bool finished = m >= a.T;                              // earlier (or no series): nothing to decide
   const long long hist_adv = a.commit_follows_done && !finished ? (long long)m * P : 0;
   const float *xb = a.x + b * a.x_stride_b + hist_adv;
   const bool apart = a.mu_q_alt && (flags & VAR_SAMPLE_PROPOSALS);
   const float *qb = apart ? a.mu_q_alt + (size_t)b * a.K * a.P : a.mu_q + b * a.x_stride_b + hist_adv;
   const bool same = qb == xb;                                  // proposals that are the draft's means
   const float *pb = a.mu_p + (size_t)b * (K + 1) * P;
+  float *const rows = accept_rows + s * stage_rows * P;
   float x0[ACCEPT_E], q0[ACCEPT_E];                            // the start of this warp's first row
 #pragma unroll
   for (int e = 0; e < ACCEPT_E; ++e) {
@@ -203,14 +221,14 @@ __global__ void __launch_bounds__(32 * ACCEPT_WARPS) accept_kernel(AcceptArgs a,
           const float dp = xv[e] - pv[e], dq = xv[e] - qv[e];
           ep = fmaf(dp, dp, ep);
           eq = fmaf(dq, dq, eq);
-          if (i < stage_rows && c < P) accept_rows[i * P + c] = pv[e];
+          if (i < stage_rows && c < P) rows[i * P + c] = pv[e];
         }
       }
       ep = warp_sum(ep) / (float)P;
       eq = warp_sum(eq) / (float)P;
       if (lane == 0 && i < K) pos_ep[i] = ep, pos_eq[i] = eq;
     }
-    __syncthreads();
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + s), "r"(32 * nw) : "memory");
     if (w == 0) {
       // Eq. 5 and the log-domain test  log u <= min(l, 0)
       bool ok = true;
@@ -233,7 +251,7 @@ __global__ void __launch_bounds__(32 * ACCEPT_WARPS) accept_kernel(AcceptArgs a,
       if (a.commit_accepted)
         for (int c = lane; c < n * P; c += 32) cb[c] = xb[c];
       for (int c = lane; c < P; c += 32) {
-        float t = n < stage_rows ? accept_rows[n * P + c] : __ldcg(pb + (size_t)n * P + c);
+        float t = n < stage_rows ? rows[n * P + c] : __ldcg(pb + (size_t)n * P + c);
         if (fallback_r != 0.f)                          // t = mu_p + r eps (Algorithm 1, correction and bonus)
           t += fallback_r * standard_normal(a.key, (uint32_t)(a.series0 + b), (uint32_t)a.round_idx, (uint32_t)n, NOISE_FALLBACK, c);
         cb[(size_t)n * P + c] = t;
@@ -261,10 +279,11 @@ __global__ void __launch_bounds__(32 * ACCEPT_WARPS) accept_kernel(AcceptArgs a,
         if (a.n_accept) a.n_accept[b] = n;
       }
     }
-  } else if (threadIdx.x == 0 && a.n_accept) {
+  } else if (w == 0 && lane == 0 && b < a.B && a.n_accept) {
     a.n_accept[b] = -1;
   }
   if (!a.st) return;
+  if (S > 1) __syncthreads();                                  // the other series' counts
   if (threadIdx.x == 0) {
     __threadfence();                                           // done[b], the time stamp: before the ticket
     last = atomicAdd(a.ticket, 1) == (int)gridDim.x - 1;

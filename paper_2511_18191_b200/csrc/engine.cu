@@ -544,10 +544,21 @@ bool f32_many(int M, int N, int K) {
 }
 bool f32_takes(const tsfm_spec *h, const void *W, int M, int N, int K) { return f32_tiles(h, W, K) && !f32_many(M, N, K); }
 
+// One series a CTA, a warp per position (eight at most), while that leaves the machine few CTAs; of more series as many share a
+// CTA of four or eight warps as keep all of them resident at once (32 warps on an SM), which also has the threads to
+// list the unfinished ones.  us a round's link, a CTA of K + 1 warps per series -> here: 3000 series, K = 7 84 -> 21, 1000 26 -> 11,
+// 500 (K = 8) 17 -> 13.5; 4000, K = 3 83 -> 20; 2000, K = 2 27 -> 13; 1000, K = 4 13 -> 10; at 256 series alone / shared K = 1 6.9 / 7.0, K = 4
+// 6.8 / 7.5, at 300, K = 20 11 / 14.
+constexpr int kAcceptAloneMaxSeries = 300;
 void launch_accept(cudaStream_t s, bool pdl, const AcceptArgs &a) {
-  const size_t rows = (size_t)(a.K + 1) * a.P * sizeof(float);
+  int nw = std::min(a.K + 1, ACCEPT_WARPS), S = 1;
+  if (a.B > kAcceptAloneMaxSeries) {
+    for (nw = 4; nw > 1 && (nw > a.K + 1 || (long)a.B * nw > 32 * 148); nw /= 2) {}
+    S = ACCEPT_WARPS / nw;
+  }
+  const size_t rows = (size_t)S * (a.K + 1) * a.P * sizeof(float);
   const bool keep = rows <= ACCEPT_STAGE_BYTES;
-  launch_ex(s, pdl, accept_kernel, dim3(a.B), dim3(32 * std::min(a.K + 1, ACCEPT_WARPS)), keep ? rows : 0, a, keep ? a.K + 1 : 0);
+  launch_ex(s, pdl, accept_kernel, dim3((a.B + S - 1) / S), dim3(32 * S * nw), keep ? rows : 0, a, nw, keep ? a.K + 1 : 0);
 }
 
 // C (op)= A . W^T through the tensor-core kernel when a plan exists, else an FMA kernel.  row_gain (fp32

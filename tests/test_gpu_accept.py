@@ -74,6 +74,12 @@ def test_accept_at_the_edges_of_its_rows_and_warps(B, K, P):
     test_accept_matches_oracle(B, K, P)
 
 
+@pytest.mark.parametrize("B,K,P", [(301, 4, 33), (303, 1, 16), (1190, 2, 40), (4737, 3, 8), (301, 32, 40)])
+def test_accept_of_several_series_per_cta(B, K, P):
+    """Four, two and one warp per series, a last CTA that is not full, boundary rows kept in shared memory or not."""
+    test_accept_matches_oracle(B, K, P)
+
+
 def test_figure1_example_with_scripted_uniforms():
     g = dict(l.split(None, 1) for l in open(os.path.join(os.path.dirname(__file__), "golden", "figure1_round.txt")) if l[0] != "#")
     K, P = int(g["K"]), 96

@@ -160,6 +160,35 @@ def test_compaction_of_finished_series_changes_nothing(name):
         assert res[0][2] == other[2]
 
 
+@pytest.mark.parametrize("B,K", [(300, 7), (1100, 1), (3000, 7), (5000, 3)])
+def test_rounds_of_many_series(B, K, tmp_path):
+    """The list of unfinished series beyond what one step takes, and the acceptance step's warps all resident at once: with compaction
+    and without it the same bits."""
+    import json
+    import paper_2511_18191_b200 as tsfm
+    wl = workload("C0", batch=B, series_recipe="c1", ctx_len=64, patch_len=16, horizon=16 * 7, K=K, target=Arch(1, 64, 1, 64), draft=Arch(1, 64, 2, 64))
+    s, ctx = series_on_device(wl)
+    res = []
+    for mode in (tsfm.TSFM_EXEC_STREAM, tsfm.TSFM_EXEC_STREAM | tsfm.TSFM_EXEC_NO_COMPACT, tsfm.TSFM_EXEC_GRAPH):
+        dec = make_decoder(wl, max_K=K, exec_mode=mode)[0]
+        with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
+            out, st = dec.forecast(ctx, wl.horizon, K, 1.5, 5)
+        res.append((out.cpu().numpy(), dec.last_trace(B, K)[0]))
+        check_stats(st, B, 7, K)
+        dec.close()
+        if len(res) == 1:
+            prof.export_chrome_trace(str(tmp_path / "t.json"))
+            ev = [e["args"] for e in json.loads((tmp_path / "t.json").read_text())["traceEvents"]
+                  if e.get("cat") == "kernel" and "accept_kernel" in e["name"]]
+            # 32 warps on an SM, or one per series; whole CTAs of eight
+            assert all(np.prod(a["grid"]) * np.prod(a["block"]) < 32 * (max(32 * 148, B) + 8) for a in ev)
+    finished_at = (res[0][1] >= 0).sum(axis=0)
+    assert finished_at.min() < finished_at.max(), "the case must desynchronise the batch"
+    for other in res[1:]:
+        np.testing.assert_array_equal(res[0][0], other[0])
+        np.testing.assert_array_equal(res[0][1], other[1])
+
+
 BOUNDS_CASES = {
     "fp32-ragged": lambda: (workload("C0", batch=6, series_recipe="c1", horizon=96 * 7 + 5), 4, 4.0),
     "bf16-small-M": lambda: (workload("C1", batch=12, horizon=96 * 10), 4, 2.0),

@@ -55,13 +55,14 @@ constexpr int kMaxGraphs = 16;                // captured forecast geometries ke
 inline size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 inline size_t elt_bytes(int dtype) { return dtype == TSFM_BF16 ? 2 : 4; }
 
+constexpr int kMaxPatch = 256;             // steps per patch
 bool arch_ok(const tsfm_arch &a, int P) {
   if (a.n_layers < 1 || a.d_model < 64 || a.n_heads < 1 || a.d_ff < 64) return false;
   if (a.d_model % a.n_heads) return false;
   const int dh = a.d_model / a.n_heads;
   if (dh != 32 && dh != 64 && dh != 128) return false;
   if (a.d_model % 64 || a.d_ff % 64) return false;
-  if (P < 16 || P > 256 || P % 16) return false;
+  if (P < 16 || P > kMaxPatch || P % 16) return false;
   return true;
 }
 // Input token length P_in (0 = P): it divides the patch length P (a patch is P / P_in tokens).
@@ -738,11 +739,23 @@ void launch_attn(tsfm_spec *h, ModelDev &m, int l, int B, const PassGeom &g, boo
   }
 }
 
-// Shared memory of an embedding of four rows a CTA, which passes of at least kEmbedFourRows rows take (see embed_kernel) where it
-// fits without opting in (tokens of up to 168 values).
-constexpr int kEmbedFourRows = 32;
+// Shared memory of an embedding of four rows a CTA (see embed_kernel); 137 KB for tokens of 256 fp32 values.
 template <typename T> constexpr size_t embed_smem(int P) {
   return 4 * P * sizeof(float) + (P % Vec16<T>::N ? 0 : 128 * (P * sizeof(T) + 16));
+}
+template <typename T> int embed_set_attr() {                   // (the largest: handles of every token length share the kernel)
+  CU_TRY(cudaFuncSetAttribute(embed_kernel<T, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)embed_smem<T>(kMaxPatch)));
+  return TSFM_OK;
+}
+// Which passes it takes, M rows to d values from tokens of P: from 32 rows on where a row is wide (d >= 512, or 256 with tokens of 64
+// values and more), elsewhere where a CTA a row would load much (rows x 128 features x P) or be many.  us a step of plain decoding
+// with one layer, one row a CTA / four, bf16: d = 64, 64 x 96 18.0 / 19.4, 256 x 96 19.1 / 20.0, 512 x 96 22.4 / 22.0; d = 128, 100 x 96
+// 18.3 / 19.2, 400 x 96 23.7 / 22.9; d = 256, 100 x 32 18.2 / 18.8, 512 x 32 27.4 / 27.8, 64 x 64 18.9 / 18.4, 400 x 64 28.6 / 26.4; d = 512, 100 x
+// 16 22.6 / 23.2, 100 x 32 23.2 / 23.8, 64 x 64 22.7 / 21.7, 400 x 96 44.5 / 39.6; d = 1024, 32 x 96 29.7 / 27.8, 400 x 96 69.7 / 56.8; tokens
+// of 176 and 256: d = 128, 64 x 176 20.3 / 20.9, 256 x 176 25.1 / 22.5, d = 512, 100 x 256 40.5 / 31.9, d = 1024, 400 x 256 122 / 72.
+bool embed_four(int M, int P, int d) {
+  if (M < 32) return false;
+  return d >= 512 || (d >= 256 && P >= 64) || (long)M * ((d + 127) / 128) * std::max(P, 25) >= 25000;
 }
 
 enum { HEAD_NONE = 0, HEAD_LAST_TO_HIST = 1, HEAD_ALL_TO_VOUT = 2 };
@@ -795,7 +808,7 @@ void run_pass(tsfm_spec *h, ModelDev &m, int B, const PassGeom &g, int head_mode
   // the RMSNorm of passes of a few thousand rows is a link in a chain: constants before the wait
   auto *norm_kernel = d > 1280 ? rmsnorm_kernel<T, false, 16> : M <= kNormEarlyMaxRows ? rmsnorm_kernel<T, true, 10> : rmsnorm_kernel<T, false, 10>;
   {
-    const bool four = M >= kEmbedFourRows && embed_smem<T>(Pi) <= 48 * 1024;
+    const bool four = embed_four(M, Pi, d);
     KTimer kt(h, KC_EMBED, (double)M * Pi * 4 + (double)d * Pi * sizeof(T) + (double)M * d * 4, 2.0 * M * Pi * d);
     if (!fold && (sizeof(T) == 4 ? f32_tiles(h, m.W_emb, Pi) : rows_tiles(h, m.W_emb, d, Pi))) {
       RowsArgs ra{};
@@ -1366,6 +1379,7 @@ int tsfm_spec_create(const tsfm_weights *target_w, const tsfm_weights *draft_w, 
       return fail(TSFM_ERR_CUDA);
   }
   prefer_max_smem_all();
+  if ((rc = cfg->dtype == TSFM_F32 ? embed_set_attr<float>() : embed_set_attr<bf16>())) return fail(rc);
   if ((rc = cfg->dtype == TSFM_F32 ? gemm_f32_init() : gemm_rows_init())) return fail(rc);
   if (h->use_tc) {
     if ((rc = gemm_sk_init())) return fail(rc);

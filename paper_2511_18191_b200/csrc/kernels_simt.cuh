@@ -224,8 +224,9 @@ __device__ __forceinline__ void cp_async16(void *smem_dst, const void *gmem_src)
 // for short tokens (point tokens: P = 1).
 // R = 1, few rows: a thread reads its own weight row before the dependency wait.  Neighbouring threads read rows 2 P bytes
 // apart, 32 lines an instruction: 1500 cycles of an SM's load path a CTA, which many rows pay over and over.
-// R = 4, from 32 rows on: the CTA's 128 weight rows are one piece of memory and come to shared memory as such (rows 16 bytes
-// apart, so that eight threads' vectors fall into different banks), once for four rows.  The same order of sums, the same bits.
+// R = 4, more rows (embed_four): the CTA's 128 weight rows are one piece of memory and come to shared memory as such (rows 16 bytes
+// apart, so that eight threads' vectors fall into different banks), once for four rows; weight rows of one or two vectors go straight
+// into registers (8000 rows of 8 bf16 values, d = 512, with one layer, norm and head: 225 -> 171 us).  The same order of sums, the same bits.
 // Bound: a round trip each for weights and tokens and the chain of P products.  us a link inside plain decoding, R = 1 -> 4:
 // 256 rows x 1024 x 96 11.9 -> 5.8, 500 x 768 x 96 16.8 -> 7.6, 256 x 512 x 64 5.4 -> 3.7, 256 x 1280 x 32 6.2 -> 3.7; 64 x 512 x 64
 // 2.1 -> 2.7, but the kernel behind finds more room: a forecast of eight patches 396 -> 380 (32 x 1024 x 96 466 -> 447, 93 x 1024 x 96
@@ -238,14 +239,14 @@ embed_kernel(const float *hist, PassGeom g, int M, int P, int d, const T *__rest
              const float *__restrict__ gain, T *__restrict__ a_out, float *__restrict__ ssq_out, int opens_round) {
   extern __shared__ __align__(16) float zs[];                  // [R][P]; R > 1: and 128 weight rows, 16 bytes apart
   __shared__ long long src[R];                                 // (R > 1) a row's token in the history, -1: no such row
-  constexpr int V = Vec16<T>::N, PRE = 12;                     // (R == 1) weight vectors fetched before the wait
+  constexpr int V = Vec16<T>::N, PRE = R == 1 ? 12 : 2;        // weight vectors fetched before the wait
   const int row0 = blockIdx.x * R, f = blockIdx.y * 128 + threadIdx.x;
   // Before the dependency wait: what does not depend on the preceding kernel -- this thread's weight row (or its
   // start), its gain, and (unless this pass opens a round, when the kernel that closed the previous round is the
   // predecessor itself) the slot lookup.
   const T *wr = W + (size_t)min(f, d - 1) * P;
-  const bool staged = R > 1 && P % V == 0;
-  typename Vec16<T>::Raw wpre[R == 1 ? PRE : 1];
+  const bool staged = R > 1 && P % V == 0 && P > PRE * V;
+  typename Vec16<T>::Raw wpre[PRE];
   unsigned char *const ws = reinterpret_cast<unsigned char *>(zs + R * P);
   const int wrow = P * (int)sizeof(T) + 16;
   if (staged) {
@@ -257,10 +258,10 @@ embed_kernel(const float *hist, PassGeom g, int M, int P, int d, const T *__rest
       r += dr, c += dc;
       if (c >= vpr) c -= vpr, ++r;
     }
-  } else if (R == 1 && P % V == 0) {
+  } else if (P % V == 0) {
 #pragma unroll
     for (int k = 0; k < PRE; ++k)
-      if (k * V < P) wpre[R == 1 ? k : 0] = Vec16<T>::raw(wr + k * V);
+      if (k * V < P) wpre[k] = Vec16<T>::raw(wr + k * V);
   }
   const float gf = a_out ? gain[min(f, d - 1)] : 0.f;
   auto token_of = [&](int row) -> long long {
@@ -322,7 +323,7 @@ embed_kernel(const float *hist, PassGeom g, int M, int P, int d, const T *__rest
     for (int k = 0; k < PRE; ++k)
       if (k * V < P) {
         float w[V];
-        Vec16<T>::unpack(wpre[R == 1 ? k : 0], w);
+        Vec16<T>::unpack(wpre[k], w);
         step(w, k * V);
       }
 #pragma unroll 4

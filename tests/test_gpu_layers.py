@@ -145,18 +145,7 @@ def test_mlp_of_a_layer_with_folded_norms_and_several_tiles_per_pair(f, B, n, ha
     assert relative(forward(w, arch, z), want[..., half * P:half * P + P]) < 1.5e-4
 
 
-@pytest.mark.parametrize("d,P,P_in,B,n", [
-    (64, 16, 16, 9, 60),              # 540 rows: rows of one block of k, 8 and 16 features a CTA
-    (192, 48, 48, 5, 103),            # half a block of k, a ragged tile of rows
-    (128, 80, 80, 3, 43),             # 129 rows: embedding row by row, head tiled
-    (1280, 32, 32, 64, 9),            # five chunks of a row
-    (320, 256, 16, 2, 320),           # a chunk and a quarter; 192 + 64 features
-    (832, 96, 96, 200, 27),           # 5400 rows: 96 and 192 features a CTA
-])
-def test_embedding_and_head_are_exact_to_fp32(d, P, P_in, B, n):
-    """Layers that add nothing between embedding, final norm and head of a bf16 model, whose rows are fp32.  The bound: sums of
-    up to 1280 products in blocks of 32, fp32 rounding (relative 2^-24 each) in embedding, square, factor and head: measured
-    1.0e-7 to 1.3e-7, and an operand that lost its last 8 bits shows as 2^-17 = 8e-6."""
+def embedding_and_head_error(d, P, P_in, B, n):
     arch = Arch(1, d, d // 64, 64)
     rng = np.random.default_rng(d + n)
     w = make_model(arch, P, 1, "bf16", patch_in=P_in)
@@ -170,18 +159,66 @@ def test_embedding_and_head_are_exact_to_fp32(d, P, P_in, B, n):
     got = dec.model_forward(0, torch.from_numpy(z).cuda()).cpu().numpy()
     dec.close()
     x = z.astype(np.float64) @ w["W_emb"].T.astype(np.float64)
-    assert relative(got, (w["g_f"] * x * rstd(x)) @ w["W_head"].T.astype(np.float64)) < 3e-7
+    return relative(got, (w["g_f"] * x * rstd(x)) @ w["W_head"].T.astype(np.float64))
+
+
+@pytest.mark.parametrize("d,P,P_in,B,n", [
+    (64, 16, 16, 9, 60),              # 540 rows: rows of one block of k, 8 and 16 features a CTA
+    (192, 48, 48, 5, 103),            # half a block of k, a ragged tile of rows
+    (128, 80, 80, 3, 43),             # 129 rows: embedding row by row, head tiled
+    (1280, 32, 32, 64, 9),            # five chunks of a row
+    (320, 256, 16, 2, 320),           # a chunk and a quarter; 192 + 64 features
+    (832, 96, 96, 200, 27),           # 5400 rows: 96 and 192 features a CTA
+])
+def test_embedding_and_head_are_exact_to_fp32(d, P, P_in, B, n):
+    """Layers that add nothing between embedding, final norm and head of a bf16 model, whose rows are fp32.  The bound: sums of
+    up to 1280 products in blocks of 32, fp32 rounding (relative 2^-24 each) in embedding, square, factor and head: measured
+    1.0e-7 to 1.3e-7, and an operand that lost its last 8 bits shows as 2^-17 = 8e-6."""
+    assert embedding_and_head_error(d, P, P_in, B, n) < 3e-7
 
 
 @pytest.mark.parametrize("d,P,P_in,B,n", [
     (128, 96, 96, 1, 31), (128, 96, 96, 2, 16),                  # row by row and four rows a block
-    (192, 32, 32, 3, 11), (64, 176, 176, 5, 7), (320, 160, 160, 67, 7),   # ragged rows and features; too long for shared memory
+    (192, 32, 32, 3, 11), (64, 176, 176, 5, 7), (320, 160, 160, 67, 7),   # ragged rows and features
     (128, 16, 1, 3, 37), (128, 16, 4, 25, 43),                   # tokens shorter than a vector, folded and not
 ])
 def test_embedding_of_few_rows(d, P, P_in, B, n):
     """The bound as above: here the embedding is one chain of up to 176 sums, whose roundings (0.42 x 2^-24 of a partial sum in the
     mean square) add up to sqrt(176 / 2) x 2.5e-8 = 2.4e-7, with the rest 2.6e-7."""
     test_embedding_and_head_are_exact_to_fp32(d, P, P_in, B, n)
+
+
+@pytest.mark.parametrize("d,P,P_in,B,n", [
+    (512, 176, 176, 3, 11), (320, 256, 256, 4, 40),              # more shared memory than a kernel has by itself
+    (640, 64, 8, 3, 23), (192, 48, 16, 35, 17), (64, 64, 8, 7, 81),   # one and two vectors in registers, folded and not
+])
+def test_embedding_of_four_rows(d, P, P_in, B, n):
+    """The chain's sqrt(P_in / 2) x 2.5e-8 (as above, 2.8e-7 for 256 values) and 1.1e-7 for the rest are the error to expect, its root
+    mean square over some thousand values; the bound is 1.3 times that."""
+    assert embedding_and_head_error(d, P, P_in, B, n) < 1.3 * math.hypot(math.sqrt(P_in / 2) * 2.5e-8, 1.1e-7)
+
+
+@pytest.mark.parametrize("dtype,simt,d,P,P_in,B,n,rows", [
+    ("f32", 1, 64, 96, 96, 11, 100, 4), ("f32", 1, 128, 256, 256, 11, 100, 4), ("bf16", 1, 256, 176, 176, 11, 100, 4),   # many rows
+    ("bf16", 0, 256, 256, 256, 4, 25, 4), ("bf16", 0, 512, 32, 32, 4, 8, 4), ("bf16", 0, 512, 32, 32, 1, 31, 1),
+    ("bf16", 0, 64, 96, 96, 4, 25, 1), ("bf16", 0, 128, 16, 16, 4, 80, 1),       # few rows of narrow models
+])
+def test_rows_that_share_an_embedding_cta(dtype, simt, d, P, P_in, B, n, rows, tmp_path):
+    import json
+    import paper_2511_18191_b200 as tsfm
+    arch = Arch(1, d, d // 32, 64)
+    w = make_model(arch, P, 1, dtype, patch_in=P_in)
+    dec = tsfm.SpecDecoder(w, None, arch, arch, P, dtype, "layer_skip", max_batch=B, max_ctx_tokens=n, max_horizon_patches=1, max_K=1,
+                           patch_in=P_in, gemm_backend=tsfm.TSFM_GEMM_SIMT if simt else tsfm.TSFM_GEMM_AUTO)
+    z = torch.zeros((B, n, P_in), device="cuda")
+    dec.model_forward(0, z)
+    with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
+        dec.model_forward(0, z)
+    dec.close()
+    prof.export_chrome_trace(str(tmp_path / "t.json"))
+    grids = [e["args"]["grid"] for e in json.loads((tmp_path / "t.json").read_text())["traceEvents"]
+             if e.get("cat") == "kernel" and "embed_kernel" in e["name"]]
+    assert not grids or grids == [[-(-B * n // rows), -(-d // 128), 1]]
 
 
 @pytest.mark.parametrize("d,f,P,P_in,B,n", [

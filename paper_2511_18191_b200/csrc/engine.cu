@@ -398,8 +398,10 @@ void prefer_max_smem_all() {
   prefer_max_smem_typed<bf16>();
   prefer_max_smem(gemm_f32_kernel<16, 16>);
   prefer_max_smem(gemm_f32_kernel<32, 32>);
-  prefer_max_smem(gemm_f32_reg_kernel<2>);
-  prefer_max_smem(gemm_f32_reg_kernel<4>);
+  prefer_max_smem(gemm_f32_reg_kernel<float, 2>);
+  prefer_max_smem(gemm_f32_reg_kernel<float, 4>);
+  prefer_max_smem(gemm_f32_reg_kernel<bf16, 2>);
+  prefer_max_smem(gemm_f32_reg_kernel<bf16, 4>);
   prefer_max_smem(gemm_rows_kernel<1>);
   prefer_max_smem(gemm_rows_kernel<3>);
   prefer_max_smem(instnorm_kernel);
@@ -522,7 +524,7 @@ inline bool pair_folds(int M, int d) { return d >= 512 ? (long)M * d <= 5l << 20
 // TSFM_GEMM_SIMT keeps to the plain kernels, which share no code with it.
 bool f32_tiles(const tsfm_spec *h, const void *W, int K) { return h->cfg.gemm_backend != TSFM_GEMM_SIMT && gemm_f32_eligible(W, K); }
 
-// Whether gemm_rows_kernel takes embedding or head of a bf16 model.
+// Whether embedding or head of a bf16 model is a contraction of tiles (gemm_rows_launch).
 bool rows_tiles(const tsfm_spec *h, const void *W, int N, int K) {
   return h->cfg.gemm_backend != TSFM_GEMM_SIMT && gemm_rows_eligible(W, N, K);
 }
@@ -759,10 +761,13 @@ bool embed_four(int M, int P, int d) {
 }
 
 enum { HEAD_NONE = 0, HEAD_LAST_TO_HIST = 1, HEAD_ALL_TO_VOUT = 2 };
-// From this many rows on the head is a tiled contraction (gemm_rows_kernel) on the bf16 path too; below it one CTA per row and
-// eight outputs, with constants fetched before the dependency wait, is shorter: 32 rows of 512 values 3.1 us (tiled 5.6), 93 of
-// 1024 7.9 (8.4), 160 of 512 9.4 (5.6), 64 of 1280 4.5 (10.3).
-constexpr int kHeadTileRows = 128;
+// Where the head of a bf16 model is a tiled contraction (gemm_rows_kernel or gemm_f32_reg_kernel): head_kernel's CTA per row and eight
+// outputs, with constants fetched before the dependency wait, is the shorter link until its CTAs (rows x P / 8) take the machine
+// several waves, and the tiled one is a chain through K (in registers up to K = 128).  us a link, head_kernel / tiled: d = 64, 128 rows to 16 1.9 / 2.4, 256 to 16 3.3 / 2.4, 190 to 32
+// 3.7 / 2.4, 64 to 64 2.3 / 2.4; d = 256, 256 to 16 2.5 / 4.2, 400 4.8 / 4.0, 190 to 32 3.9 / 4.1, 100 to 64 3.9 / 4.1, 128 4.5 / 4.2; d = 512, 256 to 32 5.2 / 5.7,
+// 400 7.3 / 6.8, 128 to 64 5.0 / 5.6, 128 to 96 7.2 / 5.6; d = 1024, 520 to 16 7.0 / 9.2, 1000 12.8 / 11.0, 400 to 32 9.4 / 11, 520 11.9 / 9.3, 190 to 64 8.7 / 8.9,
+// 93 to 96 7.9 / 8.4, 160 10.9 / 9.0; d = 1280, 64 to 32 4.5 / 10.3.
+bool head_tiled(int rows, int P, int d) { return (long)rows * P >= (d <= 64 ? 4096 : 5600 + 7 * d); }
 // Up to this many rows the separate RMSNorm kernel fetches its constants before the dependency wait.
 constexpr int kNormEarlyMaxRows = 2048;
 
@@ -872,7 +877,7 @@ void run_pass(tsfm_spec *h, ModelDev &m, int B, const PassGeom &g, int head_mode
   const double rows = head_mode == HEAD_LAST_TO_HIST ? B : Mb;
   KTimer kt(h, head_mode == HEAD_NONE ? -1 : KC_HEAD, rows * d * 4 + (double)P * d * sizeof(T) + rows * P * 4,
             2.0 * rows * P * d);
-  if (head_mode != HEAD_NONE && (sizeof(T) == 4 ? f32_tiles(h, m.W_head, d) : rows >= kHeadTileRows && rows_tiles(h, m.W_head, P, d))) {
+  if (head_mode != HEAD_NONE && (sizeof(T) == 4 ? f32_tiles(h, m.W_head, d) : head_tiled((int)rows, P, d) && rows_tiles(h, m.W_head, P, d))) {
     RowsArgs ra{};
     ra.mode = head_mode == HEAD_LAST_TO_HIST ? ROWS_HEAD_LAST : ROWS_HEAD_ALL;
     ra.epi = EPI_F32;

@@ -80,6 +80,11 @@ template <int MT, int FN> constexpr int f32_smem_bytes(int KC) {
 }
 
 __device__ __forceinline__ float4 f32_vec4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
+__device__ __forceinline__ float4 f32_vec4(const bf16 *p) {
+  const uint2 u = *reinterpret_cast<const uint2 *>(p);
+  return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xffff0000u), __uint_as_float(u.y << 16),
+                     __uint_as_float(u.y & 0xffff0000u));
+}
 
 template <int MT, int FN>
 __global__ void __launch_bounds__(256)
@@ -236,11 +241,11 @@ gemm_f32_kernel(const float *A, const float *__restrict__ W, float *C, int M, in
 // behind it in one round trip; no copy through shared memory and no barrier stands before the sum of the partial tiles.
 // Bound: one round trip to L2 and the sum of eight partial tiles.  Links of the fp32 models' forecasts, us, gemm_f32_kernel -> here:
 // K = 64 2.3 .. 2.9 -> 1.5 .. 2.1, K = 128 2.0 .. 3.6 -> 1.5 .. 2.8; a speculative forecast of one series 231 -> 207 us,
-// of 37 series of different lengths 707 -> 654.  Where it is taken: f32_in_registers.
+// of 37 series of different lengths 707 -> 654.  Where it is taken: f32_in_registers; embedding and head of bf16 models (T): rows_in_registers.
 // NV: vectors per warp, K <= 32 NV.  grid as above (z = 1), block = 256.
-template <int NV>
+template <typename T, int NV>
 __global__ void __launch_bounds__(256, NV <= 2 ? 3 : 2)
-gemm_f32_reg_kernel(const float *A, const float *__restrict__ W, float *C, int M, int N, int K, const RowsArgs ra) {
+gemm_f32_reg_kernel(const float *A, const T *__restrict__ W, float *C, int M, int N, int K, const RowsArgs ra) {
   __shared__ float red[8][256], row_ss[8][16];
   __shared__ long long src_off[16], dst_off[16];               // (modes other than ROWS_PLAIN)
   __shared__ int row_series[16];
@@ -258,7 +263,7 @@ gemm_f32_reg_kernel(const float *A, const float *__restrict__ W, float *C, int M
   for (int n = 0; n < NV; ++n) {
     const int k = (w + 8 * n) * 4;
 #pragma unroll
-    for (int j = 0; j < 2; ++j) b[n][j] = k < K && f0 + tf + 8 * j < N ? *reinterpret_cast<const float4 *>(W + (size_t)(f0 + tf + 8 * j) * K + k) : zero;
+    for (int j = 0; j < 2; ++j) b[n][j] = k < K && f0 + tf + 8 * j < N ? f32_vec4(W + (size_t)(f0 + tf + 8 * j) * K + k) : zero;
   }
   if (ra.gain) {
 #pragma unroll
@@ -375,8 +380,8 @@ static bool gemm_f32_launch(cudaStream_t st, bool pdl, const float *A, const flo
   cfg.numAttrs = pdl ? 1 : 0;
   if (small && f32_in_registers(ra.mode, M, N, K)) {
     cfg.dynamicSmemBytes = 0;
-    return (K <= 64 ? cudaLaunchKernelEx(&cfg, gemm_f32_reg_kernel<2>, A, W, C, M, N, K, ra)
-                    : cudaLaunchKernelEx(&cfg, gemm_f32_reg_kernel<4>, A, W, C, M, N, K, ra)) == cudaSuccess;
+    return (K <= 64 ? cudaLaunchKernelEx(&cfg, gemm_f32_reg_kernel<float, 2>, A, W, C, M, N, K, ra)
+                    : cudaLaunchKernelEx(&cfg, gemm_f32_reg_kernel<float, 4>, A, W, C, M, N, K, ra)) == cudaSuccess;
   }
   return (small ? cudaLaunchKernelEx(&cfg, gemm_f32_kernel<16, 16>, A, W, C, M, N, K, KC, ra)
                 : cudaLaunchKernelEx(&cfg, gemm_f32_kernel<32, 32>, A, W, C, M, N, K, KC, ra)) == cudaSuccess;

@@ -249,6 +249,15 @@ static bool gemm_rows_eligible(const void *W, int N, int K) {
   return K % 16 == 0 && K >= 16 && K <= 32768 && N % 16 == 0 && !((uintptr_t)W & 15);
 }
 
+// With K <= 128 and as many 16 x 16 tiles as the machine holds at once gemm_f32_reg_kernel is the shorter link: there is nothing to
+// overlap a row's three parts with.  us a link of plain decoding, here / there: heads from d = 64, 256 rows to 32 3.7 / 2.5, 512 to 64 4.0 /
+// 2.7, 1000 to 96 (378 tiles) 3.7 / 2.7, 512 to 256 (512) 4.6 / 6.6; from d = 128, 256 to 96 4.1 / 3.9, 1000 to 64 (252) 4.5 / 3.3, 1500 to 64
+// (376) 4.2 / 7.2; embedding, 520 rows of 16 to d = 64 3.2 / 1.5, of 64 to 128 (264) 3.5 / 2.7, of 32 to 128, 1000 rows (504) 3.5 / 4.1, of 96
+// to 128, 700 rows (352) 3.5 / 5.5.
+static bool rows_in_registers(int M, int N, int K) {
+  return K <= 128 && (long)((N + 15) / 16) * ((M + 15) / 16) <= (K <= 64 ? 3 : 2) * 148;
+}
+
 static bool gemm_rows_launch(cudaStream_t st, bool pdl, const float *A, const bf16 *W, float *C, int M, int N, int K, const RowsArgs &ra) {
   const RowsShape sh = gemm_rows_shape(M, N);
   const int nt = 8 * sh.NTW * sh.wn, row_tiles = (M - 1) / GR_ROWS + 1;
@@ -262,6 +271,12 @@ static bool gemm_rows_launch(cudaStream_t st, bool pdl, const float *A, const bf
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = pdl ? 1 : 0;
+  if (rows_in_registers(M, N, K)) {
+    cfg.gridDim = dim3((N + 15) / 16, (M + 15) / 16);
+    cfg.dynamicSmemBytes = 0;
+    return (K <= 64 ? cudaLaunchKernelEx(&cfg, gemm_f32_reg_kernel<bf16, 2>, A, W, C, M, N, K, ra)
+                    : cudaLaunchKernelEx(&cfg, gemm_f32_reg_kernel<bf16, 4>, A, W, C, M, N, K, ra)) == cudaSuccess;
+  }
   auto go = [&](auto kernel) { return cudaLaunchKernelEx(&cfg, kernel, A, W, C, M, N, K, sh.wn, ra) == cudaSuccess; };
   return sh.NTW == 3 ? go(gemm_rows_kernel<3>) : go(gemm_rows_kernel<1>);
 }

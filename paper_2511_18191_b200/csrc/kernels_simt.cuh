@@ -926,7 +926,7 @@ attn_kernel(const float *qkv, T *Kc, T *Vc,
 __device__ float head_normal(const DevState *st, int series, int k_pos, int e);   // accept.cuh
 
 template <typename T>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 1)   // (fp32: 74 registers otherwise, three CTAs on an SM)
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 0)   // (fp32: 74 registers otherwise, three CTAs on an SM)
 head_kernel(const float *x, const float *__restrict__ gain, const T *__restrict__ Wh, int d,
             int P, float eps, PassGeom g, int only_last, float *__restrict__ hist,
             float *__restrict__ vout, const DevState *st, float *__restrict__ muq, int k_pos, int K,

@@ -163,9 +163,9 @@ def embedding_and_head_error(d, P, P_in, B, n):
 
 
 @pytest.mark.parametrize("d,P,P_in,B,n", [
-    (64, 16, 16, 9, 60),              # 540 rows: rows of one block of k, 8 and 16 features a CTA
+    (64, 16, 16, 9, 60),              # 540 rows: operands in registers
     (192, 48, 48, 5, 103),            # half a block of k, a ragged tile of rows
-    (128, 80, 80, 3, 43),             # 129 rows: embedding row by row, head tiled
+    (128, 80, 80, 3, 43),             # 129 rows: embedding row by row, head tiled (in registers)
     (1280, 32, 32, 64, 9),            # five chunks of a row
     (320, 256, 16, 2, 320),           # a chunk and a quarter; 192 + 64 features
     (832, 96, 96, 200, 27),           # 5400 rows: 96 and 192 features a CTA
@@ -175,6 +175,19 @@ def test_embedding_and_head_are_exact_to_fp32(d, P, P_in, B, n):
     up to 1280 products in blocks of 32, fp32 rounding (relative 2^-24 each) in embedding, square, factor and head: measured
     1.0e-7 to 1.3e-7, and an operand that lost its last 8 bits shows as 2^-17 = 8e-6."""
     assert embedding_and_head_error(d, P, P_in, B, n) < 3e-7
+
+
+@pytest.mark.parametrize("d,P,P_in,B,n", [
+    (64, 256, 256, 9, 60), (192, 16, 16, 9, 60),   # 540 rows: tiles of 16 and 8 features
+    (192, 80, 80, 3, 43),                          # embedding row by row
+    (64, 16, 16, 60, 200),                         # rows of half a block of k
+    (64, 48, 48, 17, 104), (64, 48, 48, 17, 105),  # embeddings of 444 and 448 tiles of 16 x 16
+    (64, 96, 96, 25, 47), (64, 96, 96, 25, 48),    # heads of 444 and 450
+    (128, 112, 112, 37, 16), (128, 112, 112, 37, 17),   # embeddings of 296 and 320
+])
+def test_tiles_of_embedding_and_head(d, P, P_in, B, n):
+    """Both sides of the line between operands in registers and rows in three parts.  The bound as above."""
+    assert embedding_and_head_error(d, P, P_in, B, n) < 1.3 * math.hypot(math.sqrt(P_in / 2) * 2.5e-8, 1.1e-7)
 
 
 @pytest.mark.parametrize("d,P,P_in,B,n", [

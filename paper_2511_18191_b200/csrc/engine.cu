@@ -639,11 +639,13 @@ void gemm(tsfm_spec *h, GemmSkPlan *plan, const void *A, const void *W, void *C,
 // attention's share of scoring passes of 33 to 704 tokens, 8 to 3200 (series, head) pairs, 190 shapes: 1.1 % above the better
 // kernel on average, 17 of them more than 4 % (0.4 to 0.7 us at 8 and 32 pairs).  At 1280 pairs, us a launch, attn_tiles_kernel /
 // attn_mma_kernel: 33 tokens 13 / 27, 64 16 / 27, 96 31 / 29, 128 43 / 35, 144 60 / 68, 192 76 / 69, 256 112 / 75, 320 151 / 117; at
-// 256 pairs 64 tokens 5.4 / 7.0, 128 10.5 / 7.7, 192 13.8 / 15.5, 256 19.6 / 15.8, 704 100 / 65.  Windows of up to 100 tokens keep the
-// blocks of 64 queries whatever the grid (a test holds them there at 1280 pairs): 96 tokens 4.5 / 5.1 at 64 pairs, 18.5 / 19.4 at 800,
-// 31 / 29 at 1280, and only beyond that a loss worth the name (59 / 49 at 2048).
+// 256 pairs 64 tokens 5.4 / 7.0, 128 10.5 / 7.7, 192 13.8 / 15.5, 256 19.6 / 15.8, 704 100 / 65.  Behind cached keys (48 to 256 tokens
+// behind 240 to 1700, 8 to 1280 pairs, 144 shapes) it is 0.2 % above the better kernel on average, 4 shapes of 48 tokens behind 240
+// more than 4 %.  Windows of up to 100 tokens keep the blocks of 64 queries up to 1280 pairs, where a test holds 100 tokens (35 us
+// for 30 in the others; the rest of that range is within 8 %, 1024 pairs x 100 26 / 23); beyond, 2048 pairs x 80 tokens are 51 / 46, x 100
+// 64 / 51, 4096 x 100 125 / 95, x 65 96 / 87.
 bool attn_mma_pays(long pairs, int first, int q_len) {
-  if (first == 0 && q_len <= 100) return false;
+  if (first == 0 && q_len <= 100 && pairs <= 1280) return false;
   double tiles = 0, mma = 0;
   long n64 = 0, n128 = 0;
   for (int q = 0; q < q_len; q += 64, ++n64) {

@@ -339,7 +339,15 @@ def test_small_attention_grids_do_not_share_sms(heads, B, n, tmp_path):
 @pytest.mark.parametrize("B,n,mma", [(16, 33, False), (320, 64, False), (320, 100, False), (320, 160, False), (80, 192, False),
                                      (1, 256, True), (320, 256, True), (320, 380, True)])
 def test_blocks_of_128_queries_are_not_given_passes_that_leave_them_empty(B, n, mma, tmp_path):
-    """Windows of 33 to 200 tokens run faster in blocks of 64 queries, as long passes do in blocks of 128."""
+    """Blocks of 64 queries for windows of up to 100 tokens and up to 1280 pairs, and where a second block of 128 stays half empty;
+    blocks of 128 for long passes."""
+    (name, _, _), = attention_launches(4, B, n, tmp_path)
+    assert ("attn_mma_kernel" in name) == mma and ("attn_tiles_kernel" in name) != mma
+
+
+@pytest.mark.parametrize("B,n,mma", [(321, 100, True), (640, 80, True), (640, 48, False)])
+def test_windows_of_many_series_take_blocks_of_128_queries(B, n, mma, tmp_path):
+    """More than 1280 pairs: the waves of blocks decide for short windows too."""
     (name, _, _), = attention_launches(4, B, n, tmp_path)
     assert ("attn_mma_kernel" in name) == mma and ("attn_tiles_kernel" in name) != mma
 

@@ -480,7 +480,7 @@ def test_general_rule_variants_match_oracle(wl_name, name, kw):
 
 def test_sampled_proposals_with_many_series_bf16():
     """Sampled proposals and fallback noise at 1024 series (C3 shape, small models): the draft head
-    of such passes shares its weight loads between 8 series and adds the proposal noise itself."""
+    of such passes is a contraction of tiles and adds the proposal noise itself."""
     import paper_2511_18191_b200 as tsfm
     wl = workload("C3", draft_eps=1e-2, horizon=96 * 4, target=Arch(2, 256, 4, 512), draft=Arch(2, 256, 4, 512))
     K, tau, seed, ids = 3, 1.5, 23, [0, 511, 1023]
@@ -490,6 +490,28 @@ def test_sampled_proposals_with_many_series_bf16():
     out, st = dec.forecast(ctx, wl.horizon, K, tau, seed, variant=v)
     check_stats(st, wl.batch, wl.n_patches, K)
     nacc, ell, logu = dec.last_trace(wl.batch, K)
+    dec.close()
+    tm, dm = parity.oracle_models(wl, tw, dw)
+    var = orc.Variant(sigma_q=0.8, sample_proposals=True, fallback_noise=0.2, tempering=True)
+    parity.compare_forecast(wl, tm, dm, s, wl.horizon, K, tau, seed, out.cpu().numpy(), nacc, ids, variant=var)
+
+
+@pytest.mark.parametrize("dtype,draft,B", [
+    ("f32", Arch(1, 192, 6, 64), 5), ("f32", Arch(1, 64, 2, 64), 203), ("f32", Arch(1, 64, 2, 64), 1700),   # gemm_f32_kernel, both tiles
+    ("f32", Arch(1, 128, 2, 64), 61),                                                                        # gemm_f32_reg_kernel
+    ("bf16", Arch(1, 64, 1, 64), 203), ("bf16", Arch(1, 128, 2, 64), 203), ("bf16", Arch(1, 192, 3, 64), 203),   # ..., gemm_rows_kernel
+    ("bf16", Arch(1, 64, 1, 64), 9),                                                                         # head_kernel
+])
+def test_sampled_proposals_of_every_head(dtype, draft, B):
+    """Each kernel that a draft's head runs on adds the proposal noise and keeps the mean: one series in the middle and the last."""
+    import paper_2511_18191_b200 as tsfm
+    wl = workload("C0", batch=B, series_recipe="c1", ctx_len=96 * 3, horizon=96 * 4, dtype=dtype, target=Arch(1, 64, 1, 64), draft=draft)
+    K, tau, seed, ids = 3, 1.5, 23, [B // 2, B - 1]
+    dec, tw, dw = make_decoder(wl, batch=B, max_K=K)
+    s, ctx = series_on_device(wl, B)
+    out, st = dec.forecast(ctx, wl.horizon, K, tau, seed, variant=tsfm.tsfm_variant(0.8, 0.2, 1, 0))
+    check_stats(st, B, wl.n_patches, K)
+    nacc, ell, logu = dec.last_trace(B, K)
     dec.close()
     tm, dm = parity.oracle_models(wl, tw, dw)
     var = orc.Variant(sigma_q=0.8, sample_proposals=True, fallback_noise=0.2, tempering=True)

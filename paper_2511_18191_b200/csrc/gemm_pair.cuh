@@ -32,7 +32,10 @@
 // Scoring passes, us a contraction inside a pass, with shared staging and barriers -> here: M = 6000, d = 1024: QKV 41 -> 34.4, W1 43
 // -> 37.2, Wo 17.9 -> 17.9, W2 39 -> 39; M = 5120, d = 768: QKV (fp32) 23.5 -> 20.0, W1 26.5 -> 23.4, Wo 12.7 -> 12.4; M = 4096, d = 512:
 // 16.3 -> 16.1, 18.7 -> 14.7, 7.8 -> 7.0, W2 12.0 -> 11.5; M = 16320, d = 1280: QKV 150 -> 133, the rest within the scatter of the clock.
-// Graph replay of dependent launches, gemm_sk_kernel -> this one: M = 16320, d = 1280: QKV 158 -> 118 us
+// Plain fp32 outputs of several tiles a pair, staged in boxes of 8 KB -> of 1 KB here: 16384 x 3840 x 1280 123.0 -> 127.8 us, 10500 x 3072 x 1024
+// 55.0 -> 55.8, 6000 x 3072 x 1024 32.5 -> 31.9 (boxes of 2 KB 129 .. 140, 57 .. 60, 32 .. 33); of one tile a pair, staged / straight from
+// registers, behind W2: 576 x 3840 x 1280 11.5 / 11.8, 1280 x 3072 x 1024 12.2 / 12.7, 1000 x 2304 x 768 8.7 / 9.0.
+// Graph replay of dependent launches before the epilogue was per warp, gemm_sk_kernel -> here: M = 16320, d = 1280: QKV 158 -> 118 us
 // (1355 TFLOP/s), W1 with GELU 254 -> 160, W2 175 -> 149, Wo 67 -> 50; M = 6000, d = 1024: 47 -> 34, 74 -> 40,
 // 61 -> 44, 21 -> 16.
 // Warps 0-15 epilogue, 16 TMA producer, 17 tensor-memory allocation and MMA issue, 18-19 the rows' factors and

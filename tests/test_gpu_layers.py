@@ -211,29 +211,6 @@ def test_embedding_of_four_rows(d, P, P_in, B, n):
     assert embedding_and_head_error(d, P, P_in, B, n) < 1.3 * math.hypot(math.sqrt(P_in / 2) * 2.5e-8, 1.1e-7)
 
 
-@pytest.mark.parametrize("dtype,simt,d,P,P_in,B,n,rows", [
-    ("f32", 1, 64, 96, 96, 11, 100, 4), ("f32", 1, 128, 256, 256, 11, 100, 4), ("bf16", 1, 256, 176, 176, 11, 100, 4),   # many rows
-    ("bf16", 0, 256, 256, 256, 4, 25, 4), ("bf16", 0, 512, 32, 32, 4, 8, 4), ("bf16", 0, 512, 32, 32, 1, 31, 1),
-    ("bf16", 0, 64, 96, 96, 4, 25, 1), ("bf16", 0, 128, 16, 16, 4, 80, 1),       # few rows of narrow models
-])
-def test_rows_that_share_an_embedding_cta(dtype, simt, d, P, P_in, B, n, rows, tmp_path):
-    import json
-    import paper_2511_18191_b200 as tsfm
-    arch = Arch(1, d, d // 32, 64)
-    w = make_model(arch, P, 1, dtype, patch_in=P_in)
-    dec = tsfm.SpecDecoder(w, None, arch, arch, P, dtype, "layer_skip", max_batch=B, max_ctx_tokens=n, max_horizon_patches=1, max_K=1,
-                           patch_in=P_in, gemm_backend=tsfm.TSFM_GEMM_SIMT if simt else tsfm.TSFM_GEMM_AUTO)
-    z = torch.zeros((B, n, P_in), device="cuda")
-    dec.model_forward(0, z)
-    with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
-        dec.model_forward(0, z)
-    dec.close()
-    prof.export_chrome_trace(str(tmp_path / "t.json"))
-    grids = [e["args"]["grid"] for e in json.loads((tmp_path / "t.json").read_text())["traceEvents"]
-             if e.get("cat") == "kernel" and "embed_kernel" in e["name"]]
-    assert not grids or grids == [[-(-B * n // rows), -(-d // 128), 1]]
-
-
 @pytest.mark.parametrize("d,f,P,P_in,B,n", [
     (64, 64, 64, 64, 1, 1), (64, 64, 48, 48, 1, 17), (64, 64, 16, 16, 10, 16), (64, 64, 16, 16, 7, 23),   # up to 160 rows
     (64, 64, 32, 8, 5, 3),                                       # embedding by itself

@@ -326,11 +326,13 @@ embed_kernel(const float *hist, PassGeom g, int M, int P, int d, const T *__rest
         Vec16<T>::unpack(wpre[k], w);
         step(w, k * V);
       }
+    if constexpr (R == 1) {                                    // (R > 1: staged)
 #pragma unroll 4
-    for (int i = PRE * V; i < P; i += V) {
-      float w[V];
-      Vec16<T>::load(wr + i, w);
-      step(w, i);
+      for (int i = PRE * V; i < P; i += V) {
+        float w[V];
+        Vec16<T>::load(wr + i, w);
+        step(w, i);
+      }
     }
   } else {
     for (int i = 0; i < P; ++i) {

@@ -150,16 +150,18 @@ __device__ __forceinline__ void close_round(const AcceptArgs &a) {
 // committed count, the proposals.  The rows of mu_p stay in shared memory for the commit where they fit.  Bound: the chain
 // of round trips.  With one warp per series, that went through its positions one after the other behind the wait, and the end of
 // the round as a launch of its own, a round's two links took 10 us at K = 3 and 4, 9 of them for a single series.
-// block = 32 S nw: S series of nw warps each (see launch_accept), grid = ceil(B / S), dynamic shared memory: stage_rows rows of P
-// floats a series ((K + 1), or 0: not kept).
+// nw_log < 0: a series a CTA; otherwise eight warps, 2^nw_log of them a series (see launch_accept).  Dynamic shared memory: stage_rows rows
+// of P floats a series ((K + 1), or 0: not kept).
 constexpr int ACCEPT_WARPS = 8, ACCEPT_E = 4;                  // elements of a row that a lane has in flight
 constexpr int ACCEPT_STAGE_BYTES = 40 * 1024;
-__global__ void __launch_bounds__(32 * ACCEPT_WARPS) accept_kernel(AcceptArgs a, int nw, int stage_rows) {
+__global__ void __launch_bounds__(32 * ACCEPT_WARPS) accept_kernel(AcceptArgs a, int nw_log, int stage_rows) {
   extern __shared__ float accept_rows[];
   __shared__ float all_ep[ACCEPT_WARPS * 32], all_eq[ACCEPT_WARPS * 32];   // energies of every position of the CTA's series
   __shared__ int last;
-  const int lane = threadIdx.x & 31, s = (threadIdx.x >> 5) / nw, w = (threadIdx.x >> 5) - s * nw, S = (blockDim.x >> 5) / nw;
-  const int b = blockIdx.x * S + s;
+  const bool alone = nw_log < 0;                               // one series: all of the CTA's warps
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = alone ? blockDim.x >> 5 : 1 << nw_log;
+  const int s = alone ? 0 : warp >> nw_log, w = alone ? warp : warp & (nw - 1);
+  const int b = alone ? blockIdx.x : (blockIdx.x * (blockDim.x >> 5) + warp) >> nw_log;
   float *const pos_ep = all_ep + s * 32, *const pos_eq = all_eq + s * 32;
   const int K = a.K, P = a.P;
   int flags = 0;
@@ -283,7 +285,7 @@ __global__ void __launch_bounds__(32 * ACCEPT_WARPS) accept_kernel(AcceptArgs a,
     a.n_accept[b] = -1;
   }
   if (!a.st) return;
-  if (S > 1) __syncthreads();                                  // the other series' counts
+  if (!alone) __syncthreads();                                 // the other series' counts
   if (threadIdx.x == 0) {
     __threadfence();                                           // done[b], the time stamp: before the ticket
     last = atomicAdd(a.ticket, 1) == (int)gridDim.x - 1;

@@ -554,14 +554,15 @@ bool f32_takes(const tsfm_spec *h, const void *W, int M, int N, int K) { return 
 // 6.8 / 7.5, at 300, K = 20 11 / 14.
 constexpr int kAcceptAloneMaxSeries = 300;
 void launch_accept(cudaStream_t s, bool pdl, const AcceptArgs &a) {
-  int nw = std::min(a.K + 1, ACCEPT_WARPS), S = 1;
+  int warps = std::min(a.K + 1, ACCEPT_WARPS), S = 1, nw_log = -1;
   if (a.B > kAcceptAloneMaxSeries) {
-    for (nw = 4; nw > 1 && (nw > a.K + 1 || (long)a.B * nw > 32 * 148); nw /= 2) {}
-    S = ACCEPT_WARPS / nw;
+    warps = ACCEPT_WARPS;
+    for (nw_log = 2; nw_log > 0 && (1 << nw_log > a.K + 1 || (long)a.B << nw_log > 32 * 148); --nw_log) {}
+    S = ACCEPT_WARPS >> nw_log;
   }
   const size_t rows = (size_t)S * (a.K + 1) * a.P * sizeof(float);
   const bool keep = rows <= ACCEPT_STAGE_BYTES;
-  launch_ex(s, pdl, accept_kernel, dim3((a.B + S - 1) / S), dim3(32 * S * nw), keep ? rows : 0, a, nw, keep ? a.K + 1 : 0);
+  launch_ex(s, pdl, accept_kernel, dim3((a.B + S - 1) / S), dim3(32 * warps), keep ? rows : 0, a, nw_log, keep ? a.K + 1 : 0);
 }
 
 // C (op)= A . W^T through the tensor-core kernel when a plan exists, else an FMA kernel.  row_gain (fp32
